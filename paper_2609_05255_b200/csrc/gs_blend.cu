@@ -1,240 +1,377 @@
-// Per-tile alpha blending, forward and backward.  One CTA of 64 threads per 16x16 tile; every
-// thread owns a 2x2 pixel quad (a warp covers 16x8 pixels), so one shared-memory read of a
-// Gaussian serves four pixels and, in the backward, four pixels are summed in registers before
-// anything crosses lanes.  The tile's depth-ordered instance list is staged through shared memory
-// in batches of 128 Gaussians (64 in the backward, which also keeps the batch's gradient sums there).
+// Per-tile alpha blending, forward and backward.  Every warp works on its own (CTAs of one warp): it owns a region of a
+// tile, 8 x 8 pixels in the forward, 16 x 8, 8 x 8 or 4 x 8 in the backward, walks the tile's depth-ordered list 32
+// entries at a time with the next ones on their way, drops those that cannot reach its region, and composites the rest
+// without a branch or a vote per entry.
+//
+// What bounds both kernels is the register file, not the arithmetic pipes: a packed fp32 multiply-add with three
+// different register pairs takes three cycles of a scheduler, one with two pairs two, so the time goes with the operands
+// read.  Hence predicates instead of 0 / 1 factors in the forward and, in the backward, no shuffles or selects per entry:
+// what crosses lanes is parked in shared memory and summed later.
 #include "gs_device.cuh"
 
 namespace gs {
 namespace {
 
-constexpr int kThreads = 64;
-constexpr int kBatch = 128;
-constexpr int kBatchBwd = 64;   // the backward keeps ten accumulators per entry and warp in shared memory
 constexpr unsigned kFull = 0xffffffffu;
 constexpr float kLn2 = 0.6931471805599453f;
 
-// Top-left pixel of this thread's quad.
-__device__ __forceinline__ void quad_of(int tile, int gx, int tid, int &px, int &py) {
-  const int tx = tile % gx, ty = tile / gx;
-  const int warp = tid >> 5, lane = tid & 31;
-  px = tx * GS_TILE + 2 * (lane & 7);
-  py = ty * GS_TILE + warp * 8 + 2 * (lane >> 3);
-}
-
-// Stage one batch entry: (x, y, la, lb) (lc, o) (r, g, b, pmin).  (la, lb, lc) is the Cholesky factor
-// of the conic, scaled by sqrt(0.5 log2 e), so that exp(power) = 2^-((la dx + lb dy)^2 + (lc dy)^2):
-// a sum of two squares has no cancellation, which keeps alpha accurate to a few ulp even for
-// footprints hundreds of pixels wide (the expanded quadratic form loses 1e-4 there).
-__device__ __forceinline__ void stage_entry(uint32_t g, const float *mean2d, const float *conic_opacity,
-                                            const float *color, float4 &xyab, float2 &co, float4 &rgb) {
-  const float2 m = __ldg(reinterpret_cast<const float2 *>(mean2d) + g);
-  const float4 q = __ldg(reinterpret_cast<const float4 *>(conic_opacity) + g);
-  const float kS = 0.8493218002880191f;   // sqrt(0.5 * log2(e))
-  xyab = make_float4(m.x, m.y, kS * q.x, kS * q.y);   // q = (l11, l21, l22, opacity)
-  co = make_float2(kS * q.z, q.w);
-  // alpha >= 1/255 <=> log2 falloff >= pmin = -log2(255 o): the test is taken on the exponent, before the
-  // exponential, by the forward, the backward and the pair counter alike
-  rgb = make_float4(__ldg(color + 3 * (size_t)g), __ldg(color + 3 * (size_t)g + 1), __ldg(color + 3 * (size_t)g + 2),
-                    -__log2f(255.f * q.w));
-}
-
-// log2 of the Gaussian falloff at the four pixels of a quad; dx0, dy0 are the offsets of the
-// top-left pixel centre from the mean.  Index k = 2 * row + column.  One explicit operation order,
-// shared by the forward and the backward so that both take identical skip decisions.
-// t1[k] = la dx + lb dy is returned too: the backward needs it for the gradient of the mean.
-__device__ __forceinline__ void quad_power(float dx0, float dy0, float la, float lb, float lc, float p[4],
-                                           float t1[4], float t2[2]) {
-  // packed fp32 pairs (one instruction, two IEEE operations): the bits equal the scalar sequence
-  const float2 one = make_float2(1.f, 1.f);
-  const float2 d1 = __fadd2_rn(make_float2(dx0, dy0), one);            // (dx1, dy1)
-  const float2 a = __fmul2_rn(make_float2(la, la), make_float2(dx0, d1.x));
-  const float2 c = __fmul2_rn(make_float2(lc, lc), make_float2(dy0, d1.y));
-  const float2 s = __fmul2_rn(c, c);
-  const float2 lb2 = make_float2(lb, lb);
-  const float2 u = __ffma2_rn(lb2, make_float2(dy0, dy0), a), w = __ffma2_rn(lb2, make_float2(d1.y, d1.y), a);
-  const float2 pu = __ffma2_rn(u, u, make_float2(s.x, s.x)), pw = __ffma2_rn(w, w, make_float2(s.y, s.y));
-  t2[0] = c.x; t2[1] = c.y;
-  t1[0] = u.x; t1[1] = u.y; t1[2] = w.x; t1[3] = w.y;
-  p[0] = -pu.x; p[1] = -pu.y; p[2] = -pw.x; p[3] = -pw.y;
-}
-
-// alpha of one pixel from its log2 falloff p; false if the pair is skipped (alpha < 1/255, decided as
-// p < pmin).  raw = o * exp(power) before the clamp at 0.99.
-__device__ __forceinline__ bool alpha_of(float p, float o, float pmin, float &e2, float &raw, float &alpha) {
-  if (p < pmin) return false;
-  e2 = ex2_approx(p);             // p <= 0 by construction
-  raw = __fmul_rn(o, e2);
-  alpha = fminf(kAlphaMax, raw);
-  return true;
-}
-
-// 1.0f where a >= b or either is NaN, else 0.0f; 1.0f where a < b, else 0.0f: masks as numbers, so that what
-// depends on them runs as packed multiplies on the FMA pipe instead of selects on the ALU pipe.
-__device__ __forceinline__ float set_geu(float a, float b) {
-  float d;
-  asm("set.geu.f32.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
-  return d;
-}
-__device__ __forceinline__ float set_lt(float a, float b) {
-  float d;
-  asm("set.lt.f32.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
-  return d;
-}
-__device__ __forceinline__ float set_le(float a, float b) {
-  float d;
-  asm("set.le.f32.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
-  return d;
-}
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }   // a - b, exact products
-
-// Forward.  The four pixels of a quad travel as two packed pairs, (0, 1) and (2, 3), and the composite of an entry is
-// branch-free: "this pixel still composites" (live), "it accepts this entry" (q: alpha >= 1/255, decided on the
-// exponent) and "it stops here" (s: T - alpha T < 1e-4) are 0/1 numbers.  A pixel that skips the entry, has stopped
-// or stops here enters with weight exactly 0, which leaves its transmittance and colour sums unchanged bit for bit.
-__global__ void __launch_bounds__(kThreads) k_blend_fwd(CamDev cam, const uint32_t *__restrict__ ranges,
-                                                        const uint32_t *__restrict__ order,
-                                                        const uint32_t *__restrict__ vals,
-                                                        const float *__restrict__ mean2d,
-                                                        const float *__restrict__ conic_opacity,
-                                                        const float *__restrict__ color, uint32_t *__restrict__ sorted_tiles,
-                                                        float *__restrict__ image,
-                                                        float *__restrict__ final_T, uint32_t *__restrict__ n_contrib) {
-  dependency_wait();
-  __shared__ float4 s_xyab[kBatch];
-  __shared__ float2 s_co[kBatch];
-  __shared__ float4 s_rgb[kBatch];
-  const int tid = threadIdx.x, tile = (int)__ldg(order + blockIdx.x);
-  int px, py;
-  quad_of(tile, cam.gx, tid, px, py);
-  const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
-  const uint32_t start = __ldg(ranges + 2 * tile), end = __ldg(ranges + 2 * tile + 1);
-  // the key of every instance of this tile's stretch of the sorted list is the tile id: stores that nothing here waits for
-  if (sorted_tiles)
-    for (uint32_t p = start + tid; p < end; p += kThreads) sorted_tiles[p] = (uint32_t)tile;
-  const float in_x1 = px + 1 < cam.W ? 1.f : 0.f, in_y1 = py + 1 < cam.H ? 1.f : 0.f, in_0 = (px < cam.W && py < cam.H) ? 1.f : 0.f;
-  // T is the transmittance while the pixel composites and 0 once it has stopped (then every later weight alpha T is
-  // 0 by itself); the value it stopped with is kept in F.  Pixels outside the image start stopped.
-  float2 T01 = make_float2(in_0, in_0 * in_x1), T23 = make_float2(in_0 * in_y1, in_0 * in_x1 * in_y1);
-  const float2 zero = make_float2(0.f, 0.f), one = make_float2(1.f, 1.f);
-  float2 F01 = zero, F23 = zero;
-  float2 R01 = zero, R23 = zero, G01 = zero, G23 = zero, B01 = zero, B23 = zero;
-  uint32_t last[4] = {0u, 0u, 0u, 0u};      // position + 1 of the last composited entry
-  for (uint32_t base = start; base < end; base += kBatch) {
-    if (__syncthreads_and((T01.x + T01.y) + (T23.x + T23.y) == 0.f)) break;
-#pragma unroll
-    for (int h = 0; h < kBatch / kThreads; ++h) {
-      const int slot = tid + h * kThreads;
-      const uint32_t idx = base + slot;
-      if (idx < end) stage_entry(__ldg(vals + idx), mean2d, conic_opacity, color, s_xyab[slot], s_co[slot], s_rgb[slot]);
-    }
-    __syncthreads();
-    const int cnt = (int)min((uint32_t)kBatch, end - base);
-    float posf = 0.f;                         // position + 1 inside the batch, as a number (exact)
-    float2 last01 = zero, last23 = zero;      // the same of the last entry composited in this batch; 0 = none
-    for (int j0 = 0; j0 < cnt; j0 += 8) {
-      if (!__any_sync(kFull, (T01.x + T01.y) + (T23.x + T23.y) != 0.f)) break;   // every pixel of the warp has stopped
-      const int j1 = min(j0 + 8, cnt);
-#pragma unroll 2
-      for (int j = j0; j < j1; ++j) {
-        const float4 a = s_xyab[j];
-        const float2 c = s_co[j];
-        float p[4], t1[4], t2[2];
-        quad_power(fx - a.x, fy - a.y, a.z, a.w, c.x, p, t1, t2);
-        const float4 col = s_rgb[j];
-        posf += 1.f;
-        const float2 q01 = make_float2(set_geu(p[0], col.w), set_geu(p[1], col.w));
-        const float2 q23 = make_float2(set_geu(p[2], col.w), set_geu(p[3], col.w));
-        if (!__any_sync(kFull, (q01.x + q01.y) + (q23.x + q23.y) != 0.f)) continue;   // no pixel of the warp takes it
-        const float2 o2 = make_float2(c.y, c.y);
-        const float2 raw01 = __fmul2_rn(o2, make_float2(ex2_approx(p[0]), ex2_approx(p[1])));
-        const float2 raw23 = __fmul2_rn(o2, make_float2(ex2_approx(p[2]), ex2_approx(p[3])));
-        const float2 al01 = __fmul2_rn(q01, make_float2(fminf(kAlphaMax, raw01.x), fminf(kAlphaMax, raw01.y)));
-        const float2 al23 = __fmul2_rn(q23, make_float2(fminf(kAlphaMax, raw23.x), fminf(kAlphaMax, raw23.y)));
-        float2 w01 = __fmul2_rn(al01, T01), w23 = __fmul2_rn(al23, T23);
-        // transmittance behind this entry, T (1 - alpha) - in this form, because the backward recovers the
-        // transmittances by dividing (1 - alpha) out again and drifts if the forward rounds another expression (ten
-        // 2D-gradient values of a 1M-Gaussian view were then off by more than 1e-3 of the sum of their terms); below
-        // 1e-4 the pixel stops and the entry is not composited.
-        // A live pixel that skips the entry keeps T >= 1e-4 and cannot stop here; a stopped one has T = 0 and
-        // "stops" again with nothing to lose.
-        const float2 n01 = __fmul2_rn(T01, sub2(one, al01)), n23 = __fmul2_rn(T23, sub2(one, al23));
-        const float2 s01 = make_float2(set_lt(n01.x, kTmin), set_lt(n01.y, kTmin));
-        const float2 s23 = make_float2(set_lt(n23.x, kTmin), set_lt(n23.y, kTmin));
-        const float2 k01 = sub2(one, s01), k23 = sub2(one, s23);
-        F01 = __ffma2_rn(s01, T01, F01); F23 = __ffma2_rn(s23, T23, F23);
-        w01 = __fmul2_rn(w01, k01); w23 = __fmul2_rn(w23, k23);
-        T01 = __fmul2_rn(n01, k01); T23 = __fmul2_rn(n23, k23);
-        R01 = __ffma2_rn(make_float2(col.x, col.x), w01, R01); R23 = __ffma2_rn(make_float2(col.x, col.x), w23, R23);
-        G01 = __ffma2_rn(make_float2(col.y, col.y), w01, G01); G23 = __ffma2_rn(make_float2(col.y, col.y), w23, G23);
-        B01 = __ffma2_rn(make_float2(col.z, col.z), w01, B01); B23 = __ffma2_rn(make_float2(col.z, col.z), w23, B23);
-        // last += composited * (position - last)
-        const float2 pos2 = make_float2(posf, posf);
-        last01 = __ffma2_rn(__fmul2_rn(q01, k01), sub2(pos2, last01), last01);
-        last23 = __ffma2_rn(__fmul2_rn(q23, k23), sub2(pos2, last23), last23);
-      }
-    }
-    const uint32_t off = base - start;
-    if (last01.x != 0.f) last[0] = off + (uint32_t)last01.x;
-    if (last01.y != 0.f) last[1] = off + (uint32_t)last01.y;
-    if (last23.x != 0.f) last[2] = off + (uint32_t)last23.x;
-    if (last23.y != 0.f) last[3] = off + (uint32_t)last23.y;
-  }
-  T01 = __fadd2_rn(T01, F01); T23 = __fadd2_rn(T23, F23);    // one of the two is 0
-  const float T[4] = {T01.x, T01.y, T23.x, T23.y};
-  const float Cr[4] = {R01.x, R01.y, R23.x, R23.y}, Cg[4] = {G01.x, G01.y, G23.x, G23.y}, Cb[4] = {B01.x, B01.y, B23.x, B23.y};
-  const size_t plane = (size_t)cam.W * cam.H;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int x = px + (k & 1), y = py + (k >> 1);
-    if (x < cam.W && y < cam.H) {
-      const size_t pix = (size_t)y * cam.W + x;
-      image[pix] = fmaf(T[k], cam.bg[0], Cr[k]);
-      image[plane + pix] = fmaf(T[k], cam.bg[1], Cg[k]);
-      image[2 * plane + pix] = fmaf(T[k], cam.bg[2], Cb[k]);
-      final_T[pix] = T[k];
-      n_contrib[pix] = last[k];
-    }
-  }
-}
-
+// ---- vectors of pixels ----------------------------------------------------------------------------------------
+// A lane's pixels travel as packed fp32 pairs (one instruction, two IEEE operations) or, with one pixel per lane, as
+// plain floats; the overloads below let one body serve both.
+template <class V> __device__ __forceinline__ V bc(float x);
+template <> __device__ __forceinline__ float bc<float>(float x) { return x; }
+template <> __device__ __forceinline__ float2 bc<float2>(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float2 mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float2 mad(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float rcp_approx(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+__device__ __forceinline__ float neg(float a) { return -a; }
+__device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
+template <bool B> struct Flag { static constexpr bool value = B; };
+__device__ __forceinline__ float hsum(float a) { return a; }
+__device__ __forceinline__ float hsum(float2 a) { return a.x + a.y; }
 
-// Sum nine per-lane values over the warp with 14 shuffles instead of 45.  Values 0..7: at each of
-// the first three butterfly levels a lane keeps only the half of the values it is "responsible"
-// for and trades the other half with its partner, so the exchanged volume halves each level
-// (4 + 2 + 1 shuffles); two plain levels finish the one value left per lane.  Afterwards the
-// lanes 0, 4, .., 28 hold the totals: lane 16 * b4 + 8 * b3 + 4 * b2 owns value 4 * b4 + 2 * b3 + b2.
-// Value 8 takes a plain five-level butterfly and ends in every lane.
-__device__ __forceinline__ void warp_reduce9(const float v[9], int lane, float &mine, float &ninth) {
-  float a[4], b[2], c;
-  const bool hi16 = lane & 16, hi8 = lane & 8, hi4 = lane & 4;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float keep = hi16 ? v[4 + i] : v[i], give = hi16 ? v[i] : v[4 + i];
-    a[i] = keep + __shfl_xor_sync(kFull, give, 16);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const float keep = hi8 ? a[2 + i] : a[i], give = hi8 ? a[i] : a[2 + i];
-    b[i] = keep + __shfl_xor_sync(kFull, give, 8);
-  }
-  {
-    const float keep = hi4 ? b[1] : b[0], give = hi4 ? b[0] : b[1];
-    c = keep + __shfl_xor_sync(kFull, give, 4);
-  }
-  c += __shfl_xor_sync(kFull, c, 2);
-  c += __shfl_xor_sync(kFull, c, 1);
-  mine = c;
-  float n = v[8];
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) n += __shfl_xor_sync(kFull, n, s);
-  ninth = n;
+// ---- how a tile is shared out ------------------------------------------------------------------------------------
+// A warp owns a region of 4 NPX x 8 pixels of one tile and works through the tile's list on its own: lane (g, t) =
+// (lane / 4, lane % 4) has NPX pixels in row g from column NPX t on.
+template <int NPX> struct Share;
+template <> struct Share<4> { using V = float2; static constexpr int kVecs = 2, kWarps = 2, kColumns = 1; };
+template <> struct Share<2> { using V = float2; static constexpr int kVecs = 1, kWarps = 4, kColumns = 2; };
+template <> struct Share<1> { using V = float; static constexpr int kVecs = 1, kWarps = 8, kColumns = 4; };
+// First pixel of the warp's region.
+template <int NPX>
+__device__ __forceinline__ void region_of(int tile, int gx, int warp, int &rx, int &ry) {
+  rx = (tile % gx) * GS_TILE + (warp % Share<NPX>::kColumns) * 4 * NPX;
+  ry = (tile / gx) * GS_TILE + (warp / Share<NPX>::kColumns) * 8;
 }
+__device__ __forceinline__ float get(float v, int) { return v; }
+__device__ __forceinline__ float get(float2 v, int k) { return k ? v.y : v.x; }
+__device__ __forceinline__ void put(float &v, int, float x) { v = x; }
+__device__ __forceinline__ void put(float2 &v, int k, float x) { if (k) v.y = x; else v.x = x; }
+template <class V> struct Lanes;
+template <> struct Lanes<float> { static constexpr int value = 1; };
+template <> struct Lanes<float2> { static constexpr int value = 2; };
+
+// ---- the list, 32 entries at a time ------------------------------------------------------------------------------
+// Lane l fetches the parameters of entry l of the next 32 with asynchronous copies while the warp works on the current
+// ones (the id was loaded one round earlier still), so neither the gather nor the two dependent loads are waited for.
+struct __align__(16) RawEntries {
+  float4 conic[32];
+  float2 mean[32];
+  float color[3][32];
+};
+// Entries the warp works on.
+constexpr int kStaged = 32;
+struct __align__(16) StagedEntries {
+  float4 shape[kStaged];      // -x, -y, la, lb
+  float4 rest[kStaged];       // lc, o, position in the list, -
+  float4 rgb[kStaged];
+};
+
+__device__ __forceinline__ void copy_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async8(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async4(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+__device__ __forceinline__ void fetch_entry(RawEntries &raw, int lane, uint32_t g, const float *mean2d, const float *conic_opacity,
+                                            const float *color) {
+  copy_async16(&raw.conic[lane], conic_opacity + 4 * (size_t)g);
+  copy_async8(&raw.mean[lane], mean2d + 2 * (size_t)g);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) copy_async4(&raw.color[c][lane], color + 3 * (size_t)g + c);
+}
+
+// Can the entry reach alpha = 1/255 somewhere in the box [x0, x1] x [y0, y1] (offsets from its centre)?  The exponent
+// f = (la x + lb y)^2 + (lc y)^2 is convex, so its minimum over the box lies at the centre if the box holds it, else on
+// the vertical or the horizontal edge facing it, where it is a clamped one-dimensional minimum.  All candidates are
+// points of the box, so an error in where they lie moves the value by its square only; `slack` covers the rounding of
+// the pixels' own evaluation (|la x| below 2^15 with an error of 2^-24 each, times 2 |la x + lb y| < 6).
+__device__ __forceinline__ bool may_touch(float x0, float x1, float y0, float y1, float la, float lb, float lc, float limit) {
+  const float kSlack = 0.02f;
+  const float xn = fminf(fmaxf(0.f, x0), x1), yn = fminf(fmaxf(0.f, y0), y1);
+  const float ye = fminf(fmaxf(-xn * la * lb * rcp_approx(fmaf(lb, lb, lc * lc)), y0), y1);
+  const float xe = fminf(fmaxf(-yn * lb * rcp_approx(la), x0), x1);
+  const float u1 = fmaf(la, xn, lb * ye), v1 = lc * ye, u2 = fmaf(la, xe, lb * yn), v2 = lc * yn;
+  const float f = fminf(fmaf(u1, u1, v1 * v1), fmaf(u2, u2, v2 * v2));
+  return !(f > limit + kSlack);     // (a NaN stays in)
+}
+
+// Turns the lane's fetched entry into a staged one if it can touch the warp's region, closing ranks; returns how many
+// there are, rounded up to whole groups of kGroup with neutral entries.  `clamp`: one of them has an opacity above the alpha clamp.
+// (la, lb, lc) is the Cholesky factor of the conic, scaled by sqrt(0.5 log2 e), so that alpha = o exp(power) =
+// o 2^-((la dx + lb dy)^2 + (lc dy)^2): a sum of two squares has no cancellation, which keeps alpha accurate to a
+// few ulp even for footprints hundreds of pixels wide (the expanded quadratic form loses 1e-4 there).
+// `pos` and `id` go with the entry (its position in the list, its Gaussian).  NPX = 0 keeps every entry.
+template <int NPX, int kGroup>
+__device__ __forceinline__ int stage_entries(const RawEntries &raw, StagedEntries &st, int lane, bool valid, uint32_t pos, uint32_t id,
+                                             float rx0, float ry0, bool &clamp) {
+  const float kS = 0.8493218002880191f;   // sqrt(0.5 * log2(e))
+  float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+  float2 m = make_float2(0.f, 0.f);
+  float la = 0.f, lb = 0.f, lc = 0.f;
+  if (valid) {
+    q = raw.conic[lane]; m = raw.mean[lane];
+    la = kS * q.x; lb = kS * q.y; lc = kS * q.z;
+    const float x0 = rx0 - m.x, y0 = ry0 - m.y;
+    valid = NPX == 0 || may_touch(x0, x0 + (float)(4 * NPX - 1), y0, y0 + 7.f, la, lb, lc, __log2f(255.f * q.w));
+  }
+  const uint32_t taken = __ballot_sync(kFull, valid);
+  clamp = __any_sync(kFull, valid && !(q.w <= kAlphaMax));
+  const int count = __popc(taken);
+  if (valid) {
+    const int slot = __popc(taken & ((1u << lane) - 1u));
+    st.shape[slot] = make_float4(-m.x, -m.y, la, lb);
+    st.rest[slot] = make_float4(lc, q.w, __uint_as_float(pos), 0.f);
+    st.rgb[slot] = make_float4(raw.color[0][lane], raw.color[1][lane], raw.color[2][lane], __uint_as_float(id));
+  }
+  if (lane < (-count & (kGroup - 1))) {          // neutral: alpha = 0
+    st.shape[count + lane] = st.rest[count + lane] = st.rgb[count + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __syncwarp();
+  return (count + kGroup - 1) & ~(kGroup - 1);
+}
+
+// Alphas of a lane's pixels (fx: the centres of its columns, fy: that of its row), not yet clamped.  One explicit
+// operation order, shared by the forward, the backward and the pair counter, so that all take identical decisions.
+// (lb dy belongs to all pixels of a lane: it must not be rounded before the sum, or their errors have one sign - with
+// that, three times as many gradients of a 100k scene miss 1e-3.)
+template <int NPX>
+__device__ __forceinline__ void alphas(const float4 &shape, const float4 &rest, const typename Share<NPX>::V fx[Share<NPX>::kVecs],
+                                       float fy, typename Share<NPX>::V alpha[Share<NPX>::kVecs]) {
+  using V = typename Share<NPX>::V;
+  const float dy = __fadd_rn(fy, shape.y), c = __fmul_rn(rest.x, dy), s = __fmul_rn(c, c);
+#pragma unroll
+  for (int k = 0; k < Share<NPX>::kVecs; ++k) {
+    const V u = mad(bc<V>(shape.w), bc<V>(dy), mul(bc<V>(shape.z), add(fx[k], bc<V>(shape.x)))), f = mad(u, u, bc<V>(s));
+#pragma unroll
+    for (int i = 0; i < Lanes<V>::value; ++i) put(alpha[k], i, ex2_approx(-get(f, i)));
+    alpha[k] = mul(bc<V>(rest.y), alpha[k]);
+  }
+}
+
+// One pixel of the forward composites one entry, all by predicates.  It takes the entry if alpha >= 1/255 (q) and
+// the transmittance behind the entry, n, stays at 1e-4 or more (p); then the entry's colour is added with weight w and
+// its position noted.  T follows n either way: once it has fallen below 1e-4 no later n can pass, so the pixel has
+// stopped for good, and F keeps the transmittance it stopped with.
+__device__ __forceinline__ void composite(float alpha, float n, float w, const float4 &c, uint32_t pos1, float &T, float &F, float &R,
+                                          float &G, float &B, uint32_t &last) {
+  asm("{\n\t.reg .pred q, p;\n\t"
+      "setp.geu.f32 q, %6, %7;\n\t"
+      "setp.ge.and.f32 p, %8, %9, q;\n\t"
+      "@p fma.rn.f32 %2, %10, %11, %2;\n\t"
+      "@p fma.rn.f32 %3, %10, %12, %3;\n\t"
+      "@p fma.rn.f32 %4, %10, %13, %4;\n\t"
+      "@p mov.f32 %1, %8;\n\t"
+      "@p mov.u32 %5, %14;\n\t"
+      "@q mov.f32 %0, %8;\n\t}"
+      : "+f"(T), "+f"(F), "+f"(R), "+f"(G), "+f"(B), "+r"(last)
+      : "f"(alpha), "f"(kAlphaMin), "f"(n), "f"(kTmin), "f"(w), "f"(c.x), "f"(c.y), "f"(c.z), "r"(pos1));
+}
+
+// Forward.  Entries are taken four at a time: their alphas do not depend on one another, only the chain through T does.
+// 8 x 8 pixels per warp measured best from 16 tiles to 8160 (16 x 8 ties at 8160, 97 against 102 us at 4108, 66 against
+// 77 at 2550; two entries at a time: 1 to 2 us more where a launch is only a few warps per scheduler).
+// 1M Gaussians, 1256 x 828: 150 -> 97 us; 92 M -> 72 M warp instructions.
+constexpr int kFwdPixels = 2, kFwdGroup = 4;
+__global__ void __launch_bounds__(32) k_blend_fwd(
+    CamDev cam, const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ order, const uint32_t *__restrict__ vals,
+    const float *__restrict__ mean2d, const float *__restrict__ conic_opacity, const float *__restrict__ color,
+    uint32_t *__restrict__ sorted_tiles, float *__restrict__ image, float *__restrict__ final_T, uint32_t *__restrict__ n_contrib) {
+  dependency_wait();
+  constexpr int NPX = kFwdPixels;
+  using V = Share<NPX>::V;
+  constexpr int kVecs = Share<NPX>::kVecs, kWarps = Share<NPX>::kWarps, kLanes = Lanes<V>::value;
+  __shared__ RawEntries raw;
+  __shared__ StagedEntries st;
+  const int lane = threadIdx.x, warp = (int)(blockIdx.x % kWarps), tile = (int)__ldg(order + blockIdx.x / kWarps);
+  int rx, ry;
+  region_of<NPX>(tile, cam.gx, warp, rx, ry);
+  const int px = rx + NPX * (lane & 3), py = ry + (lane >> 2);
+  const uint32_t start = __ldg(ranges + 2 * tile), end = __ldg(ranges + 2 * tile + 1);
+  // the key of every instance of this tile's stretch of the sorted list is the tile id: stores that nothing here waits for
+  if (sorted_tiles)
+    for (uint32_t p = start + 32u * warp + lane; p < end; p += 32 * kWarps) sorted_tiles[p] = (uint32_t)tile;
+  const float fy = (float)py + 0.5f, rx0 = (float)rx + 0.5f, ry0 = (float)ry + 0.5f;
+  // T, F: transmittance (see composite); pixels outside the image start stopped
+  V fx[kVecs];
+  float T[NPX], F[NPX], R[NPX], G[NPX], B[NPX];
+  uint32_t last[NPX];                       // position + 1 of the last composited entry
+#pragma unroll
+  for (int k = 0; k < NPX; ++k) {
+    put(fx[k / kLanes], k % kLanes, (float)(px + k) + 0.5f);
+    T[k] = px + k < cam.W && py < cam.H ? 1.f : 0.f;
+    F[k] = 1.f;
+    R[k] = G[k] = B[k] = 0.f;
+    last[k] = 0u;
+  }
+  auto any_live = [&]() {
+    float t = T[0];
+#pragma unroll
+    for (int k = 1; k < NPX; ++k) t = fmaxf(t, T[k]);
+    return __any_sync(kFull, t >= kTmin);
+  };
+  const uint32_t len = end - start;
+  uint32_t id = 0;
+  if ((uint32_t)lane < len) fetch_entry(raw, lane, __ldg(vals + start + lane), mean2d, conic_opacity, color);
+  if (32u + (uint32_t)lane < len) id = __ldg(vals + start + 32u + lane);
+  for (uint32_t base = 0; base < len; base += 32) {
+    if (!any_live()) break;                 // every pixel of the region has stopped
+    copies_wait();
+    bool clamp;
+    const int count = stage_entries<NPX, kFwdGroup>(raw, st, lane, base + lane < len, base + lane + 1u, 0u, rx0, ry0, clamp);
+    if (base + 32u + lane < len) fetch_entry(raw, lane, id, mean2d, conic_opacity, color);
+    if (base + 64u + lane < len) id = __ldg(vals + start + base + 64u + lane);
+    auto work = [&](auto clamped) {
+      for (int j0 = 0; j0 < count; j0 += 8) {
+        if (j0 && !any_live()) break;
+        const int j1 = min(j0 + 8, count);
+        for (int j = j0; j < j1; j += kFwdGroup) {
+          V al[kFwdGroup][kVecs];
+#pragma unroll
+          for (int e = 0; e < kFwdGroup; ++e) {
+            alphas<NPX>(st.shape[j + e], st.rest[j + e], fx, fy, al[e]);
+            if (decltype(clamped)::value)
+#pragma unroll
+              for (int k = 0; k < kVecs; ++k)
+#pragma unroll
+                for (int i = 0; i < kLanes; ++i) put(al[e][k], i, fminf(kAlphaMax, get(al[e][k], i)));
+          }
+#pragma unroll
+          for (int e = 0; e < kFwdGroup; ++e) {
+            const float4 c = st.rgb[j + e];
+            const uint32_t pos1 = __float_as_uint(st.rest[j + e].z);
+#pragma unroll
+            for (int k = 0; k < kVecs; ++k) {
+              // transmittance behind the entry as T (1 - alpha), both roundings included: the backward recovers T by dividing
+              // (1 - alpha) out again and drifts if the forward rounds another expression (T - alpha T in one rounding: 2.4
+              // times as many gradients of a 1M scene miss 1e-3)
+              V t;
+#pragma unroll
+              for (int i = 0; i < kLanes; ++i) put(t, i, T[kLanes * k + i]);
+              const V w = mul(al[e][k], t), n = mul(t, add(bc<V>(1.f), neg(al[e][k])));
+#pragma unroll
+              for (int i = 0; i < kLanes; ++i) {
+                const int p = kLanes * k + i;
+                composite(get(al[e][k], i), get(n, i), get(w, i), c, pos1, T[p], F[p], R[p], G[p], B[p], last[p]);
+              }
+            }
+          }
+        }
+      }
+    };
+    if (clamp) work(Flag<true>()); else work(Flag<false>());
+    __syncwarp();                            // the staged entries have been read
+  }
+  copies_wait();
+  const size_t plane = (size_t)cam.W * cam.H;
+#pragma unroll
+  for (int k = 0; k < NPX; ++k)
+    if (px + k < cam.W && py < cam.H) {
+      const size_t pix = (size_t)py * cam.W + px + k;
+      const float t = F[k];
+      image[pix] = fmaf(t, cam.bg[0], R[k]);
+      image[plane + pix] = fmaf(t, cam.bg[1], G[k]);
+      image[2 * plane + pix] = fmaf(t, cam.bg[2], B[k]);
+      final_T[pix] = t;
+      n_contrib[pix] = last[k];
+    }
+}
+
+// ---- backward ----------------------------------------------------------------------------------------------------
+__device__ __forceinline__ void red_add4(float *p, float a, float b, float c, float d) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+// v if alpha >= 1/255 and the entry lies inside the pixel's walk, else 0
+__device__ __forceinline__ float select_alpha(float alpha, uint32_t pos, uint32_t nc, float v) {
+  float r;
+  asm("{\n\t.reg .pred q, p;\n\tsetp.lt.u32 q, %1, %2;\n\tsetp.geu.and.f32 p, %3, %4, q;\n\tselp.f32 %0, %5, 0f00000000, p;\n\t}"
+      : "=f"(r) : "r"(pos), "r"(nc), "f"(alpha), "f"(kAlphaMin), "f"(v));
+  return r;
+}
+
+// What the lanes leave of an entry: dp of their pixels and their colour sums, kBatch entries at a time.  Strides chosen
+// so that the reads of sum_entries meet no bank conflict: four lanes read neighbouring values of one entry, and the
+// eight (float4), sixteen (float2) or thirty-two (float) lanes that are served together cover all banks.
+constexpr int kBatch = 8, kParkStride = 36;
+template <int NPX> struct Dp;
+template <> struct Dp<4> { using T = float4; };
+template <> struct Dp<2> { using T = float2; };
+template <> struct Dp<1> { using T = float; };
+template <int NPX>
+struct __align__(16) Parked {
+  typename Dp<NPX>::T dp[kBatch * kParkStride];
+  float2 rg[kBatch * kParkStride];
+  float b[kBatch * kParkStride];
+};
+
+__device__ __forceinline__ float4 pack(const float2 v[2]) { return make_float4(v[0].x, v[0].y, v[1].x, v[1].y); }
+template <int NPX, class V>
+__device__ __forceinline__ void park(Parked<NPX> &p, int e, int lane, const V dp[Share<NPX>::kVecs], float r, float g, float b) {
+  if constexpr (NPX == 4) p.dp[e * kParkStride + lane] = pack(dp); else p.dp[e * kParkStride + lane] = dp[0];
+  p.rg[e * kParkStride + lane] = make_float2(r, g);
+  p.b[e * kParkStride + lane] = b;
+}
+// Sums over the region of entry e, in all of its four lanes: dp times 1, x, y, x^2, xy, y^2 (about the region's middle) and
+// the colours.  Lane t takes the strips of the eight lanes (g, t).
+struct Sums { float m, mx, my, mxx, mxy, myy, r, g, b; };
+__device__ __forceinline__ float sum4(float v) {
+  v += __shfl_xor_sync(kFull, v, 1);
+  return v + __shfl_xor_sync(kFull, v, 2);
+}
+template <int NPX>
+__device__ __forceinline__ Sums sum_entries(const Parked<NPX> &p, int e, int t) {
+  using V = typename Share<NPX>::V;
+  constexpr int kVecs = Share<NPX>::kVecs, kLanes = Lanes<V>::value;
+  V m[kVecs], my[kVecs], myy[kVecs];          // per column of the strip
+  float2 rg = make_float2(0.f, 0.f);
+  float b = 0.f;
+#pragma unroll
+  for (int g = 0; g < 8; ++g) {
+    const int at = e * kParkStride + 4 * g + t;
+    V v[kVecs];
+    if constexpr (NPX == 4) { const float4 q = p.dp[at]; v[0] = make_float2(q.x, q.y); v[1] = make_float2(q.z, q.w); } else v[0] = p.dp[at];
+    const float y = (float)g - 3.5f;
+#pragma unroll
+    for (int k = 0; k < kVecs; ++k) {
+      m[k] = g ? add(m[k], v[k]) : v[k];
+      my[k] = g ? mad(bc<V>(y), v[k], my[k]) : mul(bc<V>(y), v[k]);
+      myy[k] = g ? mad(bc<V>(y * y), v[k], myy[k]) : mul(bc<V>(y * y), v[k]);
+    }
+    rg = __fadd2_rn(rg, p.rg[at]);
+    b += p.b[at];
+  }
+  Sums s = {};
+#pragma unroll
+  for (int k = 0; k < NPX; ++k) {
+    const float x = (float)(NPX * t + k) + 0.5f - 2.f * NPX, c = get(m[k / kLanes], k % kLanes), cy = get(my[k / kLanes], k % kLanes);
+    s.m += c; s.mx = fmaf(x, c, s.mx); s.mxx = fmaf(x * x, c, s.mxx);
+    s.my += cy; s.mxy = fmaf(x, cy, s.mxy);
+    s.myy += get(myy[k / kLanes], k % kLanes);
+  }
+  s.m = sum4(s.m); s.mx = sum4(s.mx); s.my = sum4(s.my); s.mxx = sum4(s.mxx); s.mxy = sum4(s.mxy); s.myy = sum4(s.myy);
+  s.r = sum4(rg.x); s.g = sum4(rg.y); s.b = sum4(b);
+  return s;
+}
+template <int NPX>
+struct __align__(16) BwdArea {
+  RawEntries raw;
+  StagedEntries st;
+  Parked<NPX> parked;
+};
 
 // Backward: walk each pixel's composited entries back to front.  The transmittance in front of
 // an entry is recovered by dividing out (1 - alpha); the light arriving from behind it is summed
@@ -242,246 +379,213 @@ __device__ __forceinline__ void warp_reduce9(const float v[9], int lane, float &
 // "final pixel - prefix" cancels badly for deep entries).  Only its product with the pixel's
 // upstream gradient is needed, so one scalar per pixel carries it.
 //
-// What a pixel sends to a Gaussian's conic and mean is linear in dp = dL/d(power) times
-// (1, dx, dy, dx^2, dx dy, dy^2).  The threads therefore sum the six moments of dp in tile-local
-// pixel coordinates (half-integers up to 7.5, so the products are exact), a quad of pixels at a
-// time, and the moments are shifted to the Gaussian's own centre once per (tile, Gaussian) when
-// the batch leaves shared memory.  The opacity gradient needs no sum of its own: alpha = o exp(power)
-// where it is not clamped, so dL/do = (sum of dp) / o, the zeroth moment.  Nine values per entry cross
-// the warp: the six moments and the colour gradient (warp_reduce9); each warp owns its own copy of the
-// batch's accumulators, so no shared-memory atomics are needed; the sums leave with one global
-// atomic per value.
-// g2d row: (d colour r, g, b, d opacity) (d conic A, B, C, d mean u) (d mean v, -, -, -).
-__global__ void __launch_bounds__(kThreads, 16) k_blend_bwd(CamDev cam, const uint32_t *__restrict__ ranges,
-                                                        const uint32_t *__restrict__ order,
-                                                        const uint32_t *__restrict__ vals,
-                                                        const float *__restrict__ mean2d,
-                                                        const float *__restrict__ conic_opacity,
-                                                        const float *__restrict__ color,
-                                                        const float *__restrict__ final_T,
-                                                        const uint32_t *__restrict__ n_contrib,
-                                                        const float *__restrict__ dL_dimage, float *__restrict__ g2d) {
-  __shared__ float4 s_xyab[kBatchBwd];
-  __shared__ float2 s_co[kBatchBwd];
-  __shared__ float4 s_rgb[kBatchBwd];
-  __shared__ uint32_t s_gid[kBatchBwd];
-  __shared__ float s_acc[kThreads / 32][kBatchBwd][9];
-  __shared__ uint32_t s_max[2];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tile = (int)__ldg(order + blockIdx.x);
-  int px, py;
-  quad_of(tile, cam.gx, tid, px, py);
-  const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
-  // tile-local coordinates of the quad's pixel centres, origin at the middle of the tile
-  const float ox_tile = (float)((tile % cam.gx) * GS_TILE + GS_TILE / 2), oy_tile = (float)((tile / cam.gx) * GS_TILE + GS_TILE / 2);
-  const float X0 = fx - ox_tile, X1 = X0 + 1.f, Y0 = fy - oy_tile, Y1 = Y0 + 1.f;
-  const float XX0 = X0 * X0, XX1 = X1 * X1, YY0 = Y0 * Y0, YY1 = Y1 * Y1;
-  const uint32_t start = __ldg(ranges + 2 * tile), end = __ldg(ranges + 2 * tile + 1);
+// What a pixel sends to a Gaussian's conic and mean is linear in dp = dL/d(power) times (1, dx, dy, dx^2, dx dy, dy^2),
+// and the opacity gradient needs no sum of its own: alpha = o exp(power) where it is not clamped, so dL/do = (sum of
+// dp) / o.  Per entry nine sums over the region's pixels are due, six moments of dp and three colours.  A lane parks its
+// pixels' dp and its three colour sums in shared memory as they are; after every eight entries four lanes per entry add
+// them up, with the weights x and y (tile-local half-integers: exact) as constants, shift the moments to the Gaussian's
+// own centre and send them off with three vector reductions to the g2d row:
+// (d colour r, g, b, d opacity) (d conic A, B, C, d mean u) (d mean v, -, -, -).
+// Per entry that is 3 stores and about 20 instructions, where a butterfly of the nine sums over the warp took 19 shuffles
+// (4 cycles each), as many adds and 14 selects, and the same sums as products on the tensor cores (tf32 operands in two
+// terms) took fewer instructions but 105 register operands instead of 55: 215 against 181 us.
+//
+// 16 x 8 pixels per warp is best where the launch fills the chip (1M Gaussians, 1256 x 828: 181 us against 195 with
+// 8 x 8; 244 before); smaller regions give more warps and cull more where it does not: 8 x 8 from 2550 tiles down
+// (128 against 133 us at 2550, 69 / 68 at 1024, 30 / 39 at 294), 4 x 8 while every warp still has a scheduler of its own
+// (16 tiles: 23 against 29 us).  There, what does not depend on the carried state is worked out for four entries at a
+// time (2 to 4 us less); with 16 x 8 pixels the registers it takes cost more than it gives.
+template <int NPX>
+__global__ void __launch_bounds__(32) k_blend_bwd(
+    CamDev cam, const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ order, const uint32_t *__restrict__ vals,
+    const float *__restrict__ mean2d, const float *__restrict__ conic_opacity, const float *__restrict__ color,
+    const float *__restrict__ final_T, const uint32_t *__restrict__ n_contrib, const float *__restrict__ dL_dimage,
+    float *__restrict__ g2d) {
+  using V = typename Share<NPX>::V;
+  constexpr int kVecs = Share<NPX>::kVecs, kLanes = Lanes<V>::value, kWarps = Share<NPX>::kWarps, kGroup = NPX == 4 ? 1 : 4;
+  __shared__ BwdArea<NPX> area;
+  const int lane = threadIdx.x, warp = (int)(blockIdx.x % kWarps), tile = (int)__ldg(order + blockIdx.x / kWarps);
+  RawEntries &raw = area.raw;
+  StagedEntries &st = area.st;
+  const int g = lane >> 2, t = lane & 3;
+  int rx, ry;
+  region_of<NPX>(tile, cam.gx, warp, rx, ry);
+  const int px = rx + NPX * t, py = ry + g;
+  const uint32_t start = __ldg(ranges + 2 * tile);
+  const float fy = (float)py + 0.5f, rx0 = (float)rx + 0.5f, ry0 = (float)ry + 0.5f;
   const size_t plane = (size_t)cam.W * cam.H;
-  uint32_t nc[4];
-  float T[4], Gr[4], Gg[4], Gb[4], GS[4];
-  uint32_t wmax = 0;
+  uint32_t nc[NPX], wmax = 0;
+  V fx[kVecs], T[kVecs], Gr[kVecs], Gg[kVecs], Gb[kVecs], S[kVecs];   // S: G . (light from behind)
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int x = px + (k & 1), y = py + (k >> 1);
-    nc[k] = 0; T[k] = 1.f; Gr[k] = Gg[k] = Gb[k] = 0.f;
-    if (x < cam.W && y < cam.H) {
-      const size_t pix = (size_t)y * cam.W + x;
+  for (int k = 0; k < NPX; ++k) {
+    float tr = 1.f, gr = 0.f, gg = 0.f, gb = 0.f;
+    nc[k] = 0u;
+    if (px + k < cam.W && py < cam.H) {
+      const size_t pix = (size_t)py * cam.W + px + k;
       nc[k] = __ldg(n_contrib + pix);
-      T[k] = __ldg(final_T + pix);
-      Gr[k] = __ldg(dL_dimage + pix); Gg[k] = __ldg(dL_dimage + plane + pix); Gb[k] = __ldg(dL_dimage + 2 * plane + pix);
+      tr = __ldg(final_T + pix);
+      gr = __ldg(dL_dimage + pix); gg = __ldg(dL_dimage + plane + pix); gb = __ldg(dL_dimage + 2 * plane + pix);
     }
-    GS[k] = T[k] * fmaf(Gb[k], cam.bg[2], fmaf(Gg[k], cam.bg[1], Gr[k] * cam.bg[0]));   // G . (light from behind)
+    const int v = k / kLanes, i = k % kLanes;
+    put(fx[v], i, (float)(px + k) + 0.5f);
+    put(T[v], i, tr); put(Gr[v], i, gr); put(Gg[v], i, gg); put(Gb[v], i, gb);
+    put(S[v], i, tr * fmaf(gb, cam.bg[2], fmaf(gg, cam.bg[1], gr * cam.bg[0])));
     wmax = max(wmax, nc[k]);
   }
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) wmax = max(wmax, __shfl_xor_sync(kFull, wmax, s));
-  if (lane == 0) s_max[warp] = wmax;
-  __syncthreads();
-  const uint32_t maxc = max(s_max[0], s_max[1]);
-  if (maxc == 0 || start + maxc > end) return;   // nothing composited in this tile
-  // value that this lane holds after the reduction (lanes 0, 4, .., 28: one of 0..7; lane 1 stores value 8)
-  const int my_value = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
-  const int nbatches = (int)((maxc + kBatchBwd - 1) / kBatchBwd);
-  // pixels (0, 1) and (2, 3) as packed pairs; nGS carries minus G . (light from behind)
-  float2 T01 = make_float2(T[0], T[1]), T23 = make_float2(T[2], T[3]);
-  float2 nGS01 = make_float2(-GS[0], -GS[1]), nGS23 = make_float2(-GS[2], -GS[3]);
-  const float2 Gr01 = make_float2(Gr[0], Gr[1]), Gr23 = make_float2(Gr[2], Gr[3]);
-  const float2 Gg01 = make_float2(Gg[0], Gg[1]), Gg23 = make_float2(Gg[2], Gg[3]);
-  const float2 Gb01 = make_float2(Gb[0], Gb[1]), Gb23 = make_float2(Gb[2], Gb[3]);
-  for (int b = nbatches - 1; b >= 0; --b) {
-    __syncthreads();
-    const uint32_t first = (uint32_t)b * kBatchBwd;
-    const int cnt = (int)min((uint32_t)kBatchBwd, maxc - first);
-#pragma unroll
-    for (int h = 0; h < kBatchBwd / kThreads; ++h) {
-      const int slot = tid + h * kThreads;
-      if (slot < cnt) {
-        const uint32_t g = __ldg(vals + start + first + slot);
-        s_gid[slot] = g;
-        stage_entry(g, mean2d, conic_opacity, color, s_xyab[slot], s_co[slot], s_rgb[slot]);
-      }
-#pragma unroll
-      for (int k = 0; k < 9; ++k) s_acc[0][slot][k] = s_acc[1][slot][k] = 0.f;
+  if (wmax == 0 || wmax > __ldg(ranges + 2 * tile + 1) - start) return;   // nothing composited in this region
+  uint32_t base = (wmax - 1u) & ~31u;          // first entry of the last piece of 32
+  uint32_t id = 0;
+  if (base + lane < wmax) {
+    id = __ldg(vals + start + base + lane);
+    fetch_entry(raw, lane, id, mean2d, conic_opacity, color);
+  }
+  uint32_t id_next = base >= 32u ? __ldg(vals + start + base - 32u + lane) : 0u;
+  for (;; base -= 32u) {
+    copies_wait();
+    bool clamp;
+    const int count = stage_entries<NPX, kGroup>(raw, st, lane, base + lane < wmax, base + lane, id, rx0, ry0, clamp);
+    if (base >= 32u) {
+      id = id_next;
+      fetch_entry(raw, lane, id, mean2d, conic_opacity, color);
+      if (base >= 64u) id_next = __ldg(vals + start + base - 64u + lane);
     }
-    __syncthreads();
-    const int jtop = (int)min((uint32_t)cnt, wmax > first ? wmax - first : 0u);
-    // positions of this batch that each pixel composited: j < lim[k] (as numbers: the comparisons below make 0 / 1 masks)
-    float limf[4];
+    for (int top = count; top > 0; top = (top - 1) & ~(kBatch - 1)) {
+      const int bottom = (top - 1) & ~(kBatch - 1);
+      auto work = [&](auto clamped) {
+        constexpr bool kClamp = decltype(clamped)::value;
+        for (int j = top - kGroup; j >= bottom; j -= kGroup) {
+          // What does not depend on the carried state, for a group of entries.  A pixel that did not composite an entry (it
+          // lies beyond the pixel's walk, or alpha < 1/255) enters with alpha = 0, for which the reciprocal is 1, every
+          // product below is 0 and its carried state is unchanged.
+          V a[kGroup][kVecs], inv[kGroup][kVecs], gc[kGroup][kVecs], free[kGroup][kVecs];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) limf[k] = nc[k] > first ? (float)min(nc[k] - first, (uint32_t)kBatchBwd) : 0.f;
-    float jf = (float)jtop;
-    for (int j = jtop - 1; j >= 0; --j) {
-      const float4 a = s_xyab[j];
-      const float2 c = s_co[j];
-      float p[4], t1[4], t2[2];
-      quad_power(fx - a.x, fy - a.y, a.z, a.w, c.x, p, t1, t2);
-      const float4 col = s_rgb[j];
-      jf -= 1.f;
-      // q: the pixel composited this entry (it lies inside the pixel's walk and alpha >= 1/255), as 0 / 1
-      const float2 q01 = __fmul2_rn(make_float2(set_geu(p[0], col.w), set_geu(p[1], col.w)), make_float2(set_lt(jf, limf[0]), set_lt(jf, limf[1])));
-      const float2 q23 = __fmul2_rn(make_float2(set_geu(p[2], col.w), set_geu(p[3], col.w)), make_float2(set_lt(jf, limf[2]), set_lt(jf, limf[3])));
-      if (!__any_sync(kFull, (q01.x + q01.y) + (q23.x + q23.y) != 0.f)) continue;
-      // Branch-free from here, two packed pixel pairs: a pixel that did not composite this entry enters with
-      // alpha = 0, for which the reciprocal is 1, every product below is 0 and its carried state is unchanged.
-      const float2 o2 = make_float2(c.y, c.y), one = make_float2(1.f, 1.f), mone = make_float2(-1.f, -1.f);
-      const float2 raw01 = __fmul2_rn(o2, make_float2(ex2_approx(p[0]), ex2_approx(p[1])));
-      const float2 raw23 = __fmul2_rn(o2, make_float2(ex2_approx(p[2]), ex2_approx(p[3])));
-      const float2 al01 = __fmul2_rn(q01, make_float2(fminf(kAlphaMax, raw01.x), fminf(kAlphaMax, raw01.y)));
-      const float2 al23 = __fmul2_rn(q23, make_float2(fminf(kAlphaMax, raw23.x), fminf(kAlphaMax, raw23.y)));
-      const float2 d01 = __ffma2_rn(al01, mone, one), d23 = __ffma2_rn(al23, mone, one);
-      const float2 inv01 = make_float2(rcp_approx(d01.x), rcp_approx(d01.y)), inv23 = make_float2(rcp_approx(d23.x), rcp_approx(d23.y));
-      const float2 Tb01 = __fmul2_rn(T01, inv01), Tb23 = __fmul2_rn(T23, inv23);     // transmittance in front of this entry
-      const float2 w01 = __fmul2_rn(al01, Tb01), w23 = __fmul2_rn(al23, Tb23);
-      float v[9];
-      {
-        const float2 r = __ffma2_rn(w01, Gr01, __fmul2_rn(w23, Gr23)), g = __ffma2_rn(w01, Gg01, __fmul2_rn(w23, Gg23));
-        const float2 bl = __ffma2_rn(w01, Gb01, __fmul2_rn(w23, Gb23));
-        v[6] = r.x + r.y; v[7] = g.x + g.y; v[8] = bl.x + bl.y;
-      }
-      // d pixel / d alpha = T c - S / (1 - alpha), S = everything composited behind this entry
-      const float2 cx = make_float2(col.x, col.x), cy = make_float2(col.y, col.y), cz = make_float2(col.z, col.z);
-      const float2 gc01 = __ffma2_rn(Gb01, cz, __ffma2_rn(Gg01, cy, __fmul2_rn(Gr01, cx)));
-      const float2 gc23 = __ffma2_rn(Gb23, cz, __ffma2_rn(Gg23, cy, __fmul2_rn(Gr23, cx)));
-      const float2 da01 = __fmul2_rn(__ffma2_rn(T01, gc01, nGS01), inv01), da23 = __fmul2_rn(__ffma2_rn(T23, gc23, nGS23), inv23);
-      // clamped at 0.99: alpha does not depend on opacity and power there (mask 0)
-      const float2 e01 = __fmul2_rn(__fmul2_rn(al01, da01), make_float2(set_le(raw01.x, kAlphaMax), set_le(raw01.y, kAlphaMax)));
-      const float2 e23 = __fmul2_rn(__fmul2_rn(al23, da23), make_float2(set_le(raw23.x, kAlphaMax), set_le(raw23.y, kAlphaMax)));
-      const float dp0 = e01.x, dp1 = e01.y, dp2 = e23.x, dp3 = e23.y;
-      nGS01 = __ffma2_rn(make_float2(-w01.x, -w01.y), gc01, nGS01);
-      nGS23 = __ffma2_rn(make_float2(-w23.x, -w23.y), gc23, nGS23);
-      T01 = Tb01; T23 = Tb23;
-      {
-        const float sL = dp0 + dp2, sR = dp1 + dp3, sT = dp0 + dp1, sB = dp2 + dp3;
-        v[0] = sL + sR;
-        v[1] = fmaf(X0, sL, X1 * sR);
-        v[2] = fmaf(Y0, sT, Y1 * sB);
-        v[3] = fmaf(XX0, sL, XX1 * sR);
-        v[4] = fmaf(X0, fmaf(Y0, dp0, Y1 * dp2), X1 * fmaf(Y0, dp1, Y1 * dp3));
-        v[5] = fmaf(YY0, sT, YY1 * sB);
-        float mine, ninth;
-        warp_reduce9(v, lane, mine, ninth);
-        if ((lane & 3) == 0) s_acc[warp][j][my_value] = mine;
-        if (lane == 1) s_acc[warp][j][8] = ninth;
-      }
-    }
-    __syncthreads();
+          for (int e = kGroup - 1; e >= 0; --e) {
+            const float4 b = st.rest[j + e], c = st.rgb[j + e];
+            const uint32_t pos = __float_as_uint(b.z);
+            alphas<NPX>(st.shape[j + e], b, fx, fy, a[e]);
 #pragma unroll
-    for (int h = 0; h < kBatchBwd / kThreads; ++h) {
-      const int slot = tid + h * kThreads;
-      if (slot < cnt) {
-        float M[9];
-        bool touched = false;
+            for (int k = 0; k < kVecs; ++k) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-          M[k] = s_acc[0][slot][k] + s_acc[1][slot][k];
-          touched = touched || (M[k] != 0.f);
+              for (int i = 0; i < kLanes; ++i) {
+                const float x = get(a[e][k], i);
+                put(a[e][k], i, select_alpha(x, pos, nc[kLanes * k + i], kClamp ? fminf(kAlphaMax, x) : x));
+                if (kClamp) put(free[e][k], i, x > kAlphaMax ? 0.f : 1.f);
+              }
+              const V d = add(bc<V>(1.f), neg(a[e][k]));
+#pragma unroll
+              for (int i = 0; i < kLanes; ++i) put(inv[e][k], i, rcp_approx(get(d, i)));
+              gc[e][k] = mad(Gb[k], bc<V>(c.z), mad(Gg[k], bc<V>(c.y), mul(Gr[k], bc<V>(c.x))));
+            }
+          }
+          V dp[kGroup][kVecs], cr[kGroup], cg[kGroup], cb[kGroup];
+#pragma unroll
+          for (int e = kGroup - 1; e >= 0; --e)
+#pragma unroll
+            for (int k = 0; k < kVecs; ++k) {
+              const V Tb = mul(T[k], inv[e][k]), w = mul(a[e][k], Tb);   // transmittance in front of this entry; its weight
+              if (k == 0) { cr[e] = mul(w, Gr[k]); cg[e] = mul(w, Gg[k]); cb[e] = mul(w, Gb[k]); }
+              else { cr[e] = mad(w, Gr[k], cr[e]); cg[e] = mad(w, Gg[k], cg[e]); cb[e] = mad(w, Gb[k], cb[e]); }
+              // d pixel / d alpha = T c - S / (1 - alpha), S = everything composited behind this entry
+              dp[e][k] = mul(a[e][k], mul(mad(T[k], gc[e][k], neg(S[k])), inv[e][k]));
+              if (kClamp) dp[e][k] = mul(dp[e][k], free[e][k]);     // clamped at 0.99: alpha does not depend on opacity and power
+              S[k] = mad(w, gc[e][k], S[k]);
+              T[k] = Tb;
+            }
+#pragma unroll
+          for (int e = kGroup - 1; e >= 0; --e) park<NPX>(area.parked, j + e - bottom, lane, dp[e], hsum(cr[e]), hsum(cg[e]), hsum(cb[e]));
         }
+      };
+      if (clamp) work(Flag<true>()); else work(Flag<false>());
+      __syncwarp();
+      // four lanes per entry
+      const int e = lane >> 2, slot = bottom + e;
+      const Sums s = sum_entries<NPX>(area.parked, e, t);
+      if (slot < top) {
+        // moments about the Gaussian's centre from those about the region's: d = (X + ox, Y + oy)
+        const float4 sh = st.shape[slot], re = st.rest[slot];
+        const float ox = (float)rx + 2.f * NPX + sh.x, oy = (float)ry + 4.f + sh.y;
+        const float sx = fmaf(ox, s.m, s.mx), sy = fmaf(oy, s.m, s.my);
+        const float sxx = fmaf(ox, s.mx + sx, s.mxx);
+        const float sxy = fmaf(oy, sx, fmaf(ox, s.my, s.mxy));
+        const float syy = fmaf(oy, s.my + sy, s.myy);
+        // the staged factor is the conic's Cholesky factor times sqrt(0.5 log2 e)
+        const float A = 2.f * kLn2 * sh.z * sh.z, B = 2.f * kLn2 * sh.z * sh.w, C = 2.f * kLn2 * fmaf(sh.w, sh.w, re.x * re.x);
+        float *dst = g2d + (size_t)__float_as_uint(st.rgb[slot].w) * 12;
+        const bool touched = s.m != 0.f || s.mx != 0.f || s.my != 0.f || s.mxx != 0.f || s.mxy != 0.f || s.myy != 0.f || s.r != 0.f ||
+                             s.g != 0.f || s.b != 0.f;
         if (touched) {
-          // moments about the Gaussian's centre from the tile-local ones: d = (X + ox, Y + oy)
-          const float4 a = s_xyab[slot];
-          const float lc = s_co[slot].x, o = s_co[slot].y;
-          const float ox = ox_tile - a.x, oy = oy_tile - a.y;
-          const float sx = fmaf(ox, M[0], M[1]), sy = fmaf(oy, M[0], M[2]);
-          const float sxx = fmaf(ox, M[1] + sx, M[3]);
-          const float sxy = fmaf(oy, sx, fmaf(ox, M[2], M[4]));
-          const float syy = fmaf(oy, M[2] + sy, M[5]);
-          // the staged factor is the conic's Cholesky factor times sqrt(0.5 log2 e)
-          const float A = 2.f * kLn2 * a.z * a.z, B = 2.f * kLn2 * a.z * a.w, C = 2.f * kLn2 * fmaf(a.w, a.w, lc * lc);
-          float *dst = g2d + (size_t)s_gid[slot] * 12;
-          atomicAdd(dst + 0, M[6]); atomicAdd(dst + 1, M[7]); atomicAdd(dst + 2, M[8]); atomicAdd(dst + 3, __fdividef(M[0], o));
-          atomicAdd(dst + 4, -0.5f * sxx); atomicAdd(dst + 5, -sxy); atomicAdd(dst + 6, -0.5f * syy);
-          atomicAdd(dst + 7, fmaf(A, sx, B * sy)); atomicAdd(dst + 8, fmaf(B, sx, C * sy));
+          if (t == 0) red_add4(dst, s.r, s.g, s.b, __fdividef(s.m, re.y));
+          if (t == 1) red_add4(dst + 4, -0.5f * sxx, -sxy, -0.5f * syy, fmaf(A, sx, B * sy));
+          if (t == 2) atomicAdd(dst + 8, fmaf(B, sx, C * sy));
         }
       }
+      __syncwarp();                              // the parked values have been read
     }
+    if (base == 0u) break;
   }
 }
 
-// Measurement only: replay the forward's decisions and count, over all pixels, the list entries
-// evaluated (until each pixel stopped) and the pairs composited; and per warp (16 x 8 pixels) the
-// entries it walked and those among them that none of its live pixels accepted.
-// counts[0] += evaluated, counts[1] += composited, counts[2] += (warp, entry) steps, counts[3] += steps without a taker.
-__global__ void __launch_bounds__(kThreads) k_blend_count(CamDev cam, const uint32_t *__restrict__ ranges,
-                                                          const uint32_t *__restrict__ vals,
-                                                          const float *__restrict__ mean2d,
-                                                          const float *__restrict__ conic_opacity,
-                                                          const float *__restrict__ color,
-                                                          unsigned long long *__restrict__ counts) {
-  __shared__ float4 s_xyab[kBatch];
-  __shared__ float2 s_co[kBatch];
-  __shared__ float4 s_rgb[kBatch];
-  const int tid = threadIdx.x, tile = blockIdx.x;
-  int px, py;
-  quad_of(tile, cam.gx, tid, px, py);
-  const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
+// Measurement only: replay the forward's decisions for regions of 16 x 8 pixels and count, over all pixels, the list
+// entries evaluated (until each pixel stopped) and the pairs composited; and per region the entries walked until all of
+// its pixels stopped and those among them that none of its live pixels accepted.
+// counts[0] += evaluated, counts[1] += composited, counts[2] += (region, entry) steps, counts[3] += steps without a taker.
+__global__ void __launch_bounds__(32) k_blend_count(CamDev cam, const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ vals,
+                                                    const float *__restrict__ mean2d, const float *__restrict__ conic_opacity,
+                                                    const float *__restrict__ color, unsigned long long *__restrict__ counts) {
+  constexpr int NPX = 4;
+  __shared__ RawEntries raw;
+  __shared__ StagedEntries st;
+  const int lane = threadIdx.x, tile = blockIdx.x / 2;
+  int rx, ry;
+  region_of<NPX>(tile, cam.gx, blockIdx.x % 2, rx, ry);
+  const int px = rx + NPX * (lane & 3), py = ry + (lane >> 2);
+  const float2 fx[2] = {make_float2((float)px + 0.5f, (float)px + 1.5f), make_float2((float)px + 2.5f, (float)px + 3.5f)};
   const uint32_t start = __ldg(ranges + 2 * tile), end = __ldg(ranges + 2 * tile + 1);
-  float T[4] = {1.f, 1.f, 1.f, 1.f};
+  float T[NPX];
   unsigned live = 0;
   unsigned long long evaluated = 0, composited = 0, steps = 0, idle = 0;
 #pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (px + (k & 1) < cam.W && py + (k >> 1) < cam.H) live |= 1u << k;
-  for (uint32_t base = start; base < end; base += kBatch) {
-    if (__syncthreads_and(live == 0)) break;
-#pragma unroll
-    for (int h = 0; h < kBatch / kThreads; ++h) {
-      const int slot = tid + h * kThreads;
-      const uint32_t idx = base + slot;
-      if (idx < end) stage_entry(__ldg(vals + idx), mean2d, conic_opacity, color, s_xyab[slot], s_co[slot], s_rgb[slot]);
-    }
-    __syncthreads();
-    const int cnt = (int)min((uint32_t)kBatch, end - base);
+  for (int k = 0; k < NPX; ++k) {
+    T[k] = 1.f;
+    if (px + k < cam.W && py < cam.H) live |= 1u << k;
+  }
+  for (uint32_t base = start; base < end && __any_sync(kFull, live != 0u); base += 32) {
+    const int cnt = (int)min(32u, end - base);
+    if (lane < cnt) fetch_entry(raw, lane, __ldg(vals + base + lane), mean2d, conic_opacity, color);
+    copies_wait();
+    bool clamp;
+    stage_entries<0, 1>(raw, st, lane, lane < cnt, 0u, 0u, 0.f, 0.f, clamp);
     for (int j = 0; j < cnt; ++j) {
-      if (!__any_sync(kFull, live != 0)) break;
-      const float4 a = s_xyab[j];
-      const float2 c = s_co[j];
-      float p[4], t1[4], t2[2];
-      quad_power(fx - a.x, fy - a.y, a.z, a.w, c.x, p, t1, t2);
-      const float4 col = s_rgb[j];
+      if (!__any_sync(kFull, live != 0u)) break;
+      float2 alpha[2];
+      alphas<NPX>(st.shape[j], st.rest[j], fx, (float)py + 0.5f, alpha);
       evaluated += __popc(live);
       bool taken = false;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        float e2, raw, alpha;
-        if (!((live >> k) & 1u) || !alpha_of(p[k], c.y, col.w, e2, raw, alpha)) continue;
+      for (int k = 0; k < NPX; ++k) {
+        const float al = get(alpha[k / 2], k % 2);
+        if (!((live >> k) & 1u) || al < kAlphaMin) continue;
         taken = true;
-        const float Tn = __fadd_rn(T[k], -__fmul_rn(alpha, T[k]));
-        if (Tn < kTmin) { live &= ~(1u << k); continue; }
-        T[k] = Tn;
+        const float n = __fmul_rn(T[k], __fadd_rn(1.f, -fminf(kAlphaMax, al)));
+        if (!(n >= kTmin)) { live &= ~(1u << k); continue; }
+        T[k] = n;
         ++composited;
       }
       ++steps;
       if (!__any_sync(kFull, taken)) ++idle;
     }
+    __syncwarp();
   }
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) {
     evaluated += __shfl_xor_sync(kFull, evaluated, s);
     composited += __shfl_xor_sync(kFull, composited, s);
   }
-  if ((tid & 31) == 0) {
+  if (lane == 0) {
     atomicAdd(counts, evaluated); atomicAdd(counts + 1, composited);
-    atomicAdd(counts + 2, steps); atomicAdd(counts + 3, idle);     // warp-uniform: one lane speaks for the warp
+    atomicAdd(counts + 2, steps); atomicAdd(counts + 3, idle);     // the same in every lane
   }
 }
 
@@ -489,7 +593,7 @@ __global__ void __launch_bounds__(kThreads) k_blend_count(CamDev cam, const uint
 
 int launch_blend_count(const CamDev &cam, const uint32_t *ranges, const uint32_t *vals, const float *mean2d,
                        const float *conic_opacity, const float *color, unsigned long long *counts, cudaStream_t st) {
-  k_blend_count<<<cam.gx * cam.gy, kThreads, 0, st>>>(cam, ranges, vals, mean2d, conic_opacity, color, counts);
+  k_blend_count<<<2 * cam.gx * cam.gy, 32, 0, st>>>(cam, ranges, vals, mean2d, conic_opacity, color, counts);
   return 1;
 }
 
@@ -497,8 +601,8 @@ int launch_blend_fwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *
                      const float *mean2d,
                      const float *conic_opacity, const float *color, uint32_t *sorted_tiles, float *image, float *final_T,
                      uint32_t *n_contrib, cudaStream_t st) {
-  launch_chained(k_blend_fwd, cam.gx * cam.gy, kThreads, 0, st, cam, ranges, order, vals, mean2d, conic_opacity, color, sorted_tiles, image,
-                 final_T, n_contrib);
+  launch_chained(k_blend_fwd, cam.gx * cam.gy * Share<kFwdPixels>::kWarps, 32, 0, st, cam, ranges, order, vals, mean2d, conic_opacity,
+                 color, sorted_tiles, image, final_T, n_contrib);
   return 1;
 }
 
@@ -506,8 +610,14 @@ int launch_blend_bwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *
                      const float *mean2d,
                      const float *conic_opacity, const float *color, const float *final_T,
                      const uint32_t *n_contrib, const float *dL_dimage, float *g2d, cudaStream_t st) {
-  k_blend_bwd<<<cam.gx * cam.gy, kThreads, 0, st>>>(cam, ranges, order, vals, mean2d, conic_opacity, color, final_T,
-                                                    n_contrib, dL_dimage, g2d);
+  const int tiles = cam.gx * cam.gy;
+  auto launch = [&](auto kernel, int warps) {
+    kernel<<<tiles * warps, 32, 0, st>>>(cam, ranges, order, vals, mean2d, conic_opacity, color, final_T, n_contrib, dL_dimage, g2d);
+  };
+  // (the measurements behind the two lines are at the kernel)
+  if (tiles <= 64) launch(k_blend_bwd<1>, Share<1>::kWarps);
+  else if (tiles <= 3000) launch(k_blend_bwd<2>, Share<2>::kWarps);
+  else launch(k_blend_bwd<4>, Share<4>::kWarps);
   return 1;
 }
 
