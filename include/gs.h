@@ -181,7 +181,7 @@ typedef struct {
   float *sv_sites;        /* SV:     [n,7,7] with respect to the raw site parameters            */
 } GsGrads;
 
-/* Create / destroy a context on CUDA device `device`.  The context owns 32 bytes of counters
+/* Create / destroy a context on CUDA device `device`.  The context owns 64 bytes of counters
  * (device and pinned host) and 7.5 MB of device memory for the per-CTA partial sums of the decoder
  * gradient.  Not thread safe: use one context per host thread, and one per stream whose calls may
  * overlap on the GPU.  Returns GS_ERR_CUDA if the device cannot be used. */
@@ -215,6 +215,11 @@ GsStatus gs_preprocess_async(GsContext *ctx, const GsScene *scene, const GsCamer
  * pair_capacity (no write ever leaves the caller's buffers), the image of that view is wrong, and a
  * flag is set that gs_async_status reports. */
 #define GS_PAIRS_ON_DEVICE ((int64_t)-1)
+/* The instance count of the context's last gs_render_forward with GS_PAIRS_ON_DEVICE, as soon as it is known: waits until
+ * that view's preprocess is done, not for the kernels behind it.  A caller that queues a view first and asks afterwards
+ * has the count without ever leaving the GPU idle; a count above pair_capacity means the view's lists were cut off.  Not
+ * for views replayed from a CUDA graph: their reports carry the number of the view that was captured. */
+GsStatus gs_async_pairs(GsContext *ctx, int64_t *num_pairs_host, void *stream);
 /* Waits for `stream`, then returns GS_ERR_CAPACITY if any device-counted view on this context
  * overflowed its pair_capacity since the last call (and clears the flag), GS_ERR_INTERNAL if a kernel
  * gave up a bounded wait on one of its own bulk copies (never expected; the waits exist so that a
@@ -351,7 +356,8 @@ GsStatus gs_neural_prepass(GsContext *ctx, const GsScene *scene, const uint16_t 
  * At most 4096 stage records are kept between two collects; further ones are dropped. */
 typedef enum {
   GS_STAGE_PREPROCESS_FWD = 0, /* projection + fused colour decode                              */
-  GS_STAGE_DEPTH_SORT,         /* radix sort of the Gaussians by depth key                      */
+  GS_STAGE_DEPTH_SORT,         /* radix sort of the Gaussians by depth key (scenes of up to 32768 Gaussians: the
+                                  whole binning, which is one kernel and the expansion there)   */
   GS_STAGE_TILE_OFFSETS,       /* (the sums of tiles touched are taken by the depth sort's last pass: no time of its own) */
   GS_STAGE_KEYGEN,             /* instance emission                                             */
   GS_STAGE_TILE_SORT,          /* radix sort of the instances by tile id                        */

@@ -75,6 +75,8 @@ _lib.gs_preprocess_async.argtypes = [_vp, C.POINTER(GsScene), C.POINTER(GsCamera
 _lib.gs_preprocess_async.restype = C.c_int
 _lib.gs_async_status.argtypes = [_vp, _vp]
 _lib.gs_async_status.restype = C.c_int
+_lib.gs_async_pairs.argtypes = [_vp, C.POINTER(C.c_int64), _vp]
+_lib.gs_async_pairs.restype = C.c_int
 GS_PAIRS_ON_DEVICE = -1
 _lib.gs_render_forward.argtypes = [_vp, C.c_int64, C.POINTER(GsProjected), C.POINTER(GsCamera), C.c_int64,
                                    C.c_int64, C.POINTER(GsBinning), _vp, _vp, _vp, _vp, C.c_size_t, _vp]
@@ -135,8 +137,9 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 def _stream_handle(stream) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())   # current_stream().cuda_stream without the object
+    return stream.cuda_stream
 
 
 def make_camera(cam) -> GsCamera:
@@ -381,6 +384,13 @@ def gs_preprocess_async(ctx: Context, scene: "DeviceScene", cam: GsCamera, out: 
     ctx._check(_lib.gs_preprocess_async(ctx._h, C.byref(cs), C.byref(cam), C.byref(pp), _stream_handle(stream)))
 
 
+def gs_async_pairs(ctx: Context, stream=None) -> int:
+    """The instance count of the last device-counted gs_render_forward, as soon as that view's preprocess is done."""
+    pairs = C.c_int64(0)
+    ctx._check(_lib.gs_async_pairs(ctx._h, C.byref(pairs), _stream_handle(stream)))
+    return pairs.value
+
+
 def gs_async_status(ctx: Context, stream=None) -> None:
     """Wait for the stream; raise GsError(GS_ERR_CAPACITY) if a device-counted view overflowed its capacity."""
     ctx._check(_lib.gs_async_status(ctx._h, _stream_handle(stream)))
@@ -440,9 +450,13 @@ class Renderer:
         self.num_pairs = 0
 
     def forward(self, scene: DeviceScene, cam: GsCamera, stream=None) -> torch.Tensor:
-        self.num_pairs = gs_preprocess(self.ctx, scene, cam, self.proj, stream)
-        gs_render_forward(self.ctx, scene.n, self.proj, cam, self.num_pairs, self.pair_capacity, self.binning,
-                          self.image, self.final_T, self.n_contrib, self.workspace, stream)
+        """The whole view is queued before the host asks for the instance count, so the GPU does not wait for the host.
+        Raises GsError(GS_ERR_CAPACITY), and the image is not valid, if the view has more than pair_capacity instances."""
+        self.forward_async(scene, cam, stream)
+        self.num_pairs = gs_async_pairs(self.ctx, stream)
+        if self.num_pairs > self.pair_capacity:
+            gs_async_status(self.ctx, stream)        # raises, and clears the flag
+            raise GsError(GS_ERR_CAPACITY, "num_pairs exceeds pair_capacity")
         return self.image
 
     def forward_async(self, scene: DeviceScene, cam: GsCamera, stream=None) -> torch.Tensor:

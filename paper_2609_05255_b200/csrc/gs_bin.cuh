@@ -1,0 +1,214 @@
+// Device helpers shared by the two binning paths: the grid-wide kernels of gs_sort.cu and the one-cluster kernel of
+// gs_bin_cluster.cu.
+#pragma once
+#include "gs_device.cuh"
+
+namespace gs {
+namespace bin {
+
+constexpr unsigned kFull = 0xffffffffu;
+
+// Inclusive prefix sum over a warp.
+__device__ __forceinline__ uint32_t warp_inclusive(uint32_t v, int lane) {
+#pragma unroll
+  for (int s = 1; s < 32; s <<= 1) {
+    const uint32_t t = __shfl_up_sync(kFull, v, s);
+    if (lane >= s) v += t;
+  }
+  return v;
+}
+
+// Stable rank of a row of 32 elements inside its warp, for a radix sort: `count` and `lanes` point to the words of this
+// lane's digit in arrays that belong to the warp alone, both zero at the start of a tile.  Every lane sets its bit in the
+// digit's word, reads back which lanes share the digit, and takes the count so far plus the sharing lanes below it; the
+// highest of them moves the count on and clears the word.  About 30 cycles of a scheduler per row, whatever the width of
+// the digit - finding the sharing lanes by one ballot per digit bit takes 10 cycles a bit, the match instruction up to 250.
+__device__ __forceinline__ uint32_t rank_row(uint32_t *count, uint32_t *lanes, bool valid, int lane) {
+  if (valid) atomicOr(lanes, 1u << lane);
+  __syncwarp();
+  uint32_t m = 0, c = 0;
+  if (valid) { m = *lanes; c = *count; }
+  __syncwarp();
+  if (valid && (m >> lane) == 1u) { *count = c + __popc(m); *lanes = 0u; }
+  __syncwarp();
+  return c + __popc(m & ((1u << lane) - 1u));
+}
+
+// The stored records of a Gaussian (3 x 3 cells at most) to their places: all loads first, they are one cache line.
+__device__ __forceinline__ void copy_records(const uint32_t *cell_records, uint32_t g, uint32_t count, uint32_t at, uint32_t capacity,
+                                             uint32_t *rec_keys, uint32_t *rec_vals) {
+  const uint32_t *src = cell_records + (size_t)g * kCellSlots;
+  uint32_t rec[kCellSlots];
+#pragma unroll
+  for (int k = 0; k < kCellSlots; ++k) rec[k] = k < (int)count ? __ldg(src + k) : 0u;
+#pragma unroll
+  for (int k = 0; k < kCellSlots; ++k)
+    if (k < (int)count && at + k < capacity) {   // never past the buffers, even if the count was taken on the device
+      rec_keys[at + k] = rec[k];
+      rec_vals[at + k] = g;
+    }
+}
+
+// A Gaussian of more than 3 x 3 cells: its cell records worked out again by the whole warp - per row of cells four lanes
+// take the four tile rows, then the lanes take one cell each.  emit(place, cell, mask) is called for record number
+// `place` of the Gaussian, counted on from `first`, by the lane that owns it.
+template <class Emit>
+__device__ __forceinline__ void big_footprint(uint32_t g, uint32_t first, const uint16_t *rect, const float *mean2d,
+                                              const float *conic_opacity, int cgx, int W, int H, int lane, Emit &&emit) {
+  const ushort4 r = __ldg(reinterpret_cast<const ushort4 *>(rect) + g);
+  const float2 m = __ldg(reinterpret_cast<const float2 *>(mean2d) + g);
+  const float4 q = __ldg(reinterpret_cast<const float4 *>(conic_opacity) + g);
+  TileSpans sp;
+  sp.setup(m.x, m.y, q.x, q.y, q.z, footprint_tau(q.w), W, H);
+  const int cy0 = r.y >> 2, cy1 = ((int)r.w - 1) >> 2;
+  uint32_t p = first;
+  for (int cy = cy0; cy <= cy1; ++cy) {
+    // lanes 0..3: the tile rows of this row of cells
+    int xa = 0, xb = 0;
+    const int ty = 4 * cy + lane;
+    const bool has = lane < 4 && ty >= (int)r.y && ty < (int)r.w && sp.row(ty, r.x, r.z, xa, xb);
+    int lo = has ? (xa >> 2) : (1 << 30), hi = has ? ((xb - 1) >> 2) : -1;
+    lo = min(lo, __shfl_xor_sync(kFull, lo, 1)); hi = max(hi, __shfl_xor_sync(kFull, hi, 1));
+    lo = min(lo, __shfl_xor_sync(kFull, lo, 2)); hi = max(hi, __shfl_xor_sync(kFull, hi, 2));
+    lo = __shfl_sync(kFull, lo, 0); hi = __shfl_sync(kFull, hi, 0);
+    if (hi < lo) continue;
+    int ra[4], rb[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      ra[k] = __shfl_sync(kFull, has ? xa : 0, k);
+      rb[k] = __shfl_sync(kFull, has ? xb : 0, k);
+    }
+    for (int cb = lo; cb <= hi; cb += 32) {
+      const int cx = cb + lane;
+      if (cx <= hi) {
+        uint32_t mask = 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int a0 = max(ra[k], 4 * cx) - 4 * cx, b0 = min(rb[k], 4 * cx + 4) - 4 * cx;
+          if (b0 > a0) mask |= (((1u << (b0 - a0)) - 1u) << a0) << (4 * k);
+        }
+        emit(p + (uint32_t)(cx - lo), (uint32_t)(cy * cgx + cx), mask);
+      }
+    }
+    p += (uint32_t)(hi - lo + 1);
+  }
+}
+
+// The 16 tile counts of the records a lane holds (masks of up to 8 records), as four words of four byte counters:
+// one multiplication spreads the four bits of a tile row of the cell over the four bytes of a word.
+__device__ __forceinline__ uint32_t spread_row(uint32_t mask, int r) { return (((mask >> (4 * r)) & 15u) * 0x00204081u) & 0x01010101u; }
+__device__ __forceinline__ void count_masks(const uint32_t mask[8], uint32_t acc[4]) {
+  acc[0] = acc[1] = acc[2] = acc[3] = 0u;
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[r] += spread_row(mask[k], r);
+}
+
+// Sum over the warp of the byte counters, widened to 16 bits on the way (8 records x 32 lanes = 256 at most): tile
+// 4 r + b of the cell ends in bits [16 (b & 1), +16) of word r * 2 + (b >> 1), in every lane.
+__device__ __forceinline__ void warp_sum_counts(const uint32_t acc[4], uint32_t out[8]) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    out[2 * r] = (acc[r] & 0xffu) | ((acc[r] & 0xff00u) << 8);
+    out[2 * r + 1] = ((acc[r] >> 16) & 0xffu) | ((acc[r] >> 8) & 0xff0000u);
+  }
+#pragma unroll
+  for (int w = 0; w < 8; ++w)
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) out[w] += __shfl_xor_sync(kFull, out[w], s);
+}
+__device__ __forceinline__ uint32_t tile_count_of(const uint32_t sums[8], int t) {   // t = 4 r + b
+  return (sums[2 * (t >> 2) + ((t & 3) >> 1)] >> (16 * (t & 1))) & 0xffffu;
+}
+
+__device__ __forceinline__ void store_if(bool p, uint32_t *addr, uint32_t v) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.global.u32 [%1], %2;\n\t}" :: "r"((uint32_t)p), "l"(addr), "r"(v) : "memory");
+}
+
+// A warp writes the instances of its 8 x 32 records (consecutive in depth order, 32 at a time).  A record's slot in the
+// list of tile t is the tile's running position plus the number of lower lanes that also list t: the 16
+// indicator bits of a lane's mask are spread over four words of byte counters and one warp-wide prefix sum of those
+// four words ranks all 16 tiles at once (at most 32 per byte).  `mine`: lane t < 16 passes where tile t continues; every
+// lane keeps all 16 running positions.
+__device__ __forceinline__ void expand_records(const uint32_t mask[8], const uint32_t gid[8], uint32_t mine, uint32_t capacity,
+                                               uint32_t *out_vals, int lane) {
+  uint32_t cur[16];
+#pragma unroll
+  for (int t = 0; t < 16; ++t) cur[t] = __shfl_sync(kFull, mine, t);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const uint32_t m = mask[k];
+    if (__ballot_sync(kFull, m != 0u) == 0u) continue;
+    uint32_t incl[4], own[4], tot[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      own[r] = spread_row(m, r);
+      incl[r] = own[r];
+    }
+#pragma unroll
+    for (int sft = 1; sft < 32; sft <<= 1) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const uint32_t u = __shfl_up_sync(kFull, incl[r], sft);
+        if (lane >= sft) incl[r] += u;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) tot[r] = __shfl_sync(kFull, incl[r], 31);
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      const int r = t >> 2, sh = 8 * (t & 3);
+      // one predicated store (no branch): the lane lists tile t and the slot lies inside the buffer
+      const uint32_t pos = cur[t] + (((incl[r] - own[r]) >> sh) & 0xffu);
+      store_if(((m >> t) & 1u) != 0u && pos < capacity, out_vals + pos, gid[k]);
+      cur[t] += (tot[r] >> sh) & 0xffu;
+    }
+  }
+}
+
+// By one CTA of 1024 threads: the exclusive scan of the tile counts in tile order = the tile ranges, and the launch
+// order of the blend's warps (tiles by decreasing list length in log2 buckets: the long tiles start first and the short
+// ones fill the tail; the order inside a bucket is whatever the atomics give, it affects scheduling only, never a result).
+struct TileScan { uint32_t w[32], cnt[33], off[33]; };
+__device__ __forceinline__ void tile_scan(TileScan &s, const uint32_t *tile_counts, int num_tiles, uint32_t capacity,
+                                          uint32_t *tile_starts, uint32_t *ranges, uint32_t *order) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < 33) s.cnt[tid] = 0;
+  __syncthreads();
+  // thread t takes the tiles [t per, (t + 1) per): one pass over its counts, one scan of the thread sums
+  const int per = (num_tiles + 1023) / 1024, first = tid * per, last = min(first + per, num_tiles);
+  uint32_t sum = 0;
+  for (int t = first; t < last; ++t) {
+    const uint32_t v = __ldcg(tile_counts + t);
+    sum += v;
+    atomicAdd(&s.cnt[v ? 32 - __clz(v) : 0], 1u);
+  }
+  const uint32_t inc = warp_inclusive(sum, lane);
+  if (lane == 31) s.w[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t w = s.w[lane];
+    s.w[lane] = warp_inclusive(w, lane) - w;
+  }
+  if (tid == 0) {
+    uint32_t off = 0;
+    for (int b = 32; b >= 0; --b) { s.off[b] = off; off += s.cnt[b]; }
+  }
+  __syncthreads();
+  uint32_t start = s.w[warp] + inc - sum;
+  for (int t = first; t < last; ++t) {
+    const uint32_t v = __ldcg(tile_counts + t);
+    tile_starts[t] = start;
+    // a tile without instances: (0, 0); never past the capacity of the instance buffers (a device-side count may
+    // exceed it: the lists are then cut off and the host is told)
+    const uint32_t s0 = min(start, capacity), e0 = start + v < start ? capacity : min(start + v, capacity);
+    ranges[2 * t] = e0 > s0 ? s0 : 0u;
+    ranges[2 * t + 1] = e0 > s0 ? e0 : 0u;
+    order[atomicAdd(&s.off[v ? 32 - __clz(v) : 0], 1u)] = (uint32_t)t;
+    start += v;
+  }
+}
+
+}  // namespace bin
+}  // namespace gs

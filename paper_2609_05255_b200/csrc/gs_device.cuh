@@ -52,7 +52,9 @@ struct PreprocessArgs {
   float *mean2d, *conic_opacity, *color, *extent;
   uint32_t *depth_key, *tiles_touched, *cell_count, *cell_records;
   uint16_t *rect;
-  unsigned long long *pair_counter;
+  unsigned long long *pair_counter;   // [0] receives the instance count; [1] zero before and after: the sum so far (40 bits)
+                                      // and the CTAs that have added to it (24 bits)
+  unsigned long long *timeout; // set to 1 if a bounded wait on a bulk copy ran out (never expected)
 };
 int launch_preprocess_fwd(int app, const PreprocessArgs &a, const CamDev &cam, cudaStream_t st);
 
@@ -110,6 +112,25 @@ int launch_variant_bwd(int hidden, int layers, int nfeat, const AppearanceArgs &
 int launch_unfused_prepare(int64_t n, const float *means, const CamDev &cam, const float *g2d, const uint32_t *mask,
                            float *dirs, float *g_color, cudaStream_t st);
 
+// What the first kernel after a device-counted preprocess does with the instance count: it tells the host - `host` is a
+// word of pinned memory that receives the view's number (24 bits) above the count (40 bits): one store, nothing to wait for
+// - and raises the flag if the lists will be cut off.
+constexpr int kCountBits = 40;
+struct CountReport {
+  const unsigned long long *count;             // null: nothing to report
+  unsigned long long capacity;
+  uint32_t *overflow;
+  unsigned long long *host, view;
+#ifdef __CUDACC__
+  __device__ __forceinline__ void send() const {
+    if (!count) return;
+    const unsigned long long c = *count;
+    if (c > capacity) *overflow = 1u;
+    *reinterpret_cast<volatile unsigned long long *>(host) = view << kCountBits | c;
+  }
+#endif
+};
+
 constexpr int kWgradBlocks = 592;   // persistent blocks of the decoder-gradient kernels (4 x 148)
 
 // Sorting / binning.
@@ -136,7 +157,7 @@ size_t sort_scratch_bytes(int64_t count);
 int launch_radix_sort(const uint32_t *keys_in, const uint32_t *vals_in, uint32_t *keys_out,
                        uint32_t *vals_out, uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t count,
                        const unsigned long long *count_dev, int first_bit, int num_bits, int max_digit_bits, void *scratch,
-                       const SortEpilogue *epilogue, cudaStream_t st);
+                       const SortEpilogue *epilogue, const CountReport &report, cudaStream_t st);
 int radix_passes(int num_bits, int max_digit_bits);   // passes launch_radix_sort makes over num_bits key bits
 size_t scan_scratch_bytes(int64_t n);
 int num_scan_blocks(int64_t n);   // entries of the block sums that launch_emit_records reads
@@ -144,15 +165,34 @@ int launch_emit_records(const uint32_t *depth_order, const uint32_t *cell_count,
                         const uint16_t *rect, const float *mean2d, const float *conic_opacity, const uint32_t *block_sums,
                         uint32_t *rec_keys, uint32_t *rec_vals, unsigned long long *rec_total, uint32_t *overflow, int64_t n,
                         int cgx, int W, int H, int64_t capacity, cudaStream_t st);
-// Scratch of the expansion: chunk_first [cells + 1], chunk_counts and chunk_bases [max_chunks, 16], tile_counts and
+// Scratch of the expansion: chunk_first [cells + 1], chunk_counts and chunk_bases [max_pieces, 16], tile_counts and
 // tile_starts [tiles].
 struct CellScratch { uint32_t *chunk_first, *chunk_counts, *chunk_bases, *tile_counts, *tile_starts; };
-int max_chunks(int64_t record_capacity, int num_cells);
+int max_pieces(int64_t record_capacity, int num_cells);   // of kBinPiece records (the grid-wide expansion works in larger chunks)
 int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint32_t *cell_ranges, const CellScratch &cs,
                   int64_t record_capacity, int64_t pair_capacity, int gx, int gy, int cgx, int cgy,
                   uint32_t *sorted_vals, uint32_t *tile_ranges, uint32_t *tile_order, cudaStream_t st);
+// The whole binning in one cluster of CTAs and one expansion kernel (gs_bin_cluster.cu), for scenes that do not fill the
+// chip.  Up to 2^kClusterDigit cells.
+constexpr int kClusterDigit = 9;              // widest digit of its sorts
+constexpr int kClusterMax = 32768;            // Gaussians (2048 per CTA of the largest cluster)
+constexpr int kBinPiece = 256;                // records of one cell that a warp counts and expands
+struct ClusterBinArgs {
+  uint32_t n, capacity;                        // Gaussians; records the buffers hold
+  uint32_t pair_capacity32;
+  CountReport report;
+  uint32_t *overflow;
+  const uint32_t *depth_key, *cell_count, *cell_records;
+  const uint16_t *rect;
+  const float *mean2d, *conic_opacity;
+  uint32_t *keys, *order, *tmp_keys, *tmp_vals;                            // [n]
+  uint32_t *rec_keys, *rec_vals, *sorted_rec_keys, *sorted_rec_vals;       // [capacity]
+  uint32_t *cell_ranges, *piece_first, *piece_counts, *piece_bases, *tile_counts, *tile_starts;
+  uint32_t *tile_ranges, *tile_order, *out_vals;
+  int num_cells, cell_bits, cgx, gx, gy, W, H;
+};
+int launch_bin_cluster(const ClusterBinArgs &a, int ctas, int64_t record_bound, cudaStream_t st);
 int launch_empty_binning(uint32_t *tile_ranges, uint32_t *tile_order, int num_tiles, cudaStream_t st);
-void launch_flag_if_greater(const unsigned long long *value, unsigned long long bound, uint32_t *flag, cudaStream_t st);
 
 // Blend.
 // (sorted_tiles: the tile id of every instance of the sorted list, written by the tile's CTA on its way in)

@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_fwd(PreprocessArgs a, Cam
     if (slab_by_copy) {
       __syncwarp();                         // lane 0 has initialised the barrier
       arrived = __all_sync(kFull, bulk::wait(bulk::smem_addr(sBar + warp), 0u));
-      if (!arrived && lane == 0) atomicExch(a.pair_counter + 3, 1ull);   // reported by gs_async_status
+      if (!arrived && lane == 0) atomicExch(a.timeout, 1ull);   // reported by gs_async_status
     } else if (__any_sync(kFull, vis) && a.deg > 0 && row0 + 32 > a.n) {   // the ragged last warp
       warp_load_rows<RowOf<APP>::value>(a.sh_rest, row0, a.n, slab, lane);
     }
@@ -641,7 +641,12 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_fwd(PreprocessArgs a, Cam
     unsigned int tot = 0;
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) tot += sPairs[w];
-    if (tot) atomicAdd(a.pair_counter, (unsigned long long)tot);
+    // one atomic carries the sum and the number of CTAs it holds: the last CTA writes the count and leaves the sum at zero
+    const unsigned long long before = atomicAdd(a.pair_counter + 1, (1ull << 40) | tot);
+    if ((before >> 40) == gridDim.x - 1) {
+      a.pair_counter[0] = (before & ((1ull << 40) - 1)) + tot;
+      a.pair_counter[1] = 0ull;
+    }
   }
 }
 

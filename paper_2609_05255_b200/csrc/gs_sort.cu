@@ -9,17 +9,18 @@
 //     records, one scan for the start of every tile and of every chunk inside it, then each chunk writes its
 //     instances, the lanes that share a tile finding their slots with one ballot.
 // The result is the instance list ordered by (tile, depth key, index), with its per-tile ranges.
-#include "gs_device.cuh"
+#include "gs_bin.cuh"
 
 namespace gs {
 namespace {
+
+using namespace bin;
 
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kItems = 16;
 constexpr int kSortTile = kSortThreads * kItems;   // 4096 elements per block iteration
 constexpr int kMaxSortBlocks = 444;                // 3 resident CTAs x 148 SMs: one full wave
-constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxDigitBits = 11;  // widest radix digit: 2048 bins
 constexpr int kScanBlock = 256;   // Gaussians per block of the tiles-touched prefix sum and per CTA of the instance emission
 
@@ -68,8 +69,9 @@ __device__ __forceinline__ BlockRange block_range(int64_t count) {
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *__restrict__ keys, int64_t count,
                                                              const unsigned long long *__restrict__ count_dev,
                                                              int shift, int bits,
-                                                             uint32_t *__restrict__ table, SortEpilogue ep) {
+                                                             uint32_t *__restrict__ table, SortEpilogue ep, CountReport report) {
   dependency_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) report.send();
   // the arrays the scatter of this pass accumulates into start from their neutral values
   if (ep.block_sums)
     for (int i = blockIdx.x * kSortThreads + threadIdx.x; i < ep.num_block_sums; i += gridDim.x * kSortThreads) ep.block_sums[i] = 0u;
@@ -315,10 +317,6 @@ __global__ void __launch_bounds__(kSortThreads, BITS <= 9 ? 3 : 2) k_radix_scatt
   }
 }
 
-__global__ void k_flag_if_greater(const unsigned long long *__restrict__ value, unsigned long long bound, uint32_t *__restrict__ flag) {
-  if (*value > bound) *flag = 1u;
-}
-
 __global__ void k_iota(uint32_t *__restrict__ out, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (uint32_t)i;
@@ -326,8 +324,8 @@ __global__ void k_iota(uint32_t *__restrict__ out, int n) {
 
 // ---- cell records in depth order ---------------------------------------------------------------
 // Every Gaussian, in depth order, writes its records (cell id << 16 | tile mask) and its id.  A Gaussian of at most
-// 3 x 3 cells copies what the preprocess stored; a larger one is worked out again by its whole warp: per row of cells
-// four lanes take the four tile rows, then the lanes take one cell each.
+// 3 x 3 cells copies what the preprocess stored; a larger one is worked out again by a warp.  The large ones are the near
+// ones, side by side in this order, so a CTA collects its own and shares them out over its warps.
 __global__ void __launch_bounds__(kScanBlock) k_emit_records(
     const uint32_t *__restrict__ order, const uint32_t *__restrict__ cell_count, const uint32_t *__restrict__ cell_records,
     const uint16_t *__restrict__ rect, const float *__restrict__ mean2d, const float *__restrict__ conic_opacity,
@@ -336,6 +334,8 @@ __global__ void __launch_bounds__(kScanBlock) k_emit_records(
     uint32_t *__restrict__ overflow) {
   dependency_wait();
   __shared__ uint32_t s_w[kScanBlock / 32], s_before[kScanBlock / 32];
+  __shared__ uint32_t s_big[kScanBlock], s_big_at[kScanBlock], s_num_big;
+  if (threadIdx.x == 0) s_num_big = 0u;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t i = (int64_t)blockIdx.x * kScanBlock + tid;
   uint32_t g = 0, cc = 0;
@@ -367,62 +367,21 @@ __global__ void __launch_bounds__(kScanBlock) k_emit_records(
     *rec_total = (unsigned long long)off + cnt;
     if (off + cnt > capacity) *overflow = 1u;                    // more records than the buffers hold: tell the host
   }
-  if (cnt && !(cc & kCellBig)) {
-    const uint32_t *src = cell_records + (size_t)g * kCellSlots;
-    for (uint32_t k = 0; k < cnt; ++k) {
-      if (off + k < capacity) {   // never past the buffers, even if the count was taken on the device
-        rec_keys[off + k] = __ldg(src + k);
-        rec_vals[off + k] = g;
-      }
-    }
+  if (cnt && !(cc & kCellBig)) copy_records(cell_records, g, cnt, off, capacity, rec_keys, rec_vals);
+  if (cc & kCellBig) {
+    const uint32_t slot = atomicAdd(&s_num_big, 1u);
+    s_big[slot] = g;
+    s_big_at[slot] = off;
   }
-  uint32_t big = __ballot_sync(kFull, (cc & kCellBig) != 0u);
-  while (big) {
-    const int src = __ffs(big) - 1;
-    big &= big - 1;
-    const uint32_t s_g = __shfl_sync(kFull, g, src);
-    uint32_t p = __shfl_sync(kFull, off, src);
-    // the owner's projected values reach every lane by a broadcast load
-    const ushort4 r = __ldg(reinterpret_cast<const ushort4 *>(rect) + s_g);
-    const float2 m = __ldg(reinterpret_cast<const float2 *>(mean2d) + s_g);
-    const float4 q = __ldg(reinterpret_cast<const float4 *>(conic_opacity) + s_g);
-    TileSpans sp;
-    sp.setup(m.x, m.y, q.x, q.y, q.z, footprint_tau(q.w), W, H);
-    const int cy0 = r.y >> 2, cy1 = ((int)r.w - 1) >> 2;
-    for (int cy = cy0; cy <= cy1; ++cy) {
-      // lanes 0..3: the tile rows of this row of cells
-      int xa = 0, xb = 0;
-      const int ty = 4 * cy + lane;
-      const bool has = lane < 4 && ty >= (int)r.y && ty < (int)r.w && sp.row(ty, r.x, r.z, xa, xb);
-      int lo = has ? (xa >> 2) : (1 << 30), hi = has ? ((xb - 1) >> 2) : -1;
-      lo = min(lo, __shfl_xor_sync(kFull, lo, 1)); hi = max(hi, __shfl_xor_sync(kFull, hi, 1));
-      lo = min(lo, __shfl_xor_sync(kFull, lo, 2)); hi = max(hi, __shfl_xor_sync(kFull, hi, 2));
-      lo = __shfl_sync(kFull, lo, 0); hi = __shfl_sync(kFull, hi, 0);
-      if (hi < lo) continue;
-      int ra[4], rb[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        ra[k] = __shfl_sync(kFull, has ? xa : 0, k);
-        rb[k] = __shfl_sync(kFull, has ? xb : 0, k);
+  __syncthreads();
+  for (uint32_t b = warp; b < s_num_big; b += kScanBlock / 32) {
+    const uint32_t bg = s_big[b];
+    big_footprint(bg, s_big_at[b], rect, mean2d, conic_opacity, cgx, W, H, lane, [&](uint32_t dst, uint32_t cell, uint32_t mask) {
+      if (dst < capacity) {
+        rec_keys[dst] = (cell << 16) | mask;
+        rec_vals[dst] = bg;
       }
-      for (int cb = lo; cb <= hi; cb += 32) {
-        const int cx = cb + lane;
-        if (cx <= hi) {
-          uint32_t mask = 0u;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int a0 = max(ra[k], 4 * cx) - 4 * cx, b0 = min(rb[k], 4 * cx + 4) - 4 * cx;
-            if (b0 > a0) mask |= (((1u << (b0 - a0)) - 1u) << a0) << (4 * k);
-          }
-          const uint32_t dst = p + (uint32_t)(cx - lo);
-          if (dst < capacity) {
-            rec_keys[dst] = ((uint32_t)(cy * cgx + cx) << 16) | mask;
-            rec_vals[dst] = s_g;
-          }
-        }
-      }
-      p += (uint32_t)(hi - lo + 1);
-    }
+    });
   }
 }
 
@@ -488,35 +447,6 @@ __device__ __forceinline__ bool chunk_of(uint32_t q, const uint32_t *__restrict_
   return true;
 }
 
-// The 16 tile counts of the records a lane holds (masks of up to 8 records), as four words of four byte counters:
-// one multiplication spreads the four bits of a tile row of the cell over the four bytes of a word.
-__device__ __forceinline__ void count_masks(const uint32_t mask[8], int have, uint32_t acc[4]) {
-  acc[0] = acc[1] = acc[2] = acc[3] = 0u;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const uint32_t m = k < have ? mask[k] : 0u;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) acc[r] += (((m >> (4 * r)) & 15u) * 0x00204081u) & 0x01010101u;
-  }
-}
-
-// Sum over the warp of the byte counters, widened to 16 bits on the way (8 records x 32 lanes = 256 at most): tile
-// 4 r + b of the cell ends in bits [16 (b & 1), +16) of word r * 2 + (b >> 1), in every lane.
-__device__ __forceinline__ void warp_sum_counts(const uint32_t acc[4], uint32_t out[8]) {
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    out[2 * r] = (acc[r] & 0xffu) | ((acc[r] & 0xff00u) << 8);
-    out[2 * r + 1] = ((acc[r] >> 16) & 0xffu) | ((acc[r] >> 8) & 0xff0000u);
-  }
-#pragma unroll
-  for (int w = 0; w < 8; ++w)
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) out[w] += __shfl_xor_sync(kFull, out[w], s);
-}
-__device__ __forceinline__ uint32_t tile_count_of(const uint32_t sums[8], int t) {   // t = 4 r + b
-  return (sums[2 * (t >> 2) + ((t & 3) >> 1)] >> (16 * (t & 1))) & 0xffffu;
-}
-
 constexpr int kExpandThreads = 256;
 constexpr int kExpandWarps = kExpandThreads / 32;
 
@@ -539,7 +469,7 @@ __global__ void __launch_bounds__(kExpandThreads) k_chunk_counts(const uint32_t 
     mask[k] = idx < end ? (__ldg(rec_keys + idx) & 0xffffu) : 0u;
   }
   uint32_t acc[4], sums[8];
-  count_masks(mask, 8, acc);
+  count_masks(mask, acc);
   warp_sum_counts(acc, sums);
   if (lane < 16) s_cnt[warp][lane] = tile_count_of(sums, lane);
   __syncthreads();
@@ -578,71 +508,16 @@ __global__ void __launch_bounds__(256) k_cell_prefix(const uint32_t *__restrict_
   if (tx < gx && ty < gy) tile_counts[ty * gx + tx] = run;
 }
 
-// One CTA: the exclusive scan of the tile counts in tile order = the tile ranges, and the launch order of the blend
-// CTAs (tiles by decreasing list length in log2 buckets: the long tiles start first and the short ones fill the tail;
-// the order inside a bucket is whatever the atomics give, it affects scheduling only, never a result).
 __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t *__restrict__ tile_counts, int num_tiles, uint32_t capacity,
                                                     uint32_t *__restrict__ tile_starts, uint32_t *__restrict__ ranges,
                                                     uint32_t *__restrict__ order) {
   dependency_wait();
-  __shared__ uint32_t s_w[32];
-  __shared__ uint32_t s_cnt[33], s_off[33];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < 33) s_cnt[tid] = 0;
-  __syncthreads();
-  // thread t takes the tiles [t per, (t + 1) per): one pass over its counts, one scan of the thread sums
-  const int per = (num_tiles + 1023) / 1024, first = tid * per, last = min(first + per, num_tiles);
-  uint32_t sum = 0;
-  for (int t = first; t < last; ++t) {
-    const uint32_t v = tile_counts[t];
-    sum += v;
-    atomicAdd(&s_cnt[v ? 32 - __clz(v) : 0], 1u);
-  }
-  uint32_t inc = sum;
-#pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const uint32_t u = __shfl_up_sync(kFull, inc, s);
-    if (lane >= s) inc += u;
-  }
-  if (lane == 31) s_w[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t w = s_w[lane], winc = w;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const uint32_t u = __shfl_up_sync(kFull, winc, s);
-      if (lane >= s) winc += u;
-    }
-    s_w[lane] = winc - w;
-  }
-  if (tid == 0) {
-    uint32_t off = 0;
-    for (int b = 32; b >= 0; --b) { s_off[b] = off; off += s_cnt[b]; }
-  }
-  __syncthreads();
-  uint32_t start = s_w[warp] + inc - sum;
-  for (int t = first; t < last; ++t) {
-    const uint32_t v = tile_counts[t];
-    tile_starts[t] = start;
-    // a tile without instances: (0, 0); never past the capacity of the instance buffers (a device-side count may
-    // exceed it: the lists are then cut off and the host is told)
-    const uint32_t s0 = min(start, capacity), e0 = start + v < start ? capacity : min(start + v, capacity);
-    ranges[2 * t] = e0 > s0 ? s0 : 0u;
-    ranges[2 * t + 1] = e0 > s0 ? e0 : 0u;
-    order[atomicAdd(&s_off[v ? 32 - __clz(v) : 0], 1u)] = (uint32_t)t;
-    start += v;
-  }
+  __shared__ TileScan s;
+  tile_scan(s, tile_counts, num_tiles, capacity, tile_starts, ranges, order);
 }
 
-__device__ __forceinline__ void store_if(bool p, uint32_t *addr, uint32_t v) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.global.u32 [%1], %2;\n\t}" :: "r"((uint32_t)p), "l"(addr), "r"(v) : "memory");
-}
-
-// Per chunk: write its instances.  A warp's records are consecutive in depth order, 32 at a time.  A record's slot
-// in the list of tile t is the tile's running position plus the number of lower lanes that also list t: the 16
-// indicator bits of a lane's mask are spread over four words of byte counters and one warp-wide prefix sum of those
-// four words ranks all 16 tiles at once (at most 32 per byte).  The running positions start from the tile's range,
-// the chunk's offset inside it and what the warps before this one hold; every lane keeps all 16 of them.
+// Per chunk: write its instances.  The running positions of the tiles start from the tile's range, the chunk's offset
+// inside it and what the warps before this one hold.
 __global__ void __launch_bounds__(kExpandThreads) k_expand(const uint32_t *__restrict__ rec_keys, const uint32_t *__restrict__ rec_vals,
                                                            const uint32_t *__restrict__ cell_ranges,
                                                            const uint32_t *__restrict__ chunk_first, int num_cells,
@@ -664,11 +539,11 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand(const uint32_t *__res
     gid[k] = ok ? __ldg(rec_vals + idx) : 0u;
   }
   uint32_t acc[4], sums[8];
-  count_masks(mask, 8, acc);
+  count_masks(mask, acc);
   warp_sum_counts(acc, sums);
   if (lane < 16) s_cnt[warp][lane] = tile_count_of(sums, lane);
   __syncthreads();
-  // lane t < 16 works out where tile t of the cell continues, then every lane takes a copy of all 16
+  // lane t < 16 works out where tile t of the cell continues
   const int tx0 = 4 * (cell % cgx), ty0 = 4 * (cell / cgx);
   uint32_t mine = 0;
   if (lane < 16) {
@@ -678,38 +553,7 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand(const uint32_t *__res
       for (int w = 0; w < warp; ++w) mine += s_cnt[w][lane];
     }
   }
-  uint32_t cur[16];
-#pragma unroll
-  for (int t = 0; t < 16; ++t) cur[t] = __shfl_sync(kFull, mine, t);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const uint32_t m = mask[k];
-    if (__ballot_sync(kFull, m != 0u) == 0u) continue;
-    uint32_t incl[4], own[4], tot[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      own[r] = (((m >> (4 * r)) & 15u) * 0x00204081u) & 0x01010101u;
-      incl[r] = own[r];
-    }
-#pragma unroll
-    for (int sft = 1; sft < 32; sft <<= 1) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const uint32_t u = __shfl_up_sync(kFull, incl[r], sft);
-        if (lane >= sft) incl[r] += u;
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) tot[r] = __shfl_sync(kFull, incl[r], 31);
-#pragma unroll
-    for (int t = 0; t < 16; ++t) {
-      const int r = t >> 2, sh = 8 * (t & 3);
-      // one predicated store (no branch): the lane lists tile t and the slot lies inside the buffer
-      const uint32_t pos = cur[t] + (((incl[r] - own[r]) >> sh) & 0xffu);
-      store_if(((m >> t) & 1u) != 0u && pos < capacity, out_vals + pos, gid[k]);
-      cur[t] += (tot[r] >> sh) & 0xffu;
-    }
-  }
+  expand_records(mask, gid, mine, capacity, out_vals, lane);
 }
 
 }  // namespace
@@ -737,23 +581,23 @@ void launch_scatter(int blocks, const uint32_t *src_k, const uint32_t *src_v, ui
 int launch_radix_sort(const uint32_t *keys_in, const uint32_t *vals_in, uint32_t *keys_out, uint32_t *vals_out,
                        uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t count, const unsigned long long *count_dev,
                        int first_bit, int num_bits, int max_digit_bits, void *scratch, const SortEpilogue *epilogue,
-                       cudaStream_t st) {
+                       const CountReport &report, cudaStream_t st) {
   if (count <= 0) return 0;
-  const int blocks = sort_blocks(count);
   const int passes = radix_passes(num_bits, max_digit_bits);
   int bits = (num_bits + passes - 1) / passes;     // digits of equal width: 13 bits sort as 7 + 6 under a limit of 8
   if (bits < 4) bits = 4;                          // (bits above the keys' range are zero: sorting on them changes nothing)
+  const int blocks = sort_blocks(count);
   uint32_t *table = static_cast<uint32_t *>(scratch);
   uint32_t *totals = table + ((size_t)blocks << bits);
   const uint32_t *src_k = keys_in, *src_v = vals_in;
-  const SortEpilogue none = {nullptr, 0u, nullptr, 0, nullptr, 0, 0, nullptr};
+  const SortEpilogue none = {};
   for (int p = 0; p < passes; ++p) {
     const bool to_out = ((passes - 1 - p) % 2) == 0;
     uint32_t *dst_k = to_out ? keys_out : tmp_keys, *dst_v = to_out ? vals_out : tmp_vals;
     const SortEpilogue ep = (p == passes - 1 && epilogue) ? *epilogue : none;
     const int mode = ep.block_sums ? 1 : ep.ranges ? 2 : 0;
     const int shift = first_bit + bits * p;
-    launch_chained(k_radix_hist, blocks, kSortThreads, 0, st, src_k, count, count_dev, shift, bits, table, ep);
+    launch_chained(k_radix_hist, blocks, kSortThreads, 0, st, src_k, count, count_dev, shift, bits, table, ep, p == 0 ? report : CountReport{});
     launch_chained(k_radix_scan_rows, 1 << bits, 256, 0, st, table, blocks, totals);
 #define GS_ARGS blocks, src_k, src_v, dst_k, dst_v, count, count_dev, shift, table, totals, ep, st
 #define GS_SCATTER(B)                                             \
@@ -800,12 +644,12 @@ int launch_emit_records(const uint32_t *depth_order, const uint32_t *cell_count,
   return 1;
 }
 
-int max_chunks(int64_t record_capacity, int num_cells) { return (int)((record_capacity + kCellChunk - 1) / kCellChunk) + num_cells; }
+int max_pieces(int64_t record_capacity, int num_cells) { return (int)((record_capacity + kBinPiece - 1) / kBinPiece) + num_cells; }
 
 int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint32_t *cell_ranges, const CellScratch &cs,
                   int64_t record_capacity, int64_t pair_capacity, int gx, int gy, int cgx, int cgy,
                   uint32_t *sorted_vals, uint32_t *tile_ranges, uint32_t *tile_order, cudaStream_t st) {
-  const int num_cells = cgx * cgy, chunks = max_chunks(record_capacity, num_cells);
+  const int num_cells = cgx * cgy, chunks = (int)((record_capacity + kCellChunk - 1) / kCellChunk) + num_cells;
   const uint32_t cap = pair_capacity > 0xffffffffll ? 0xffffffffu : (uint32_t)pair_capacity;
   launch_chained(k_cell_chunks, 1, 1024, 0, st, cell_ranges, num_cells, cs.chunk_first);
   launch_chained(k_chunk_counts, chunks, kExpandThreads, 0, st, rec_keys, cell_ranges, cs.chunk_first, num_cells, cs.chunk_counts);
@@ -815,10 +659,6 @@ int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint
   launch_chained(k_expand, chunks, kExpandThreads, 0, st, rec_keys, rec_vals, cell_ranges, cs.chunk_first, num_cells, cs.chunk_bases,
                  cs.tile_starts, gx, gy, cgx, cap, sorted_vals);
   return 5;
-}
-
-void launch_flag_if_greater(const unsigned long long *value, unsigned long long bound, uint32_t *flag, cudaStream_t st) {
-  k_flag_if_greater<<<1, 1, 0, st>>>(value, bound, flag);
 }
 
 // No record was sorted (no Gaussian, or none that reaches a tile): every tile is empty.
