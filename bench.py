@@ -456,7 +456,7 @@ STAGE_KERNELS = {
     "tile_sort": "k_radix_hist, k_radix_scan_rows, k_radix_scatter<9>: one stable pass on the cell id",
     "tile_ranges": "k_cell_chunks, k_chunk_counts, k_cell_prefix, k_tile_scan, k_expand: records -> per-tile lists",
     "blend_fwd": "k_blend_fwd", "blend_bwd": "k_blend_bwd",
-    "preprocess_bwd": "k_preprocess_bwd_sparse (zero rows at once, the Gaussians with a gradient in full batches) + k_wgrad_reduce"}
+    "preprocess_bwd": "k_preprocess_bwd_sparse (the Gaussians with a gradient in full batches; the zero rows are written by k_blend_bwd) + k_wgrad_reduce"}
 
 
 def stage_roofline(stage, arm, views, n, peaks, alu_peak):

@@ -230,18 +230,19 @@ FwdWorkspace carve_fwd(void *ws, int64_t n, int64_t cap, int width, int height) 
   return w;
 }
 
-// Backward scratch: the 2D gradients [n,12], then (used by the separate-pass path only) directions, dL/dcolor and
-// dL/dd as [n,3] each, then the flags of the Gaussians that received a gradient.
-struct BwdWorkspace { float *g2d, *dirs, *g_color, *g_dirs; uint32_t *flags; size_t bytes; };
+// Backward scratch: the 2D gradients [n,12] and the flags of the Gaussians that received one (cleared together), then (used
+// by the separate-pass path only) directions, dL/dcolor and dL/dd as [n,3] each.
+struct BwdWorkspace { float *g2d, *dirs, *g_color, *g_dirs; uint32_t *flags; size_t cleared, bytes; };
 BwdWorkspace carve_bwd(void *ws, int64_t n) {
   Carver c{static_cast<char *>(ws), 0};
   const size_t nn = (size_t)(n > 0 ? n : 1);
   BwdWorkspace w;
   w.g2d = c.take<float>(nn * 12);
+  w.flags = c.take<uint32_t>((nn + 31) / 32);     // one bit per Gaussian
+  w.cleared = c.used;
   w.dirs = c.take<float>(nn * 3);
   w.g_color = c.take<float>(nn * 3);
   w.g_dirs = c.take<float>(nn * 3);
-  w.flags = c.take<uint32_t>((nn + 31) / 32);     // one bit per Gaussian: it received a gradient
   w.bytes = c.used;
   return w;
 }
@@ -543,13 +544,28 @@ GsStatus gs_render_backward(GsContext *ctx, const GsScene *scene, const GsCamera
   const BwdWorkspace bw = carve_bwd(workspace, n);
   float *g2d = bw.g2d;
   const bool ext = unfused(scene);
+  // A decoder variant on the tcgen05 kernels works on the Gaussians that received a gradient only
+  const bool gathered = ext && scene->app == GS_APP_NEURAL && !default_decoder(scene) && ctx->decoder_engine != GS_ENGINE_WARP_MMA &&
+                        scene->active_degree > 0;
   if (ext && n > 0 && bad_ptr(proj->tiles_touched)) return fail(ctx, GS_ERR_INVALID_ARG, "proj->tiles_touched is NULL or misaligned");
   if (n > 0) {
-    if ((st = check_cuda(ctx, cudaMemsetAsync(g2d, 0, (size_t)n * 12 * sizeof(float), s), "memset")) != GS_OK) return st;
+    if ((st = check_cuda(ctx, cudaMemsetAsync(g2d, 0, bw.cleared, s), "memset")) != GS_OK) return st;
+    ZeroRows zeros = {};
+    const uint64_t m = (uint64_t)n;
+    zeros.add(grads->means, 3 * m); zeros.add(grads->log_scales, 3 * m); zeros.add(grads->quats, 4 * m); zeros.add(grads->opacity_logits, m);
+    if (!ext || gathered) {    // (a dense appearance backward writes all rows itself)
+      zeros.add(grads->base_color, 3 * m);
+      if (scene->app == GS_APP_SH) zeros.add(grads->sh_rest, GS_SH_REST * m);
+      else if (scene->app == GS_APP_SV) zeros.add(grads->sv_sites, GS_SV_ROW * m);
+      else zeros.add(grads->features, decoder_arch(scene).nfeat * m);
+    }
     if (num_pairs > 0) {
       StageTimer t(ctx, GS_STAGE_BLEND_BWD, s);
       t.done(launch_blend_bwd(cd, bin->tile_ranges, bin->tile_order, bin->sorted_vals, proj->mean2d, proj->conic_opacity, proj->color,
-                              final_T, n_contrib, dL_dimage, g2d, s));
+                              final_T, n_contrib, dL_dimage, g2d, bw.flags, zeros, s));
+    } else {
+      for (int k = 0; k < zeros.count; ++k)
+        if ((st = check_cuda(ctx, cudaMemsetAsync(zeros.ptr[k], 0, zeros.floats[k] * sizeof(float), s), "memset")) != GS_OK) return st;
     }
   }
   PreprocessBwdArgs a;
@@ -559,33 +575,26 @@ GsStatus gs_render_backward(GsContext *ctx, const GsScene *scene, const GsCamera
   a.features = reinterpret_cast<const __half *>(scene->features);
   a.weights = reinterpret_cast<const __half *>(scene->mlp_weights);
   a.deg = scene->active_degree; a.act = scene->color_activation;
-  a.rect = proj->rect; a.g2d = g2d;
+  a.g2d = g2d;
   a.g_means = grads->means; a.g_log_scales = grads->log_scales; a.g_quats = grads->quats;
   a.g_logits = grads->opacity_logits; a.g_base = grads->base_color;
   a.g_sh_rest = scene->app == GS_APP_SV ? grads->sv_sites : grads->sh_rest;
   a.g_features = grads->features; a.w_partials = ctx->d_w_partials; a.g_weights = grads->mlp_weights;
   a.gd_in = bw.g_dirs;
   a.flags = bw.flags;
-  a.nfeat = scene->app == GS_APP_NEURAL ? decoder_arch(scene).nfeat : 8;
-  a.timeout = ctx->d_counter + 3;
   if (n == 0 && scene->app == GS_APP_NEURAL) {
     const DecoderArch d = decoder_arch(scene);
     return check_cuda(ctx, cudaMemsetAsync(grads->mlp_weights, 0, sizeof(float) * variant_num_weights(d.hidden, d.layers), s), "memset");
   }
-  bool flags_ready = false;
   if (ext && n > 0) {   // the appearance backward as a pass of its own, through dense arrays in the workspace
     AppearanceArgs ap = appearance_args(ctx, scene);
     ap.dirs = bw.dirs; ap.g_color = bw.g_color; ap.mask = proj->tiles_touched;
     ap.g_base = grads->base_color; ap.g_sh_rest = scene->app == GS_APP_SV ? grads->sv_sites : grads->sh_rest;
     ap.g_features = grads->features; ap.g_dirs = bw.g_dirs;
     ap.w_partials = ctx->d_w_partials; ap.g_weights = grads->mlp_weights;
-    // A decoder variant on the tcgen05 kernels works on the Gaussians that received a gradient only: the flag bits
-    // (and the zero rows of everyone else) are taken first, and serve the projection backward below as well.
-    flags_ready = scene->app == GS_APP_NEURAL && !default_decoder(scene) && ctx->decoder_engine != GS_ENGINE_WARP_MMA && scene->active_degree > 0;
     StageTimer t(ctx, GS_STAGE_APPEARANCE_BWD, s);
     int launches = 0;
-    if (flags_ready) {   // directions and dL/dcolor are taken from the means and the 2D gradient rows in the kernel itself
-      launches = launch_bwd_flags(a, true, s);
+    if (gathered) {   // directions and dL/dcolor are taken from the means and the 2D gradient rows in the kernel itself
       ap.flags = bw.flags;
       ap.means = scene->means; ap.g2d = g2d;
       ap.oc[0] = cd.oc[0]; ap.oc[1] = cd.oc[1]; ap.oc[2] = cd.oc[2];
@@ -596,7 +605,7 @@ GsStatus gs_render_backward(GsContext *ctx, const GsScene *scene, const GsCamera
   }
   {
     StageTimer t(ctx, GS_STAGE_PREPROCESS_BWD, s);
-    t.done(launch_preprocess_bwd(ext ? kAppExternal : kernel_app(scene), a, cd, s, flags_ready));
+    t.done(launch_preprocess_bwd(ext ? kAppExternal : kernel_app(scene), a, cd, s));
   }
   return check_cuda(ctx, cudaGetLastError(), "render_backward launch");
 }

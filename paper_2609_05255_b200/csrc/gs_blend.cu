@@ -303,6 +303,18 @@ __device__ __forceinline__ float select_alpha(float alpha, uint32_t pos, uint32_
   return r;
 }
 
+// One warp's slice of the rows that start as zeros.
+__device__ __forceinline__ void zero_rows(const ZeroRows &z, int lane) {
+#pragma unroll 1
+  for (int k = 0; k < z.count; ++k) {
+    float4 *p = reinterpret_cast<float4 *>(z.ptr[k]) + (uint64_t)blockIdx.x * z.slice[k];
+    const uint64_t quads = z.floats[k] >> 2, from = (uint64_t)blockIdx.x * z.slice[k];
+    const uint32_t count = from < quads ? (uint32_t)min(quads - from, (uint64_t)z.slice[k]) : 0u;
+    for (uint32_t i = lane; i < count; i += 32) __stcs(p + i, make_float4(0.f, 0.f, 0.f, 0.f));
+    if (blockIdx.x == 0 && lane < (int)(z.floats[k] & 3u)) z.ptr[k][4 * quads + lane] = 0.f;
+  }
+}
+
 // What the lanes leave of an entry: dp of their pixels and their colour sums, kBatch entries at a time.  Strides chosen
 // so that the reads of sum_entries meet no bank conflict: four lanes read neighbouring values of one entry, and the
 // eight (float4), sixteen (float2) or thirty-two (float) lanes that are served together cover all banks.
@@ -390,6 +402,12 @@ struct __align__(16) BwdArea {
 // (4 cycles each), as many adds and 14 selects, and the same sums as products on the tensor cores (tf32 operands in two
 // terms) took fewer instructions but 105 register operands instead of 55: 215 against 181 us.
 //
+// The kernel leaves the memory idle, so its warps also write what needs no arithmetic: every gradient row that is zero
+// because its Gaussian received nothing (in a scene with occlusion most of them: 94 % of the listed Gaussians of a view of
+// 1M).  All rows are zeroed here, each warp a slice on its way out
+// (on its way in, the first wave writes them all at once and the others' reads wait behind that: 23 us more at 1M); a bit per Gaussian says who received a gradient, and the
+// projection and appearance backward gathers those alone.
+//
 // 16 x 8 pixels per warp is best where the launch fills the chip (1M Gaussians, 1256 x 828: 181 us against 195 with
 // 8 x 8; 244 before); smaller regions give more warps and cull more where it does not: 8 x 8 from 2550 tiles down
 // (128 against 133 us at 2550, 69 / 68 at 1024, 30 / 39 at 294), 4 x 8 while every warp still has a scheduler of its own
@@ -400,7 +418,7 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
     CamDev cam, const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ order, const uint32_t *__restrict__ vals,
     const float *__restrict__ mean2d, const float *__restrict__ conic_opacity, const float *__restrict__ color,
     const float *__restrict__ final_T, const uint32_t *__restrict__ n_contrib, const float *__restrict__ dL_dimage,
-    float *__restrict__ g2d) {
+    float *__restrict__ g2d, uint32_t *__restrict__ flags, ZeroRows zeros) {
   using V = typename Share<NPX>::V;
   constexpr int kVecs = Share<NPX>::kVecs, kLanes = Lanes<V>::value, kWarps = Share<NPX>::kWarps, kGroup = NPX == 4 ? 1 : 4;
   __shared__ BwdArea<NPX> area;
@@ -434,7 +452,10 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
   }
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) wmax = max(wmax, __shfl_xor_sync(kFull, wmax, s));
-  if (wmax == 0 || wmax > __ldg(ranges + 2 * tile + 1) - start) return;   // nothing composited in this region
+  if (wmax == 0 || wmax > __ldg(ranges + 2 * tile + 1) - start) {   // nothing composited in this region
+    zero_rows(zeros, lane);
+    return;
+  }
   uint32_t base = (wmax - 1u) & ~31u;          // first entry of the last piece of 32
   uint32_t id = 0;
   if (base + lane < wmax) {
@@ -512,19 +533,22 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
         const float syy = fmaf(oy, s.my + sy, s.myy);
         // the staged factor is the conic's Cholesky factor times sqrt(0.5 log2 e)
         const float A = 2.f * kLn2 * sh.z * sh.z, B = 2.f * kLn2 * sh.z * sh.w, C = 2.f * kLn2 * fmaf(sh.w, sh.w, re.x * re.x);
-        float *dst = g2d + (size_t)__float_as_uint(st.rgb[slot].w) * 12;
+        const uint32_t gid = __float_as_uint(st.rgb[slot].w);
+        float *dst = g2d + (size_t)gid * 12;
         const bool touched = s.m != 0.f || s.mx != 0.f || s.my != 0.f || s.mxx != 0.f || s.mxy != 0.f || s.myy != 0.f || s.r != 0.f ||
                              s.g != 0.f || s.b != 0.f;
         if (touched) {
           if (t == 0) red_add4(dst, s.r, s.g, s.b, __fdividef(s.m, re.y));
           if (t == 1) red_add4(dst + 4, -0.5f * sxx, -sxy, -0.5f * syy, fmaf(A, sx, B * sy));
           if (t == 2) atomicAdd(dst + 8, fmaf(B, sx, C * sy));
+          if (t == 3) atomicOr(flags + (gid >> 5), 1u << (gid & 31u));
         }
       }
       __syncwarp();                              // the parked values have been read
     }
     if (base == 0u) break;
   }
+  zero_rows(zeros, lane);
 }
 
 // Measurement only: replay the forward's decisions for regions of 16 x 8 pixels and count, over all pixels, the list
@@ -609,10 +633,15 @@ int launch_blend_fwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *
 int launch_blend_bwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
                      const float *mean2d,
                      const float *conic_opacity, const float *color, const float *final_T,
-                     const uint32_t *n_contrib, const float *dL_dimage, float *g2d, cudaStream_t st) {
+                     const uint32_t *n_contrib, const float *dL_dimage, float *g2d, uint32_t *flags, const ZeroRows &zeros,
+                     cudaStream_t st) {
   const int tiles = cam.gx * cam.gy;
   auto launch = [&](auto kernel, int warps) {
-    kernel<<<tiles * warps, 32, 0, st>>>(cam, ranges, order, vals, mean2d, conic_opacity, color, final_T, n_contrib, dL_dimage, g2d);
+    ZeroRows z = zeros;
+    const uint64_t ctas = (uint64_t)tiles * warps;
+    for (int k = 0; k < z.count; ++k) z.slice[k] = (uint32_t)(((z.floats[k] >> 2) + ctas - 1) / ctas);
+    kernel<<<tiles * warps, 32, 0, st>>>(cam, ranges, order, vals, mean2d, conic_opacity, color, final_T, n_contrib, dL_dimage, g2d,
+                                        flags, z);
   };
   // (the measurements behind the two lines are at the kernel)
   if (tiles <= 64) launch(k_blend_bwd<1>, Share<1>::kWarps);

@@ -63,21 +63,14 @@ struct PreprocessBwdArgs {
   const float *means, *log_scales, *quats, *logits, *base_color, *sh_rest;
   const __half *features, *weights;
   int deg, act;
-  const uint16_t *rect;
   const float *g2d;            // [n,12]: dL/dcolor(3), dL/dopacity, dL/dconic(3), dL/dmean2d(2), pad
-  unsigned long long *timeout; // set to 1 if a bounded wait on a bulk copy ran out (never expected)
   const float *gd_in;          // kAppExternal only: [n,3] dL/dd from the separate appearance backward
-  uint32_t *flags;             // scratch, one bit per Gaussian: it received a gradient in this view
-  int nfeat;                   // features per Gaussian of g_features (8, or 16 for the raw-feature decoder variants)
+  const uint32_t *flags;       // one bit per Gaussian: it received a gradient in this view (only their rows are written)
   float *g_means, *g_log_scales, *g_quats, *g_logits, *g_base, *g_sh_rest, *g_features;
   float *w_partials;           // [kWgradBlocks, 816]
   float *g_weights;            // [816]
 };
-// flags_ready (kAppExternal): launch_bwd_flags has run on these arguments already.
-int launch_preprocess_bwd(int app, const PreprocessBwdArgs &a, const CamDev &cam, cudaStream_t st, bool flags_ready = false);
-// The flag bits (who received a gradient) and the zero rows of everyone else: projection gradients, and with
-// appearance_rows also base colour and features.
-int launch_bwd_flags(const PreprocessBwdArgs &a, bool appearance_rows, cudaStream_t st);
+int launch_preprocess_bwd(int app, const PreprocessBwdArgs &a, const CamDev &cam, cudaStream_t st);
 
 struct AppearanceArgs {
   int64_t n;
@@ -199,10 +192,21 @@ int launch_empty_binning(uint32_t *tile_ranges, uint32_t *tile_order, int num_ti
 int launch_blend_fwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
                       const float *mean2d, const float *conic_opacity, const float *color, uint32_t *sorted_tiles,
                       float *image, float *final_T, uint32_t *n_contrib, cudaStream_t st);
+// Gradient arrays whose rows start as zeros (16-byte aligned): the backward then writes the rows of the Gaussians that
+// received a gradient.
+struct ZeroRows {
+  static constexpr int kMost = 8;
+  float *ptr[kMost];
+  uint64_t floats[kMost];
+  uint32_t slice[kMost];        // groups of four floats that one warp writes (set by the launch)
+  int count;
+  void add(float *p, uint64_t n) { if (n) { ptr[count] = p; floats[count++] = n; } }
+};
+// Also sets the flag bit of every Gaussian that received a gradient, and fills `zeros`.
 int launch_blend_bwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
                       const float *mean2d, const float *conic_opacity, const float *color,
                       const float *final_T, const uint32_t *n_contrib, const float *dL_dimage,
-                      float *g2d, cudaStream_t st);
+                      float *g2d, uint32_t *flags, const ZeroRows &zeros, cudaStream_t st);
 
 int launch_neural_fold(int64_t n, const __half *features, const __half *weights, __half *preact, cudaStream_t st);
 int launch_neural_prepass(int64_t n, int deg, int act, const float *means, const float *logits, const float *base_color,

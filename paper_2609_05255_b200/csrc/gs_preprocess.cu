@@ -55,6 +55,12 @@ __device__ __forceinline__ void warp_store_rows(float *g, int64_t row0, int64_t 
   __syncwarp();
 }
 
+// A float on its own way into shared memory, no register held.
+__device__ __forceinline__ void copy_async4(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // ---- 1D bulk copies (tensor memory accelerator) with bounded waits ------------------------------------------
 // load(): one lane arms the warp's mbarrier with the byte count and starts the copy; wait(): every lane polls the
 // barrier's phase, at most about a second in all; store(): shared -> global as a bulk group of the issuing lane.
@@ -293,6 +299,7 @@ __device__ __forceinline__ void reload_fence() { asm volatile("" ::: "memory"); 
 constexpr int kReduceGroups = 16;
 __global__ void __launch_bounds__(32 * kReduceGroups) k_wgrad_reduce(const float *__restrict__ partials, int nblocks,
                                                                     float *__restrict__ out) {
+  dependency_wait();
   __shared__ float s_part[kReduceGroups][32];
   const int k = blockIdx.x * 32 + threadIdx.x, grp = threadIdx.y;
   float s = 0.f;
@@ -315,7 +322,7 @@ __global__ void __launch_bounds__(32 * kReduceGroups) k_wgrad_reduce(const float
   }
 }
 inline void launch_wgrad_reduce(const float *partials, int nblocks, float *out, cudaStream_t st) {
-  k_wgrad_reduce<<<(GS_MLP_WEIGHTS + 31) / 32, dim3(32, kReduceGroups), 0, st>>>(partials, nblocks, out);
+  launch_chained(k_wgrad_reduce, (GS_MLP_WEIGHTS + 31) / 32, dim3(32, kReduceGroups), 0, st, partials, nblocks, out);
 }
 
 // ---- projection -----------------------------------------------------------------------------
@@ -767,212 +774,26 @@ constexpr size_t kBwdSmemNN = sizeof(mlp::Weights) + kWarps * sizeof(mlp::WarpSt
 static_assert(kWarps * sizeof(mlp::WarpStage) >= kWarps * GS_MLP_WEIGHTS * sizeof(float), "partial sums reuse the staging areas");
 static_assert(sizeof(mlp::Weights) % 16 == 0, "staging areas must stay 16-byte aligned");
 
-template <int APP>
-__global__ void __launch_bounds__(kBlock) k_preprocess_bwd(PreprocessBwdArgs a, CamDev cam) {
-  dependency_wait();
-  extern __shared__ __align__(16) float smem[];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float *slab = smem + warp * SlabOf<APP>::value;   // SH / SV: this warp's slab of parameter rows
-  mlp::Weights &sWt = *reinterpret_cast<mlp::Weights *>(smem);
-  mlp::WarpStage *sStage = reinterpret_cast<mlp::WarpStage *>(reinterpret_cast<unsigned char *>(smem) + sizeof(mlp::Weights));
-  mlp::WeightGrad dW;
-  if (IsNeural<APP>::value) {
-    mlp::load_weights(a.weights, sWt, tid, kBlock);
-    dW.clear();
-    __syncthreads();
-  }
-  // SH / Spherical Voronoi: the warp's slab of parameter rows comes in by one bulk copy and its slab of gradient
-  // rows leaves by one (a ragged last warp uses plain loads and stores)
-  __shared__ unsigned long long sBar[kWarps];
-  uint32_t slab_parity = 0u;
-  if (Explicit<APP>::value && lane == 0) {
-    bulk::barrier_init(bulk::smem_addr(sBar + warp));
-    bulk::fence_barrier_init();
-  }
-  __syncwarp();
-  const int64_t nchunks = (a.n + kBlock - 1) / kBlock;
-  for (int64_t chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
-    reload_fence();
-    const int64_t i = chunk * kBlock + tid;
-    const int64_t row0 = chunk * kBlock + warp * 32;
-    const bool in = i < a.n;
-    // Every input row of this Gaussian is requested here, before anything depends on one of them (also for
-    // culled Gaussians, whose rows are then ignored): one memory round trip per trip of the loop instead of one
-    // per branch that needs a value.
-    bool vis = false;
-    float gd[3] = {0.f, 0.f, 0.f};
-    float mu[3] = {0.f, 0.f, 0.f}, ls[3] = {0.f, 0.f, 0.f}, q[4] = {1.f, 0.f, 0.f, 0.f}, logit = 0.f;
-    float4 ga = make_float4(0.f, 0.f, 0.f, 0.f), gb = ga, gc = ga;
-    float base_in[3] = {0.f, 0.f, 0.f};
-    uint4 feat_raw = make_uint4(0u, 0u, 0u, 0u);
-    float dx = 0.f, dy = 0.f, dz = 0.f;
-    if (in) {
-      const ushort4 rc = __ldg(reinterpret_cast<const ushort4 *>(a.rect) + i);
-      load3(a.means, i, mu);
-      load3(a.log_scales, i, ls);
-      const float4 q4 = __ldg(reinterpret_cast<const float4 *>(a.quats) + i);
-      logit = __ldg(a.logits + i);
-      const float4 *g2 = reinterpret_cast<const float4 *>(a.g2d) + 3 * i;
-      ga = g2[0]; gb = g2[1]; gc = g2[2];   // (gr, gg, gb, go) (gA, gB, gC, gu) (gv, -, -, -)
-      if (APP != kAppExternal) load3(a.base_color, i, base_in);
-      else load3(a.gd_in, i, gd);
-      if (IsNeural<APP>::value) feat_raw = __ldg(reinterpret_cast<const uint4 *>(a.features) + i);
-      q[0] = q4.x; q[1] = q4.y; q[2] = q4.z; q[3] = q4.w;
-      vis = rc.z > rc.x && rc.w > rc.y;
-    }
-    const bool warp_vis = __any_sync(kFull, vis);
-    const bool full_warp = row0 + 32 <= a.n;
-    const bool slab_by_copy = Explicit<APP>::value && warp_vis && a.deg > 0 && full_warp;
-    if (Explicit<APP>::value && lane == 0) {
-      bulk::wait_stores_read();          // an earlier trip's gradient slab has left shared memory
-      if (slab_by_copy)
-        bulk::load(bulk::smem_addr(slab), a.sh_rest + row0 * RowOf<APP>::value, SlabOf<APP>::value * sizeof(float),
-                   bulk::smem_addr(sBar + warp));
-    }
-    if (Explicit<APP>::value) __syncwarp();
-    if (vis) {
-      const float vx = mu[0] - cam.oc[0], vy = mu[1] - cam.oc[1], vz = mu[2] - cam.oc[2];
-      const float vi = rsqrtf(vx * vx + vy * vy + vz * vz);
-      dx = vx * vi; dy = vy * vi; dz = vz * vi;
-    }
-    // ---- appearance backward
-    float gp[3] = {0.f, 0.f, 0.f};
-    if (APP == kAppExternal) {
-      // dL/dd came from the separate appearance backward (zero rows for culled Gaussians)
-    } else if (Explicit<APP>::value) {
-      if (row0 < a.n) {
-        bool arrived = true;
-        if (slab_by_copy) {
-          arrived = __all_sync(kFull, bulk::wait(bulk::smem_addr(sBar + warp), slab_parity));
-          slab_parity ^= 1u;
-          if (!arrived && lane == 0 && a.timeout) atomicExch(a.timeout, 1ull);   // reported by gs_async_status
-        } else if (warp_vis && a.deg > 0) {
-          warp_load_rows<RowOf<APP>::value>(a.sh_rest, row0, a.n, slab, lane);
-        }
-        float *row = slab + lane * RowOf<APP>::value;
-        if (vis && arrived) {
-          float pre[3];
-          const float (&base)[3] = base_in;
-          SvCarry cy;
-          if (a.deg > 0) explicit_pre<APP>(row, base, dx, dy, dz, a.deg, pre, cy);
-          else { pre[0] = base[0] + 0.5f; pre[1] = base[1] + 0.5f; pre[2] = base[2] + 0.5f; }
-          gp[0] = color_act_grad_z(a.act, pre[0]) * ga.x; gp[1] = color_act_grad_z(a.act, pre[1]) * ga.y;
-          gp[2] = color_act_grad_z(a.act, pre[2]) * ga.z;
-          explicit_bwd<APP>(row, gp, dx, dy, dz, a.deg, cy, gd);
-        } else {
-#pragma unroll
-          for (int k = 0; k < RowOf<APP>::value; ++k) row[k] = 0.f;
-        }
-        if (full_warp) {
-          bulk::fence_generic_writes();     // the lanes' rows become visible to the copy engine
-          __syncwarp();
-          if (lane == 0) bulk::store(a.g_sh_rest + row0 * RowOf<APP>::value, bulk::smem_addr(slab), SlabOf<APP>::value * sizeof(float));
-        } else {
-          warp_store_rows<RowOf<APP>::value>(a.g_sh_rest, row0, a.n, slab, lane);
-        }
-      }
-    } else {
-      float gf[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      float base[3] = {0.f, 0.f, 0.f};
-      const float gcol[3] = {ga.x, ga.y, ga.z};
-      if (vis) { base[0] = base_in[0]; base[1] = base_in[1]; base[2] = base_in[2]; }
-      if (warp_vis && a.deg > 0) {   // the whole warp goes through the decoder; culled lanes feed zeros
-        float x[32];
-        if (vis) {
-          float f[8];
-          unpack_features(feat_raw, f);
-          decoder_inputs(dx, dy, dz, f, a.deg, x);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 32; ++k) x[k] = 0.f;
-        }
-        decode_backward_warp<Split<APP>::value>(sWt, sStage[warp], lane, vis, x, dx, dy, dz, a.deg, a.act, base, gcol, dW, gp, gf, gd);
-      } else if (vis) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) gp[c] = color_act_grad_z(a.act, base[c] + 0.5f) * gcol[c];
-      }
-      if (in) {
-        float4 *gfp = reinterpret_cast<float4 *>(a.g_features) + 2 * i;
-        gfp[0] = make_float4(gf[0], gf[1], gf[2], gf[3]);
-        gfp[1] = make_float4(gf[4], gf[5], gf[6], gf[7]);
-      }
-    }
-    // ---- geometry backward
-    if (in) {
-      GeoGrads gg;
-      if (vis) {
-        gg = project_backward(mu, ls, q, logit, cam, gb.x, gb.y, gb.z, gb.w, gc.x, ga.w, gd);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) { gg.mu[k] = 0.f; gg.ls[k] = 0.f; }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) gg.q[k] = 0.f;
-        gg.logit = 0.f;
-      }
-      store3(a.g_means, i, gg.mu[0], gg.mu[1], gg.mu[2]);
-      store3(a.g_log_scales, i, gg.ls[0], gg.ls[1], gg.ls[2]);
-      reinterpret_cast<float4 *>(a.g_quats)[i] = make_float4(gg.q[0], gg.q[1], gg.q[2], gg.q[3]);
-      a.g_logits[i] = gg.logit;
-      if (APP != kAppExternal) store3(a.g_base, i, gp[0], gp[1], gp[2]);
-    }
-  }
-  if (IsNeural<APP>::value) {
-    weight_grad_flush(dW, reinterpret_cast<float *>(sStage), a.w_partials + (size_t)blockIdx.x * GS_MLP_WEIGHTS, tid);
-  }
-  if (Explicit<APP>::value && lane == 0) bulk::wait_stores_done();
-}
-
 // ---- preprocess backward over the Gaussians that received a gradient -------------------------------------------
 // A Gaussian whose nine 2D gradients are all zero - culled, or listed in tiles but composited by no pixel of this view
-// because the pixels it covers saturated in front of it - gets zero gradients whatever its parameters are.  In a
-// scene with occlusion that is most of them (config 3: 94 % of the visible Gaussians of a view).  Two kernels:
-// k_bwd_flags streams over all Gaussians at full occupancy, writes the zero rows and leaves one bit per Gaussian
-// (set = it received a gradient); k_preprocess_bwd_sparse, persistent, gathers the flagged ones in index order and,
-// whenever kBlock of them are queued, runs them through the decoder and projection backward, one per thread, with
-// every lane busy.  A CTA's run of flag words is fixed by the grid, so the order of all sums is the same from run to
-// run.
-constexpr int kFlagThreads = 256;
-template <bool kBase, bool kFeatures>
-__global__ void __launch_bounds__(kFlagThreads) k_bwd_flags(PreprocessBwdArgs a) {
-  dependency_wait();
-  const int64_t i = (int64_t)blockIdx.x * kFlagThreads + threadIdx.x;
-  bool active = false;
-  if (i < a.n) {
-    const ushort4 rc = __ldg(reinterpret_cast<const ushort4 *>(a.rect) + i);
-    if (rc.z > rc.x && rc.w > rc.y) {
-      const float4 *g2 = reinterpret_cast<const float4 *>(a.g2d) + 3 * i;
-      const float4 ga = g2[0], gb = g2[1];
-      const float gv = a.g2d[12 * i + 8];
-      active = ga.x != 0.f || ga.y != 0.f || ga.z != 0.f || ga.w != 0.f || gb.x != 0.f || gb.y != 0.f || gb.z != 0.f ||
-               gb.w != 0.f || gv != 0.f;
-    }
-    if (!active) {
-      store3(a.g_means, i, 0.f, 0.f, 0.f);
-      store3(a.g_log_scales, i, 0.f, 0.f, 0.f);
-      reinterpret_cast<float4 *>(a.g_quats)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      a.g_logits[i] = 0.f;
-      if (kBase) store3(a.g_base, i, 0.f, 0.f, 0.f);
-      if (kFeatures) {
-        const int quads = a.nfeat == 16 ? 4 : 2;
-        float4 *gfp = reinterpret_cast<float4 *>(a.g_features) + quads * i;
-        for (int q = 0; q < quads; ++q) gfp[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-  }
-  const unsigned ballot = __ballot_sync(kFull, active);
-  if ((threadIdx.x & 31) == 0 && i < a.n) a.flags[i >> 5] = ballot;    // (i is a multiple of 32 here)
-}
-
+// because the pixels it covers saturated in front of it - gets zero gradients whatever its parameters are; the blend
+// backward has written those rows, and one bit per Gaussian that says who is left.  This kernel, persistent, gathers the
+// flagged ones in index order and, whenever kBlock of them are queued, runs them through the appearance and projection
+// backward, one per thread, with every lane busy.  A CTA's run of flag words is fixed by the grid, so the order of all sums
+// is the same from run to run.  What bounds it is the chain of latencies (flag words, gathered rows, decoder), not the
+// bytes: 51 k of 1M Gaussians in a view have a gradient.
+// SH and Spherical Voronoi rows are gathered and scattered row by row through the warp's slab, a row being 45 or 49
+// neighbouring floats.
 template <int APP>
 __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdArgs a, CamDev cam) {
   dependency_wait();
-  static_assert(IsNeural<APP>::value || APP == kAppExternal, "the neural model, or the projection alone");
   extern __shared__ __align__(16) float smem[];
   constexpr int kWordsPerRound = kBlock / 4;             // flag words (of 32 Gaussians) looked at per round
   __shared__ uint32_t s_queue[2 * 32 * kWordsPerRound];  // a power of two above 32 * kWordsPerRound + kBlock - 1
   __shared__ int s_warp_count[kWarps];
   constexpr int kMask = 2 * 32 * kWordsPerRound - 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float *slab = smem + warp * SlabOf<APP>::value;     // SH / SV: this warp's slab of parameter rows
   mlp::Weights &sWt = *reinterpret_cast<mlp::Weights *>(smem);
   mlp::WarpStage *sStage = reinterpret_cast<mlp::WarpStage *>(reinterpret_cast<unsigned char *>(smem) + sizeof(mlp::Weights));
   mlp::WeightGrad dW;
@@ -987,6 +808,16 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
   auto process = [&](int count) {
     const bool has = tid < count;
     const int64_t i = has ? (int64_t)s_queue[(q_head + tid) & kMask] : 0;
+    const int rows = min(32, count - warp * 32);
+    if (Explicit<APP>::value && a.deg > 0) {   // the parameter rows, on their way while the rest is loaded
+      constexpr int kRow = Explicit<APP>::value ? RowOf<APP>::value : 1;
+#pragma unroll 4
+      for (int r = 0; r < rows; ++r) {
+        const float *src = a.sh_rest + (int64_t)s_queue[(q_head + warp * 32 + r) & kMask] * kRow;
+        copy_async4(slab + r * kRow + lane, src + lane);
+        if (lane + 32 < kRow) copy_async4(slab + r * kRow + 32 + lane, src + 32 + lane);
+      }
+    }
     float gd[3] = {0.f, 0.f, 0.f};
     float mu[3] = {0.f, 0.f, 0.f}, ls[3] = {0.f, 0.f, 0.f}, q[4] = {1.f, 0.f, 0.f, 0.f}, logit = 0.f;
     float4 ga = make_float4(0.f, 0.f, 0.f, 0.f), gb = ga, gc = ga;
@@ -1009,7 +840,32 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
       dx = vx * vi; dy = vy * vi; dz = vz * vi;
     }
     float gp[3] = {0.f, 0.f, 0.f};
-    if (IsNeural<APP>::value) {
+    if (Explicit<APP>::value) {
+      constexpr int kRow = Explicit<APP>::value ? RowOf<APP>::value : 1;
+      float *row = slab + lane * kRow;
+      if (a.deg > 0) {
+        copies_wait();
+        __syncwarp();
+      }
+      if (has) {
+        float pre[3] = {base[0] + 0.5f, base[1] + 0.5f, base[2] + 0.5f};
+        SvCarry cy;
+        if (a.deg > 0) explicit_pre<APP>(row, base, dx, dy, dz, a.deg, pre, cy);
+        gp[0] = color_act_grad_z(a.act, pre[0]) * ga.x; gp[1] = color_act_grad_z(a.act, pre[1]) * ga.y;
+        gp[2] = color_act_grad_z(a.act, pre[2]) * ga.z;
+        if (a.deg > 0) explicit_bwd<APP>(row, gp, dx, dy, dz, a.deg, cy, gd);
+      }
+      if (a.deg > 0) {                          // (degree 0 leaves the zeros)
+        __syncwarp();
+#pragma unroll 4
+        for (int r = 0; r < rows; ++r) {
+          float *dst = a.g_sh_rest + (int64_t)s_queue[(q_head + warp * 32 + r) & kMask] * kRow;
+          dst[lane] = slab[r * kRow + lane];
+          if (lane + 32 < kRow) dst[32 + lane] = slab[r * kRow + 32 + lane];
+        }
+        __syncwarp();
+      }
+    } else if (IsNeural<APP>::value) {
       float gf[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       const float gcol[3] = {ga.x, ga.y, ga.z};
       if (warp * 32 < count && a.deg > 0) {     // the whole warp goes through the decoder; lanes past the count feed zeros
@@ -1043,7 +899,7 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
     }
   };
 
-  // The flags of k_bwd_flags, one bit per Gaussian, say who is left.  Every CTA takes one contiguous run of flag words
+  // Every CTA takes one contiguous run of flag words
   // (equal to within a word whatever the grid) and reads it kWordsPerRound words at a time: thread t looks at byte
   // t % 4 of word t / 4, an exclusive scan over the CTA gives its place in the queue, and it writes the indices of its
   // set bits there - index order, the same from run to run.
@@ -1343,47 +1199,26 @@ int launch_unfused_prepare(int64_t n, const float *means, const CamDev &cam, con
   return 1;
 }
 
-int launch_bwd_flags(const PreprocessBwdArgs &a, bool appearance_rows, cudaStream_t st) {
-  if (a.n == 0) return 0;
-  const int blocks = (int)((a.n + kFlagThreads - 1) / kFlagThreads);
-  if (appearance_rows) launch_chained(k_bwd_flags<true, true>, blocks, kFlagThreads, 0, st, a);
-  else launch_chained(k_bwd_flags<false, false>, blocks, kFlagThreads, 0, st, a);
-  return 1;
+namespace {
+template <int APP>
+int launch_bwd_sparse(size_t smem, const PreprocessBwdArgs &a, const CamDev &cam, cudaStream_t st) {
+  opt_in_smem(k_preprocess_bwd_sparse<APP>, smem);
+  const int wave = resident_blocks<k_preprocess_bwd_sparse<APP>>(smem, IsNeural<APP>::value ? kWgradBlocks : 1 << 20), chunks = grid_for(a.n);
+  const int blocks = chunks < wave ? chunks : wave;
+  launch_chained(k_preprocess_bwd_sparse<APP>, blocks, kBlock, smem, st, a, cam);
+  if (!IsNeural<APP>::value) return 1;
+  launch_wgrad_reduce(a.w_partials, blocks, a.g_weights, st);
+  return 2;
 }
+}  // namespace
 
-int launch_preprocess_bwd(int app, const PreprocessBwdArgs &a, const CamDev &cam, cudaStream_t st, bool flags_ready) {
-  if (app == GS_APP_SH) {
-    if (a.n == 0) return 0;
-    opt_in_smem(k_preprocess_bwd<GS_APP_SH>, kBwdSmemSH);
-    launch_chained(k_preprocess_bwd<GS_APP_SH>, grid_for(a.n), kBlock, kBwdSmemSH, st, a, cam);
-    return 1;
-  } else if (app == GS_APP_SV) {
-    if (a.n == 0) return 0;
-    opt_in_smem(k_preprocess_bwd<GS_APP_SV>, kBwdSmemSV);
-    launch_chained(k_preprocess_bwd<GS_APP_SV>, grid_for(a.n), kBlock, kBwdSmemSV, st, a, cam);
-    return 1;
-  } else if (app == kAppExternal) {
-    if (a.n == 0) return 0;
-    if (!flags_ready) launch_bwd_flags(a, false, st);
-    const int wave = resident_blocks<k_preprocess_bwd_sparse<kAppExternal>>(sizeof(mlp::Weights), 1 << 20), chunks = grid_for(a.n);
-    launch_chained(k_preprocess_bwd_sparse<kAppExternal>, chunks < wave ? chunks : wave, kBlock, sizeof(mlp::Weights), st, a, cam);
-    return flags_ready ? 1 : 2;
-  } else {
-    if (app == kAppNeuralHalf) {
-      opt_in_smem(k_preprocess_bwd_sparse<kAppNeuralHalf>, kBwdSmemNN);
-      const int blocks = resident_blocks<k_preprocess_bwd_sparse<kAppNeuralHalf>>(kBwdSmemNN);
-      if (a.n > 0) launch_chained(k_bwd_flags<true, true>, (int)((a.n + kFlagThreads - 1) / kFlagThreads), kFlagThreads, 0, st, a);
-      launch_chained(k_preprocess_bwd_sparse<kAppNeuralHalf>, blocks, kBlock, kBwdSmemNN, st, a, cam);
-      launch_wgrad_reduce(a.w_partials, blocks, a.g_weights, st);
-      return 3;
-    }
-    opt_in_smem(k_preprocess_bwd_sparse<GS_APP_NEURAL>, kBwdSmemNN);
-    const int blocks = resident_blocks<k_preprocess_bwd_sparse<GS_APP_NEURAL>>(kBwdSmemNN);
-    if (a.n > 0) launch_chained(k_bwd_flags<true, true>, (int)((a.n + kFlagThreads - 1) / kFlagThreads), kFlagThreads, 0, st, a);
-    launch_chained(k_preprocess_bwd_sparse<GS_APP_NEURAL>, blocks, kBlock, kBwdSmemNN, st, a, cam);
-    launch_wgrad_reduce(a.w_partials, blocks, a.g_weights, st);
-    return 3;
-  }
+int launch_preprocess_bwd(int app, const PreprocessBwdArgs &a, const CamDev &cam, cudaStream_t st) {
+  if (a.n == 0) return 0;
+  if (app == GS_APP_SH) return launch_bwd_sparse<GS_APP_SH>(kBwdSmemSH, a, cam, st);
+  if (app == GS_APP_SV) return launch_bwd_sparse<GS_APP_SV>(kBwdSmemSV, a, cam, st);
+  if (app == kAppExternal) return launch_bwd_sparse<kAppExternal>(sizeof(mlp::Weights), a, cam, st);
+  if (app == kAppNeuralHalf) return launch_bwd_sparse<kAppNeuralHalf>(kBwdSmemNN, a, cam, st);
+  return launch_bwd_sparse<GS_APP_NEURAL>(kBwdSmemNN, a, cam, st);
 }
 
 template <int APP, bool BWD>
