@@ -53,7 +53,7 @@ struct PreprocessArgs {
   uint32_t *depth_key, *tiles_touched, *cell_count, *cell_records;
   uint16_t *rect;
   unsigned long long *pair_counter;   // [0] receives the instance count; [1] zero before and after: the sum so far (40 bits)
-                                      // and the CTAs that have added to it (24 bits)
+                                      // and the warps that have added to it (24 bits)
   unsigned long long *timeout; // set to 1 if a bounded wait on a bulk copy ran out (never expected)
 };
 int launch_preprocess_fwd(int app, const PreprocessArgs &a, const CamDev &cam, cudaStream_t st);

@@ -329,8 +329,6 @@ inline void launch_wgrad_reduce(const float *partials, int nblocks, float *out, 
 struct Geo {
   bool valid;
   float u, v, A, B, C, o, ex, ey, tau;   // (A, B, C) = (l11, l21, l22), the Cholesky factor of the conic
-  uint32_t zbits;
-  float dirx, diry, dirz;
 };
 
 __device__ __forceinline__ void quat_rot(float r, float x, float y, float z, float R[9]) {
@@ -352,20 +350,23 @@ __device__ __forceinline__ float cov_det(const float N[6], float a, float c) {
   return cx * cx + cy * cy + cz * cz + kDilation * ((a - kDilation) + (c - kDilation)) + kDilation * kDilation;
 }
 
+// The depth: one fp32 FMA chain, identical bits on any IEEE machine.
+__device__ __forceinline__ float depth_of(const float mu[3], const CamDev &cam) {
+  return __fmaf_rn(cam.R[8], mu[2], __fmaf_rn(cam.R[7], mu[1], __fmaf_rn(cam.R[6], mu[0], cam.t[2])));
+}
+
 // Everything the backward needs again is recomputed there; this is the forward only.
 __device__ __forceinline__ Geo project(const float mu[3], const float ls[3], const float q[4],
                                        float logit, const CamDev &cam) {
   Geo g;
   g.valid = false;
-  g.zbits = 0xffffffffu;
   bool fin = finite_f(logit);
 #pragma unroll
   for (int k = 0; k < 3; ++k) fin = fin && finite_f(mu[k]) && finite_f(ls[k]);
 #pragma unroll
   for (int k = 0; k < 4; ++k) fin = fin && finite_f(q[k]);
   if (!fin) return g;
-  // the depth key: one fp32 FMA chain, identical bits on any IEEE machine
-  const float z32 = __fmaf_rn(cam.R[8], mu[2], __fmaf_rn(cam.R[7], mu[1], __fmaf_rn(cam.R[6], mu[0], cam.t[2])));
+  const float z32 = depth_of(mu, cam);
   if (!(z32 >= cam.near_plane) || !(z32 <= cam.far_plane)) return g;
   // The values that leave this function are compared with the oracle's within 1e-5-ish relative bounds; the
   // integers of the tile stage are derived from the STORED values by operations that are rounded correctly
@@ -412,14 +413,10 @@ __device__ __forceinline__ Geo project(const float mu[3], const float ls[3], con
   const float u = fmaf(cam.fx, rx, cam.cx), v = fmaf(cam.fy, ry, cam.cy);
   if (!finite_f(u) || !finite_f(v) || !finite_f(ex) || !finite_f(ey)) return g;
   g.valid = true;
-  g.zbits = __float_as_uint(z32);
   // Cholesky factor of the conic Q = cov^-1 = L L^T, straight from the covariance entries (no
   // cancellation even for needle-like splats): l22 = 1/sqrt(c), l11 = sqrt(c/det), l21 = -b/sqrt(c det)
   const float isd = rsqrtf(det), l22 = rsqrtf(c);
   g.u = u; g.v = v; g.A = c * l22 * isd; g.B = -b * l22 * isd; g.C = l22; g.o = o; g.ex = ex; g.ey = ey; g.tau = tau;
-  const float vx = mu[0] - cam.oc[0], vy = mu[1] - cam.oc[1], vz = mu[2] - cam.oc[2];
-  const float vi = rsqrtf(vx * vx + vy * vy + vz * vz);
-  g.dirx = vx * vi; g.diry = vy * vi; g.dirz = vz * vi;
   return g;
 }
 
@@ -441,90 +438,87 @@ __device__ __forceinline__ void load3(const float *p, int64_t i, float v[3]) {
   v[0] = __ldg(p + 3 * i); v[1] = __ldg(p + 3 * i + 1); v[2] = __ldg(p + 3 * i + 2);
 }
 
-// Per-warp shared memory of the cooperative tile-row evaluation: span parameters, rectangle and cell masks of the 32
-// owners, and the list of (owner << 8 | row) pairs.
-struct RowStage {
-  float par[32][8];
-  int4 geo[32];
-  uint32_t mask[32][9];
-  uint32_t tiles[32];
-  unsigned short list[32 * 12];
+// What the projection leaves of a warp's visible Gaussians for the second half of the preprocess: 64 slots in which they
+// wait until there are 32, or 32 where every lane goes on with its own.
+template <int kSlots>
+struct Projections {
+  float la[kSlots], lb[kSlots], lc[kSlots], tau[kSlots];   // la and tau become TileSpans' ila and taup
+  float2 centre[kSlots];
+  ushort4 rect[kSlots];                    // (tx0, ty0, tx1, ty1)
+  uint32_t id[kSlots];
 };
+// Per-warp shared memory of the second half's tile rows: what else TileSpans needs of the 32 owners, their
+// cell masks (sixteen bits per cell), and the owners of the rows in order, with the place of everyone's first.
+struct RowStage {
+  float dys[32], eyp[32];
+  uint32_t mask[32][5];
+  unsigned short first[32];
+  unsigned char list[32 * 12];
+};
+template <int kSlots>
+__device__ __forceinline__ TileSpans spans_of(const Projections<kSlots> &w, const RowStage &rs, int slot, int owner, const CamDev &cam) {
+  TileSpans sp;
+  sp.u = w.centre[slot].x; sp.v = w.centre[slot].y; sp.dys = rs.dys[owner]; sp.eyp = rs.eyp[owner];
+  sp.ila = w.la[slot]; sp.lb = w.lb[slot]; sp.lc = w.lc[slot]; sp.taup = w.tau[slot];
+  sp.W = cam.W; sp.H = cam.H;
+  return sp;
+}
 
+// Forward.  Every warp works on its own: it projects its run of Gaussians 32 at a time (the next ones' parameters on their
+// way) and writes what does not depend on the tiles; then the visible ones have their tiles counted and their colours
+// decoded.  What bounds it is the number of instructions (1800 a batch of 32), so idle lanes are what there is to save:
+// 60 % of a scene that surrounds the camera are culled, 12 % of one seen from outside.  With the neural model the visible
+// ones are queued and go through the second half 32 at a time, every lane busy: 3M in such a scene 255 -> 154 us, 1.5M seen
+// from outside 144 -> 125.  With SH or Spherical Voronoi every lane goes on with its own: the parameter rows of 32
+// neighbours are one piece of memory that one bulk copy brings in during the projection, and gathering them row by row
+// costs what the idle lanes do (2M SH in a scene with 60 % culled 146 us either way, 1M 84 against 95; 87 before).
+// One atomic per warp carries the instance count.
 template <int APP>
-__global__ void __launch_bounds__(kBlock) k_preprocess_fwd(PreprocessArgs a, CamDev cam) {
+__global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_preprocess_fwd(PreprocessArgs a, CamDev cam) {
   dependency_wait();
-  __shared__ __align__(16) RowStage sRows[kWarps];
-  __shared__ __align__(16) float sData[Explicit<APP>::value ? kWarps * SlabOf<APP>::value : 4];
-  __shared__ __align__(16) unsigned char sNN[IsNeural<APP>::value ? kWarps * sizeof(StageFwd) : 16];
-  StageFwd *sStage = reinterpret_cast<StageFwd *>(sNN);   // unused for SH
-  __shared__ unsigned int sPairs[kWarps];
+  constexpr bool kQueue = !Explicit<APP>::value;
+  constexpr int kSlots = kQueue ? 64 : 32;
+  // the stage of the tile rows, which the neural decoder's operands replace afterwards; the slab of parameter rows
+  constexpr size_t kStage = IsNeural<APP>::value && sizeof(StageFwd) > sizeof(RowStage) ? sizeof(StageFwd) : sizeof(RowStage);
+  __shared__ __align__(16) unsigned char sStages[kWarps][(kStage + 15) / 16 * 16];
+  __shared__ __align__(16) float sData[kQueue ? 4 : kWarps * SlabOf<APP>::value];
+  __shared__ __align__(16) Projections<kSlots> sProjections[kWarps];
   __shared__ unsigned long long sBar[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t i = (int64_t)blockIdx.x * kBlock + tid;
-  const int64_t row0 = (int64_t)blockIdx.x * kBlock + warp * 32;
-  const bool in = i < a.n;
-  Geo g;
-  g.valid = false;
-  int rect[4] = {0, 0, 0, 0};
-  bool vis = false;
-  float mu[3] = {0.f, 0.f, 0.f}, ls[3] = {0.f, 0.f, 0.f}, q[4] = {1.f, 0.f, 0.f, 0.f}, logit = 0.f;
-  if (in) {
-    load3(a.means, i, mu);
-    load3(a.log_scales, i, ls);
-    const float4 q4 = __ldg(reinterpret_cast<const float4 *>(a.quats) + i);
-    q[0] = q4.x; q[1] = q4.y; q[2] = q4.z; q[3] = q4.w;
-    logit = __ldg(a.logits + i);
+  Projections<kSlots> &wait = sProjections[warp];
+  float *slab = sData + (kQueue ? 0 : warp * SlabOf<APP>::value);   // SH / Spherical Voronoi: 32 parameter rows
+  const uint32_t bar = bulk::smem_addr(sBar + warp);
+  uint32_t parity = 0u;
+  bool copying = false, gave_up = false;      // a bulk copy is on its way; one never came
+  if (!kQueue && lane == 0) {
+    bulk::barrier_init(bar);
+    bulk::fence_barrier_init();
   }
-  // SH / Spherical Voronoi: the warp's slab of parameter rows is one contiguous piece of memory.  Unless the depth
-  // test already culls the whole warp, a bulk copy brings it in while the projection below runs (a ragged last
-  // warp uses plain loads further down).
-  bool slab_by_copy = false;
-  if (Explicit<APP>::value && a.deg > 0 && row0 + 32 <= a.n) {
-    const float z = __fmaf_rn(cam.R[8], mu[2], __fmaf_rn(cam.R[7], mu[1], __fmaf_rn(cam.R[6], mu[0], cam.t[2])));
-    slab_by_copy = __any_sync(kFull, z >= cam.near_plane && z <= cam.far_plane);
-    if (slab_by_copy && lane == 0) {
-      const uint32_t bar = bulk::smem_addr(sBar + warp);
-      bulk::barrier_init(bar);
-      bulk::fence_barrier_init();
-      bulk::load(bulk::smem_addr(sData + warp * SlabOf<APP>::value), a.sh_rest + row0 * RowOf<APP>::value,
-                 SlabOf<APP>::value * sizeof(float), bar);
+  __syncwarp();
+  unsigned int instances = 0;
+
+  // the second half for the Gaussians in the slots [head, head + 32), one per lane (`in`: this lane has one)
+  auto finish = [&](int head, bool in) {
+    RowStage &rs = *reinterpret_cast<RowStage *>(sStages[warp]);
+    const int mine = head + lane;
+    const int64_t i = in ? (int64_t)wait.id[mine] : 0;
+    float mu[3] = {0.f, 0.f, 0.f}, base[3] = {0.f, 0.f, 0.f};
+    uint4 feat_raw = make_uint4(0u, 0u, 0u, 0u);
+    const ushort4 rect = in ? wait.rect[mine] : make_ushort4(0, 0, 0, 0);
+    if (in) {                                  // for the colour, further down
+      load3(a.means, i, mu);
+      if (APP != kAppExternal) load3(a.base_color, i, base);
+      if (IsNeural<APP>::value && a.deg > 0) feat_raw = __ldg(reinterpret_cast<const uint4 *>(a.features) + i);
     }
-  }
-  if (in) {
-    g = project(mu, ls, q, logit, cam);
-    if (g.valid) vis = tile_rect(g.u, g.v, g.ex, g.ey, cam, rect);
-  }
-  // tiles the ellipse really meets inside its bounding rectangle, and the same by cells of 4 x 4 tiles: one
-  // record (cell id, mask of the tiles met) per cell, which is what the binning sorts.
-  unsigned int tiles = 0, nrec = 0;
-  bool stored = false;
-  {
-    TileSpans sp;
-    if (vis) sp.setup(g.u, g.v, g.A, g.B, g.C, g.tau, cam.W, cam.H);
-    const int cx0 = rect[0] >> 2, cx1 = (rect[2] - 1) >> 2, cy0 = rect[1] >> 2, cy1 = (rect[3] - 1) >> 2;
-    stored = vis && cx1 - cx0 <= 2 && cy1 - cy0 <= 2;          // at most 3 x 3 cells: the records fit the Gaussian's slots
-    if (vis && !stored) {
-      // a large footprint is only counted here (the record emission works its cells out again): a row of cells
-      // contributes the cells from the leftmost to the rightmost tile met in its tile rows
-      for (int cy = cy0; cy <= cy1; ++cy) {
-        int lo = 1 << 30, hi = -1;
-        const int ta = max(rect[1], 4 * cy), tb = min(rect[3], 4 * cy + 4);
-        for (int ty = ta; ty < tb; ++ty) {
-          int xa, xb;
-          if (!sp.row(ty, rect[0], rect[2], xa, xb)) continue;
-          tiles += (unsigned)(xb - xa);
-          lo = min(lo, xa >> 2); hi = max(hi, (xb - 1) >> 2);
-        }
-        if (hi >= lo) nrec += (unsigned)(hi - lo + 1);
-      }
-    }
-    // The tile rows of the other footprints are evaluated by the warp together, one (Gaussian, tile row) per lane
+    // tiles the ellipse really meets inside its bounding rectangle, and the same by cells of 4 x 4 tiles: one
+    // record (cell id, mask of the tiles met) per cell, which is what the binning sorts.
+    unsigned int tiles = 0, nrec = 0;
+    const int cx0 = rect.x >> 2, cx1 = ((int)rect.z - 1) >> 2, cy0 = rect.y >> 2, cy1 = ((int)rect.w - 1) >> 2;
+    const bool stored = in && cx1 - cx0 <= 2 && cy1 - cy0 <= 2;          // at most 3 x 3 cells: the records fit the Gaussian's slots
+    // The tile rows of the footprints are evaluated by the warp together, one (Gaussian, tile row) per lane
     // and round: lanes own very different numbers of rows (1 to 12), and a loop per lane would idle most of them.
-    // Each owner parks its span parameters and the list of its rows in shared memory; a row's tiles go into the
-    // owner's cell masks with shared-memory atomics (integer OR / add: any order gives the same bits).
-    RowStage &rs = sRows[warp];
-    const int rows = stored ? rect[3] - rect[1] : 0;
+    // A row's tiles go into the owner's cell masks with shared-memory ORs (any order gives the same bits).
+    const int rows = stored ? rect.w - rect.y : 0;
     int incl = rows;
 #pragma unroll
     for (int sft = 1; sft < 32; sft <<= 1) {
@@ -532,126 +526,198 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_fwd(PreprocessArgs a, Cam
       if (lane >= sft) incl += t;
     }
     const int total = __shfl_sync(kFull, incl, 31);
-    if (stored) {
-      float *par = rs.par[lane];
-      par[0] = sp.u; par[1] = sp.v; par[2] = sp.ila; par[3] = sp.lb; par[4] = sp.lc; par[5] = sp.taup; par[6] = sp.dys; par[7] = sp.eyp;
-      rs.geo[lane] = make_int4(rect[0], rect[2], rect[1], cx0);
+    if (in) {
+      TileSpans sp;
+      sp.setup(wait.centre[mine].x, wait.centre[mine].y, wait.la[mine], wait.lb[mine], wait.lc[mine], wait.tau[mine], cam.W, cam.H);
+      wait.la[mine] = sp.ila; wait.tau[mine] = sp.taup;
+      rs.dys[lane] = sp.dys; rs.eyp[lane] = sp.eyp;
+      rs.first[lane] = (unsigned short)(incl - rows);
 #pragma unroll
-      for (int j = 0; j < 9; ++j) rs.mask[lane][j] = 0u;
-      rs.tiles[lane] = 0u;
-      for (int k = 0; k < rows; ++k) rs.list[incl - rows + k] = (unsigned short)((lane << 8) | k);
+      for (int j = 0; j < 5; ++j) rs.mask[lane][j] = 0u;
+      for (int k = 0; k < rows; ++k) rs.list[incl - rows + k] = (unsigned char)lane;
     }
     __syncwarp();
-    for (int base = 0; base < total; base += 32) {
-      if (base + lane < total) {
-        const unsigned e = rs.list[base + lane];
-        const int o = (int)(e >> 8), k = (int)(e & 255u);
-        const float *par = rs.par[o];
-        TileSpans so;
-        so.u = par[0]; so.v = par[1]; so.ila = par[2]; so.lb = par[3]; so.lc = par[4]; so.taup = par[5]; so.dys = par[6]; so.eyp = par[7];
-        so.W = cam.W; so.H = cam.H;
-        const int4 ge = rs.geo[o];      // (tx0, tx1, ty0, first cell column)
-        const int ty = ge.z + k;
-        int xa, xb;
-        if (so.row(ty, ge.x, ge.y, xa, xb)) {
-          atomicAdd(&rs.tiles[o], (unsigned)(xb - xa));
-          // the row's tiles as bits counted from the first column of the first cell (at most 12), a nibble per cell
-          const uint32_t bits = ((1u << (xb - xa)) - 1u) << (xa - 4 * ge.w);
-          const int cyi = (ty >> 2) - (ge.z >> 2), sh = 4 * (ty & 3);
+    for (int at = lane; at < total; at += 32) {
+      const int o = rs.list[at];
+      const ushort4 r = wait.rect[head + o];
+      const int ty = r.y + at - rs.first[o];
+      int xa, xb;
+      if (spans_of(wait, rs, head + o, o, cam).row(ty, r.x, r.z, xa, xb)) {
+        // the row's tiles as bits counted from the first column of the first cell (at most 12), a nibble per cell
+        const uint32_t bits = ((1u << (xb - xa)) - 1u) << (xa - (r.x & ~3));
+        const int cell0 = 3 * ((ty >> 2) - (r.y >> 2)), sh = 4 * (ty & 3);
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const uint32_t nib = (bits >> (4 * c)) & 15u;
-            if (nib) atomicOr(&rs.mask[o][3 * cyi + c], nib << sh);
-          }
+        for (int c = 0; c < 3; ++c) {
+          const uint32_t nib = (bits >> (4 * c)) & 15u;
+          if (nib) atomicOr(&rs.mask[o][(cell0 + c) >> 1], nib << (sh + 16 * ((cell0 + c) & 1)));
         }
       }
     }
+    // A large footprint is only counted here (the record emission works its cells out again), a tile row per lane: a row
+    // of cells contributes the cells from the leftmost to the rightmost tile met in its four tile rows.
+    for (uint32_t big = __ballot_sync(kFull, in && !stored); big; big &= big - 1) {
+      const int o = __ffs(big) - 1;
+      const ushort4 r = wait.rect[head + o];
+      const TileSpans sp = spans_of(wait, rs, head + o, o, cam);
+      unsigned t = 0, c = 0;
+      for (int ty0 = r.y & ~3; ty0 < r.w; ty0 += 32) {
+        const int ty = ty0 + lane;
+        int xa = 0, xb = 0;
+        const bool has = ty >= r.y && ty < r.w && sp.row(ty, r.x, r.z, xa, xb);
+        int lo = has ? xa >> 2 : 1 << 30, hi = has ? (xb - 1) >> 2 : -1;
+        lo = min(lo, __shfl_xor_sync(kFull, lo, 1)); hi = max(hi, __shfl_xor_sync(kFull, hi, 1));
+        lo = min(lo, __shfl_xor_sync(kFull, lo, 2)); hi = max(hi, __shfl_xor_sync(kFull, hi, 2));
+        if (has) t += (unsigned)(xb - xa);
+        if ((lane & 3) == 0 && hi >= lo) c += (unsigned)(hi - lo + 1);
+      }
+      t = __reduce_add_sync(kFull, t); c = __reduce_add_sync(kFull, c);
+      if (lane == o) { tiles = t; nrec = c; }
+    }
     __syncwarp();
     if (stored) {
-      tiles = rs.tiles[lane];
       uint32_t *slot = a.cell_records + (size_t)i * kCellSlots;
 #pragma unroll
       for (int j = 0; j < 9; ++j) {
-        const uint32_t m = rs.mask[lane][j];
+        const uint32_t m = (rs.mask[lane][j >> 1] >> (16 * (j & 1))) & 0xffffu;
+        tiles += (unsigned)__popc(m);
         if (m) slot[nrec++] = ((uint32_t)((cy0 + j / 3) * cam.cgx + cx0 + j % 3) << 16) | m;
       }
     }
-    if (vis && tiles == 0) { vis = false; nrec = 0; rect[0] = rect[1] = rect[2] = rect[3] = 0; }
-  }
-  // ---- fused colour decode for the Gaussians that survived culling
-  float pre[3] = {0.f, 0.f, 0.f};
-  if (Explicit<APP>::value) {   // SH or Spherical Voronoi: parameter rows through the warp's slab
-    float *slab = sData + warp * SlabOf<APP>::value;
-    bool arrived = true;
-    if (slab_by_copy) {
-      __syncwarp();                         // lane 0 has initialised the barrier
-      arrived = __all_sync(kFull, bulk::wait(bulk::smem_addr(sBar + warp), 0u));
-      if (!arrived && lane == 0) atomicExch(a.timeout, 1ull);   // reported by gs_async_status
-    } else if (__any_sync(kFull, vis) && a.deg > 0 && row0 + 32 > a.n) {   // the ragged last warp
-      warp_load_rows<RowOf<APP>::value>(a.sh_rest, row0, a.n, slab, lane);
+    const bool vis = tiles > 0;
+    if (!vis) nrec = 0;
+    __syncwarp();
+    // ---- fused colour decode
+    float pre[3] = {base[0] + 0.5f, base[1] + 0.5f, base[2] + 0.5f};
+    float dx = 0.f, dy = 0.f, dz = 0.f;
+    if (vis) {
+      const float vx = mu[0] - cam.oc[0], vy = mu[1] - cam.oc[1], vz = mu[2] - cam.oc[2];
+      const float vi = rsqrtf(vx * vx + vy * vy + vz * vz);
+      dx = vx * vi; dy = vy * vi; dz = vz * vi;
     }
-    if (vis && arrived) {
-      float base[3];
-      load3(a.base_color, i, base);
-      SvCarry cy;
-      explicit_pre<APP>(slab + lane * RowOf<APP>::value, base, g.dirx, g.diry, g.dirz, a.deg, pre, cy);
+    if (Explicit<APP>::value) {   // SH or Spherical Voronoi
+      if (copying) {
+        if (!__all_sync(kFull, bulk::wait(bar, parity))) gave_up = true;
+        parity ^= 1u;
+      }
+      if (vis && !gave_up) {
+        SvCarry cy;
+        explicit_pre<APP>(slab + lane * RowOf<APP>::value, base, dx, dy, dz, a.deg, pre, cy);
+      }
+    } else if (IsNeural<APP>::value) {
+      if (a.deg > 0 && __any_sync(kFull, vis)) {   // the whole warp decodes; culled lanes feed zeros
+        float x[32], A[3];
+        if (vis) {
+          float f[8];
+          unpack_features(feat_raw, f);
+          decoder_inputs(dx, dy, dz, f, a.deg, x);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 32; ++k) x[k] = 0.f;
+        }
+        mlp::Activations act;
+        // the lane's 14 words of the forward's weight operands come straight from global memory (1.6 KB that stay in L1)
+        const mlp::FwdFrags F = mlp::load_fwd_frags(a.weights, lane);
+        decode_warp<Split<APP>::value>(F, *reinterpret_cast<StageFwd *>(sStages[warp]), lane, x, act, A);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) pre[c] += A[c];
+      }
     }
-  } else if (IsNeural<APP>::value) {
-    float A[3] = {0.f, 0.f, 0.f};
-    if (a.deg > 0 && __any_sync(kFull, vis)) {   // the whole warp decodes; culled lanes feed zeros
-      float x[32];
+    if (in) {
       if (vis) {
-        float f[8];
-        load_features(a.features, i, f);
-        decoder_inputs(g.dirx, g.diry, g.dirz, f, a.deg, x);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) x[k] = 0.f;
+        if (APP == kAppExternal) {   // the separate appearance pass reads the direction here and writes the colour over it
+          a.color[3 * i] = dx; a.color[3 * i + 1] = dy; a.color[3 * i + 2] = dz;
+        } else {
+          a.color[3 * i] = color_act_z(a.act, pre[0]); a.color[3 * i + 1] = color_act_z(a.act, pre[1]); a.color[3 * i + 2] = color_act_z(a.act, pre[2]);
+        }
       }
-      mlp::Activations act;
-      // the lane's 14 words of the forward's weight operands come straight from global memory (1.6 KB that stay in L1)
-      const mlp::FwdFrags F = mlp::load_fwd_frags(a.weights, lane);
-      decode_warp<Split<APP>::value>(F, sStage[warp], lane, x, act, A);
+      a.depth_key[i] = vis ? __float_as_uint(depth_of(mu, cam)) : 0xffffffffu;
+      a.tiles_touched[i] = tiles;
+      a.cell_count[i] = nrec | ((nrec && !stored) ? kCellBig : 0u);
+      if (!vis) reinterpret_cast<ushort4 *>(a.rect)[i] = make_ushort4(0, 0, 0, 0);
     }
+    instances += tiles;
+    __syncwarp();
+  };
+
+  const int64_t warps = (int64_t)gridDim.x * kWarps;
+  const int64_t per = ((a.n + warps - 1) / warps + 31) & ~(int64_t)31;
+  const int64_t begin = min(a.n, ((int64_t)blockIdx.x * kWarps + warp) * per), end = min(a.n, begin + per);
+  float mu[3] = {0.f, 0.f, 0.f}, ls[3], logit;
+  float4 q4;
+  auto load = [&](int64_t i) {
+    if (i < end) {
+      load3(a.means, i, mu);
+      load3(a.log_scales, i, ls);
+      q4 = __ldg(reinterpret_cast<const float4 *>(a.quats) + i);
+      logit = __ldg(a.logits + i);
+    }
+  };
+  load(begin + lane);
+  int head = 0, waiting = 0;                       // the same in every lane
+  for (int64_t i0 = begin; i0 < end || waiting > 0; i0 += 32) {
+    reload_fence();
+    const int64_t i = i0 + lane;
+    bool vis = false;
+    Geo g;
+    int rect[4];
+    ushort4 tiles4 = make_ushort4(0, 0, 0, 0);
+    if (!kQueue && a.deg > 0) {
+      // the slab of parameter rows, unless the depth test culls the whole warp (the ragged last rows by plain loads)
+      const float z = depth_of(mu, cam);
+      const bool wanted = __any_sync(kFull, i < end && z >= cam.near_plane && z <= cam.far_plane);
+      copying = wanted && i0 + 32 <= end;
+      if (copying && lane == 0) bulk::load(bulk::smem_addr(slab), a.sh_rest + i0 * RowOf<APP>::value, SlabOf<APP>::value * sizeof(float), bar);
+      if (wanted && !copying) warp_load_rows<RowOf<APP>::value>(a.sh_rest, i0, a.n, slab, lane);
+    }
+    if (i < end) {
+      const float q[4] = {q4.x, q4.y, q4.z, q4.w};
+      g = project(mu, ls, q, logit, cam);
+      load(i + 32);
+      if (g.valid) {   // also for footprints that reach no tile: the tile stage is checked from these values
+        vis = tile_rect(g.u, g.v, g.ex, g.ey, cam, rect);
+        reinterpret_cast<float2 *>(a.mean2d)[i] = make_float2(g.u, g.v);
+        reinterpret_cast<float4 *>(a.conic_opacity)[i] = make_float4(g.A, g.B, g.C, g.o);
+      }
+      if (a.extent) reinterpret_cast<float4 *>(a.extent)[i] = g.valid ? make_float4(g.ex, g.ey, g.tau, 0.f) : make_float4(-1.f, -1.f, 0.f, 0.f);
+      if (!vis) {
+        a.depth_key[i] = 0xffffffffu;
+        a.tiles_touched[i] = 0u;
+        a.cell_count[i] = 0u;
+        rect[0] = rect[1] = rect[2] = rect[3] = 0;
+      }
+      tiles4 = make_ushort4((unsigned short)rect[0], (unsigned short)rect[1], (unsigned short)rect[2], (unsigned short)rect[3]);
+      reinterpret_cast<ushort4 *>(a.rect)[i] = tiles4;
+    }
+    const uint32_t found = __ballot_sync(kFull, vis);
     if (vis) {
-      float base[3];
-      load3(a.base_color, i, base);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) pre[c] = base[c] + 0.5f + A[c];
+      const int slot = kQueue ? (head + waiting + __popc(found & ((1u << lane) - 1u))) & 63 : lane;
+      wait.la[slot] = g.A; wait.lb[slot] = g.B; wait.lc[slot] = g.C; wait.tau[slot] = g.tau;
+      wait.centre[slot] = make_float2(g.u, g.v); wait.rect[slot] = tiles4; wait.id[slot] = (uint32_t)i;
+    }
+    __syncwarp();
+    if (kQueue) {
+      waiting += __popc(found);
+      if (waiting >= 32 || i0 + 32 >= end) {
+        const int count = min(waiting, 32);
+        if (count > 0) finish(head, lane < count);
+        head ^= 32;
+        waiting -= count;
+      }
+    } else if (found) {
+      finish(0, vis);
+    } else if (copying) {                          // not wanted after all
+      if (!__all_sync(kFull, bulk::wait(bar, parity))) gave_up = true;
+      parity ^= 1u;
     }
   }
-  if (in) {
-    if (g.valid) {   // also for footprints that reach no tile: the tile stage is checked from these values
-      reinterpret_cast<float2 *>(a.mean2d)[i] = make_float2(g.u, g.v);
-      reinterpret_cast<float4 *>(a.conic_opacity)[i] = make_float4(g.A, g.B, g.C, g.o);
-    }
-    if (vis) {
-      if (APP == kAppExternal) {   // the separate appearance pass reads the direction here and writes the colour over it
-        a.color[3 * i] = g.dirx; a.color[3 * i + 1] = g.diry; a.color[3 * i + 2] = g.dirz;
-      } else {
-        a.color[3 * i] = color_act_z(a.act, pre[0]); a.color[3 * i + 1] = color_act_z(a.act, pre[1]); a.color[3 * i + 2] = color_act_z(a.act, pre[2]);
-      }
-    }
-    a.depth_key[i] = vis ? g.zbits : 0xffffffffu;
-    a.tiles_touched[i] = tiles;
-    a.cell_count[i] = nrec | ((nrec && !stored) ? kCellBig : 0u);   // (vis was cleared if no tile is met: nrec = 0)
-    reinterpret_cast<ushort4 *>(a.rect)[i] = make_ushort4((unsigned short)rect[0], (unsigned short)rect[1],
-                                                          (unsigned short)rect[2], (unsigned short)rect[3]);
-    if (a.extent) reinterpret_cast<float4 *>(a.extent)[i] = g.valid ? make_float4(g.ex, g.ey, g.tau, 0.f) : make_float4(-1.f, -1.f, 0.f, 0.f);
-  }
-  // ---- total number of (Gaussian, tile) instances
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) tiles += __shfl_xor_sync(kFull, tiles, s);
-  if (lane == 0) sPairs[warp] = tiles;
-  __syncthreads();
-  if (tid == 0) {
-    unsigned int tot = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) tot += sPairs[w];
-    // one atomic carries the sum and the number of CTAs it holds: the last CTA writes the count and leaves the sum at zero
-    const unsigned long long before = atomicAdd(a.pair_counter + 1, (1ull << 40) | tot);
-    if ((before >> 40) == gridDim.x - 1) {
-      a.pair_counter[0] = (before & ((1ull << 40) - 1)) + tot;
+  if (gave_up && lane == 0) atomicExch(a.timeout, 1ull);   // reported by gs_async_status
+  // ---- total number of (Gaussian, tile) instances: one atomic carries the sum and the number of warps it holds; the last
+  // warp writes the count and leaves the sum at zero
+  instances = __reduce_add_sync(kFull, instances);
+  if (lane == 0) {
+    const unsigned long long before = atomicAdd(a.pair_counter + 1, (1ull << 40) | instances);
+    if ((before >> 40) == (unsigned long long)warps - 1) {
+      a.pair_counter[0] = (before & ((1ull << 40) - 1)) + instances;
       a.pair_counter[1] = 0ull;
     }
   }
@@ -1182,14 +1248,22 @@ int resident_blocks(size_t smem_bytes, int cap = kWgradBlocks) {
 
 }  // namespace
 
+namespace {
+template <int APP>
+int launch_fwd(const PreprocessArgs &a, const CamDev &cam, cudaStream_t st) {
+  const int wave = resident_blocks<k_preprocess_fwd<APP>>(0, 1 << 20), chunks = grid_for(a.n);
+  launch_chained(k_preprocess_fwd<APP>, chunks < wave ? chunks : wave, kBlock, 0, st, a, cam);
+  return 1;
+}
+}  // namespace
+
 int launch_preprocess_fwd(int app, const PreprocessArgs &a, const CamDev &cam, cudaStream_t st) {
   if (a.n == 0) return 0;
-  if (app == GS_APP_SH) launch_chained(k_preprocess_fwd<GS_APP_SH>, grid_for(a.n), kBlock, 0, st, a, cam);
-  else if (app == GS_APP_SV) launch_chained(k_preprocess_fwd<GS_APP_SV>, grid_for(a.n), kBlock, 0, st, a, cam);
-  else if (app == kAppExternal) launch_chained(k_preprocess_fwd<kAppExternal>, grid_for(a.n), kBlock, 0, st, a, cam);
-  else if (app == kAppNeuralHalf) launch_chained(k_preprocess_fwd<kAppNeuralHalf>, grid_for(a.n), kBlock, 0, st, a, cam);
-  else launch_chained(k_preprocess_fwd<GS_APP_NEURAL>, grid_for(a.n), kBlock, 0, st, a, cam);
-  return 1;
+  if (app == GS_APP_SH) return launch_fwd<GS_APP_SH>(a, cam, st);
+  if (app == GS_APP_SV) return launch_fwd<GS_APP_SV>(a, cam, st);
+  if (app == kAppExternal) return launch_fwd<kAppExternal>(a, cam, st);
+  if (app == kAppNeuralHalf) return launch_fwd<kAppNeuralHalf>(a, cam, st);
+  return launch_fwd<GS_APP_NEURAL>(a, cam, st);
 }
 
 int launch_unfused_prepare(int64_t n, const float *means, const CamDev &cam, const float *g2d, const uint32_t *mask,
