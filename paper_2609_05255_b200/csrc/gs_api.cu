@@ -199,6 +199,7 @@ struct FwdWorkspace {
   uint32_t *cell_ranges;                                 // [cells, 2]
   CellScratch cells;
   unsigned long long *rec_total;                         // number of records, written by the emission
+  uint32_t *num_big;                                     // of the one-cluster binning
   void *sort_table;
   size_t bytes;
 };
@@ -225,6 +226,7 @@ FwdWorkspace carve_fwd(void *ws, int64_t n, int64_t cap, int width, int height) 
   w.cells.tile_counts = c.take<uint32_t>((size_t)gx * gy);
   w.cells.tile_starts = c.take<uint32_t>((size_t)gx * gy);
   w.rec_total = c.take<unsigned long long>(1);
+  w.num_big = c.take<uint32_t>(1);
   w.sort_table = c.take<char>(sort_scratch_bytes((int64_t)(nn > cc ? nn : cc)));
   w.bytes = c.used;
   return w;
@@ -450,7 +452,7 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
   // 103.  A CTA for every 64 Gaussians, up to 16 (1000 Gaussians: 33 us on 16 CTAs, 36 on 4).
   if (sorted && n <= kClusterMax && num_cells <= (1 << kClusterDigit)) {
     ClusterBinArgs b = {};
-    b.n = (uint32_t)n; b.capacity = cap32; b.pair_capacity32 = cap32; b.report = report; b.overflow = overflow;
+    b.n = (uint32_t)n; b.capacity = cap32; b.pair_capacity32 = cap32; b.report = report; b.overflow = overflow; b.num_big = w.num_big;
     b.depth_key = proj->depth_key; b.cell_count = proj->cell_count; b.cell_records = proj->cell_records; b.rect = proj->rect;
     b.mean2d = proj->mean2d; b.conic_opacity = proj->conic_opacity;
     b.keys = w.sorted_depth; b.order = bin->depth_order; b.tmp_keys = w.tmp_keys; b.tmp_vals = w.tmp_vals;

@@ -34,21 +34,6 @@ __device__ __forceinline__ uint32_t rank_row(uint32_t *count, uint32_t *lanes, b
   return c + __popc(m & ((1u << lane) - 1u));
 }
 
-// The stored records of a Gaussian (3 x 3 cells at most) to their places: all loads first, they are one cache line.
-__device__ __forceinline__ void copy_records(const uint32_t *cell_records, uint32_t g, uint32_t count, uint32_t at, uint32_t capacity,
-                                             uint32_t *rec_keys, uint32_t *rec_vals) {
-  const uint32_t *src = cell_records + (size_t)g * kCellSlots;
-  uint32_t rec[kCellSlots];
-#pragma unroll
-  for (int k = 0; k < kCellSlots; ++k) rec[k] = k < (int)count ? __ldg(src + k) : 0u;
-#pragma unroll
-  for (int k = 0; k < kCellSlots; ++k)
-    if (k < (int)count && at + k < capacity) {   // never past the buffers, even if the count was taken on the device
-      rec_keys[at + k] = rec[k];
-      rec_vals[at + k] = g;
-    }
-}
-
 // A Gaussian of more than 3 x 3 cells: its cell records worked out again by the whole warp - per row of cells four lanes
 // take the four tile rows, then the lanes take one cell each.  emit(place, cell, mask) is called for record number
 // `place` of the Gaussian, counted on from `first`, by the lane that owns it.

@@ -182,6 +182,7 @@ struct ClusterBinArgs {
   uint32_t *rec_keys, *rec_vals, *sorted_rec_keys, *sorted_rec_vals;       // [capacity]
   uint32_t *cell_ranges, *piece_first, *piece_counts, *piece_bases, *tile_counts, *tile_starts;
   uint32_t *tile_ranges, *tile_order, *out_vals;
+  uint32_t *num_big;                           // scratch: Gaussians whose records wait for a warp
   int num_cells, cell_bits, cgx, gx, gy, W, H;
 };
 int launch_bin_cluster(const ClusterBinArgs &a, int ctas, int64_t record_bound, cudaStream_t st);
