@@ -199,6 +199,7 @@ struct FwdWorkspace {
   uint32_t *cell_ranges;                                 // [cells, 2]
   CellScratch cells;
   unsigned long long *rec_total;                         // number of records, written by the emission
+  unsigned long long *num_visible;                       // Gaussians not culled, written by the depth sort
   uint32_t *num_big;                                     // of the one-cluster binning
   void *sort_table;
   size_t bytes;
@@ -226,6 +227,7 @@ FwdWorkspace carve_fwd(void *ws, int64_t n, int64_t cap, int width, int height) 
   w.cells.tile_counts = c.take<uint32_t>((size_t)gx * gy);
   w.cells.tile_starts = c.take<uint32_t>((size_t)gx * gy);
   w.rec_total = c.take<unsigned long long>(1);
+  w.num_visible = c.take<unsigned long long>(1);
   w.num_big = c.take<uint32_t>(1);
   w.sort_table = c.take<char>(sort_scratch_bytes((int64_t)(nn > cc ? nn : cc)));
   w.bytes = c.used;
@@ -467,19 +469,22 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
     t.done(launch_bin_cluster(b, ctas, num_pairs, s));
   } else if (sorted) {
     // stage 1: Gaussians by depth key (stable => ties keep the index order); the last pass also leaves the cell records
-    // per 256 sorted Gaussians, from which their emission takes its offsets
+    // per 256 sorted Gaussians, from which their emission takes its offsets.  Depths that a camera lets be zero or negative
+    // have no key bit to spare for the culled ones, which are then sorted with the others.
+    unsigned long long *num_visible = cam->near_plane > 0.f ? w.num_visible : nullptr;
     {
       StageTimer t(ctx, GS_STAGE_DEPTH_SORT, s);
-      const SortEpilogue ep = {proj->cell_count, ~kCellBig, w.block_sums, num_scan_blocks(n), nullptr, 0, 0, nullptr};
-      t.done(launch_radix_sort(proj->depth_key, nullptr, w.sorted_depth, bin->depth_order, w.tmp_keys, w.tmp_vals,
-                               n, nullptr, 0, 32, 8, w.sort_table, &ep, report, s));
+      SortEpilogue ep = {};
+      ep.counts = proj->cell_count; ep.count_mask = ~kCellBig; ep.block_sums = w.block_sums; ep.num_block_sums = num_scan_blocks(n);
+      t.done(launch_depth_sort(proj->depth_key, w.sorted_depth, bin->depth_order, w.tmp_keys, w.tmp_vals, n, num_visible, w.sort_table,
+                               ep, report, s));
     }
     // stage 2: one record per (Gaussian, cell of 4 x 4 tiles) in depth order, then a stable sort by cell id alone,
     // whose last pass finds where every cell's records begin and end
     {
       StageTimer t(ctx, GS_STAGE_KEYGEN, s);
       t.done(launch_emit_records(bin->depth_order, proj->cell_count, proj->cell_records, proj->rect, proj->mean2d,
-                                 proj->conic_opacity, w.block_sums, w.rec_keys, w.rec_vals, w.rec_total, overflow, n, cd.cgx,
+                                 proj->conic_opacity, w.block_sums, num_visible, w.rec_keys, w.rec_vals, w.rec_total, overflow, n, cd.cgx,
                                  cd.W, cd.H, pair_capacity, s));
     }
     // two buffers serve the passes: an odd number of passes ends in the other one, an even number back in the first
@@ -489,7 +494,8 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
     uint32_t *sorted_rkeys = odd ? w.tmp_rkeys : w.rec_keys, *sorted_rvals = odd ? w.tmp_rvals : w.rec_vals;
     {
       StageTimer t(ctx, GS_STAGE_TILE_SORT, s);
-      const SortEpilogue ep = {nullptr, 0u, nullptr, 0, w.cell_ranges, num_cells, 16, nullptr};
+      SortEpilogue ep = {};
+      ep.ranges = w.cell_ranges; ep.num_ranges = num_cells; ep.key_shift = 16;
       // the count lives on the device; its host-side bound: a record holds at least one instance
       t.done(launch_radix_sort(w.rec_keys, w.rec_vals, sorted_rkeys, sorted_rvals, odd ? w.rec_keys : w.tmp_rkeys,
                                odd ? w.rec_vals : w.tmp_rvals, num_pairs, w.rec_total, 16, cell_bits, kCellDigit, w.sort_table, &ep, CountReport{}, s));

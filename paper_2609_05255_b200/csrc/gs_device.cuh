@@ -141,6 +141,9 @@ struct SortEpilogue {
   int num_ranges;
   int key_shift;
   uint32_t *overflow;
+  // depth sort: the number of visible Gaussians, and the place of the culled ones behind them, found by the first pass
+  unsigned long long *visible;
+  uint32_t *final_vals;
 };
 size_t sort_scratch_bytes(int64_t count);
 // LSD radix sort of (key, val) pairs on bits [first_bit, first_bit + num_bits), in digits of at most max_digit_bits
@@ -151,12 +154,17 @@ int launch_radix_sort(const uint32_t *keys_in, const uint32_t *vals_in, uint32_t
                        uint32_t *vals_out, uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t count,
                        const unsigned long long *count_dev, int first_bit, int num_bits, int max_digit_bits, void *scratch,
                        const SortEpilogue *epilogue, const CountReport &report, cudaStream_t st);
+// The depth order: ids by (key, id) ascending, where a key is the bits of a float, or 0xffffffff: culled Gaussians, behind
+// all others.  keys / tmp_keys / tmp_vals [n] are scratch.  With visible != nullptr all floats are positive; it receives
+// the number of Gaussians that are not culled, and the epilogue's block sums cover those.
+int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order, uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t n,
+                      unsigned long long *visible, void *scratch, const SortEpilogue &epilogue, const CountReport &report, cudaStream_t st);
 int radix_passes(int num_bits, int max_digit_bits);   // passes launch_radix_sort makes over num_bits key bits
 size_t scan_scratch_bytes(int64_t n);
 int num_scan_blocks(int64_t n);   // entries of the block sums that launch_emit_records reads
 int launch_emit_records(const uint32_t *depth_order, const uint32_t *cell_count, const uint32_t *cell_records,
                         const uint16_t *rect, const float *mean2d, const float *conic_opacity, const uint32_t *block_sums,
-                        uint32_t *rec_keys, uint32_t *rec_vals, unsigned long long *rec_total, uint32_t *overflow, int64_t n,
+                        const unsigned long long *visible, uint32_t *rec_keys, uint32_t *rec_vals, unsigned long long *rec_total, uint32_t *overflow, int64_t n,
                         int cgx, int W, int H, int64_t capacity, cudaStream_t st);
 // Scratch of the expansion: chunk_first [cells + 1], chunk_counts and chunk_bases [max_pieces, 16], tile_counts and
 // tile_starts [tiles].
