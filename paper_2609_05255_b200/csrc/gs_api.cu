@@ -488,22 +488,21 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
                                  cd.W, cd.H, pair_capacity, s));
     }
     // two buffers serve the passes: an odd number of passes ends in the other one, an even number back in the first
+    // (up to 512 cells, 2048 x 1024 pixels, sort in one pass)
     const int cell_bits = id_bits(num_cells);
-    constexpr int kCellDigit = 9;   // up to 512 cells (2048 x 1024 pixels) sort in one pass
-    const bool odd = (radix_passes(cell_bits, kCellDigit) & 1) != 0;
+    const bool odd = radix_passes(cell_bits) == 1;
     uint32_t *sorted_rkeys = odd ? w.tmp_rkeys : w.rec_keys, *sorted_rvals = odd ? w.tmp_rvals : w.rec_vals;
     {
       StageTimer t(ctx, GS_STAGE_TILE_SORT, s);
       SortEpilogue ep = {};
-      ep.ranges = w.cell_ranges; ep.num_ranges = num_cells; ep.key_shift = 16;
+      ep.ranges = w.cell_ranges; ep.num_ranges = num_cells; ep.key_shift = 16; ep.chunk_first = w.cells.chunk_first;
       // the count lives on the device; its host-side bound: a record holds at least one instance
-      t.done(launch_radix_sort(w.rec_keys, w.rec_vals, sorted_rkeys, sorted_rvals, odd ? w.rec_keys : w.tmp_rkeys,
-                               odd ? w.rec_vals : w.tmp_rvals, num_pairs, w.rec_total, 16, cell_bits, kCellDigit, w.sort_table, &ep, CountReport{}, s));
+      t.done(launch_record_sort(w.rec_keys, w.rec_vals, w.tmp_rkeys, w.tmp_rvals, num_pairs, w.rec_total, cell_bits, w.sort_table, ep, s));
     }
     // stage 3: the records of every cell, still in depth order, expanded into the lists of its 16 tiles
     {
       StageTimer t(ctx, GS_STAGE_TILE_RANGES, s);
-      t.done(launch_expand(sorted_rkeys, sorted_rvals, w.cell_ranges, w.cells, num_pairs, pair_capacity, cd.gx, cd.gy, cd.cgx,
+      t.done(launch_expand(sorted_rkeys, sorted_rvals, w.cell_ranges, w.cells, odd, num_pairs, pair_capacity, cd.gx, cd.gy, cd.cgx,
                            cd.cgy, bin->sorted_vals, bin->tile_ranges, bin->tile_order, s));
     }
   } else {

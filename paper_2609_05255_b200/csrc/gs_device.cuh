@@ -135,31 +135,29 @@ struct SortEpilogue {
   uint32_t count_mask;
   uint32_t *block_sums;
   int num_block_sums;
-  // record sort: [start, end) of every id = key >> key_shift in the sorted list (an id that does not occur is left at
-  // (0xffffffff, 0)), and the flag raised when the device-side count exceeded the capacity
+  // record sort: [start, end) of every id = key >> key_shift in the sorted list (an id that does not occur has an empty
+  // range), and the number of expansion chunks of the ids before each
   uint32_t *ranges;
   int num_ranges;
   int key_shift;
-  uint32_t *overflow;
+  uint32_t *chunk_first;
   // depth sort: the number of visible Gaussians, and the place of the culled ones behind them, found by the first pass
   unsigned long long *visible;
   uint32_t *final_vals;
 };
 size_t sort_scratch_bytes(int64_t count);
-// LSD radix sort of (key, val) pairs on bits [first_bit, first_bit + num_bits), in digits of at most max_digit_bits
-// (4 .. 11; wide digits save passes but take registers and shared memory: they pay for short keys only).  If vals_in == nullptr the values are
-// the element indices.  Result lands in keys_out / vals_out; tmp_* are same-sized alternates.  `count` bounds the
-// number of elements (and sizes the grid); with count_dev the true number is read on the device.
-int launch_radix_sort(const uint32_t *keys_in, const uint32_t *vals_in, uint32_t *keys_out,
-                       uint32_t *vals_out, uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t count,
-                       const unsigned long long *count_dev, int first_bit, int num_bits, int max_digit_bits, void *scratch,
-                       const SortEpilogue *epilogue, const CountReport &report, cudaStream_t st);
+// Stable sort of the cell records (keys: cell << 16 | tile mask) by cell, in radix_passes() passes: an odd number ends in
+// other_keys / other_vals, an even one in keys / vals.  `count` bounds the number of records (and sizes the grid), the true
+// number is read on the device.  With one pass it also leaves the chunks of the expansion.  Comes after launch_depth_sort,
+// which prepares the scratch it shares with it.
+int launch_record_sort(uint32_t *keys, uint32_t *vals, uint32_t *other_keys, uint32_t *other_vals, int64_t count,
+                       const unsigned long long *count_dev, int cell_bits, void *scratch, const SortEpilogue &epilogue, cudaStream_t st);
+int radix_passes(int num_bits);
 // The depth order: ids by (key, id) ascending, where a key is the bits of a float, or 0xffffffff: culled Gaussians, behind
 // all others.  keys / tmp_keys / tmp_vals [n] are scratch.  With visible != nullptr all floats are positive; it receives
 // the number of Gaussians that are not culled, and the epilogue's block sums cover those.
 int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order, uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t n,
                       unsigned long long *visible, void *scratch, const SortEpilogue &epilogue, const CountReport &report, cudaStream_t st);
-int radix_passes(int num_bits, int max_digit_bits);   // passes launch_radix_sort makes over num_bits key bits
 size_t scan_scratch_bytes(int64_t n);
 int num_scan_blocks(int64_t n);   // entries of the block sums that launch_emit_records reads
 int launch_emit_records(const uint32_t *depth_order, const uint32_t *cell_count, const uint32_t *cell_records,
@@ -170,7 +168,7 @@ int launch_emit_records(const uint32_t *depth_order, const uint32_t *cell_count,
 // tile_starts [tiles].
 struct CellScratch { uint32_t *chunk_first, *chunk_counts, *chunk_bases, *tile_counts, *tile_starts; };
 int max_pieces(int64_t record_capacity, int num_cells);   // of kBinPiece records (the grid-wide expansion works in larger chunks)
-int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint32_t *cell_ranges, const CellScratch &cs,
+int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint32_t *cell_ranges, const CellScratch &cs, bool chunks_known,
                   int64_t record_capacity, int64_t pair_capacity, int gx, int gy, int cgx, int cgy,
                   uint32_t *sorted_vals, uint32_t *tile_ranges, uint32_t *tile_order, cudaStream_t st);
 // The whole binning in one cluster of CTAs and one expansion kernel (gs_bin_cluster.cu), for scenes that do not fill the

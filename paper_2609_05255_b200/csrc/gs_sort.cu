@@ -1,4 +1,4 @@
-// Ordering and binning: a stable LSD radix sort (digits of 4 to 11 bits, keys staged and ranked in shared
+// Ordering and binning: a stable LSD radix sort (digits of 4 to 9 bits, keys staged and ranked in shared
 // memory, no inter-block waiting) and the kernels that turn its output into per-tile lists.
 //
 // (1) The Gaussians are sorted once by their 32-bit depth key (ties keep the index order: the sort is stable).
@@ -21,7 +21,7 @@ constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kItems = 16;
 constexpr int kSortTile = kSortThreads * kItems;   // 4096 elements per block iteration
 constexpr int kMaxSortBlocks = 444;                // 3 resident CTAs x 148 SMs: one full wave
-constexpr int kMaxDigitBits = 11;  // widest radix digit: 2048 bins
+constexpr int kMaxDigitBits = 9;   // widest radix digit: 512 bins
 constexpr int kScanBlock = 256;   // Gaussians per block of the tiles-touched prefix sum and per CTA of the instance emission
 
 
@@ -71,34 +71,44 @@ __device__ __forceinline__ BlockRange block_range(int64_t count) {
 // scene: the four passes 147 us before, XXX now, the emission 68 and XXX).
 __device__ __forceinline__ uint32_t rotated(uint32_t key) { return __funnelshift_l(key, key, 1); }
 
-// Digit histogram of each block's contiguous range: table[digit][block] (digits of up to kMaxDigitBits bits).
+// Where a block's elements of a digit go follows from the digits of all blocks before it.  Blocks are taken in groups of
+// about the square root of their number: a block adds its digits to its group's sums, and the scatter adds up the groups
+// before its own and the blocks before it in its group - 43 loads at most, where a kernel of its own scanned the
+// rows before (444 blocks: 4.4 us, and a launch in each pass).
+constexpr int kMaxGroups = 22;                   // ceil(sqrt(kMaxSortBlocks)), also the largest group
+constexpr int kGroupTables = 6;                  // four passes of the depth sort, two of the record sort
+static_assert(kMaxGroups * kMaxGroups >= kMaxSortBlocks, "groups");
+int group_size(int blocks) { int g = 1; while (g * g < blocks) ++g; return g; }
+
+// Digit histogram of each block's contiguous range: table[block][digit], added to groups[block / group][digit] unless
+// `groups` is null (it is not cleared yet: the first pass, whose block clears the tables of the passes to come).
 template <bool ROTATE>
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *__restrict__ keys, int64_t count,
                                                              const unsigned long long *__restrict__ count_dev,
-                                                             int shift, int bits,
-                                                             uint32_t *__restrict__ table, SortEpilogue ep, CountReport report) {
+                                                             int shift, int bits, uint32_t *__restrict__ table,
+                                                             uint32_t *__restrict__ groups, int group,
+                                                             uint32_t *__restrict__ clear, int clear_words, SortEpilogue ep,
+                                                             CountReport report) {
   dependency_wait();
   if (blockIdx.x == 0 && threadIdx.x == 0) report.send();
+  for (int i = blockIdx.x * kSortThreads + threadIdx.x; i < clear_words; i += gridDim.x * kSortThreads) clear[i] = 0u;
   // the arrays the scatter of this pass accumulates into start from their neutral values
   if (ep.block_sums)
     for (int i = blockIdx.x * kSortThreads + threadIdx.x; i < ep.num_block_sums; i += gridDim.x * kSortThreads) ep.block_sums[i] = 0u;
-  if (ep.ranges)
+  if (ep.ranges && !ep.chunk_first)
     for (int i = blockIdx.x * kSortThreads + threadIdx.x; i < 2 * ep.num_ranges; i += gridDim.x * kSortThreads)
       ep.ranges[i] = (i & 1) ? 0u : 0xffffffffu;
-  if (count_dev) {
-    const int64_t c = (int64_t)__ldg(count_dev);                    // the true length lives on the device
-    if (ep.overflow && c > count && blockIdx.x == 0 && threadIdx.x == 0) *ep.overflow = 1u;   // lists were cut off: tell the host
-    count = min(count, c);
-  }
-  // up to 256 digits: one histogram per warp (fewer collisions); more: two shared by the warps
-  __shared__ uint32_t s_hist[2 << kMaxDigitBits];
+  if (count_dev) count = min(count, (int64_t)__ldg(count_dev));     // the true length lives on the device
+  // up to 256 digits: one histogram per warp (fewer collisions); more: four shared by the warps
+  __shared__ uint32_t s_hist[kSortWarps << 8];
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int nb = 1 << bits, copies = nb <= 256 ? kSortWarps : 2;
+  const int nb = 1 << bits, copies = nb <= 256 ? kSortWarps : kSortWarps / 2;
   const uint32_t mask = (uint32_t)nb - 1u;
   for (int k = tid; k < copies * nb; k += kSortThreads) s_hist[k] = 0;
   __syncthreads();
   const BlockRange r = block_range(count);
   uint32_t *mine = s_hist + (warp % copies) * nb;
+#pragma unroll 4
   for (int64_t i = r.begin + tid; i < r.end; i += kSortThreads) {
     const uint32_t k = __ldg(keys + i);
     atomicAdd(mine + (((ROTATE ? rotated(k) : k) >> shift) & mask), 1u);
@@ -107,42 +117,20 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *__r
   for (int d = tid; d < nb; d += kSortThreads) {
     uint32_t t = 0;
     for (int w = 0; w < copies; ++w) t += s_hist[w * nb + d];
-    table[(size_t)d * gridDim.x + blockIdx.x] = t;   // digit-major: one contiguous row per digit
+    table[(blockIdx.x << bits) + d] = t;
+    if (groups && t) atomicAdd(groups + ((blockIdx.x / group) << bits) + d, t);
   }
 }
 
-// Per digit (one CTA each): exclusive scan of the row of per-block counts, in place, and the row
-// total.  Done once per pass here instead of by every scatter CTA.
-__global__ void __launch_bounds__(256) k_radix_scan_rows(uint32_t *__restrict__ table, int nblocks,
-                                                         uint32_t *__restrict__ totals) {
+// The groups' sums of the first pass: one CTA per group.
+__global__ void __launch_bounds__(1 << 8) k_group_sums(const uint32_t *__restrict__ table, int nblocks, int group,
+                                                       uint32_t *__restrict__ groups) {
   dependency_wait();
-  __shared__ uint32_t s_w[8];
-  __shared__ uint32_t s_carry;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t *row = table + (size_t)blockIdx.x * nblocks;
-  if (tid == 0) s_carry = 0;
-  __syncthreads();
-  for (int base = 0; base < nblocks; base += 256) {
-    const int i = base + tid;
-    const uint32_t v = i < nblocks ? row[i] : 0u;
-    uint32_t inc = v;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, inc, s);
-      if (lane >= s) inc += t;
-    }
-    if (lane == 31) s_w[warp] = inc;
-    __syncthreads();
-    uint32_t off = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) off += (w < warp) ? s_w[w] : 0u;
-    const uint32_t carry = s_carry;
-    if (i < nblocks) row[i] = carry + off + inc - v;
-    __syncthreads();
-    if (tid == 255) s_carry = carry + off + inc;
-    __syncthreads();
-  }
-  if (tid == 0) totals[blockIdx.x] = s_carry;
+  const int first = blockIdx.x * group, last = min(nblocks, first + group);
+  uint32_t t = 0;
+#pragma unroll 8
+  for (int b = first; b < last; ++b) t += __ldg(table + (b << 8) + threadIdx.x);
+  groups[(blockIdx.x << 8) + threadIdx.x] = t;
 }
 
 // Exclusive prefix sums over kSortThreads * DPT values in thread-major order (thread t holds values t * DPT ..): each
@@ -181,12 +169,13 @@ template <int BITS> constexpr size_t scatter_smem_bytes() {
 // equal ids = key >> key_shift (last pass of the record sort: inside a block's run of one digit the keys are
 // non-decreasing, because the earlier passes ordered the lower bits, so a change of id between neighbours of a run
 // is a boundary; the two ends of a run may continue in another block and enter with an atomic min / max), 3 the first
-// pass of the depth sort: keys come as they are, the largest digit's elements go to their final place and are counted out.
+// pass of the depth sort: keys come as they are, the largest digit's elements go to their final place and are counted out,
+// 4 the record sort in a single pass: the digits' totals are the ranges, and the chunks of the expansion follow from them.
 template <int BITS, int EP>
 __global__ void __launch_bounds__(kSortThreads, BITS <= 9 ? 3 : 2) k_radix_scatter(
     const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in, uint32_t *__restrict__ keys_out,
     uint32_t *__restrict__ vals_out, int64_t count, const unsigned long long *__restrict__ count_dev, int shift,
-    const uint32_t *__restrict__ table, const uint32_t *__restrict__ totals, int nblocks, SortEpilogue ep) {
+    const uint32_t *__restrict__ table, const uint32_t *__restrict__ groups, int group, SortEpilogue ep) {
   dependency_wait();
   constexpr int NB = BITS <= 8 ? 256 : (1 << BITS);   // entries of the digit arrays
   constexpr int DPT = NB / kSortThreads;              // digits per thread
@@ -199,18 +188,48 @@ __global__ void __launch_bounds__(kSortThreads, BITS <= 9 ? 3 : 2) k_radix_scatt
   if (count_dev) count = min(count, (int64_t)__ldg(count_dev));
   constexpr uint32_t kDigitMask = (1u << BITS) - 1u;
 
-  // global base of every digit for this block: all smaller digits everywhere (scan of the row
-  // totals) + the same digit in the blocks before this one (the row prefix from k_radix_scan_rows)
+  // global base of every digit for this block: all smaller digits everywhere + the same digit in the blocks before
   {
-    uint32_t tot[DPT], start[DPT];
+    uint32_t tot[DPT] = {}, before[DPT] = {}, start[DPT];
+    if (tid * DPT <= (int)kDigitMask) {
+      const int own = (int)blockIdx.x / group, num = ((int)gridDim.x + group - 1) / group, in_group = (int)blockIdx.x - own * group;
+      uint32_t v[kMaxGroups][DPT], u[kMaxGroups][DPT];     // all in flight together: in two halves the pass took 3 us more
 #pragma unroll
-    for (int j = 0; j < DPT; ++j) { const int d = tid * DPT + j; tot[j] = d <= (int)kDigitMask ? __ldg(totals + d) : 0u; }
+      for (int g = 0; g < kMaxGroups; ++g)
+#pragma unroll
+        for (int j = 0; j < DPT; ++j) {
+          v[g][j] = g < num ? __ldg(groups + (g << BITS) + tid * DPT + j) : 0u;
+          u[g][j] = g < in_group ? __ldg(table + ((own * group + g) << BITS) + tid * DPT + j) : 0u;
+        }
+#pragma unroll
+      for (int g = 0; g < kMaxGroups; ++g)
+#pragma unroll
+        for (int j = 0; j < DPT; ++j) {
+          tot[j] += v[g][j];
+          before[j] += u[g][j] + (g < own ? v[g][j] : 0u);
+        }
+    }
     block_exclusive_scan<DPT>(tot, start, s_warp_tot, tid);
 #pragma unroll
     for (int j = 0; j < DPT; ++j) {
       const int d = tid * DPT + j;
-      s_base[d] = start[j] + (d <= (int)kDigitMask ? __ldg(table + (size_t)d * nblocks + blockIdx.x) : 0u);
+      s_base[d] = start[j] + before[j];
       if (EP == 3 && blockIdx.x == 0 && d == (int)kDigitMask) *ep.visible = start[j];
+    }
+    if (EP == 4 && blockIdx.x == gridDim.x - 1) {       // (its range is the shortest)
+      uint32_t chunks[DPT], first[DPT];
+#pragma unroll
+      for (int j = 0; j < DPT; ++j) chunks[j] = (tot[j] + kCellChunk - 1) / kCellChunk;
+      block_exclusive_scan<DPT>(chunks, first, s_warp_tot, tid);
+#pragma unroll
+      for (int j = 0; j < DPT; ++j) {
+        const int d = tid * DPT + j;
+        if (d < ep.num_ranges) {
+          ep.ranges[2 * d] = start[j]; ep.ranges[2 * d + 1] = start[j] + tot[j];
+          ep.chunk_first[d] = first[j];
+        }
+        if (d == NB - 1) ep.chunk_first[ep.num_ranges] = first[j] + chunks[j];
+      }
     }
   }
 
@@ -287,43 +306,47 @@ __global__ void __launch_bounds__(kSortThreads, BITS <= 9 ? 3 : 2) k_radix_scatt
       s_vals[pos] = val[it];
     }
     __syncthreads();
-    for (int j0 = 0; j0 < valid_count; j0 += kSortThreads) {
-      const int j = j0 + tid;
-      const bool ok = j < valid_count;
-      uint32_t k = 0, d = 0, gpos = 0, v = 0;
-      if (ok) {
-        k = s_keys[j];
-        d = (k >> shift) & kDigitMask;
-        gpos = s_base[d] + ((uint32_t)j - s_digit_start[d]);
-        v = s_vals[j];
+    constexpr int kOut = 4;                             // rows written together, so that what they wait for overlaps
+    for (int j0 = 0; j0 < valid_count; j0 += kOut * kSortThreads) {
+      uint32_t gpos[kOut], count_of[kOut];
+#pragma unroll
+      for (int h = 0; h < kOut; ++h) {
+        const int j = j0 + h * kSortThreads + tid;
+        const bool ok = j < valid_count;
+        gpos[h] = count_of[h] = 0u;
+        if (!ok) continue;
+        const uint32_t k = s_keys[j], d = (k >> shift) & kDigitMask, v = s_vals[j], run_first = s_digit_start[d];
+        gpos[h] = s_base[d] + ((uint32_t)j - run_first);
+        if (EP == 1) count_of[h] = __ldg(ep.counts + v) & ep.count_mask;
         if (EP == 3 && d == kDigitMask) {
-          ep.final_vals[gpos] = v;
+          ep.final_vals[gpos[h]] = v;
         } else {
-          keys_out[gpos] = k;
-          vals_out[gpos] = v;
+          keys_out[gpos[h]] = k;
+          vals_out[gpos[h]] = v;
+        }
+        if (EP == 2) {
+          const uint32_t run_end = d == kDigitMask ? (uint32_t)valid_count : s_digit_start[d + 1];   // slots past the input hold no run
+          const uint32_t id = k >> ep.key_shift;
+          if ((uint32_t)j == run_first) atomicMin(ep.ranges + 2 * id, gpos[h]);
+          else if ((s_keys[j - 1] >> ep.key_shift) != id) ep.ranges[2 * id] = gpos[h];
+          if ((uint32_t)j + 1 == run_end) atomicMax(ep.ranges + 2 * id + 1, gpos[h] + 1);
+          else if ((s_keys[j + 1] >> ep.key_shift) != id) ep.ranges[2 * id + 1] = gpos[h] + 1;
         }
       }
       if (EP == 1) {
-        // the Gaussian's count, added to the sum of its block of kScanBlock sorted positions; a warp whose
-        // lanes all fall into one block (the usual case: a run is contiguous) adds once
-        uint32_t tt = ok ? (__ldg(ep.counts + v) & ep.count_mask) : 0u;
-        const uint32_t blk = gpos / kScanBlock, blk0 = __shfl_sync(kFull, blk, 0);
-        if (__all_sync(kFull, !ok || blk == blk0)) {
 #pragma unroll
-          for (int sft = 16; sft > 0; sft >>= 1) tt += __shfl_xor_sync(kFull, tt, sft);
-          if (lane == 0 && tt) atomicAdd(ep.block_sums + blk0, tt);
-        } else if (tt) {
-          atomicAdd(ep.block_sums + blk, tt);
+        for (int h = 0; h < kOut; ++h) {
+          // the Gaussian's count, added to the sum of its block of kScanBlock sorted positions; a warp whose
+          // lanes all fall into one block (the usual case: a run is contiguous) adds once
+          const bool ok = j0 + h * kSortThreads + tid < valid_count;
+          const uint32_t blk = gpos[h] / kScanBlock, blk0 = __shfl_sync(kFull, blk, 0);
+          if (__all_sync(kFull, !ok || blk == blk0)) {
+            const uint32_t sum = __reduce_add_sync(kFull, count_of[h]);
+            if (lane == 0 && sum) atomicAdd(ep.block_sums + blk0, sum);
+          } else if (count_of[h]) {
+            atomicAdd(ep.block_sums + blk, count_of[h]);
+          }
         }
-      }
-      if (EP == 2 && ok) {
-        const uint32_t run_first = s_digit_start[d];
-        const uint32_t run_end = d == kDigitMask ? (uint32_t)valid_count : s_digit_start[d + 1];   // slots past the input hold no run
-        const uint32_t id = k >> ep.key_shift;
-        if ((uint32_t)j == run_first) atomicMin(ep.ranges + 2 * id, gpos);
-        else if ((s_keys[j - 1] >> ep.key_shift) != id) ep.ranges[2 * id] = gpos;
-        if ((uint32_t)j + 1 == run_end) atomicMax(ep.ranges + 2 * id + 1, gpos + 1);
-        else if ((s_keys[j + 1] >> ep.key_shift) != id) ep.ranges[2 * id + 1] = gpos + 1;
       }
     }
     __syncthreads();
@@ -594,12 +617,18 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand(const uint32_t *__res
 
 }  // namespace
 
-size_t sort_scratch_bytes(int64_t count) { return ((size_t)sort_blocks(count) + 1) * (1 << kMaxDigitBits) * sizeof(uint32_t); }
+size_t sort_scratch_bytes(int64_t count) {
+  return ((size_t)sort_blocks(count) + kGroupTables * kMaxGroups) * (1 << kMaxDigitBits) * sizeof(uint32_t);
+}
 
 namespace {
+// The groups' sums of pass `p` of a view (the four of the depth sort, then the record sort's).
+uint32_t *group_table(void *scratch, int p) { return static_cast<uint32_t *>(scratch) + ((size_t)p * kMaxGroups << kMaxDigitBits); }
+uint32_t *block_table(void *scratch) { return group_table(scratch, kGroupTables); }
+
 template <int BITS, int EP>
 void launch_scatter(int blocks, const uint32_t *src_k, const uint32_t *src_v, uint32_t *dst_k, uint32_t *dst_v, int64_t count,
-                    const unsigned long long *count_dev, int shift, const uint32_t *table, const uint32_t *totals,
+                    const unsigned long long *count_dev, int shift, const uint32_t *table, const uint32_t *groups,
                     const SortEpilogue &ep, cudaStream_t st) {
   constexpr size_t smem = scatter_smem_bytes<BITS>();
   static bool opted[64] = {};
@@ -610,55 +639,48 @@ void launch_scatter(int blocks, const uint32_t *src_k, const uint32_t *src_v, ui
     opted[dev] = true;
   }
   launch_chained(k_radix_scatter<BITS, EP>, blocks, kSortThreads, smem, st, src_k, src_v, dst_k, dst_v, count, count_dev, shift, table,
-                 totals, blocks, ep);
+                 groups, group_size(blocks), ep);
 }
 }  // namespace
 
-int launch_radix_sort(const uint32_t *keys_in, const uint32_t *vals_in, uint32_t *keys_out, uint32_t *vals_out,
-                       uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t count, const unsigned long long *count_dev,
-                       int first_bit, int num_bits, int max_digit_bits, void *scratch, const SortEpilogue *epilogue,
-                       const CountReport &report, cudaStream_t st) {
-  if (count <= 0) return 0;
-  const int passes = radix_passes(num_bits, max_digit_bits);
-  int bits = (num_bits + passes - 1) / passes;     // digits of equal width: 13 bits sort as 7 + 6 under a limit of 8
+int radix_passes(int num_bits) { return num_bits <= kMaxDigitBits ? 1 : 2; }
+
+int launch_record_sort(uint32_t *keys, uint32_t *vals, uint32_t *other_keys, uint32_t *other_vals, int64_t count,
+                       const unsigned long long *count_dev, int cell_bits, void *scratch, const SortEpilogue &epilogue, cudaStream_t st) {
+  const int passes = radix_passes(cell_bits);
+  int bits = (cell_bits + passes - 1) / passes;    // digits of equal width: 13 bits sort as 7 + 6
   if (bits < 4) bits = 4;                          // (bits above the keys' range are zero: sorting on them changes nothing)
-  const int blocks = sort_blocks(count);
-  uint32_t *table = static_cast<uint32_t *>(scratch);
-  uint32_t *totals = table + ((size_t)blocks << bits);
-  const uint32_t *src_k = keys_in, *src_v = vals_in;
-  const SortEpilogue none = {};
+  const int blocks = sort_blocks(count), group = group_size(blocks);
+  uint32_t *table = block_table(scratch);
   for (int p = 0; p < passes; ++p) {
-    const bool to_out = ((passes - 1 - p) % 2) == 0;
-    uint32_t *dst_k = to_out ? keys_out : tmp_keys, *dst_v = to_out ? vals_out : tmp_vals;
-    const SortEpilogue ep = (p == passes - 1 && epilogue) ? *epilogue : none;
-    const int mode = ep.ranges ? 2 : 0;
-    const int shift = first_bit + bits * p;
-    launch_chained(k_radix_hist<false>, blocks, kSortThreads, 0, st, src_k, count, count_dev, shift, bits, table, ep, p == 0 ? report : CountReport{});
-    launch_chained(k_radix_scan_rows, 1 << bits, 256, 0, st, table, blocks, totals);
-#define GS_ARGS blocks, src_k, src_v, dst_k, dst_v, count, count_dev, shift, table, totals, ep, st
-#define GS_SCATTER(B)                                             \
-  case B:                                                         \
-    if (mode == 2) launch_scatter<B, 2>(GS_ARGS);                 \
-    else launch_scatter<B, 0>(GS_ARGS);                           \
-    break;
+    const uint32_t *src_k = p ? other_keys : keys, *src_v = p ? other_vals : vals;
+    uint32_t *dst_k = p ? keys : other_keys, *dst_v = p ? vals : other_vals, *groups = group_table(scratch, 4 + p);
+    const int mode = p < passes - 1 ? 0 : passes == 1 ? 4 : 2, shift = 16 + bits * p;
+    SortEpilogue ep = {};
+    if (mode) ep = epilogue;
+    if (mode == 2) ep.chunk_first = nullptr;
+    launch_chained(k_radix_hist<false>, blocks, kSortThreads, 0, st, src_k, count, count_dev, shift, bits, table, groups, group,
+                   (uint32_t *)nullptr, 0, ep, CountReport{});
+#define GS_SCATTER(B, EP) launch_scatter<B, EP>(blocks, src_k, src_v, dst_k, dst_v, count, count_dev, shift, table, groups, ep, st)
+#define GS_SCATTER_TWO(B) if (mode == 2) GS_SCATTER(B, 2); else if (mode == 4) GS_SCATTER(B, 4); else GS_SCATTER(B, 0); break;
     switch (bits) {
-      GS_SCATTER(4) GS_SCATTER(5) GS_SCATTER(6) GS_SCATTER(7) GS_SCATTER(8) GS_SCATTER(9) GS_SCATTER(10)
-      default:
-        if (mode == 2) launch_scatter<11, 2>(GS_ARGS);
-        else launch_scatter<11, 0>(GS_ARGS);
+      case 4: GS_SCATTER(4, 4); break;             // (one pass; two passes have digits of five to eight bits)
+      case 9: GS_SCATTER(9, 4); break;
+      case 5: GS_SCATTER_TWO(5)
+      case 6: GS_SCATTER_TWO(6)
+      case 7: GS_SCATTER_TWO(7)
+      default: GS_SCATTER_TWO(8)
     }
+#undef GS_SCATTER_TWO
 #undef GS_SCATTER
-#undef GS_ARGS
-    src_k = dst_k;
-    src_v = dst_v;
   }
-  return 3 * passes;
+  return 2 * passes;
 }
 
 int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order, uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t n,
                       unsigned long long *visible, void *scratch, const SortEpilogue &epilogue, const CountReport &report, cudaStream_t st) {
-  const int blocks = sort_blocks(n);
-  uint32_t *table = static_cast<uint32_t *>(scratch), *totals = table + ((size_t)blocks << 8);
+  const int blocks = sort_blocks(n), group = group_size(blocks);
+  uint32_t *table = block_table(scratch);
   SortEpilogue ep[4] = {};
   if (visible) {
     ep[0].visible = visible;
@@ -667,22 +689,17 @@ int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order
   ep[3] = epilogue;
   for (int p = 0; p < 4; ++p) {
     const uint32_t *src_k = p == 0 ? depth_key : p & 1 ? tmp_keys : keys, *src_v = p == 0 ? nullptr : p & 1 ? tmp_vals : order;
-    uint32_t *dst_k = p & 1 ? keys : tmp_keys, *dst_v = p & 1 ? order : tmp_vals;
+    uint32_t *dst_k = p & 1 ? keys : tmp_keys, *dst_v = p & 1 ? order : tmp_vals, *groups = group_table(scratch, p);
     const unsigned long long *count = p == 0 ? nullptr : visible;
-    launch_chained(p == 0 && visible ? k_radix_hist<true> : k_radix_hist<false>, blocks, kSortThreads, 0, st, src_k, n, count, 8 * p, 8, table, ep[p],
-                   p == 0 ? report : CountReport{});
-    launch_chained(k_radix_scan_rows, 256, 256, 0, st, table, blocks, totals);
-    if (p == 0 && visible) launch_scatter<8, 3>(blocks, src_k, src_v, dst_k, dst_v, n, count, 8 * p, table, totals, ep[p], st);
-    else if (p < 3) launch_scatter<8, 0>(blocks, src_k, src_v, dst_k, dst_v, n, count, 8 * p, table, totals, ep[p], st);
-    else launch_scatter<8, 1>(blocks, src_k, src_v, dst_k, dst_v, n, count, 8 * p, table, totals, ep[p], st);
+    const int clear_words = p == 0 ? (int)(block_table(scratch) - group_table(scratch, 1)) : 0;
+    launch_chained(p == 0 && visible ? k_radix_hist<true> : k_radix_hist<false>, blocks, kSortThreads, 0, st, src_k, n, count, 8 * p, 8, table,
+                   p == 0 ? (uint32_t *)nullptr : groups, group, group_table(scratch, 1), clear_words, ep[p], p == 0 ? report : CountReport{});
+    if (p == 0) launch_chained(k_group_sums, (blocks + group - 1) / group, 256, 0, st, table, blocks, group, groups);
+    if (p == 0 && visible) launch_scatter<8, 3>(blocks, src_k, src_v, dst_k, dst_v, n, count, 8 * p, table, groups, ep[p], st);
+    else if (p < 3) launch_scatter<8, 0>(blocks, src_k, src_v, dst_k, dst_v, n, count, 8 * p, table, groups, ep[p], st);
+    else launch_scatter<8, 1>(blocks, src_k, src_v, dst_k, dst_v, n, count, 8 * p, table, groups, ep[p], st);
   }
-  return 12;
-}
-
-int radix_passes(int num_bits, int max_digit_bits) {
-  const int m = max_digit_bits < 4 ? 4 : max_digit_bits > kMaxDigitBits ? kMaxDigitBits : max_digit_bits;
-  const int p = (num_bits + m - 1) / m;
-  return p < 1 ? 1 : p;
+  return 9;
 }
 
 size_t scan_scratch_bytes(int64_t n) { return (size_t)((n + kScanBlock - 1) / kScanBlock + 1) * sizeof(uint32_t); }
@@ -701,19 +718,19 @@ int launch_emit_records(const uint32_t *depth_order, const uint32_t *cell_count,
 
 int max_pieces(int64_t record_capacity, int num_cells) { return (int)((record_capacity + kBinPiece - 1) / kBinPiece) + num_cells; }
 
-int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint32_t *cell_ranges, const CellScratch &cs,
+int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint32_t *cell_ranges, const CellScratch &cs, bool chunks_known,
                   int64_t record_capacity, int64_t pair_capacity, int gx, int gy, int cgx, int cgy,
                   uint32_t *sorted_vals, uint32_t *tile_ranges, uint32_t *tile_order, cudaStream_t st) {
   const int num_cells = cgx * cgy, chunks = (int)((record_capacity + kCellChunk - 1) / kCellChunk) + num_cells;
   const uint32_t cap = pair_capacity > 0xffffffffll ? 0xffffffffu : (uint32_t)pair_capacity;
-  launch_chained(k_cell_chunks, 1, 1024, 0, st, cell_ranges, num_cells, cs.chunk_first);
+  if (!chunks_known) launch_chained(k_cell_chunks, 1, 1024, 0, st, cell_ranges, num_cells, cs.chunk_first);
   launch_chained(k_chunk_counts, chunks, kExpandThreads, 0, st, rec_keys, cell_ranges, cs.chunk_first, num_cells, cs.chunk_counts);
   launch_chained(k_cell_prefix, (num_cells + 7) / 8, 256, 0, st, cs.chunk_first, cs.chunk_counts, gx, gy, cgx, num_cells, cs.chunk_bases,
                  cs.tile_counts);
   launch_chained(k_tile_scan, 1, 1024, 0, st, cs.tile_counts, gx * gy, cap, cs.tile_starts, tile_ranges, tile_order);
   launch_chained(k_expand, chunks, kExpandThreads, 0, st, rec_keys, rec_vals, cell_ranges, cs.chunk_first, num_cells, cs.chunk_bases,
                  cs.tile_starts, gx, gy, cgx, cap, sorted_vals);
-  return 5;
+  return chunks_known ? 4 : 5;
 }
 
 // No record was sorted (no Gaussian, or none that reaches a tile): every tile is empty.
