@@ -222,6 +222,7 @@ FwdWorkspace carve_fwd(void *ws, int64_t n, int64_t cap, int width, int height) 
   w.tmp_rvals = c.take<uint32_t>(cc);
   w.cell_ranges = c.take<uint32_t>((size_t)cells * 2);
   w.cells.chunk_first = c.take<uint32_t>((size_t)cells + 1);
+  w.cells.chunks = c.take<uint4>(pieces);
   w.cells.chunk_counts = c.take<uint32_t>(pieces * 16);
   w.cells.chunk_bases = c.take<uint32_t>(pieces * 16);
   w.cells.tile_counts = c.take<uint32_t>((size_t)gx * gy);
@@ -495,7 +496,7 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
     {
       StageTimer t(ctx, GS_STAGE_TILE_SORT, s);
       SortEpilogue ep = {};
-      ep.ranges = w.cell_ranges; ep.num_ranges = num_cells; ep.key_shift = 16; ep.chunk_first = w.cells.chunk_first;
+      ep.ranges = w.cell_ranges; ep.num_ranges = num_cells; ep.key_shift = 16; ep.chunk_first = w.cells.chunk_first; ep.chunks = w.cells.chunks;
       // the count lives on the device; its host-side bound: a record holds at least one instance
       t.done(launch_record_sort(w.rec_keys, w.rec_vals, w.tmp_rkeys, w.tmp_rvals, num_pairs, w.rec_total, cell_bits, w.sort_table, ep, s));
     }

@@ -155,43 +155,66 @@ __device__ __forceinline__ void expand_records(const uint32_t mask[8], const uin
 // By one CTA of 1024 threads: the exclusive scan of the tile counts in tile order = the tile ranges, and the launch
 // order of the blend's warps (tiles by decreasing list length in log2 buckets: the long tiles start first and the short
 // ones fill the tail; the order inside a bucket is whatever the atomics give, it affects scheduling only, never a result).
-struct TileScan { uint32_t w[32], cnt[33], off[33]; };
+// Thread t takes the tiles [t per, (t + 1) per) of a strip of 1024 per, all loads in flight together (a loop over `per`
+// dependent turns took 10.6 us for the 4161 tiles of a 1256 x 828 image, now 8.1).
+struct TileScan { uint32_t w[32], cnt[33], off[33], all; };
 __device__ __forceinline__ void tile_scan(TileScan &s, const uint32_t *tile_counts, int num_tiles, uint32_t capacity,
                                           uint32_t *tile_starts, uint32_t *ranges, uint32_t *order) {
+  constexpr int kMost = 8;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = min((num_tiles + 1023) / 1024, kMost), strip = 1024 * per;
   if (tid < 33) s.cnt[tid] = 0;
   __syncthreads();
-  // thread t takes the tiles [t per, (t + 1) per): one pass over its counts, one scan of the thread sums
-  const int per = (num_tiles + 1023) / 1024, first = tid * per, last = min(first + per, num_tiles);
-  uint32_t sum = 0;
-  for (int t = first; t < last; ++t) {
-    const uint32_t v = __ldcg(tile_counts + t);
-    sum += v;
-    atomicAdd(&s.cnt[v ? 32 - __clz(v) : 0], 1u);
-  }
-  const uint32_t inc = warp_inclusive(sum, lane);
-  if (lane == 31) s.w[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    const uint32_t w = s.w[lane];
-    s.w[lane] = warp_inclusive(w, lane) - w;
-  }
-  if (tid == 0) {
-    uint32_t off = 0;
-    for (int b = 32; b >= 0; --b) { s.off[b] = off; off += s.cnt[b]; }
+  uint32_t v[kMost];
+  auto load = [&](int base) {
+#pragma unroll
+    for (int k = 0; k < kMost; ++k) {
+      const int t = base + tid * per + k;
+      v[k] = k < per && t < num_tiles ? __ldcg(tile_counts + t) : 0u;
+    }
+  };
+  for (int base = 0; base < num_tiles; base += strip) {
+    load(base);
+#pragma unroll
+    for (int k = 0; k < kMost; ++k)
+      if (k < per && base + tid * per + k < num_tiles) atomicAdd(&s.cnt[32 - __clz(v[k])], 1u);
   }
   __syncthreads();
-  uint32_t start = s.w[warp] + inc - sum;
-  for (int t = first; t < last; ++t) {
-    const uint32_t v = __ldcg(tile_counts + t);
-    tile_starts[t] = start;
-    // a tile without instances: (0, 0); never past the capacity of the instance buffers (a device-side count may
-    // exceed it: the lists are then cut off and the host is told)
-    const uint32_t s0 = min(start, capacity), e0 = start + v < start ? capacity : min(start + v, capacity);
-    ranges[2 * t] = e0 > s0 ? s0 : 0u;
-    ranges[2 * t + 1] = e0 > s0 ? e0 : 0u;
-    order[atomicAdd(&s.off[v ? 32 - __clz(v) : 0], 1u)] = (uint32_t)t;
-    start += v;
+  if (warp == 0) {                             // lane l: bucket 32 - l, the longest lists first
+    const uint32_t c = s.cnt[32 - lane], inc = warp_inclusive(c, lane);
+    s.off[32 - lane] = inc - c;
+    if (lane == 31) s.off[0] = inc;
+  }
+  uint32_t carry = 0;
+  for (int base = 0; base < num_tiles; base += strip) {
+    if (strip < num_tiles) load(base);
+    uint32_t sum = 0;
+#pragma unroll
+    for (int k = 0; k < kMost; ++k) sum += v[k];
+    const uint32_t inc = warp_inclusive(sum, lane);
+    if (lane == 31) s.w[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+      const uint32_t w = s.w[lane], winc = warp_inclusive(w, lane);
+      s.w[lane] = winc - w;
+      if (lane == 31) s.all = winc;
+    }
+    __syncthreads();
+    uint32_t start = carry + s.w[warp] + inc - sum;
+    carry += s.all;
+#pragma unroll
+    for (int k = 0; k < kMost; ++k) {
+      const int t = base + tid * per + k;
+      if (k >= per || t >= num_tiles) continue;
+      tile_starts[t] = start;
+      // a tile without instances: (0, 0); never past the capacity of the instance buffers (a device-side count may
+      // exceed it: the lists are then cut off and the host is told)
+      const uint32_t s0 = min(start, capacity), e0 = start + v[k] < start ? capacity : min(start + v[k], capacity);
+      reinterpret_cast<uint2 *>(ranges)[t] = e0 > s0 ? make_uint2(s0, e0) : make_uint2(0u, 0u);
+      order[atomicAdd(&s.off[32 - __clz(v[k])], 1u)] = (uint32_t)t;
+      start += v[k];
+    }
+    __syncthreads();
   }
 }
 

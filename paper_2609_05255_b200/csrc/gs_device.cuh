@@ -136,11 +136,12 @@ struct SortEpilogue {
   uint32_t *block_sums;
   int num_block_sums;
   // record sort: [start, end) of every id = key >> key_shift in the sorted list (an id that does not occur has an empty
-  // range), and the number of expansion chunks of the ids before each
+  // range), and the chunks of the expansion: the number of those of the ids before each, and (begin, end, id) of them all
   uint32_t *ranges;
   int num_ranges;
   int key_shift;
   uint32_t *chunk_first;
+  uint4 *chunks;
   // depth sort: the number of visible Gaussians, and the place of the culled ones behind them, found by the first pass
   unsigned long long *visible;
   uint32_t *final_vals;
@@ -164,9 +165,9 @@ int launch_emit_records(const uint32_t *depth_order, const uint32_t *cell_count,
                         const uint16_t *rect, const float *mean2d, const float *conic_opacity, const uint32_t *block_sums,
                         const unsigned long long *visible, uint32_t *rec_keys, uint32_t *rec_vals, unsigned long long *rec_total, uint32_t *overflow, int64_t n,
                         int cgx, int W, int H, int64_t capacity, cudaStream_t st);
-// Scratch of the expansion: chunk_first [cells + 1], chunk_counts and chunk_bases [max_pieces, 16], tile_counts and
+// Scratch of the expansion: chunk_first [cells + 1], chunks, chunk_counts and chunk_bases [max_pieces, 16], tile_counts and
 // tile_starts [tiles].
-struct CellScratch { uint32_t *chunk_first, *chunk_counts, *chunk_bases, *tile_counts, *tile_starts; };
+struct CellScratch { uint32_t *chunk_first, *chunk_counts, *chunk_bases, *tile_counts, *tile_starts; uint4 *chunks; };
 int max_pieces(int64_t record_capacity, int num_cells);   // of kBinPiece records (the grid-wide expansion works in larger chunks)
 int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint32_t *cell_ranges, const CellScratch &cs, bool chunks_known,
                   int64_t record_capacity, int64_t pair_capacity, int gx, int gy, int cgx, int cgy,

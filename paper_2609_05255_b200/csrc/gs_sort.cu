@@ -9,6 +9,7 @@
 //     records, one scan for the start of every tile and of every chunk inside it, then each chunk writes its
 //     instances, the lanes that share a tile finding their slots with one ballot.
 // The result is the instance list ordered by (tile, depth key, index), with its per-tile ranges.
+#include <algorithm>
 #include "gs_bin.cuh"
 
 namespace gs {
@@ -68,7 +69,7 @@ __device__ __forceinline__ BlockRange block_range(int64_t count) {
 // The depth keys are sorted with their bits rotated: the sign bit, which only culled Gaussians have set, comes last.  The
 // first of the four passes then has the culled ones in a digit of their own (visible ones have even digits), the largest,
 // and puts them where they belong for good; the other passes and the record emission see the visible ones only (1.2 of 3 million in a view from inside a
-// scene: the four passes 147 us before, XXX now, the emission 68 and XXX).
+// scene: the four passes 147 us before, 107 now, the emission 68 and 50).
 __device__ __forceinline__ uint32_t rotated(uint32_t key) { return __funnelshift_l(key, key, 1); }
 
 // Where a block's elements of a digit go follows from the digits of all blocks before it.  Blocks are taken in groups of
@@ -228,8 +229,17 @@ __global__ void __launch_bounds__(kSortThreads, BITS <= 9 ? 3 : 2) k_radix_scatt
           ep.ranges[2 * d] = start[j]; ep.ranges[2 * d + 1] = start[j] + tot[j];
           ep.chunk_first[d] = first[j];
         }
-        if (d == NB - 1) ep.chunk_first[ep.num_ranges] = first[j] + chunks[j];
+        s_warp_cnt[d] = first[j]; s_warp_cnt[NB + d] = start[j]; s_warp_cnt[2 * NB + d] = start[j] + tot[j];
+        if (d == NB - 1) s_warp_tot[0] = ep.chunk_first[ep.num_ranges] = first[j] + chunks[j];
       }
+      __syncthreads();
+      for (uint32_t q = tid; q < s_warp_tot[0]; q += kSortThreads) {
+        int lo = 0;                                     // the last digit whose chunks begin at q or before
+        for (int step = NB / 2; step > 0; step /= 2) lo += s_warp_cnt[lo + step] <= q ? step : 0;
+        const uint32_t begin = s_warp_cnt[NB + lo] + (q - s_warp_cnt[lo]) * kCellChunk;
+        ep.chunks[q] = make_uint4(begin, min(begin + kCellChunk, s_warp_cnt[2 * NB + lo]), (uint32_t)lo, 0u);
+      }
+      __syncthreads();
     }
   }
 
@@ -490,53 +500,54 @@ __global__ void __launch_bounds__(1024) k_cell_chunks(const uint32_t *__restrict
   if (tid == 0) chunk_first[num_cells] = s_carry;
 }
 
-// The cell and the record range of chunk q, or false if there is no such chunk.
-__device__ __forceinline__ bool chunk_of(uint32_t q, const uint32_t *__restrict__ chunk_first, const uint32_t *__restrict__ cell_ranges,
-                                         int num_cells, int &cell, uint32_t &begin, uint32_t &end) {
-  if (q >= __ldg(chunk_first + num_cells)) return false;
-  int lo = 0, hi = num_cells - 1;     // largest c with chunk_first[c] <= q (cells without records share a value: take the last)
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(chunk_first + mid) <= q) lo = mid; else hi = mid - 1;
+// ... and which records they are: (begin, end, cell) of every chunk.  One warp per cell.
+__global__ void __launch_bounds__(256) k_chunk_list(const uint32_t *__restrict__ cell_ranges, const uint32_t *__restrict__ chunk_first,
+                                                    int num_cells, uint4 *__restrict__ chunks) {
+  dependency_wait();
+  const int lane = threadIdx.x & 31, cell = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (cell >= num_cells) return;
+  const uint32_t s0 = __ldg(cell_ranges + 2 * cell), e0 = __ldg(cell_ranges + 2 * cell + 1);
+  const uint32_t q0 = __ldg(chunk_first + cell), q1 = __ldg(chunk_first + cell + 1);
+  for (uint32_t q = q0 + lane; q < q1; q += 32) {
+    const uint32_t begin = s0 + (q - q0) * kCellChunk;
+    chunks[q] = make_uint4(begin, min(begin + (uint32_t)kCellChunk, e0), (uint32_t)cell, 0u);
   }
-  cell = lo;
-  const uint32_t s0 = __ldg(cell_ranges + 2 * lo), e0 = __ldg(cell_ranges + 2 * lo + 1);
-  begin = s0 + (q - __ldg(chunk_first + lo)) * kCellChunk;
-  end = min(begin + (uint32_t)kCellChunk, e0);
-  return true;
 }
 
+// The two kernels below work on chunks.  Their number is known on the device only, and the host's bound (a record for every
+// instance) is several times too high: a wave of CTAs goes through the chunks there are.
 constexpr int kExpandThreads = 256;
 constexpr int kExpandWarps = kExpandThreads / 32;
 
 // Per chunk: how many instances it holds for each of the 16 tiles of its cell.
-__global__ void __launch_bounds__(kExpandThreads) k_chunk_counts(const uint32_t *__restrict__ rec_keys,
-                                                                 const uint32_t *__restrict__ cell_ranges,
-                                                                 const uint32_t *__restrict__ chunk_first, int num_cells,
-                                                                 uint32_t *__restrict__ chunk_counts) {
+constexpr int kCountBlocks = 148 * 6;
+__global__ void __launch_bounds__(kExpandThreads, 6) k_chunk_counts(const uint32_t *__restrict__ rec_keys, const uint4 *__restrict__ chunks,
+                                                                    const uint32_t *__restrict__ num_chunks, uint32_t *__restrict__ chunk_counts) {
   dependency_wait();
-  __shared__ uint32_t s_cnt[kExpandWarps][16];
+  __shared__ uint32_t s_cnt[2][kExpandWarps][16];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int cell;
-  uint32_t begin, end;
-  if (!chunk_of(blockIdx.x, chunk_first, cell_ranges, num_cells, cell, begin, end)) return;
-  // warp w holds records [begin + 256 w, + 256): lane l the records 256 w + 32 k + l, k = 0..7
-  uint32_t mask[8];
+  const uint32_t num = __ldg(num_chunks);
+  int round = 0;                       // (two sets of counters: one barrier per chunk)
+  for (uint32_t q = blockIdx.x; q < num; q += gridDim.x, round ^= 1) {
+    const uint4 c = __ldg(chunks + q);
+    // warp w holds records [begin + 256 w, + 256): lane l the records 256 w + 32 k + l, k = 0..7
+    uint32_t mask[8];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const uint32_t idx = begin + (uint32_t)(256 * warp + 32 * k + lane);
-    mask[k] = idx < end ? (__ldg(rec_keys + idx) & 0xffffu) : 0u;
-  }
-  uint32_t acc[4], sums[8];
-  count_masks(mask, acc);
-  warp_sum_counts(acc, sums);
-  if (lane < 16) s_cnt[warp][lane] = tile_count_of(sums, lane);
-  __syncthreads();
-  if (tid < 16) {
-    uint32_t t = 0;
+    for (int k = 0; k < 8; ++k) {
+      const uint32_t idx = c.x + (uint32_t)(256 * warp + 32 * k + lane);
+      mask[k] = idx < c.y ? (__ldg(rec_keys + idx) & 0xffffu) : 0u;
+    }
+    uint32_t acc[4], sums[8];
+    count_masks(mask, acc);
+    warp_sum_counts(acc, sums);
+    if (lane < 16) s_cnt[round][warp][lane] = tile_count_of(sums, lane);
+    __syncthreads();
+    if (tid < 16) {
+      uint32_t t = 0;
 #pragma unroll
-    for (int w = 0; w < kExpandWarps; ++w) t += s_cnt[w][tid];
-    chunk_counts[(size_t)blockIdx.x * 16 + tid] = t;
+      for (int w = 0; w < kExpandWarps; ++w) t += s_cnt[round][w][tid];
+      chunk_counts[(size_t)q * 16 + tid] = t;
+    }
   }
 }
 
@@ -577,42 +588,43 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t *__restrict__
 
 // Per chunk: write its instances.  The running positions of the tiles start from the tile's range, the chunk's offset
 // inside it and what the warps before this one hold.
-__global__ void __launch_bounds__(kExpandThreads) k_expand(const uint32_t *__restrict__ rec_keys, const uint32_t *__restrict__ rec_vals,
-                                                           const uint32_t *__restrict__ cell_ranges,
-                                                           const uint32_t *__restrict__ chunk_first, int num_cells,
-                                                           const uint32_t *__restrict__ chunk_bases,
-                                                           const uint32_t *__restrict__ tile_starts, int gx, int gy, int cgx,
-                                                           uint32_t capacity, uint32_t *__restrict__ out_vals) {
+// Bound by the instructions of the ranking and by latency: a CTA used to search its chunk's cell (eight dependent loads),
+// and two of three CTAs found that they had no chunk.  1M Gaussians, 2.0M records, 7.9M instances: the expansion 55 us before, 50 now.
+constexpr int kExpandBlocks = 148 * 4;
+__global__ void __launch_bounds__(kExpandThreads, 4) k_expand(const uint32_t *__restrict__ rec_keys, const uint32_t *__restrict__ rec_vals,
+                                                              const uint4 *__restrict__ chunks, const uint32_t *__restrict__ num_chunks,
+                                                              const uint32_t *__restrict__ chunk_bases,
+                                                              const uint32_t *__restrict__ tile_starts, int gx, int gy, int cgx,
+                                                              uint32_t capacity, uint32_t *__restrict__ out_vals) {
   dependency_wait();
-  __shared__ uint32_t s_cnt[kExpandWarps][16];
+  __shared__ uint32_t s_cnt[2][kExpandWarps][16];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int cell;
-  uint32_t begin, end;
-  if (!chunk_of(blockIdx.x, chunk_first, cell_ranges, num_cells, cell, begin, end)) return;
-  uint32_t mask[8], gid[8];
+  const uint32_t num = __ldg(num_chunks);
+  int round = 0;
+  for (uint32_t q = blockIdx.x; q < num; q += gridDim.x, round ^= 1) {
+    const uint4 c = __ldg(chunks + q);
+    uint32_t mask[8], gid[8];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const uint32_t idx = begin + (uint32_t)(256 * warp + 32 * k + lane);
-    const bool ok = idx < end;
-    mask[k] = ok ? (__ldg(rec_keys + idx) & 0xffffu) : 0u;
-    gid[k] = ok ? __ldg(rec_vals + idx) : 0u;
-  }
-  uint32_t acc[4], sums[8];
-  count_masks(mask, acc);
-  warp_sum_counts(acc, sums);
-  if (lane < 16) s_cnt[warp][lane] = tile_count_of(sums, lane);
-  __syncthreads();
-  // lane t < 16 works out where tile t of the cell continues
-  const int tx0 = 4 * (cell % cgx), ty0 = 4 * (cell / cgx);
-  uint32_t mine = 0;
-  if (lane < 16) {
-    const int tx = tx0 + (lane & 3), ty = ty0 + (lane >> 2);
-    if (tx < gx && ty < gy) {   // (a tile of the cell outside the image has no instances)
-      mine = __ldg(tile_starts + ty * gx + tx) + __ldg(chunk_bases + (size_t)blockIdx.x * 16 + lane);
-      for (int w = 0; w < warp; ++w) mine += s_cnt[w][lane];
+    for (int k = 0; k < 8; ++k) {
+      const uint32_t idx = c.x + (uint32_t)(256 * warp + 32 * k + lane);
+      const bool ok = idx < c.y;
+      mask[k] = ok ? (__ldg(rec_keys + idx) & 0xffffu) : 0u;
+      gid[k] = ok ? __ldg(rec_vals + idx) : 0u;
     }
+    // lane t < 16 works out where tile t of the cell continues
+    const int tx = 4 * ((int)c.z % cgx) + (lane & 3), ty = 4 * ((int)c.z / cgx) + (lane >> 2);
+    uint32_t mine = 0;
+    if (lane < 16 && tx < gx && ty < gy)      // (a tile of the cell outside the image has no instances)
+      mine = __ldg(tile_starts + ty * gx + tx) + __ldg(chunk_bases + (size_t)q * 16 + lane);
+    uint32_t acc[4], sums[8];
+    count_masks(mask, acc);
+    warp_sum_counts(acc, sums);
+    if (lane < 16) s_cnt[round][warp][lane] = tile_count_of(sums, lane);
+    __syncthreads();
+    if (lane < 16)
+      for (int w = 0; w < warp; ++w) mine += s_cnt[round][w][lane];
+    expand_records(mask, gid, mine, capacity, out_vals, lane);
   }
-  expand_records(mask, gid, mine, capacity, out_vals, lane);
 }
 
 }  // namespace
@@ -722,15 +734,18 @@ int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint
                   int64_t record_capacity, int64_t pair_capacity, int gx, int gy, int cgx, int cgy,
                   uint32_t *sorted_vals, uint32_t *tile_ranges, uint32_t *tile_order, cudaStream_t st) {
   const int num_cells = cgx * cgy, chunks = (int)((record_capacity + kCellChunk - 1) / kCellChunk) + num_cells;
-  const uint32_t cap = pair_capacity > 0xffffffffll ? 0xffffffffu : (uint32_t)pair_capacity;
-  if (!chunks_known) launch_chained(k_cell_chunks, 1, 1024, 0, st, cell_ranges, num_cells, cs.chunk_first);
-  launch_chained(k_chunk_counts, chunks, kExpandThreads, 0, st, rec_keys, cell_ranges, cs.chunk_first, num_cells, cs.chunk_counts);
+  const uint32_t cap = pair_capacity > 0xffffffffll ? 0xffffffffu : (uint32_t)pair_capacity, *num_chunks = cs.chunk_first + num_cells;
+  if (!chunks_known) {
+    launch_chained(k_cell_chunks, 1, 1024, 0, st, cell_ranges, num_cells, cs.chunk_first);
+    launch_chained(k_chunk_list, (num_cells + 7) / 8, 256, 0, st, cell_ranges, cs.chunk_first, num_cells, cs.chunks);
+  }
+  launch_chained(k_chunk_counts, std::min(chunks, kCountBlocks), kExpandThreads, 0, st, rec_keys, cs.chunks, num_chunks, cs.chunk_counts);
   launch_chained(k_cell_prefix, (num_cells + 7) / 8, 256, 0, st, cs.chunk_first, cs.chunk_counts, gx, gy, cgx, num_cells, cs.chunk_bases,
                  cs.tile_counts);
   launch_chained(k_tile_scan, 1, 1024, 0, st, cs.tile_counts, gx * gy, cap, cs.tile_starts, tile_ranges, tile_order);
-  launch_chained(k_expand, chunks, kExpandThreads, 0, st, rec_keys, rec_vals, cell_ranges, cs.chunk_first, num_cells, cs.chunk_bases,
+  launch_chained(k_expand, std::min(chunks, kExpandBlocks), kExpandThreads, 0, st, rec_keys, rec_vals, cs.chunks, num_chunks, cs.chunk_bases,
                  cs.tile_starts, gx, gy, cgx, cap, sorted_vals);
-  return chunks_known ? 4 : 5;
+  return chunks_known ? 4 : 6;
 }
 
 // No record was sorted (no Gaussian, or none that reaches a tile): every tile is empty.
