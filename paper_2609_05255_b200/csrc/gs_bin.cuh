@@ -34,48 +34,74 @@ __device__ __forceinline__ uint32_t rank_row(uint32_t *count, uint32_t *lanes, b
   return c + __popc(m & ((1u << lane) - 1u));
 }
 
-// A Gaussian of more than 3 x 3 cells: its cell records worked out again by the whole warp - per row of cells four lanes
-// take the four tile rows, then the lanes take one cell each.  emit(place, cell, mask) is called for record number
-// `place` of the Gaussian, counted on from `first`, by the lane that owns it.
-template <class Emit>
-__device__ __forceinline__ void big_footprint(uint32_t g, uint32_t first, const uint16_t *rect, const float *mean2d,
-                                              const float *conic_opacity, int cgx, int W, int H, int lane, Emit &&emit) {
-  const ushort4 r = __ldg(reinterpret_cast<const ushort4 *>(rect) + g);
-  const float2 m = __ldg(reinterpret_cast<const float2 *>(mean2d) + g);
-  const float4 q = __ldg(reinterpret_cast<const float4 *>(conic_opacity) + g);
-  TileSpans sp;
-  sp.setup(m.x, m.y, q.x, q.y, q.z, footprint_tau(q.w), W, H);
-  const int cy0 = r.y >> 2, cy1 = ((int)r.w - 1) >> 2;
-  uint32_t p = first;
-  for (int cy = cy0; cy <= cy1; ++cy) {
-    // lanes 0..3: the tile rows of this row of cells
-    int xa = 0, xb = 0;
-    const int ty = 4 * cy + lane;
-    const bool has = lane < 4 && ty >= (int)r.y && ty < (int)r.w && sp.row(ty, r.x, r.z, xa, xb);
-    int lo = has ? (xa >> 2) : (1 << 30), hi = has ? ((xb - 1) >> 2) : -1;
-    lo = min(lo, __shfl_xor_sync(kFull, lo, 1)); hi = max(hi, __shfl_xor_sync(kFull, hi, 1));
-    lo = min(lo, __shfl_xor_sync(kFull, lo, 2)); hi = max(hi, __shfl_xor_sync(kFull, hi, 2));
-    lo = __shfl_sync(kFull, lo, 0); hi = __shfl_sync(kFull, hi, 0);
-    if (hi < lo) continue;
-    int ra[4], rb[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      ra[k] = __shfl_sync(kFull, has ? xa : 0, k);
-      rb[k] = __shfl_sync(kFull, has ? xb : 0, k);
+// Gaussians of more than 3 x 3 cells: their cell records worked out again by the whole warp.  The warp takes the numbers
+// start, start + stride, ... below total; entry(number, g, at) gives the Gaussian and the place of its first record, and
+// emit(place, g, cell, mask) is called for each record by the lane that owns it.
+// A lane loads and prepares one Gaussian each; then, Gaussian by Gaussian, the lanes take the 32 tile rows of eight rows of
+// cells together, and one record each.  (A row of cells at a time on four lanes, and each Gaussian's loads before its rows:
+// 16.1 us for the emission of a view of 100 000 Gaussians, of which 170 are large, now 12.8.)
+template <class Entry, class Emit>
+__device__ __forceinline__ void big_footprints(uint32_t start, uint32_t stride, uint32_t total, const uint16_t *rect, const float *mean2d,
+                                               const float *conic_opacity, int cgx, int W, int H, int lane, Entry &&entry, Emit &&emit) {
+  for (uint32_t first = start; first < total; first += 32u * stride) {
+    uint32_t my_g = 0, my_at = 0, my_x = 0, my_y = 0;       // columns and rows of tiles: begin | end << 16
+    TileSpans mine = {};
+    if (first + lane * stride < total) {
+      entry(first + lane * stride, my_g, my_at);
+      const ushort4 r = __ldg(reinterpret_cast<const ushort4 *>(rect) + my_g);
+      const float2 m = __ldg(reinterpret_cast<const float2 *>(mean2d) + my_g);
+      const float4 q = __ldg(reinterpret_cast<const float4 *>(conic_opacity) + my_g);
+      mine.setup(m.x, m.y, q.x, q.y, q.z, footprint_tau(q.w), W, H);
+      my_x = r.x | (uint32_t)r.z << 16;
+      my_y = r.y | (uint32_t)r.w << 16;
     }
-    for (int cb = lo; cb <= hi; cb += 32) {
-      const int cx = cb + lane;
-      if (cx <= hi) {
-        uint32_t mask = 0u;
+    const int held = (int)min(32u, (total - first + stride - 1) / stride);
+    for (int o = 0; o < held; ++o) {
+      TileSpans sp;
+      sp.u = __shfl_sync(kFull, mine.u, o); sp.v = __shfl_sync(kFull, mine.v, o); sp.ila = __shfl_sync(kFull, mine.ila, o);
+      sp.lb = __shfl_sync(kFull, mine.lb, o); sp.lc = __shfl_sync(kFull, mine.lc, o); sp.taup = __shfl_sync(kFull, mine.taup, o);
+      sp.dys = __shfl_sync(kFull, mine.dys, o); sp.eyp = __shfl_sync(kFull, mine.eyp, o); sp.W = W; sp.H = H;
+      const uint32_t g = __shfl_sync(kFull, my_g, o), x = __shfl_sync(kFull, my_x, o), y = __shfl_sync(kFull, my_y, o);
+      uint32_t at = __shfl_sync(kFull, my_at, o);
+      const int y0 = (int)(y & 0xffffu), y1 = (int)(y >> 16);
+      for (int cy0 = y0 >> 2; 4 * cy0 < y1; cy0 += 8) {
+        // lane 4 r + k: tile row k of row of cells cy0 + r
+        int xa = 0, xb = 0;
+        const int ty = 4 * cy0 + lane;
+        const bool has = ty >= y0 && ty < y1 && sp.row(ty, (int)(x & 0xffffu), (int)(x >> 16), xa, xb);
+        if (!has) xa = xb = 0;
+        int lo = has ? (xa >> 2) : (1 << 30), hi = has ? ((xb - 1) >> 2) : -1;
+        lo = min(lo, __shfl_xor_sync(kFull, lo, 1)); hi = max(hi, __shfl_xor_sync(kFull, hi, 1));
+        lo = min(lo, __shfl_xor_sync(kFull, lo, 2)); hi = max(hi, __shfl_xor_sync(kFull, hi, 2));
+        const int cells = max(hi - lo + 1, 0);
+        int end = cells;                                    // records up to and including this row of cells
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int a0 = max(ra[k], 4 * cx) - 4 * cx, b0 = min(rb[k], 4 * cx + 4) - 4 * cx;
-          if (b0 > a0) mask |= (((1u << (b0 - a0)) - 1u) << a0) << (4 * k);
+        for (int s = 4; s < 32; s <<= 1) {
+          const int t = __shfl_up_sync(kFull, end, s);
+          if (lane >= s) end += t;
         }
-        emit(p + (uint32_t)(cx - lo), (uint32_t)(cy * cgx + cx), mask);
+        const int all = __shfl_sync(kFull, end, 31);
+        for (int j0 = 0; j0 < all; j0 += 32) {
+          const int j = j0 + lane;
+          int r = 0;                                        // record j lies in the row of cells r
+#pragma unroll
+          for (int s = 4; s > 0; s >>= 1) {
+            const int e = __shfl_sync(kFull, end, 4 * (r + s - 1));
+            if (j >= e) r += s;
+          }
+          r = min(r, 7);
+          const int cx = __shfl_sync(kFull, lo, 4 * r) + j - __shfl_sync(kFull, end - cells, 4 * r);
+          uint32_t mask = 0u;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int a0 = max(__shfl_sync(kFull, xa, 4 * r + k), 4 * cx) - 4 * cx, b0 = min(__shfl_sync(kFull, xb, 4 * r + k), 4 * cx + 4) - 4 * cx;
+            if (b0 > a0) mask |= (((1u << (b0 - a0)) - 1u) << a0) << (4 * k);
+          }
+          if (j < all) emit(at + (uint32_t)j, g, (uint32_t)((cy0 + r) * cgx + cx), mask);
+        }
+        at += (uint32_t)all;
       }
     }
-    p += (uint32_t)(hi - lo + 1);
   }
 }
 

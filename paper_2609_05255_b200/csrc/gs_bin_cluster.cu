@@ -373,16 +373,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_bin_cluster(ClusterBinArgs a) {
   cluster_sync();
   {
     const uint32_t waiting = __ldcg(a.num_big);
-    for (uint32_t b = rank + ctas * warp; b < waiting; b += ctas * kWarps) {
-      const uint32_t bg = __ldcg(a.tmp_vals + b);
-      big_footprint(bg, __ldcg(a.tmp_keys + b), a.rect, a.mean2d, a.conic_opacity, a.cgx, a.W, a.H, lane,
-                    [&](uint32_t dst, uint32_t cell, uint32_t tiles) {
-                      if (dst < capacity) {
-                        a.rec_keys[dst] = (cell << 16) | tiles;
-                        a.rec_vals[dst] = bg;
-                      }
-                    });
-    }
+    big_footprints(rank + ctas * warp, ctas * kWarps, waiting, a.rect, a.mean2d, a.conic_opacity, a.cgx, a.W, a.H, lane,
+                   [&](uint32_t b, uint32_t &bg, uint32_t &place) { bg = __ldcg(a.tmp_vals + b); place = __ldcg(a.tmp_keys + b); },
+                   [&](uint32_t dst, uint32_t bg, uint32_t cell, uint32_t tiles) {
+                     if (dst < capacity) {
+                       a.rec_keys[dst] = (cell << 16) | tiles;
+                       a.rec_vals[dst] = bg;
+                     }
+                   });
     if (waiting) cluster_sync();
   }
   // ---- records by cell

@@ -392,7 +392,9 @@ __device__ __forceinline__ void copy_records(const uint32_t *cell_records, uint3
 // Every Gaussian, in depth order, writes its records (cell id << 16 | tile mask) and its id.  A Gaussian of at most
 // 3 x 3 cells copies what the preprocess stored; a larger one is worked out again by a warp.  The large ones are the near
 // ones, side by side in this order, so a CTA collects its own and shares them out over its warps.
-__global__ void __launch_bounds__(kScanBlock) k_emit_records(
+// Eight CTAs per SM, although the large ones' path then spills: the copies wait for random rows (at five CTAs 55 instead of
+// 50 us in a view of 1.2 million).
+__global__ void __launch_bounds__(kScanBlock, 8) k_emit_records(
     const uint32_t *__restrict__ order, const uint32_t *__restrict__ cell_count, const uint32_t *__restrict__ cell_records,
     const uint16_t *__restrict__ rect, const float *__restrict__ mean2d, const float *__restrict__ conic_opacity,
     const uint32_t *__restrict__ block_sums, const unsigned long long *__restrict__ visible, int64_t n, int cgx, int W, int H, uint32_t capacity,
@@ -443,15 +445,14 @@ __global__ void __launch_bounds__(kScanBlock) k_emit_records(
     s_big_at[slot] = off;
   }
   __syncthreads();
-  for (uint32_t b = warp; b < s_num_big; b += kScanBlock / 32) {
-    const uint32_t bg = s_big[b];
-    big_footprint(bg, s_big_at[b], rect, mean2d, conic_opacity, cgx, W, H, lane, [&](uint32_t dst, uint32_t cell, uint32_t mask) {
-      if (dst < capacity) {
-        rec_keys[dst] = (cell << 16) | mask;
-        rec_vals[dst] = bg;
-      }
-    });
-  }
+  big_footprints(warp, kScanBlock / 32, s_num_big, rect, mean2d, conic_opacity, cgx, W, H, lane,
+                 [&](uint32_t b, uint32_t &bg, uint32_t &at) { bg = s_big[b]; at = s_big_at[b]; },
+                 [&](uint32_t dst, uint32_t bg, uint32_t cell, uint32_t mask) {
+                   if (dst < capacity) {
+                     rec_keys[dst] = (cell << 16) | mask;
+                     rec_vals[dst] = bg;
+                   }
+                 });
 }
 
 // ---- from the sorted records of a cell to the lists of its tiles ----------------------------------
