@@ -356,7 +356,7 @@ GsStatus gs_neural_prepass(GsContext *ctx, const GsScene *scene, const uint16_t 
  * At most 4096 stage records are kept between two collects; further ones are dropped. */
 typedef enum {
   GS_STAGE_PREPROCESS_FWD = 0, /* projection + fused colour decode                              */
-  GS_STAGE_DEPTH_SORT,         /* radix sort of the Gaussians by depth key (scenes of up to 32768 Gaussians: the
+  GS_STAGE_DEPTH_SORT,         /* radix sort of the Gaussians by depth key (scenes of up to 8192 Gaussians: the
                                   whole binning, which is one kernel and the expansion there)   */
   GS_STAGE_TILE_OFFSETS,       /* (the sums of tiles touched are taken by the depth sort's last pass: no time of its own) */
   GS_STAGE_KEYGEN,             /* instance emission                                             */

@@ -450,9 +450,10 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
   }
   const int num_cells = cd.cgx * cd.cgy;
   const uint32_t cap32 = pair_capacity > 0xffffffffll ? 0xffffffffu : (uint32_t)pair_capacity;
-  // Up to 32768 Gaussians the whole binning is one cluster's work: 16 SMs, but two launches instead of 21.  Measured (the
-  // binning alone): 1000 Gaussians 33 against 81 us, 20 000 58 against 85; at 100 000 the 16 SMs are too few, 131 against
-  // 103.  A CTA for every 64 Gaussians, up to 16 (1000 Gaussians: 33 us on 16 CTAs, 36 on 4).
+  // Up to 8192 Gaussians the whole binning is one cluster's work: 16 SMs, but two launches instead of 12.  Steps measured
+  // with the cluster and with the chain: 2100 Gaussians 115.0 and 118.5 us, 8000 in a small image 87.6 and 88.3, in one of
+  // 640 x 480 113.5 and 112.3, 12 000 143.7 and 142.8, 16 000 137.0 and 131.3, 32 000 138.5 and 132.0.  A CTA for every
+  // 64 Gaussians, up to 16 (1000 Gaussians: 33 us on 16 CTAs, 36 on 4).
   if (sorted && n <= kClusterMax && num_cells <= (1 << kClusterDigit)) {
     ClusterBinArgs b = {};
     b.n = (uint32_t)n; b.capacity = cap32; b.pair_capacity32 = cap32; b.report = report; b.overflow = overflow; b.num_big = w.num_big;

@@ -7,9 +7,8 @@
 // hardware barriers instead, and exchange digit histograms through distributed shared memory.  Keys and records go
 // through global memory between the passes (a few MB that stay in L2).
 // The results are the same bits as those of the grid-wide chain: both are stable sorts.
-// The same kernel as a cooperative grid of one CTA per SM, meeting at a counter in memory, measured 2 % of a step faster at
-// 100 000 Gaussians, 2 % slower at 300 000 and 6 % at a million (barriers of 2 us, and every CTA reading every other's
-// digits): the scenes in between take the chain.
+// The same kernel as a cooperative grid of one CTA per SM, for larger scenes, was no faster than the chain (barriers of
+// 2 us, and every CTA reads every other's digits): a step on 100 000 Gaussians 212 against 217 us, on a million 642 against 604.
 #include "gs_bin.cuh"
 
 namespace gs {
@@ -33,7 +32,7 @@ struct Shared {
   uint32_t base[kBins];                        // where this CTA's next element of a digit goes
   uint32_t tile_count[kBins], tile_start[kBins];
   uint32_t piece_first[kBins + 1];
-  uint32_t warp_sum[kWarps], part[kRows * kWarps];
+  uint32_t warp_sum[kWarps];
   uint32_t lowest, highest, records;           // (read by the others)
   uint32_t all_lowest, all_highest, records_before, all_records;
   TileScan scan;
@@ -310,22 +309,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_bin_cluster(ClusterBinArgs a) {
     }
   }
 
-  // ---- one record per (Gaussian, cell of 4 x 4 tiles), in depth order.  First everyone's number of records, for the places
-  // (ids and counts of the first tile stay in shared memory), then the records, kTile Gaussians at a time.
-  uint32_t mine = 0, own_records;
-  for (uint32_t first = 0; first < count; first += kTile) {
-    uint32_t g[kRows], cc[kRows];
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) { const uint32_t i = first + r * kThreads + tid; g[r] = i < count ? __ldcg(a.order + begin + i) : 0u; }
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) { const uint32_t i = first + r * kThreads + tid; cc[r] = i < count ? __ldg(a.cell_count + g[r]) : 0u; }
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-      mine += cc[r] & ~kCellBig;
-      if (first == 0) { s.vals[r * kThreads + tid] = g[r]; s.keys[r * kThreads + tid] = cc[r]; }
-    }
-  }
-  block_exclusive(s, mine, own_records);
+  // ---- one record per (Gaussian, cell of 4 x 4 tiles), in depth order: a thread per Gaussian for the places
+  static_assert(kClusterMax <= 16 * kThreads, "a thread has one Gaussian at most");
+  const uint32_t g = tid < count ? __ldcg(a.order + begin + tid) : 0u, cc = tid < count ? __ldg(a.cell_count + g) : 0u, cnt = cc & ~kCellBig;
+  uint32_t own_records;
+  const uint32_t place = block_exclusive(s, cnt, own_records);
   if (tid == 0) s.records = own_records;
   cluster_sync();
   if (tid < ctas) {
@@ -336,39 +324,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_bin_cluster(ClusterBinArgs a) {
   __syncthreads();
   const uint32_t capacity = a.capacity, first_record = s.records_before;
   if (rank == 0 && tid == 0 && s.all_records > capacity) *a.overflow = 1u;      // more records than the buffers hold
-  uint32_t at = first_record;
-  for (uint32_t first = 0; first < count; first += kTile) {
-    const int rows = (int)min((count - first + kThreads - 1) / kThreads, (uint32_t)kRows);
-    if (first) {
-      __syncthreads();
-      for (int r = 0; r < rows; ++r) {
-        const uint32_t i = first + r * kThreads + tid, g = i < count ? __ldcg(a.order + begin + i) : 0u;
-        s.vals[r * kThreads + tid] = g;
-        s.keys[r * kThreads + tid] = i < count ? __ldg(a.cell_count + g) : 0u;
-      }
-    }
-    // places: one scan of the sums of all rows' warps
-    for (int r = 0; r < rows; ++r) {
-      const uint32_t sum = __reduce_add_sync(kFull, s.keys[r * kThreads + tid] & ~kCellBig);
-      if (lane == 0) s.part[r * kWarps + warp] = sum;
-    }
-    __syncthreads();
-    uint32_t total;
-    const uint32_t sums = tid < rows * kWarps ? s.part[tid] : 0u, places = block_exclusive(s, sums, total);
-    if (tid < rows * kWarps) s.part[tid] = places;
-    __syncthreads();
-    for (int r = 0; r < rows; ++r) {
-      const uint32_t g = s.vals[r * kThreads + tid], cc = s.keys[r * kThreads + tid], cnt = cc & ~kCellBig;
-      const uint32_t off = at + s.part[r * kWarps + warp] + warp_inclusive(cnt, lane) - cnt;
-      if (cc & kCellBig) {                     // large footprints wait for a warp, below
-        const uint32_t slot = atomicAdd(a.num_big, 1u);
-        a.tmp_vals[slot] = g; a.tmp_keys[slot] = off;
-      }
-      copy_records(a.cell_records, g, (cc & kCellBig) ? 0u : cnt, off, capacity, a.rec_keys, a.rec_vals,
-                   reinterpret_cast<unsigned char *>(s.count) + warp * 32 * kCellSlots, lane);
-    }
-    at += total;
+  if (cc & kCellBig) {                         // large footprints wait for a warp, below
+    const uint32_t slot = atomicAdd(a.num_big, 1u);
+    a.tmp_vals[slot] = g; a.tmp_keys[slot] = first_record + place;
   }
+  copy_records(a.cell_records, g, (cc & kCellBig) ? 0u : cnt, first_record + place, capacity, a.rec_keys, a.rec_vals,
+               reinterpret_cast<unsigned char *>(s.count) + warp * 32 * kCellSlots, lane);
   // large footprints are worked out by a warp each; the near ones are the large ones, so they are shared out over the cluster
   cluster_sync();
   {

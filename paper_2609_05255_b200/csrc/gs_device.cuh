@@ -175,7 +175,7 @@ int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint
 // The whole binning in one cluster of CTAs and one expansion kernel (gs_bin_cluster.cu), for scenes that do not fill the
 // chip.  Up to 2^kClusterDigit cells.
 constexpr int kClusterDigit = 9;              // widest digit of its sorts
-constexpr int kClusterMax = 32768;            // Gaussians (2048 per CTA of the largest cluster)
+constexpr int kClusterMax = 8192;             // Gaussians (512 per CTA of the largest cluster)
 constexpr int kBinPiece = 256;                // records of one cell that a warp counts and expands
 struct ClusterBinArgs {
   uint32_t n, capacity;                        // Gaussians; records the buffers hold
@@ -395,7 +395,8 @@ __device__ __forceinline__ float tanh_fast(float y) {
   return fmaf(-2.f, r, 1.f);
 }
 
-// Programmatic dependent launch.  The kernels of the binning (gs_sort.cu) form chains of short, dependent launches (27 per view).
+// Programmatic dependent launch.  The kernels of the binning (gs_sort.cu) form chains of short, dependent launches (12 per view, 16 of a
+// large scene).
 // Launched with the attribute below, a kernel may be placed on the SMs as soon as the CTAs of its predecessor in the
 // stream have exited, without waiting for the predecessor's completion to be processed; dependency_wait() returns once
 // the predecessor has completed and its writes are visible, and every kernel here calls it before its first access to

@@ -1,4 +1,4 @@
-"""Binning of small scenes runs in one cluster of CTAs (up to 32768 Gaussians and 512 cells of 64 x 64 pixels), in which up
+"""Binning of small scenes runs in one cluster of CTAs (up to 8192 Gaussians and 512 cells of 64 x 64 pixels), in which up
 to 2048 Gaussians are ordered by counting and more by a radix sort; larger ones take the grid-wide kernels.  On both sides
 of these lines the instance lists must be the ones the projected arrays call for: ordered by (tile, depth key, index),
 every Gaussian as often as it touches tiles, with the ranges and the depth order that go with them."""
@@ -36,7 +36,7 @@ def _check(sc, cam):
     return gpu
 
 
-@pytest.mark.parametrize("n", [1, 2, 33, 1025, 2047, 2048, 2049, 5000, 16385, 32767, 32768, 32769])
+@pytest.mark.parametrize("n", [1, 2, 33, 1025, 2047, 2048, 2049, 5000, 8191, 8192, 8193, 16385, 32769])
 def test_scene_sizes(n):
     sc = scenes.box_scene(n, 3.0, -1.0, 8.0, -3.5, 0.8, 1.0, scenes.APP_NEURAL, seed=500 + n)      # some behind the camera
     _check(sc, scenes.identity_camera(333, 217, 300.0))
@@ -51,7 +51,7 @@ def test_image_sizes_and_large_footprints(width, height):
         assert np.any(spans[gpu.visible] > 2)                            # footprints of more than 3 x 3 cells
 
 
-@pytest.mark.parametrize("n", [1500, 20011])
+@pytest.mark.parametrize("n", [1500, 8000, 20011])
 def test_equal_depths_keep_the_index_order(n):
     sc = scenes.box_scene(n, 2.0, 3.0, 3.0, -3.0, 0.5, 1.0, scenes.APP_SH, seed=3)
     assert np.all(sc.means[:, 2] == 3.0)
