@@ -6,6 +6,8 @@
 // and one 8-bit RGBA texel per Gaussian as the result.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "gs_device.cuh"
 #include "gs_mlp_mma.cuh"
 
@@ -15,6 +17,7 @@ namespace {
 constexpr int kFoldThreads = 128;
 constexpr int kPrepassThreads = 128;
 constexpr int kPrepassWarps = kPrepassThreads / 32;
+constexpr int kPrepassBlocks = 8;   // resident CTAs per SM: the most that 64 registers allow (nine spill: 64 us instead of 56)
 constexpr int kXRow = 12;   // 32-bit words per staged input row: 8 half pairs + 4 pad (conflict-free fragment reads)
 
 __global__ void __launch_bounds__(kFoldThreads) k_neural_fold(int64_t n, const __half *__restrict__ features,
@@ -58,14 +61,23 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
   const __half2 p = __floats2half2_rn(a, b);
   return *reinterpret_cast<const uint32_t *>(&p);
 }
+__device__ __forceinline__ uint32_t pack_relu(float a, float b) {              // (rounding keeps the sign)
+  const __half2 p = __hmax2(__floats2half2_rn(a, b), __float2half2_rn(0.f));
+  return *reinterpret_cast<const uint32_t *>(&p);
+}
 __device__ __forceinline__ uint32_t pack_weights(const __half *w, int idx) {   // w[idx], w[idx + 1]; idx is even
   return __ldg(reinterpret_cast<const uint32_t *>(w + idx));
 }
 
-// One warp per 32 Gaussians.  Lane L prepares row L (direction, SH basis, base colour, alpha byte);
+// One warp per 32 Gaussians at a time.  Lane L prepares row L (direction, SH basis, base colour, alpha byte);
 // the rows reach the tensor-core fragment layout through a small shared-memory tile; the weights
 // live in ten registers per lane for the whole kernel.
-__global__ void __launch_bounds__(kPrepassThreads) k_neural_prepass(int64_t n, int deg, int act, const float *__restrict__ means,
+// Bound by instruction issue (70 % of the slots, ALU pipe 63 %; 192 MB need 29 us): the warps are persistent, so that the weights
+// are read once, all addresses are 32-bit offsets from the warp's rows, the rectifiers work on packed halves, and degree 3
+// has an instance without the selects of the others.  3M Gaussians: 61.3 us before, 56.0 now.  Prefetching the next rows
+// takes registers that are worth more as warps (64.5).
+template <bool kFull3>   // degree 3: all direction inputs in use
+__global__ void __launch_bounds__(kPrepassThreads, kPrepassBlocks) k_neural_prepass(int64_t n, int deg, int act, const float *__restrict__ means,
                                                                     const float *__restrict__ logits,
                                                                     const float *__restrict__ base_color,
                                                                     const __half *__restrict__ preact,
@@ -91,85 +103,98 @@ __global__ void __launch_bounds__(kPrepassThreads) k_neural_prepass(int64_t n, i
   w3b1 = g < 3 ? pack_weights(weights, kMlpW3 + g * GS_MLP_HIDDEN + 2 * t + 8) : 0u;
   const int na = (deg + 1) * (deg + 1);
 
-  const int64_t row0 = ((int64_t)blockIdx.x * kPrepassWarps + warp) * 32;
-  if (row0 >= n) return;
-  const int64_t i = row0 + lane;
-  // ---- this lane's Gaussian: direction, direction inputs, base colour, alpha
-  float4 c = make_float4(0.f, 0.f, 0.f, 0.f);   // base colour and the alpha texel value
-  {
-    float Y[16];
+  const int64_t row_first = ((int64_t)blockIdx.x * kPrepassWarps + warp) * 32;
+#pragma unroll 1
+  for (int64_t row0 = row_first; row0 < n; row0 += (int64_t)gridDim.x * kPrepassThreads) {
+    const int rows = (int)min(n - row0, (int64_t)32);     // of this warp; what lies at row0 is addressed by 32-bit offsets
+    const bool in = lane < rows;
+    // ---- the pre-activations of this lane's fragment rows, then its own Gaussian: direction, direction inputs, base
+    // colour, alpha
+    uint32_t pre[2][2][2];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) Y[k] = 0.f;
-    if (i < n) {
-      const float dx = __ldg(means + 3 * i) - ex, dy = __ldg(means + 3 * i + 1) - ey, dz = __ldg(means + 3 * i + 2) - ez;
-      const float inv = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-      sh_basis(dx * inv, dy * inv, dz * inv, Y);
-      const float o = 1.f / (1.f + __expf(-__ldg(logits + i)));
-      c = make_float4(__ldg(base_color + 3 * i), __ldg(base_color + 3 * i + 1), __ldg(base_color + 3 * i + 2),
-                      floorf(fmaf(fminf(fmaxf(o, 0.f), 1.f), 255.f, 0.5f)));
+    for (int r = 0; r < 4; ++r) {
+      const uint32_t *p = reinterpret_cast<const uint32_t *>(preact + 16 * row0) + (uint32_t)(8 * min(8 * r + g, rows - 1) + t);
+      pre[r >> 1][0][r & 1] = __ldg(p);
+      pre[r >> 1][1][r & 1] = __ldg(p + 4);
     }
-    Y[0] = 0.f;   // folded into the pre-activations
+    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);   // base colour and the alpha texel value
+    {
+      float Y[16];
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      s_x[warp][lane][k] = pack_half2(2 * k < na ? Y[2 * k] : 0.f, 2 * k + 1 < na ? Y[2 * k + 1] : 0.f);
-  }
-  __syncwarp();
-  float y[2][4];
+      for (int k = 0; k < 16; ++k) Y[k] = 0.f;
+      if (in) {
+        const float *mean = means + 3 * row0 + (uint32_t)(3 * lane), *base = base_color + 3 * row0 + (uint32_t)(3 * lane);
+        const float dx = __ldg(mean) - ex, dy = __ldg(mean + 1) - ey, dz = __ldg(mean + 2) - ez;
+        const float inv = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+        sh_basis(dx * inv, dy * inv, dz * inv, Y);
+        const float o = 1.f / (1.f + __expf(-__ldg(logits + row0 + (uint32_t)lane)));
+        c = make_float4(__ldg(base), __ldg(base + 1), __ldg(base + 2),
+                        fmaf(fminf(fmaxf(o, 0.f), 1.f), 255.f, 0.5f));
+      }
+      Y[0] = 0.f;   // folded into the pre-activations
 #pragma unroll
-  for (int mt = 0; mt < 2; ++mt) {
-    const int r0 = mt * 16 + g, r1 = r0 + 8;
-    uint32_t a[4] = {s_x[warp][r0][t], s_x[warp][r1][t], s_x[warp][r0][t + 4], s_x[warp][r1][t + 4]};
-    // ---- layer 1, accumulators start at the folded pre-activations
-    float h[2][4];
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      const int64_t ra = row0 + r0 < n ? row0 + r0 : n - 1, rb = row0 + r1 < n ? row0 + r1 : n - 1;
-      const uint32_t p0 = __ldg(reinterpret_cast<const uint32_t *>(preact + 16 * ra + nt * 8 + 2 * t));
-      const uint32_t p1 = __ldg(reinterpret_cast<const uint32_t *>(preact + 16 * rb + nt * 8 + 2 * t));
-      const float2 f0 = __half22float2(*reinterpret_cast<const __half2 *>(&p0));
-      const float2 f1 = __half22float2(*reinterpret_cast<const __half2 *>(&p1));
-      h[nt][0] = f0.x; h[nt][1] = f0.y; h[nt][2] = f1.x; h[nt][3] = f1.y;
-      if (deg > 0) mlp::mma16816(h[nt], a, w1b0[nt], w1b1[nt]);
+      for (int k = 0; k < 8; ++k)
+        s_x[warp][lane][k] = kFull3 ? pack_half2(Y[2 * k], Y[2 * k + 1])
+                                    : pack_half2(2 * k < na ? Y[2 * k] : 0.f, 2 * k + 1 < na ? Y[2 * k + 1] : 0.f);
     }
-    // ---- layer 2: the ReLU'd outputs of two column tiles are one A fragment
-    a[0] = pack_half2(fmaxf(h[0][0], 0.f), fmaxf(h[0][1], 0.f)); a[1] = pack_half2(fmaxf(h[0][2], 0.f), fmaxf(h[0][3], 0.f));
-    a[2] = pack_half2(fmaxf(h[1][0], 0.f), fmaxf(h[1][1], 0.f)); a[3] = pack_half2(fmaxf(h[1][2], 0.f), fmaxf(h[1][3], 0.f));
+    __syncwarp();
+    float y[2][4];
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      h[nt][0] = h[nt][1] = h[nt][2] = h[nt][3] = 0.f;
-      mlp::mma16816(h[nt], a, w2b0[nt], w2b1[nt]);
-    }
-    // ---- layer 3 (three outputs, padded to eight columns)
-    a[0] = pack_half2(fmaxf(h[0][0], 0.f), fmaxf(h[0][1], 0.f)); a[1] = pack_half2(fmaxf(h[0][2], 0.f), fmaxf(h[0][3], 0.f));
-    a[2] = pack_half2(fmaxf(h[1][0], 0.f), fmaxf(h[1][1], 0.f)); a[3] = pack_half2(fmaxf(h[1][2], 0.f), fmaxf(h[1][3], 0.f));
-    y[mt][0] = y[mt][1] = y[mt][2] = y[mt][3] = 0.f;
-    mlp::mma16816(y[mt], a, w3b0, w3b1);
-  }
-  // ---- the three outputs go back from the fragment layout (lanes t = 0 hold outputs 0, 1 of rows g and
-  // g + 8, lanes t = 1 output 2) to one row per lane, so that every lane finishes its own Gaussian
+    for (int mt = 0; mt < 2; ++mt) {
+      const int r0 = mt * 16 + g, r1 = r0 + 8;
+      uint32_t a[4] = {s_x[warp][r0][t], s_x[warp][r1][t], s_x[warp][r0][t + 4], s_x[warp][r1][t + 4]};
+      // ---- layer 1, accumulators start at the folded pre-activations
+      float h[2][4];
 #pragma unroll
-  for (int mt = 0; mt < 2; ++mt) {
-    if (t == 0) {
-      s_y[warp][mt * 16 + g][0] = y[mt][0]; s_y[warp][mt * 16 + g][1] = y[mt][1];
-      s_y[warp][mt * 16 + g + 8][0] = y[mt][2]; s_y[warp][mt * 16 + g + 8][1] = y[mt][3];
-    } else if (t == 1) {
-      s_y[warp][mt * 16 + g][2] = y[mt][0];
-      s_y[warp][mt * 16 + g + 8][2] = y[mt][2];
-    }
-  }
-  __syncwarp();
-  if (i < n) {
-    float col[3];
-    unsigned q[3];
+      for (int nt = 0; nt < 2; ++nt) {
+        const float2 f0 = __half22float2(*reinterpret_cast<const __half2 *>(&pre[mt][nt][0]));
+        const float2 f1 = __half22float2(*reinterpret_cast<const __half2 *>(&pre[mt][nt][1]));
+        h[nt][0] = f0.x; h[nt][1] = f0.y; h[nt][2] = f1.x; h[nt][3] = f1.y;
+        if (kFull3 || deg > 0) mlp::mma16816(h[nt], a, w1b0[nt], w1b1[nt]);
+      }
+      // ---- layer 2: the ReLU'd outputs of two column tiles are one A fragment
+      a[0] = pack_relu(h[0][0], h[0][1]); a[1] = pack_relu(h[0][2], h[0][3]);
+      a[2] = pack_relu(h[1][0], h[1][1]); a[3] = pack_relu(h[1][2], h[1][3]);
 #pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-      // tanh(a) = 1 - 2 / (exp(2a) + 1); the fast exponential and division are far inside the texel's step
-      const float res = deg > 0 ? 1.f - __fdividef(2.f, __expf(2.f * s_y[warp][lane][ch]) + 1.f) : 0.f;
-      col[ch] = color_act_z(act, (ch == 0 ? c.x : ch == 1 ? c.y : c.z) + 0.5f + res);
-      q[ch] = (unsigned)floorf(fmaf(fminf(col[ch], 1.f), 255.f, 0.5f));
+      for (int nt = 0; nt < 2; ++nt) {
+        h[nt][0] = h[nt][1] = h[nt][2] = h[nt][3] = 0.f;
+        mlp::mma16816(h[nt], a, w2b0[nt], w2b1[nt]);
+      }
+      // ---- layer 3 (three outputs, padded to eight columns)
+      a[0] = pack_relu(h[0][0], h[0][1]); a[1] = pack_relu(h[0][2], h[0][3]);
+      a[2] = pack_relu(h[1][0], h[1][1]); a[3] = pack_relu(h[1][2], h[1][3]);
+      y[mt][0] = y[mt][1] = y[mt][2] = y[mt][3] = 0.f;
+      mlp::mma16816(y[mt], a, w3b0, w3b1);
     }
-    rgba[i] = make_uchar4((unsigned char)q[0], (unsigned char)q[1], (unsigned char)q[2], (unsigned char)c.w);
-    if (color) { color[3 * i] = col[0]; color[3 * i + 1] = col[1]; color[3 * i + 2] = col[2]; }
+    // ---- the three outputs go back from the fragment layout (lanes t = 0 hold outputs 0, 1 of rows g and
+    // g + 8, lanes t = 1 output 2) to one row per lane, so that every lane finishes its own Gaussian
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+      if (t == 0) {
+        s_y[warp][mt * 16 + g][0] = y[mt][0]; s_y[warp][mt * 16 + g][1] = y[mt][1];
+        s_y[warp][mt * 16 + g + 8][0] = y[mt][2]; s_y[warp][mt * 16 + g + 8][1] = y[mt][3];
+      } else if (t == 1) {
+        s_y[warp][mt * 16 + g][2] = y[mt][0];
+        s_y[warp][mt * 16 + g + 8][2] = y[mt][2];
+      }
+    }
+    __syncwarp();
+    if (in) {
+      float col[3];
+      unsigned q[3];
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch) {
+        // tanh(a) = 1 - 2 / (exp(2a) + 1); the fast exponential and division are far inside the texel's step
+        const float res = kFull3 || deg > 0 ? 1.f - __fdividef(2.f, __expf(2.f * s_y[warp][lane][ch]) + 1.f) : 0.f;
+        col[ch] = color_act_z(act, (ch == 0 ? c.x : ch == 1 ? c.y : c.z) + 0.5f + res);
+        q[ch] = (unsigned)fmaf(fminf(col[ch], 1.f), 255.f, 0.5f);   // (rounds down)
+      }
+      reinterpret_cast<uint32_t *>(rgba + row0)[lane] = q[0] | q[1] << 8 | q[2] << 16 | (unsigned)c.w << 24;
+      if (color) {
+        float *out = color + 3 * row0 + (uint32_t)(3 * lane);
+        out[0] = col[0]; out[1] = col[1]; out[2] = col[2];
+      }
+    }
   }
 }
 
@@ -185,7 +210,8 @@ int launch_neural_prepass(int64_t n, int deg, int act, const float *means, const
                           const __half *preact, const __half *weights, const float eye[3], uint8_t *rgba, float *color,
                           cudaStream_t st) {
   if (n <= 0) return 0;
-  k_neural_prepass<<<(unsigned)((n + kPrepassThreads - 1) / kPrepassThreads), kPrepassThreads, 0, st>>>(
+  const int64_t blocks = std::min<int64_t>((n + kPrepassThreads - 1) / kPrepassThreads, 148 * kPrepassBlocks);
+  (deg >= 3 ? k_neural_prepass<true> : k_neural_prepass<false>)<<<(unsigned)blocks, kPrepassThreads, 0, st>>>(
       n, deg, act, means, logits, base_color, preact, weights, eye[0], eye[1], eye[2], reinterpret_cast<uchar4 *>(rgba), color);
   return 1;
 }
