@@ -451,10 +451,10 @@ def ncu_constants():
 # Names of the timed stages (the C ABI's stage enumeration) and the kernels behind them.
 STAGE_KERNELS = {
     "preprocess_fwd": "k_preprocess_fwd (projection, fused appearance, cell records of 4x4 tiles)",
-    "depth_sort": "4 x (k_radix_hist, k_radix_scan_rows, k_radix_scatter<8>) on the 32-bit depth keys of all Gaussians",
+    "depth_sort": "4 x (k_radix_hist, k_radix_scatter<8>) on the 32-bit depth keys, culled Gaussians placed by the first pass, k_group_sums",
     "keygen": "k_emit_records: (cell id, 16-bit tile mask) records in depth order",
-    "tile_sort": "k_radix_hist, k_radix_scan_rows, k_radix_scatter<9>: one stable pass on the cell id",
-    "tile_ranges": "k_cell_chunks, k_chunk_counts, k_cell_prefix, k_tile_scan, k_expand: records -> per-tile lists",
+    "tile_sort": "k_radix_hist, k_radix_scatter<9>: one stable pass on the cell id, cell ranges and chunks from its totals",
+    "tile_ranges": "k_chunk_counts, k_cell_prefix, k_tile_scan, k_expand: records -> per-tile lists",
     "blend_fwd": "k_blend_fwd", "blend_bwd": "k_blend_bwd",
     "preprocess_bwd": "k_preprocess_bwd_sparse (the Gaussians with a gradient in full batches; the zero rows are written by k_blend_bwd) + k_wgrad_reduce"}
 

@@ -133,17 +133,18 @@ __device__ __forceinline__ uint32_t tile_count_of(const uint32_t sums[8], int t)
   return (sums[2 * (t >> 2) + ((t & 3) >> 1)] >> (16 * (t & 1))) & 0xffffu;
 }
 
-__device__ __forceinline__ void store_if(bool p, uint32_t *addr, uint32_t v) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.global.u32 [%1], %2;\n\t}" :: "r"((uint32_t)p), "l"(addr), "r"(v) : "memory");
+__device__ __forceinline__ void store_if(uint32_t p, uint32_t *addr, uint32_t v) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.global.u32 [%1], %2;\n\t}" :: "r"(p), "l"(addr), "r"(v) : "memory");
 }
 
 // A warp writes the instances of its 8 x 32 records (consecutive in depth order, 32 at a time).  A record's slot in the
 // list of tile t is the tile's running position plus the number of lower lanes that also list t: the 16
 // indicator bits of a lane's mask are spread over four words of byte counters and one warp-wide prefix sum of those
 // four words ranks all 16 tiles at once (at most 32 per byte).  `mine`: lane t < 16 passes where tile t continues; every
-// lane keeps all 16 running positions.
-__device__ __forceinline__ void expand_records(const uint32_t mask[8], const uint32_t gid[8], uint32_t mine, uint32_t capacity,
-                                               uint32_t *out_vals, int lane) {
+// lane keeps all 16 running positions.  kInside: no position reaches the capacity, so that a store needs its mask bit only.
+template <bool kInside>
+__device__ __forceinline__ void expand_rows(const uint32_t mask[8], const uint32_t gid[8], uint32_t mine, uint32_t capacity,
+                                            uint32_t *out_vals, int lane) {
   uint32_t cur[16];
 #pragma unroll
   for (int t = 0; t < 16; ++t) cur[t] = __shfl_sync(kFull, mine, t);
@@ -172,10 +173,18 @@ __device__ __forceinline__ void expand_records(const uint32_t mask[8], const uin
       const int r = t >> 2, sh = 8 * (t & 3);
       // one predicated store (no branch): the lane lists tile t and the slot lies inside the buffer
       const uint32_t pos = cur[t] + (((incl[r] - own[r]) >> sh) & 0xffu);
-      store_if(((m >> t) & 1u) != 0u && pos < capacity, out_vals + pos, gid[k]);
+      store_if(kInside || pos < capacity ? m & (1u << t) : 0u, out_vals + pos, gid[k]);
       cur[t] += (tot[r] >> sh) & 0xffu;
     }
   }
+}
+// `count`: instances that the warp writes for tile `lane` (lanes below 16).
+__device__ __forceinline__ void expand_records(const uint32_t mask[8], const uint32_t gid[8], uint32_t mine, uint32_t count,
+                                               uint32_t capacity, uint32_t *out_vals, int lane) {
+  if (__all_sync(kFull, lane >= 16 || (mine <= capacity && count <= capacity - mine)))
+    expand_rows<true>(mask, gid, mine, capacity, out_vals, lane);
+  else
+    expand_rows<false>(mask, gid, mine, capacity, out_vals, lane);
 }
 
 // By one CTA of 1024 threads: the exclusive scan of the tile counts in tile order = the tile ranges, and the launch

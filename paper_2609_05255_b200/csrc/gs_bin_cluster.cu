@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand_pieces(ClusterBinArgs
     const int tx = 4 * (lo % a.cgx) + (lane & 3), ty = 4 * (lo / a.cgx) + (lane >> 2);
     uint32_t mine = 0;                         // (a tile of the cell outside the image has no instances)
     if (lane < 16 && tx < a.gx && ty < a.gy) mine = __ldg(a.tile_starts + ty * a.gx + tx) + __ldg(a.piece_bases + (size_t)q * 16 + lane);
-    expand_records(tiles, gid, mine, a.pair_capacity32, a.out_vals, lane);
+    expand_records(tiles, gid, mine, kBinPiece, a.pair_capacity32, a.out_vals, lane);    // (kBinPiece at most)
   }
 }
 
