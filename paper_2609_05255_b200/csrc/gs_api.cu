@@ -192,7 +192,7 @@ struct Carver {
 };
 
 struct FwdWorkspace {
-  uint32_t *sorted_depth, *tmp_keys, *tmp_vals;          // [n]
+  uint32_t *sorted_depth, *tmp_keys, *tmp_vals;          // [n] keys of the depth sort; the first ends as the sorted record counts
   uint32_t *block_sums;                                  // cell records per 256 depth-sorted Gaussians
   uint32_t *rec_keys, *rec_vals, *tmp_rkeys, *tmp_rvals; // [pair_capacity]: cell records (never more than instances, save for
                                                          // slivers that reach a cell's rows but none of its tiles)
@@ -477,7 +477,7 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
     {
       StageTimer t(ctx, GS_STAGE_DEPTH_SORT, s);
       SortEpilogue ep = {};
-      ep.counts = proj->cell_count; ep.count_mask = ~kCellBig; ep.block_sums = w.block_sums; ep.num_block_sums = num_scan_blocks(n);
+      ep.counts = proj->cell_count; ep.block_sums = w.block_sums; ep.num_block_sums = num_scan_blocks(n);
       t.done(launch_depth_sort(proj->depth_key, w.sorted_depth, bin->depth_order, w.tmp_keys, w.tmp_vals, n, num_visible, w.sort_table,
                                ep, report, s));
     }
@@ -485,7 +485,7 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
     // whose last pass finds where every cell's records begin and end
     {
       StageTimer t(ctx, GS_STAGE_KEYGEN, s);
-      t.done(launch_emit_records(bin->depth_order, proj->cell_count, proj->cell_records, proj->rect, proj->mean2d,
+      t.done(launch_emit_records(bin->depth_order, w.sorted_depth, proj->cell_records, proj->rect, proj->mean2d,
                                  proj->conic_opacity, w.block_sums, num_visible, w.rec_keys, w.rec_vals, w.rec_total, overflow, n, cd.cgx,
                                  cd.W, cd.H, pair_capacity, s));
     }

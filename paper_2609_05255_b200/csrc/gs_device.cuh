@@ -129,10 +129,10 @@ constexpr int kWgradBlocks = 592;   // persistent blocks of the decoder-gradient
 // Sorting / binning.
 // What the scatter of the last pass of a sort adds on its way out (nothing where the pointers are null).
 struct SortEpilogue {
-  // depth sort: sums of a per-Gaussian count (counts[id] & count_mask) per 256 consecutive Gaussians of the sorted
-  // order, from which the record emission takes its offsets; cleared by the same pass
+  // depth sort: sums of the Gaussians' record counts (counts[id], without the flag of a large footprint) per 256
+  // consecutive Gaussians of the sorted order, from which the record emission takes its offsets; cleared by the same pass
   const uint32_t *counts;
-  uint32_t count_mask;
+  uint32_t id_mask;             // bits of a sorted value that are the id (all: no count travels with it)
   uint32_t *block_sums;
   int num_block_sums;
   // record sort: [start, end) of every id = key >> key_shift in the sorted list (an id that does not occur has an empty
@@ -155,13 +155,13 @@ int launch_record_sort(uint32_t *keys, uint32_t *vals, uint32_t *other_keys, uin
                        const unsigned long long *count_dev, int cell_bits, void *scratch, const SortEpilogue &epilogue, cudaStream_t st);
 int radix_passes(int num_bits);
 // The depth order: ids by (key, id) ascending, where a key is the bits of a float, or 0xffffffff: culled Gaussians, behind
-// all others.  keys / tmp_keys / tmp_vals [n] are scratch.  With visible != nullptr all floats are positive; it receives
+// all others.  tmp_keys / tmp_vals [n] are scratch, keys [n] receives the record counts in that order.  With visible != nullptr all floats are positive; it receives
 // the number of Gaussians that are not culled, and the epilogue's block sums cover those.
 int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order, uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t n,
                       unsigned long long *visible, void *scratch, const SortEpilogue &epilogue, const CountReport &report, cudaStream_t st);
 size_t scan_scratch_bytes(int64_t n);
 int num_scan_blocks(int64_t n);   // entries of the block sums that launch_emit_records reads
-int launch_emit_records(const uint32_t *depth_order, const uint32_t *cell_count, const uint32_t *cell_records,
+int launch_emit_records(const uint32_t *depth_order, const uint32_t *sorted_count, const uint32_t *cell_records,
                         const uint16_t *rect, const float *mean2d, const float *conic_opacity, const uint32_t *block_sums,
                         const unsigned long long *visible, uint32_t *rec_keys, uint32_t *rec_vals, unsigned long long *rec_total, uint32_t *overflow, int64_t n,
                         int cgx, int W, int H, int64_t capacity, cudaStream_t st);

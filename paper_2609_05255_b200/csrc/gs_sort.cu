@@ -70,6 +70,13 @@ __device__ __forceinline__ BlockRange block_range(int64_t count) {
 // first of the four passes then has the culled ones in a digit of their own (visible ones have even digits), the largest,
 // and puts them where they belong for good; the other passes and the record emission see the visible ones only (1.2 of 3 million in a view from inside a
 // scene: the four passes 147 us before, 107 now, the emission 68 and 50).
+// What the emission needs to know of a Gaussian first, how many records it has (nine at most, unless its footprint is large),
+// travels with its id in the upper bits of the sorted value, where ids leave room: read in order by the first pass, where the
+// last pass and the emission fetched it from random rows (emission of 1M Gaussians 33.4 us before, 30.3 now, of 1.5M 46.2
+// and 41.6; the sort itself takes as long as before).
+constexpr int kIdBits = 28;
+constexpr uint32_t kCountUnknown = 15u;        // a large footprint: to be looked up
+static_assert(kCellSlots < (int)kCountUnknown, "counts of the stored records fit");
 __device__ __forceinline__ uint32_t rotated(uint32_t key) { return __funnelshift_l(key, key, 1); }
 
 // Where a block's elements of a digit go follows from the digits of all blocks before it.  Blocks are taken in groups of
@@ -167,7 +174,8 @@ template <int BITS> constexpr size_t scatter_smem_bytes() {
 // digit arrays hold max(256, 2^BITS) entries, thread t looking after digits t * DPT ..).  Slots past the
 // end of the input carry the largest digit and sit at the end of the last tile, so they rank after
 // every real key and are never written.
-// EP selects the epilogue: 0 none, 1 block sums of a per-Gaussian count (last pass of the depth sort), 2 ranges of
+// EP selects the epilogue: 0 none, 1 the last pass of the depth sort: leaves the Gaussians' record counts in place of the
+// keys, and their sums per block of sorted positions, 2 ranges of
 // equal ids = key >> key_shift (last pass of the record sort: inside a block's run of one digit the keys are
 // non-decreasing, because the earlier passes ordered the lower bits, so a change of id between neighbours of a run
 // is a boundary; the two ends of a run may continue in another block and enter with an atomic min / max), 3 the first
@@ -293,6 +301,10 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
       const int64_t idx = tile_begin + local;
       key[it] = ok ? (EP == 3 ? rotated(__ldg(keys_in + idx)) : __ldg(keys_in + idx)) : 0xffffffffu;
       val[it] = ok ? (vals_in ? __ldg(vals_in + idx) : (uint32_t)idx) : 0u;
+      if (EP == 3 && ok && ep.id_mask != ~0u) {
+        const uint32_t c = __ldg(ep.counts + idx);
+        val[it] |= min(c, kCountUnknown) << kIdBits;    // (a large footprint's count has its top bit set)
+      }
     }
 #pragma unroll
     for (int it = 0; it < kItems; ++it) {
@@ -364,9 +376,13 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
         if (!ok) continue;
         const uint32_t k = s_keys[j], d = (k >> shift) & kDigitMask, v = s_vals[j], run_first = s_digit_start[d];
         gpos[h] = s_base[d] + ((uint32_t)j - run_first);
-        if (EP == 1) count_of[h] = __ldg(ep.counts + v) & ep.count_mask;
-        if (EP == 3 && d == kDigitMask) {
-          ep.final_vals[gpos[h]] = v;
+        if (EP == 1) {
+          const uint32_t id = v & ep.id_mask, c = ep.id_mask != ~0u && v >> kIdBits != kCountUnknown ? v >> kIdBits : __ldg(ep.counts + id);
+          keys_out[gpos[h]] = c;
+          vals_out[gpos[h]] = id;
+          count_of[h] = c & ~kCellBig;
+        } else if (EP == 3 && d == kDigitMask) {
+          ep.final_vals[gpos[h]] = v & ep.id_mask;
         } else {
           keys_out[gpos[h]] = k;
           vals_out[gpos[h]] = v;
@@ -387,16 +403,18 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
       if (EP == 1) {
 #pragma unroll
         for (int h = 0; h < kOut; ++h) {
-          // the Gaussian's count, added to the sum of its block of kScanBlock sorted positions; a warp whose
-          // lanes all fall into one block (the usual case: a run is contiguous) adds once
+          // the Gaussian's count, added to the sum of its block of kScanBlock sorted positions: once per warp for the first
+          // lane's block and once for the last one's (runs of this digit are long, so that hardly any lane has another)
           const bool ok = j0 + h * kSortThreads + tid < valid_count;
-          const uint32_t blk = gpos[h] / kScanBlock, blk0 = __shfl_sync(kFull, blk, 0);
-          if (__all_sync(kFull, !ok || blk == blk0)) {
-            const uint32_t sum = __reduce_add_sync(kFull, count_of[h]);
-            if (lane == 0 && sum) atomicAdd(ep.block_sums + blk0, sum);
-          } else if (count_of[h]) {
-            atomicAdd(ep.block_sums + blk, count_of[h]);
-          }
+          const uint32_t any = __ballot_sync(kFull, ok);
+          if (!any) continue;
+          const int last = 31 - __clz(any);
+          const uint32_t blk = gpos[h] / kScanBlock, blk0 = __shfl_sync(kFull, blk, 0), blk1 = __shfl_sync(kFull, blk, last);
+          const bool in0 = blk == blk0, in1 = !in0 && blk == blk1;
+          const uint32_t sum0 = __reduce_add_sync(kFull, in0 && ok ? count_of[h] : 0u), sum1 = __reduce_add_sync(kFull, in1 && ok ? count_of[h] : 0u);
+          if (lane == 0 && sum0) atomicAdd(ep.block_sums + blk0, sum0);
+          if (lane == last && sum1) atomicAdd(ep.block_sums + blk1, sum1);
+          if (ok && !in0 && !in1 && count_of[h]) atomicAdd(ep.block_sums + blk, count_of[h]);
         }
       }
     }
@@ -436,7 +454,7 @@ __device__ __forceinline__ void copy_records(const uint32_t *cell_records, uint3
 // Eight CTAs per SM, although the large ones' path then spills: the copies wait for random rows (at five CTAs 55 instead of
 // 50 us in a view of 1.2 million).
 __global__ void __launch_bounds__(kScanBlock, 8) k_emit_records(
-    const uint32_t *__restrict__ order, const uint32_t *__restrict__ cell_count, const uint32_t *__restrict__ cell_records,
+    const uint32_t *__restrict__ order, const uint32_t *__restrict__ sorted_count, const uint32_t *__restrict__ cell_records,
     const uint16_t *__restrict__ rect, const float *__restrict__ mean2d, const float *__restrict__ conic_opacity,
     const uint32_t *__restrict__ block_sums, const unsigned long long *__restrict__ visible, int64_t n, int cgx, int W, int H, uint32_t capacity,
     uint32_t *__restrict__ rec_keys, uint32_t *__restrict__ rec_vals, unsigned long long *__restrict__ rec_total,
@@ -453,7 +471,7 @@ __global__ void __launch_bounds__(kScanBlock, 8) k_emit_records(
   uint32_t g = 0, cc = 0;
   if (i < n) {
     g = __ldg(order + i);
-    cc = __ldg(cell_count + g);
+    cc = __ldg(sorted_count + i);
   }
   const uint32_t cnt = cc & ~kCellBig;
   uint32_t inc = cnt;
@@ -738,11 +756,14 @@ int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order
   const int blocks = sort_blocks(n), group = group_size(blocks);
   uint32_t *table = block_table(scratch);
   SortEpilogue ep[4] = {};
+  ep[3] = epilogue;
+  ep[3].id_mask = ~0u;
   if (visible) {
     ep[0].visible = visible;
     ep[0].final_vals = order;
+    ep[0].counts = epilogue.counts;
+    ep[0].id_mask = ep[3].id_mask = n <= (int64_t)1 << kIdBits ? (1u << kIdBits) - 1u : ~0u;
   }
-  ep[3] = epilogue;
   const bool direct = blocks <= kDirectBlocks && visible;
   // digit tables of the passes, where each has its own: those of the passes to come lie together, after the groups' tables
   const auto pass_table = [&](int p) { return table + ((size_t)((p + 3) & 3) * blocks << 8); };
@@ -772,13 +793,13 @@ int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order
 size_t scan_scratch_bytes(int64_t n) { return (size_t)((n + kScanBlock - 1) / kScanBlock + 1) * sizeof(uint32_t); }
 int num_scan_blocks(int64_t n) { return (int)((n + kScanBlock - 1) / kScanBlock); }
 
-int launch_emit_records(const uint32_t *depth_order, const uint32_t *cell_count, const uint32_t *cell_records,
+int launch_emit_records(const uint32_t *depth_order, const uint32_t *sorted_count, const uint32_t *cell_records,
                         const uint16_t *rect, const float *mean2d, const float *conic_opacity, const uint32_t *block_sums,
                         const unsigned long long *visible, uint32_t *rec_keys, uint32_t *rec_vals, unsigned long long *rec_total, uint32_t *overflow, int64_t n,
                         int cgx, int W, int H, int64_t capacity, cudaStream_t st) {
   if (n <= 0) return 0;
   const uint32_t cap = capacity > 0xffffffffll ? 0xffffffffu : (uint32_t)capacity;
-  launch_chained(k_emit_records, num_scan_blocks(n), kScanBlock, 0, st, depth_order, cell_count, cell_records, rect, mean2d, conic_opacity,
+  launch_chained(k_emit_records, num_scan_blocks(n), kScanBlock, 0, st, depth_order, sorted_count, cell_records, rect, mean2d, conic_opacity,
                  block_sums, visible, n, cgx, W, H, cap, rec_keys, rec_vals, rec_total, overflow);
   return 1;
 }
