@@ -2,7 +2,7 @@
 // order, records ordered by cell, instances counted per tile, tile ranges - in ONE kernel of one thread-block cluster,
 // and a second one that writes the instance lists.
 //
-// For such scenes the grid-wide chain of gs_sort.cu (21 launches) is bound by the launches: each of its kernels has a
+// For such scenes the grid-wide chain of gs_sort.cu (12 launches) is bound by the launches: each of its kernels has a
 // few microseconds of work at most.  Here the up to 16 CTAs of a cluster, 1024 threads each on an SM of its own, meet at
 // hardware barriers instead, and exchange digit histograms through distributed shared memory.  Keys and records go
 // through global memory between the passes (a few MB that stay in L2).

@@ -1,13 +1,14 @@
 // Ordering and binning: a stable LSD radix sort (digits of 4 to 9 bits, keys staged and ranked in shared
 // memory, no inter-block waiting) and the kernels that turn its output into per-tile lists.
 //
-// (1) The Gaussians are sorted once by their 32-bit depth key (ties keep the index order: the sort is stable).
+// (1) The Gaussians are sorted once by their 32-bit depth key (ties keep the index order: the sort is stable), culled ones
+//     leaving after the first of the four passes.
 // (2) In that order every Gaussian emits one record per CELL of 4 x 4 tiles that its footprint reaches - the cell id
 //     and a 16-bit mask of the tiles met inside the cell, as the preprocess left them - and the records are sorted by
 //     cell id alone (a quarter of the elements and fewer bits than a sort of the (Gaussian, tile) instances).
 // (3) A cell's records, still in depth order, are expanded into the lists of its 16 tiles: counts per chunk of 2048
 //     records, one scan for the start of every tile and of every chunk inside it, then each chunk writes its
-//     instances, the lanes that share a tile finding their slots with one ballot.
+//     instances, a warp ranking 32 records for all 16 tiles with one prefix sum of byte counters.
 // The result is the instance list ordered by (tile, depth key, index), with its per-tile ranges.
 #include <algorithm>
 #include "gs_bin.cuh"
