@@ -394,12 +394,15 @@ GsStatus gs_async_pairs(GsContext *ctx, int64_t *num_pairs_host, void *stream) {
   *num_pairs_host = 0;
   GsStatus st;
   if (ctx->reports) {
-    // The view's first binning kernel writes the count with the view's number; the kernels behind it need not be waited for.  Should the stream have drained (or failed) without it, the copy below has the answer.
+    // The view's first binning kernel writes the count with the view's number; the kernels behind it need not be waited for.
+    // Should the stream have drained (or failed) without it, or the count be too large for the word, the copy below has the
+    // answer.
     volatile unsigned long long *h = ctx->h_counter + 8;
     for (unsigned spins = 1;; ++spins) {
       const unsigned long long v = *h;
       if (v >> kCountBits == ctx->views) {
-        *num_pairs_host = (int64_t)(v & ((1ull << kCountBits) - 1));
+        if ((v & kCountMost) == kCountMost) break;
+        *num_pairs_host = (int64_t)(v & kCountMost);
         return GS_OK;
       }
       if ((spins & 4095u) == 0 && cudaStreamQuery(s) != cudaErrorNotReady) break;

@@ -44,6 +44,9 @@ constexpr int kAppExternal = 3;
 // split ones: GsScene.decoder_precision = GS_DECODER_HALF.  Same kernels, same weights, same layout.
 constexpr int kAppNeuralHalf = 4;
 
+// Instances of a view: below 2^31 Gaussians with at most 2^20 tiles each (65536 cells of 16).  The 13 bits left in a word
+// of 64 count the warps of the preprocess (888 CTAs of four on a B200).
+constexpr int kSumBits = 51;
 struct PreprocessArgs {
   int64_t n;
   const float *means, *log_scales, *quats, *logits, *base_color, *sh_rest;
@@ -52,8 +55,8 @@ struct PreprocessArgs {
   float *mean2d, *conic_opacity, *color, *extent;
   uint32_t *depth_key, *tiles_touched, *cell_count, *cell_records;
   uint16_t *rect;
-  unsigned long long *pair_counter;   // [0] receives the instance count; [1] zero before and after: the sum so far (40 bits)
-                                      // and the warps that have added to it (24 bits)
+  unsigned long long *pair_counter;   // [0] receives the instance count; [1] zero before and after: the sum so far (kSumBits)
+                                      // and, above it, the warps that have added to it
   unsigned long long *timeout; // set to 1 if a bounded wait on a bulk copy ran out (never expected)
 };
 int launch_preprocess_fwd(int app, const PreprocessArgs &a, const CamDev &cam, cudaStream_t st);
@@ -107,8 +110,10 @@ int launch_unfused_prepare(int64_t n, const float *means, const CamDev &cam, con
 
 // What the first kernel after a device-counted preprocess does with the instance count: it tells the host - `host` is a
 // word of pinned memory that receives the view's number (24 bits) above the count (40 bits): one store, nothing to wait for
-// - and raises the flag if the lists will be cut off.
+// - and raises the flag if the lists will be cut off.  A count that the 40 bits cannot hold goes as their largest value, at
+// which the host reads the word on the device instead.
 constexpr int kCountBits = 40;
+constexpr unsigned long long kCountMost = (1ull << kCountBits) - 1;
 struct CountReport {
   const unsigned long long *count;             // null: nothing to report
   unsigned long long capacity;
@@ -119,7 +124,7 @@ struct CountReport {
     if (!count) return;
     const unsigned long long c = *count;
     if (c > capacity) *overflow = 1u;
-    *reinterpret_cast<volatile unsigned long long *>(host) = view << kCountBits | c;
+    *reinterpret_cast<volatile unsigned long long *>(host) = view << kCountBits | (c < kCountMost ? c : kCountMost);
   }
 #endif
 };

@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_prepro
     bulk::fence_barrier_init();
   }
   __syncwarp();
-  unsigned int instances = 0;
+  unsigned long long instances = 0;            // (of a lane: its run of Gaussians may hold 2^32 and more)
 
   // the second half for the Gaussians in the slots [head, head + 32), one per lane (`in`: this lane has one)
   auto finish = [&](int head, bool in) {
@@ -713,11 +713,12 @@ __global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_prepro
   if (gave_up && lane == 0) atomicExch(a.timeout, 1ull);   // reported by gs_async_status
   // ---- total number of (Gaussian, tile) instances: one atomic carries the sum and the number of warps it holds; the last
   // warp writes the count and leaves the sum at zero
-  instances = __reduce_add_sync(kFull, instances);
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) instances += __shfl_xor_sync(kFull, instances, s);
   if (lane == 0) {
-    const unsigned long long before = atomicAdd(a.pair_counter + 1, (1ull << 40) | instances);
-    if ((before >> 40) == (unsigned long long)warps - 1) {
-      a.pair_counter[0] = (before & ((1ull << 40) - 1)) + instances;
+    const unsigned long long before = atomicAdd(a.pair_counter + 1, (1ull << kSumBits) | instances);
+    if (before >> kSumBits == (unsigned long long)warps - 1) {
+      a.pair_counter[0] = (before & ((1ull << kSumBits) - 1)) + instances;
       a.pair_counter[1] = 0ull;
     }
   }
@@ -1251,7 +1252,8 @@ int resident_blocks(size_t smem_bytes, int cap = kWgradBlocks) {
 namespace {
 template <int APP>
 int launch_fwd(const PreprocessArgs &a, const CamDev &cam, cudaStream_t st) {
-  const int wave = resident_blocks<k_preprocess_fwd<APP>>(0, 1 << 20), chunks = grid_for(a.n);
+  constexpr int kMost = ((1 << (64 - kSumBits)) - 1) / kWarps;      // CTAs whose warps the counter has room for
+  const int wave = resident_blocks<k_preprocess_fwd<APP>>(0, kMost), chunks = grid_for(a.n);
   launch_chained(k_preprocess_fwd<APP>, chunks < wave ? chunks : wave, kBlock, 0, st, a, cam);
   return 1;
 }
