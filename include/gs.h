@@ -217,8 +217,11 @@ GsStatus gs_preprocess_async(GsContext *ctx, const GsScene *scene, const GsCamer
 #define GS_PAIRS_ON_DEVICE ((int64_t)-1)
 /* The instance count of the context's last gs_render_forward with GS_PAIRS_ON_DEVICE, as soon as it is known: waits until
  * that view's preprocess is done, not for the kernels behind it.  A caller that queues a view first and asks afterwards
- * has the count without ever leaving the GPU idle; a count above pair_capacity means the view's lists were cut off.  Not
- * for views replayed from a CUDA graph: their reports carry the number of the view that was captured. */
+ * has the count without ever leaving the GPU idle; a count above pair_capacity means the view's lists were cut off.  A
+ * view issued while its stream is captured into a CUDA graph sends no report: after a replay the call waits for the
+ * stream and returns the count of the replay.  (A replay is not a call: where another device-counted view was issued on the
+ * context after the capture, the answer is about that one, and graphs want a context of their own.)  GS_ERR_INVALID_ARG
+ * on a stream that is being captured. */
 GsStatus gs_async_pairs(GsContext *ctx, int64_t *num_pairs_host, void *stream);
 /* Waits for `stream`, then returns GS_ERR_CAPACITY if any device-counted view on this context
  * overflowed its pair_capacity since the last call (and clears the flag), GS_ERR_INTERNAL if a kernel

@@ -23,8 +23,8 @@ struct GsContext {
                                       // [4..7] the four words of gs_profile_blend_counts
   unsigned long long *h_counter;      // pinned host memory the device sees: [0], [2..7] mirror the words above; [8] the last
                                       // device-counted view's report (CountReport)
-  unsigned long long views;           // device-counted views issued so far
-  bool reports;                       // the last of them reports its count to the host by itself
+  unsigned long long views;           // number of the last device-counted view that reports (kViewMask)
+  bool reports;                       // the last device-counted view reports its count to the host by itself
   float *d_w_partials;                // device: per-CTA partial sums of the decoder gradient ([kWgradBlocks, 816];
                                       // sized for the decoder variants' largest case as well)
   char error[256];
@@ -175,6 +175,14 @@ GsStatus scene_ok(GsContext *ctx, const GsScene *s) {
   if (s->n > 0 && (bad_ptr(s->means) || bad_ptr(s->log_scales) || bad_ptr(s->quats) || bad_ptr(s->opacity_logits)))
     return fail(ctx, GS_ERR_INVALID_ARG, "a geometry array is NULL or misaligned");
   return GS_OK;
+}
+
+// Is the stream being captured into a graph?  (The legacy stream cannot be, but asking fails while another one is.)
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
 }
 
 // ---- workspace layout -------------------------------------------------------------------------
@@ -392,6 +400,7 @@ GsStatus gs_async_pairs(GsContext *ctx, int64_t *num_pairs_host, void *stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaSetDevice(ctx->device);
   *num_pairs_host = 0;
+  if (capturing(s)) return fail(ctx, GS_ERR_INVALID_ARG, "gs_async_pairs on a stream that is being captured");
   GsStatus st;
   if (ctx->reports) {
     // The view's first binning kernel writes the count with the view's number; the kernels behind it need not be waited for.
@@ -447,9 +456,10 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
   uint32_t *overflow = reinterpret_cast<uint32_t *>(ctx->d_counter + 2);
   CountReport report = {};
   if (on_device) {
-    ctx->reports = sorted;
-    ctx->views = (ctx->views + 1) & 0xffffffull;
-    report = {count_dev, (unsigned long long)pair_capacity, overflow, ctx->h_counter + 8, ctx->views};
+    // (a view that goes into a graph sends no report: its replays would all carry the same number)
+    ctx->reports = sorted && !capturing(s);
+    if (ctx->reports) ctx->views = (ctx->views + 1) & kViewMask;
+    report = {count_dev, (unsigned long long)pair_capacity, overflow, ctx->reports ? ctx->h_counter + 8 : nullptr, ctx->views};
   }
   const int num_cells = cd.cgx * cd.cgy;
   const uint32_t cap32 = pair_capacity > 0xffffffffll ? 0xffffffffu : (uint32_t)pair_capacity;

@@ -113,18 +113,18 @@ int launch_unfused_prepare(int64_t n, const float *means, const CamDev &cam, con
 // - and raises the flag if the lists will be cut off.  A count that the 40 bits cannot hold goes as their largest value, at
 // which the host reads the word on the device instead.
 constexpr int kCountBits = 40;
-constexpr unsigned long long kCountMost = (1ull << kCountBits) - 1;
+constexpr unsigned long long kCountMost = (1ull << kCountBits) - 1, kViewMask = (1ull << (64 - kCountBits)) - 1;
 struct CountReport {
   const unsigned long long *count;             // null: nothing to report
   unsigned long long capacity;
   uint32_t *overflow;
-  unsigned long long *host, view;
+  unsigned long long *host, view;              // host null: no report
 #ifdef __CUDACC__
   __device__ __forceinline__ void send() const {
     if (!count) return;
     const unsigned long long c = *count;
     if (c > capacity) *overflow = 1u;
-    *reinterpret_cast<volatile unsigned long long *>(host) = view << kCountBits | (c < kCountMost ? c : kCountMost);
+    if (host) *reinterpret_cast<volatile unsigned long long *>(host) = view << kCountBits | (c < kCountMost ? c : kCountMost);
   }
 #endif
 };

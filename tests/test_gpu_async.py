@@ -81,3 +81,41 @@ def test_empty_scene_through_the_async_calls():
     bg = torch.tensor(np.asarray(cam_h.background, np.float32), device=ctx.device)
     assert torch.equal(r.image, bg[:, None, None].expand(3, 64, 64))
     ctx.close()
+
+
+def _pairs_of_views(api, ctx, ds, cam):
+    probe = api.alloc_projected(ds.n, ctx.device, False)
+    return api.gs_preprocess(ctx, ds, cam, probe)
+
+
+def test_pairs_of_a_replayed_graph_are_those_of_the_replay():
+    torch, api, ctx, ds, cam, w = _setup()
+    W, H = w.cameras[0].width, w.cameras[0].height
+    other = api.Context(0)
+    before = _pairs_of_views(api, other, ds, cam)
+    r = api.Renderer(ctx, ds.n, W, H, ds.app, pair_capacity=int(before * 1.3) + 777)
+    r.forward(ds, cam)
+    assert r.num_pairs == before
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        r.forward_async(ds, cam, stream=stream)
+        with pytest.raises(api.GsError) as e:
+            api.gs_async_pairs(ctx, stream=stream)               # refused, and the capture stays whole
+        assert e.value.status == api.GS_ERR_INVALID_ARG
+    with torch.cuda.stream(stream):
+        graph.replay()
+        assert api.gs_async_pairs(ctx) == before
+        ds.means[: ds.n // 2] = 1e3                              # half of the scene leaves the view
+        after = _pairs_of_views(api, other, ds, cam)
+        assert 0 < after < before
+        torch.cuda._sleep(20_000_000)                            # the replay is still to come when the count is asked for
+        graph.replay()
+        assert api.gs_async_pairs(ctx) == after
+    # a view issued by a call answers for itself again
+    torch.cuda.synchronize()
+    r.forward(ds, cam)
+    assert r.num_pairs == after
+    del graph
+    ctx.close(); other.close()
