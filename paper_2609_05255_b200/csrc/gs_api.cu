@@ -457,7 +457,7 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
   CountReport report = {};
   if (on_device) {
     // (a view that goes into a graph sends no report: its replays would all carry the same number)
-    ctx->reports = sorted && !capturing(s);
+    ctx->reports = !capturing(s);
     if (ctx->reports) ctx->views = (ctx->views + 1) & kViewMask;
     report = {count_dev, (unsigned long long)pair_capacity, overflow, ctx->reports ? ctx->h_counter + 8 : nullptr, ctx->views};
   }
@@ -522,7 +522,7 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
     }
   } else {
     StageTimer t(ctx, GS_STAGE_TILE_RANGES, s);
-    t.done(launch_empty_binning(bin->tile_ranges, bin->tile_order, num_tiles, s));
+    t.done(launch_empty_binning(bin->tile_ranges, bin->tile_order, num_tiles, report, s));
   }
   {
     StageTimer t(ctx, GS_STAGE_BLEND_FWD, s);

@@ -198,7 +198,7 @@ struct ClusterBinArgs {
   int num_cells, cell_bits, cgx, gx, gy, W, H;
 };
 int launch_bin_cluster(const ClusterBinArgs &a, int ctas, int64_t record_bound, cudaStream_t st);
-int launch_empty_binning(uint32_t *tile_ranges, uint32_t *tile_order, int num_tiles, cudaStream_t st);
+int launch_empty_binning(uint32_t *tile_ranges, uint32_t *tile_order, int num_tiles, const CountReport &report, cudaStream_t st);
 
 // Blend.
 // (sorted_tiles: the tile id of every instance of the sorted list, written by the tile's CTA on its way in)

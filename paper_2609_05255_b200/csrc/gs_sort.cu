@@ -426,7 +426,8 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
   }
 }
 
-__global__ void k_iota(uint32_t *__restrict__ out, int n) {
+__global__ void k_iota(uint32_t *__restrict__ out, int n, CountReport report) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) report.send();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (uint32_t)i;
 }
@@ -825,10 +826,10 @@ int launch_expand(const uint32_t *rec_keys, const uint32_t *rec_vals, const uint
   return chunks_known ? 4 : 6;
 }
 
-// No record was sorted (no Gaussian, or none that reaches a tile): every tile is empty.
-int launch_empty_binning(uint32_t *tile_ranges, uint32_t *tile_order, int num_tiles, cudaStream_t st) {
+// No record is sorted (no Gaussian, none that reaches a tile, or no room for an instance): every tile is empty.
+int launch_empty_binning(uint32_t *tile_ranges, uint32_t *tile_order, int num_tiles, const CountReport &report, cudaStream_t st) {
   cudaMemsetAsync(tile_ranges, 0, (size_t)num_tiles * 2 * sizeof(uint32_t), st);
-  k_iota<<<(num_tiles + 255) / 256, 256, 0, st>>>(tile_order, num_tiles);
+  k_iota<<<(num_tiles + 255) / 256, 256, 0, st>>>(tile_order, num_tiles, report);
   return 1;
 }
 

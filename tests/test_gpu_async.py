@@ -119,3 +119,26 @@ def test_pairs_of_a_replayed_graph_are_those_of_the_replay():
     assert r.num_pairs == after
     del graph
     ctx.close(); other.close()
+
+
+def test_a_capacity_of_zero_overflows_like_any_other():
+    torch, api, ctx, ds, cam, w = _setup(n=5_003)
+    W, H = w.cameras[0].width, w.cameras[0].height
+    P = _pairs_of_views(api, ctx, ds, cam)
+    full = api.Renderer(ctx, ds.n, W, H, ds.app, pair_capacity=P)
+    none = api.Renderer(ctx, ds.n, W, H, ds.app, pair_capacity=0)
+    full.forward_async(ds, cam)
+    assert api.gs_async_pairs(ctx) == P
+    api.gs_async_status(ctx)                                     # within the capacity
+    assert api.gs_async_pairs(ctx) == P                          # asked again, after the stream has drained
+    none.forward_async(ds, cam)
+    assert api.gs_async_pairs(ctx) == P
+    with pytest.raises(api.GsError) as e:
+        api.gs_async_status(ctx)
+    assert e.value.status == api.GS_ERR_CAPACITY
+    empty = api.upload_scene(scenes.config1(0).scene, ctx.device)
+    e = api.Renderer(ctx, 0, 64, 64, empty.app, pair_capacity=0)
+    e.forward_async(empty, api.make_camera(scenes.identity_camera(64, 64, 64.0)))
+    assert api.gs_async_pairs(ctx) == 0
+    api.gs_async_status(ctx)
+    ctx.close()
