@@ -28,6 +28,7 @@ struct GsContext {
   float *d_w_partials;                // device: per-CTA partial sums of the decoder gradient ([kWgradBlocks, 816];
                                       // sized for the decoder variants' largest case as well)
   char error[256];
+  int cluster_limit;                  // CTAs of the largest cluster that the one-cluster binning can have (0: none)
   int decoder_engine;                 // GsDecoderEngine of the separate-pass forward
   bool profiling;
   std::vector<StageRecord> records;   // stage timings since the last collect
@@ -286,6 +287,7 @@ GsStatus gs_create(int device, GsContext **out) {
   ctx->d_counter = nullptr; ctx->h_counter = nullptr; ctx->d_w_partials = nullptr;
   ctx->profiling = false;
   ctx->views = 0; ctx->reports = false;
+  ctx->cluster_limit = bin_cluster_limit();
   ctx->decoder_engine = GS_ENGINE_AUTO;
   if (cudaMalloc(&ctx->d_counter, 8 * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMemset(ctx->d_counter, 0, 8 * sizeof(unsigned long long)) != cudaSuccess ||
@@ -465,9 +467,10 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
   const uint32_t cap32 = pair_capacity > 0xffffffffll ? 0xffffffffu : (uint32_t)pair_capacity;
   // Up to 8192 Gaussians the whole binning is one cluster's work: 16 SMs, but two launches instead of 12.  Steps measured
   // with the cluster and with the chain: 2100 Gaussians 115.0 and 118.5 us, 8000 in a small image 87.6 and 88.3, in one of
-  // 640 x 480 113.5 and 112.3, 12 000 143.7 and 142.8, 16 000 137.0 and 131.3, 32 000 138.5 and 132.0.  A CTA for every
-  // 64 Gaussians, up to 16 (1000 Gaussians: 33 us on 16 CTAs, 36 on 4).
-  if (sorted && n <= kClusterMax && num_cells <= (1 << kClusterDigit)) {
+  // 640 x 480 113.5 and 112.3, 12 000 143.7 and 142.8, 16 000 137.0 and 131.3, 32 000 138.5 and 132.0.
+  const int ctas = sorted ? cluster_ctas(n, num_cells, ctx->cluster_limit) : 0;
+  bool binned = !sorted;
+  if (ctas > 0) {
     ClusterBinArgs b = {};
     b.n = (uint32_t)n; b.capacity = cap32; b.pair_capacity32 = cap32; b.report = report; b.overflow = overflow; b.num_big = w.num_big;
     b.depth_key = proj->depth_key; b.cell_count = proj->cell_count; b.cell_records = proj->cell_records; b.rect = proj->rect;
@@ -478,11 +481,12 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
     b.piece_bases = w.cells.chunk_bases; b.tile_counts = w.cells.tile_counts; b.tile_starts = w.cells.tile_starts;
     b.tile_ranges = bin->tile_ranges; b.tile_order = bin->tile_order; b.out_vals = bin->sorted_vals;
     b.num_cells = num_cells; b.cell_bits = id_bits(num_cells); b.cgx = cd.cgx; b.gx = cd.gx; b.gy = cd.gy; b.W = cd.W; b.H = cd.H;
-    int ctas = 1;
-    while (ctas < 16 && (int64_t)ctas * 64 < n) ctas *= 2;
     StageTimer t(ctx, GS_STAGE_DEPTH_SORT, s);
-    t.done(launch_bin_cluster(b, ctas, num_pairs, s));
-  } else if (sorted) {
+    const int launches = launch_bin_cluster(b, ctas, num_pairs, s);
+    t.done(launches);
+    binned = launches > 0;
+  }
+  if (!binned) {
     // stage 1: Gaussians by depth key (stable => ties keep the index order); the last pass also leaves the cell records
     // per 256 sorted Gaussians, from which their emission takes its offsets.  Depths that a camera lets be zero or negative
     // have no key bit to spare for the culled ones, which are then sorted with the others.
@@ -520,7 +524,8 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
       t.done(launch_expand(sorted_rkeys, sorted_rvals, w.cell_ranges, w.cells, odd, num_pairs, pair_capacity, cd.gx, cd.gy, cd.cgx,
                            cd.cgy, bin->sorted_vals, bin->tile_ranges, bin->tile_order, s));
     }
-  } else {
+  }
+  if (!sorted) {
     StageTimer t(ctx, GS_STAGE_TILE_RANGES, s);
     t.done(launch_empty_binning(bin->tile_ranges, bin->tile_order, num_tiles, report, s));
   }

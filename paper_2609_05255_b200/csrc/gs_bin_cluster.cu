@@ -441,24 +441,43 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand_pieces(ClusterBinArgs
 
 }  // namespace
 
-int launch_bin_cluster(const ClusterBinArgs &a, int ctas, int64_t record_bound, cudaStream_t st) {
-  static bool opted[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !opted[dev]) {
-    cudaFuncSetAttribute(k_bin_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
-    cudaFuncSetAttribute(k_bin_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    opted[dev] = true;
-  }
+namespace {
+// Dependent launch of `ctas` CTAs as one cluster; attr has room for two.
+cudaLaunchConfig_t cluster_config(int ctas, cudaLaunchAttribute attr[2], cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = ctas; cfg.blockDim = kThreads; cfg.dynamicSmemBytes = sizeof(Shared); cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = ctas; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
-  cudaLaunchKernelEx(&cfg, k_bin_cluster, a);
+  return cfg;
+}
+}  // namespace
+
+int bin_cluster_limit() {
+  int limit = 0;
+  if (cudaFuncSetAttribute(k_bin_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared)) == cudaSuccess &&
+      cudaFuncSetAttribute(k_bin_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    for (int ctas = kClusterCtas; ctas >= 1 && !limit; ctas /= 2) {
+      cudaLaunchAttribute attr[2];
+      cudaLaunchConfig_t cfg = cluster_config(ctas, attr, nullptr);
+      cfg.numAttrs = 1;
+      int active = 0;
+      if (cudaOccupancyMaxActiveClusters(&active, k_bin_cluster, &cfg) == cudaSuccess && active > 0) limit = ctas;
+    }
+  }
+  cudaGetLastError();                          // a refusal is an answer
+  return limit;
+}
+
+int launch_bin_cluster(const ClusterBinArgs &a, int ctas, int64_t record_bound, cudaStream_t st) {
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = cluster_config(ctas, attr, st);
+  if (cudaLaunchKernelEx(&cfg, k_bin_cluster, a) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
   const int64_t warps = (record_bound + kBinPiece - 1) / kBinPiece + a.num_cells, blocks = (warps + 3) / 4;
   launch_chained(k_expand_pieces, (int)(blocks < 148 * 12 ? blocks : 148 * 12), kExpandThreads, 0, st, a);
   return 2;

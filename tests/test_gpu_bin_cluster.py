@@ -51,6 +51,13 @@ def test_image_sizes_and_large_footprints(width, height):
         assert np.any(spans[gpu.visible] > 2)                            # footprints of more than 3 x 3 cells
 
 
+@pytest.mark.parametrize("n", [1, 33, 1025, 8192])
+def test_few_gaussians_through_the_grid_wide_kernels(n):
+    """561 cells are too many for the cluster: the way that small scenes take where a cluster cannot be launched."""
+    sc = scenes.box_scene(n, 3.0, -1.0, 8.0, -3.5, 0.8, 1.0, scenes.APP_NEURAL, seed=600 + n)
+    _check(sc, scenes.identity_camera(2049, 1025, 1500.0))
+
+
 @pytest.mark.parametrize("n", [1500, 8000, 20011])
 def test_equal_depths_keep_the_index_order(n):
     sc = scenes.box_scene(n, 2.0, 3.0, 3.0, -3.0, 0.5, 1.0, scenes.APP_SH, seed=3)
