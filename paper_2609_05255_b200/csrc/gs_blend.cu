@@ -7,6 +7,8 @@
 // different register pairs takes three cycles of a scheduler, one with two pairs two, so the time goes with the operands
 // read.  Hence predicates instead of 0 / 1 factors in the forward and, in the backward, no shuffles or selects per entry:
 // what crosses lanes is parked in shared memory and summed later.
+#include <algorithm>
+
 #include "gs_device.cuh"
 
 namespace gs {
@@ -304,6 +306,7 @@ __device__ __forceinline__ float select_alpha(float alpha, uint32_t pos, uint32_
 }
 
 // One warp's slice of the rows that start as zeros.
+constexpr int kZeroWarps = 148 * 2;           // at least; see launch_blend_bwd
 __device__ __forceinline__ void zero_rows(const ZeroRows &z, int lane) {
 #pragma unroll 1
   for (int k = 0; k < z.count; ++k) {
@@ -422,7 +425,12 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
   using V = typename Share<NPX>::V;
   constexpr int kVecs = Share<NPX>::kVecs, kLanes = Lanes<V>::value, kWarps = Share<NPX>::kWarps, kGroup = NPX == 4 ? 1 : 4;
   __shared__ BwdArea<NPX> area;
-  const int lane = threadIdx.x, warp = (int)(blockIdx.x % kWarps), tile = (int)__ldg(order + blockIdx.x / kWarps);
+  const int lane = threadIdx.x;
+  if (blockIdx.x >= (unsigned)(cam.gx * cam.gy * kWarps)) {      // a warp without a region, see launch_blend_bwd
+    zero_rows(zeros, lane);
+    return;
+  }
+  const int warp = (int)(blockIdx.x % kWarps), tile = (int)__ldg(order + blockIdx.x / kWarps);
   RawEntries &raw = area.raw;
   StagedEntries &st = area.st;
   const int g = lane >> 2, t = lane & 3;
@@ -636,12 +644,18 @@ int launch_blend_bwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *
                      const uint32_t *n_contrib, const float *dL_dimage, float *g2d, uint32_t *flags, const ZeroRows &zeros,
                      cudaStream_t st) {
   const int tiles = cam.gx * cam.gy;
+  // The rows that start as zeros are shared out over all warps of the grid.  An image of few tiles does not have the warps
+  // for that - 16 x 16 pixels of a scene of 3M have 8, and 708 MB of SH gradients: 1473 us, now 120 - so warps without a
+  // region make up what is missing to two per SM, each with 4 KB at least.  (One per SM: 121 us for 16 x 16 pixels, 134 for
+  // 64 x 64 of the same scene; two 120 and 120, four 121 and 123, eight 126 and 126, sixteen 129 and 137.)
+  uint64_t quads = 0;
+  for (int k = 0; k < zeros.count; ++k) quads += zeros.floats[k] >> 2;
+  const int zero_warps = (int)std::min<uint64_t>(kZeroWarps, quads / 256);
   auto launch = [&](auto kernel, int warps) {
     ZeroRows z = zeros;
-    const uint64_t ctas = (uint64_t)tiles * warps;
+    const int ctas = std::max(tiles * warps, zero_warps);
     for (int k = 0; k < z.count; ++k) z.slice[k] = (uint32_t)(((z.floats[k] >> 2) + ctas - 1) / ctas);
-    kernel<<<tiles * warps, 32, 0, st>>>(cam, ranges, order, vals, mean2d, conic_opacity, color, final_T, n_contrib, dL_dimage, g2d,
-                                        flags, z);
+    kernel<<<ctas, 32, 0, st>>>(cam, ranges, order, vals, mean2d, conic_opacity, color, final_T, n_contrib, dL_dimage, g2d, flags, z);
   };
   // (the measurements behind the two lines are at the kernel)
   if (tiles <= 64) launch(k_blend_bwd<1>, Share<1>::kWarps);
