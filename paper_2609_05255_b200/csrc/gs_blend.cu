@@ -411,11 +411,20 @@ struct __align__(16) BwdArea {
 // (on its way in, the first wave writes them all at once and the others' reads wait behind that: 23 us more at 1M); a bit per Gaussian says who received a gradient, and the
 // projection and appearance backward gathers those alone.
 //
-// 16 x 8 pixels per warp is best where the launch fills the chip (1M Gaussians, 1256 x 828: 181 us against 195 with
-// 8 x 8; 244 before); smaller regions give more warps and cull more where it does not: 8 x 8 from 2550 tiles down
-// (128 against 133 us at 2550, 69 / 68 at 1024, 30 / 39 at 294), 4 x 8 while every warp still has a scheduler of its own
-// (16 tiles: 23 against 29 us).  There, what does not depend on the carried state is worked out for four entries at a
-// time (2 to 4 us less); with 16 x 8 pixels the registers it takes cost more than it gives.
+// 16 x 8 pixels per warp is best where the launch fills the chip; smaller regions give more warps and cull more where it
+// does not, and where a few long lists make the time.  Measured with all three (4 x 8, 8 x 8, 16 x 8; us, zero rows
+// included) from 25 to 9600 tiles, for scenes of 5000 to 100 000 Gaussians in a box, 300 000 and 1M in clusters, drawn and
+// with all opacities 0.1, and 2M over depths of 1 to 50:
+//     100 tiles   box of 100 000  45  51  92    of 5000  35  41  74    (128: 37 41 70, but 45 33 55; clusters 86 125 332)
+//     361         box of 100 000  55  49  74    clusters of 300 000  90 102 217
+//    2700         box of 100 000 197 129 119    clusters of 1M 234 166 178    deep 336 330 469
+//    3200                                       clusters of 1M 260 182 188    deep 363 301 530
+//    4108                                       clusters of 1M 303 207 205    deep 404 303 459
+//    7500                                       clusters of 1M 483 313 289    deep 611 408 414
+// So 4 x 8 up to 100 tiles, where all scenes agree, and 8 x 8 up to 4000, where those in clusters change over (the deep one
+// changes over at 7500, the box of 100 000 at 1200, by 10 % at most; 5000 Gaussians at 400: 74 against 53 us at 960 tiles).
+// In the two smaller ones, what does not depend on the carried state is worked out for four entries at a time (2 to 4 us
+// less); with 16 x 8 pixels the registers it takes cost more than it gives.
 template <int NPX>
 __global__ void __launch_bounds__(32) k_blend_bwd(
     CamDev cam, const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ order, const uint32_t *__restrict__ vals,
@@ -658,8 +667,8 @@ int launch_blend_bwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *
     kernel<<<ctas, 32, 0, st>>>(cam, ranges, order, vals, mean2d, conic_opacity, color, final_T, n_contrib, dL_dimage, g2d, flags, z);
   };
   // (the measurements behind the two lines are at the kernel)
-  if (tiles <= 64) launch(k_blend_bwd<1>, Share<1>::kWarps);
-  else if (tiles <= 3000) launch(k_blend_bwd<2>, Share<2>::kWarps);
+  if (tiles <= 100) launch(k_blend_bwd<1>, Share<1>::kWarps);
+  else if (tiles <= 4000) launch(k_blend_bwd<2>, Share<2>::kWarps);
   else launch(k_blend_bwd<4>, Share<4>::kWarps);
   return 1;
 }

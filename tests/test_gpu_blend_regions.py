@@ -1,5 +1,5 @@
 """The blend kernels give every warp a region of a tile and choose its size by the number of tiles (backward: 4 x 8 pixels
-up to 64 tiles, 8 x 8 up to 3000, 16 x 8 beyond); lists go through shared memory 32 entries at a time, in groups of four,
+up to 100 tiles, 8 x 8 up to 4000, 16 x 8 beyond); lists go through shared memory 32 entries at a time, in groups of four,
 and what the lanes park is summed every eight entries.  Checked against the oracle at the edges of all of these: tile
 counts on either side of the two lines, ragged images, lists of about 32 and 64 entries, opacities above the alpha clamp."""
 import numpy as np
@@ -28,6 +28,12 @@ def test_image_sizes_at_the_lines_between_region_sizes(oracle, width, height):
     sc = scenes.box_scene(3000, 2.0, 2.0, 6.0, -3.0, 0.5, 1.0, scenes.APP_SH, seed=31)
     cam = scenes.identity_camera(width, height, float(max(width, height)), background=(0.2, 0.1, 0.3))
     _check(oracle, sc, cam)
+
+
+@pytest.mark.parametrize("width,height", [(160, 160), (1601, 16), (800, 1280), (1022, 1008)])       # 100, 101, 4000, 4032 tiles
+def test_on_either_side_of_the_lines(oracle, width, height):
+    sc = scenes.box_scene(3000, 2.0, 2.0, 6.0, -3.0, 0.5, 1.0, scenes.APP_SH, seed=32)
+    _check(oracle, sc, scenes.identity_camera(width, height, float(max(width, height)), background=(0.2, 0.1, 0.3)))
 
 
 @pytest.mark.parametrize("n", [1, 3, 4, 5, 7, 8, 9, 31, 32, 33, 40, 63, 64, 65])
