@@ -72,6 +72,7 @@ struct PreprocessBwdArgs {
   float *g_means, *g_log_scales, *g_quats, *g_logits, *g_base, *g_sh_rest, *g_features;
   float *w_partials;           // [kWgradBlocks, 816]
   float *g_weights;            // [816]
+  unsigned long long *timeout; // set to 1 if a bounded wait on a bulk copy ran out (never expected)
 };
 int launch_preprocess_bwd(int app, const PreprocessBwdArgs &a, const CamDev &cam, cudaStream_t st);
 

@@ -833,10 +833,7 @@ __device__ __forceinline__ void store3(float *p, int64_t i, float a, float b, fl
   p[3 * i] = a; p[3 * i + 1] = b; p[3 * i + 2] = c;
 }
 
-// Shared memory of the backward kernels (dynamic): SH: kWarps slabs of coefficient rows.
-// Neural: weights [816] | kWarps operand slabs [32][100] (reused as [kWarps][816] at the end).
-constexpr size_t kBwdSmemSH = sizeof(float) * kWarps * SlabOf<GS_APP_SH>::value;
-constexpr size_t kBwdSmemSV = sizeof(float) * kWarps * SlabOf<GS_APP_SV>::value;
+// Shared memory of the neural backward kernels (dynamic): weights [816] | kWarps operand slabs [32][100] (reused as [kWarps][816] at the end).
 constexpr size_t kBwdSmemNN = sizeof(mlp::Weights) + kWarps * sizeof(mlp::WarpStage);
 static_assert(kWarps * sizeof(mlp::WarpStage) >= kWarps * GS_MLP_WEIGHTS * sizeof(float), "partial sums reuse the staging areas");
 static_assert(sizeof(mlp::Weights) % 16 == 0, "staging areas must stay 16-byte aligned");
@@ -849,10 +846,10 @@ static_assert(sizeof(mlp::Weights) % 16 == 0, "staging areas must stay 16-byte a
 // backward, one per thread, with every lane busy.  A CTA's run of flag words is fixed by the grid, so the order of all sums
 // is the same from run to run.  What bounds it is the chain of latencies (flag words, gathered rows, decoder), not the
 // bytes: 51 k of 1M Gaussians in a view have a gradient.
-// SH and Spherical Voronoi rows are gathered and scattered row by row through the warp's slab, a row being 45 or 49
-// neighbouring floats.
+// (The explicit models have a kernel of their own, below.)
 template <int APP>
 __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdArgs a, CamDev cam) {
+  static_assert(!Explicit<APP>::value, "k_preprocess_bwd_explicit");
   dependency_wait();
   extern __shared__ __align__(16) float smem[];
   constexpr int kWordsPerRound = kBlock / 4;             // flag words (of 32 Gaussians) looked at per round
@@ -860,7 +857,6 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
   __shared__ int s_warp_count[kWarps];
   constexpr int kMask = 2 * 32 * kWordsPerRound - 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float *slab = smem + warp * SlabOf<APP>::value;     // SH / SV: this warp's slab of parameter rows
   mlp::Weights &sWt = *reinterpret_cast<mlp::Weights *>(smem);
   mlp::WarpStage *sStage = reinterpret_cast<mlp::WarpStage *>(reinterpret_cast<unsigned char *>(smem) + sizeof(mlp::Weights));
   mlp::WeightGrad dW;
@@ -875,16 +871,6 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
   auto process = [&](int count) {
     const bool has = tid < count;
     const int64_t i = has ? (int64_t)s_queue[(q_head + tid) & kMask] : 0;
-    const int rows = min(32, count - warp * 32);
-    if (Explicit<APP>::value && a.deg > 0) {   // the parameter rows, on their way while the rest is loaded
-      constexpr int kRow = Explicit<APP>::value ? RowOf<APP>::value : 1;
-#pragma unroll 4
-      for (int r = 0; r < rows; ++r) {
-        const float *src = a.sh_rest + (int64_t)s_queue[(q_head + warp * 32 + r) & kMask] * kRow;
-        copy_async4(slab + r * kRow + lane, src + lane);
-        if (lane + 32 < kRow) copy_async4(slab + r * kRow + 32 + lane, src + 32 + lane);
-      }
-    }
     float gd[3] = {0.f, 0.f, 0.f};
     float mu[3] = {0.f, 0.f, 0.f}, ls[3] = {0.f, 0.f, 0.f}, q[4] = {1.f, 0.f, 0.f, 0.f}, logit = 0.f;
     float4 ga = make_float4(0.f, 0.f, 0.f, 0.f), gb = ga, gc = ga;
@@ -907,32 +893,7 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
       dx = vx * vi; dy = vy * vi; dz = vz * vi;
     }
     float gp[3] = {0.f, 0.f, 0.f};
-    if (Explicit<APP>::value) {
-      constexpr int kRow = Explicit<APP>::value ? RowOf<APP>::value : 1;
-      float *row = slab + lane * kRow;
-      if (a.deg > 0) {
-        copies_wait();
-        __syncwarp();
-      }
-      if (has) {
-        float pre[3] = {base[0] + 0.5f, base[1] + 0.5f, base[2] + 0.5f};
-        SvCarry cy;
-        if (a.deg > 0) explicit_pre<APP>(row, base, dx, dy, dz, a.deg, pre, cy);
-        gp[0] = color_act_grad_z(a.act, pre[0]) * ga.x; gp[1] = color_act_grad_z(a.act, pre[1]) * ga.y;
-        gp[2] = color_act_grad_z(a.act, pre[2]) * ga.z;
-        if (a.deg > 0) explicit_bwd<APP>(row, gp, dx, dy, dz, a.deg, cy, gd);
-      }
-      if (a.deg > 0) {                          // (degree 0 leaves the zeros)
-        __syncwarp();
-#pragma unroll 4
-        for (int r = 0; r < rows; ++r) {
-          float *dst = a.g_sh_rest + (int64_t)s_queue[(q_head + warp * 32 + r) & kMask] * kRow;
-          dst[lane] = slab[r * kRow + lane];
-          if (lane + 32 < kRow) dst[32 + lane] = slab[r * kRow + 32 + lane];
-        }
-        __syncwarp();
-      }
-    } else if (IsNeural<APP>::value) {
+    if (IsNeural<APP>::value) {
       float gf[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       const float gcol[3] = {ga.x, ga.y, ga.z};
       if (warp * 32 < count && a.deg > 0) {     // the whole warp goes through the decoder; lanes past the count feed zeros
@@ -1008,6 +969,167 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
   if (IsNeural<APP>::value) {
     weight_grad_flush(dW, reinterpret_cast<float *>(sStage), a.w_partials + (size_t)blockIdx.x * GS_MLP_WEIGHTS, tid);
   }
+}
+
+// ---- the same for the explicit models, SH and Spherical Voronoi ----
+// Bound by memory: a Gaussian with a gradient reads and writes its parameter row of 45 or 49 floats and as much again of
+// geometry.  A CTA takes 128 flag words of its run at a time, one per thread.  Where a word has at least kDenseWord
+// Gaussians with a gradient (a view of a scene that is not opaque yet: all words), its 32 rows come in by one bulk copy and
+// their gradients leave by one, zeros among them; the Gaussians of the thinner words are listed, and gathered and scattered
+// row by row, 32 at a time.  The four warps take the words and the batches in turn, on their own.
+// 1M Gaussians, 1256 x 828, SH / Spherical Voronoi: 29 / 31 us where 6 % have a gradient, 78 / 82 at 29 %, 108 / 116 at 87 %
+// (all opacities 0.1).  Without the whole words and with batches of 128 behind barriers 34 / 32, 84 / 83 and 132 / 138; a dense
+// kernel over all Gaussians, which writes the zero rows too, 83 / 103 at any share.  From 16 or 24 Gaussians on instead of
+// 20: 1 to 4 us more where words hold about that many.  Warps with runs and queues of their own: 5 us more at 300 000 Gaussians (half-full
+// batches), and one place in the code for whole words and batches: inlined twice it took 10 us more in small scenes (cold code).
+constexpr int kDenseWord = 20;
+template <int APP>
+__global__ void __launch_bounds__(kBlock) k_preprocess_bwd_explicit(PreprocessBwdArgs a, CamDev cam) {
+  static_assert(Explicit<APP>::value, "k_preprocess_bwd_sparse");
+  dependency_wait();
+  constexpr int kRow = RowOf<APP>::value;
+  constexpr uint32_t kBytes = SlabOf<APP>::value * sizeof(float);
+  extern __shared__ __align__(16) float smem[];
+  __shared__ unsigned short s_list[32 * kBlock];      // Gaussians of the thin words, counted from the first of the round
+  __shared__ uint32_t s_dense[kBlock];                // flags of the dense words, ...
+  __shared__ unsigned char s_which[kBlock];           // ... and which they are
+  __shared__ int s_counts[kWarps];                    // of a warp: listed Gaussians | dense words << 16
+  __shared__ unsigned long long s_bar[kWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float *slab = smem + warp * SlabOf<APP>::value;
+  const uint32_t bar = bulk::smem_addr(s_bar + warp);
+  if (lane == 0) {
+    bulk::barrier_init(bar);
+    bulk::fence_barrier_init();
+  }
+  uint32_t parity = 0u;
+  bool gave_up = false;             // a bulk copy never came
+
+  const int64_t words = (a.n + 31) / 32;
+  const int64_t begin = words * blockIdx.x / gridDim.x, end = words * (blockIdx.x + 1) / gridDim.x;
+  for (int64_t w0 = begin; w0 < end; w0 += kBlock) {
+    const int64_t w = w0 + tid;
+    const uint32_t word = w < end ? __ldg(a.flags + w) : 0u;
+    const bool dense = a.deg > 0 && __popc(word) >= kDenseWord && 32 * w + 32 <= a.n;
+    const int own = dense ? 1 << 16 : __popc(word);
+    int incl = own;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const int t = __shfl_up_sync(kFull, incl, s);
+      if (lane >= s) incl += t;
+    }
+    if (lane == 31) s_counts[warp] = incl;
+    __syncthreads();                // (the round before is over, too)
+    int first = incl - own, all = 0;
+#pragma unroll
+    for (int k = 0; k < kWarps; ++k) { const int c = s_counts[k]; first += k < warp ? c : 0; all += c; }
+    if (dense) {
+      s_dense[first >> 16] = word;
+      s_which[first >> 16] = (unsigned char)tid;
+    } else {
+      int at = first & 0xffff;
+      for (uint32_t bits = word; bits; bits &= bits - 1u) s_list[at++] = (unsigned short)(32 * tid + __ffs(bits) - 1);
+    }
+    __syncthreads();
+    const int num_dense = all >> 16, listed = all & 0xffff, jobs = num_dense + (listed + 31) / 32;
+    for (int job = warp; job < jobs && !gave_up; job += kWarps) {
+      reload_fence();
+      // 32 Gaussians, one per lane: the rows of a whole word, or the next of the list
+      const bool whole = job < num_dense;
+      const int at = 32 * (job - num_dense), count = whole ? 32 : min(32, listed - at);
+      int64_t row0 = 32 * w0;
+      bool has;
+      int64_t i;
+      if (whole) {
+        row0 += 32 * s_which[job];
+        i = row0 + lane;
+        has = (s_dense[job] >> lane) & 1u;
+        bulk::fence_generic_writes();           // what the lanes wrote to the slab comes before the copy
+      } else {
+        has = lane < count;
+        i = row0 + (has ? s_list[at + lane] : 0);
+      }
+      __syncwarp();
+      if (lane == 0) {
+        bulk::wait_stores_read();               // the gradients of the word before have left the slab
+        if (whole) bulk::load(bulk::smem_addr(slab), a.sh_rest + row0 * kRow, kBytes, bar);
+      }
+      __syncwarp();
+      if (!whole && a.deg > 0) {
+#pragma unroll 4
+        for (int r = 0; r < count; ++r) {
+          const float *src = a.sh_rest + (int64_t)__shfl_sync(kFull, (uint32_t)i, r) * kRow;
+          copy_async4(slab + r * kRow + lane, src + lane);
+          if (lane + 32 < kRow) copy_async4(slab + r * kRow + 32 + lane, src + 32 + lane);
+        }
+      }
+      float mu[3] = {0.f, 0.f, 0.f}, ls[3] = {0.f, 0.f, 0.f}, base[3] = {0.f, 0.f, 0.f}, logit = 0.f;
+      float4 q4 = make_float4(1.f, 0.f, 0.f, 0.f), ga = make_float4(0.f, 0.f, 0.f, 0.f), gb = ga, gc = ga;
+      float dx = 0.f, dy = 0.f, dz = 1.f;
+      if (has) {
+        load3(a.means, i, mu);
+        load3(a.log_scales, i, ls);
+        q4 = __ldg(reinterpret_cast<const float4 *>(a.quats) + i);
+        logit = __ldg(a.logits + i);
+        const float4 *g2 = reinterpret_cast<const float4 *>(a.g2d) + 3 * i;
+        ga = g2[0]; gb = g2[1]; gc = g2[2];
+        load3(a.base_color, i, base);
+        const float vx = mu[0] - cam.oc[0], vy = mu[1] - cam.oc[1], vz = mu[2] - cam.oc[2];
+        const float vi = rsqrtf(vx * vx + vy * vy + vz * vz);
+        dx = vx * vi; dy = vy * vi; dz = vz * vi;
+      }
+      if (whole) {
+        if (!__all_sync(kFull, bulk::wait(bar, parity))) {
+          gave_up = true;                     // nothing more for this warp, which meets the others all the same
+          continue;
+        }
+        parity ^= 1u;
+      } else if (a.deg > 0) {
+        copies_wait();
+        __syncwarp();
+      }
+      float *row = slab + lane * kRow;
+      float gp[3] = {0.f, 0.f, 0.f}, gd[3] = {0.f, 0.f, 0.f};
+      if (has) {
+        float pre[3] = {base[0] + 0.5f, base[1] + 0.5f, base[2] + 0.5f};
+        SvCarry cy;
+        if (a.deg > 0) explicit_pre<APP>(row, base, dx, dy, dz, a.deg, pre, cy);
+        gp[0] = color_act_grad_z(a.act, pre[0]) * ga.x; gp[1] = color_act_grad_z(a.act, pre[1]) * ga.y;
+        gp[2] = color_act_grad_z(a.act, pre[2]) * ga.z;
+        if (a.deg > 0) explicit_bwd<APP>(row, gp, dx, dy, dz, a.deg, cy, gd);
+      } else if (whole) {
+#pragma unroll
+        for (int k = 0; k < kRow; ++k) row[k] = 0.f;
+      }
+      if (whole) {
+        bulk::fence_generic_writes();           // the lanes' rows become visible to the copy engine
+        __syncwarp();
+        if (lane == 0) bulk::store(a.g_sh_rest + row0 * kRow, bulk::smem_addr(slab), kBytes);
+      } else if (a.deg > 0) {                   // (degree 0 leaves the zeros)
+        __syncwarp();
+#pragma unroll 4
+        for (int r = 0; r < count; ++r) {
+          float *dst = a.g_sh_rest + (int64_t)__shfl_sync(kFull, (uint32_t)i, r) * kRow;
+          dst[lane] = slab[r * kRow + lane];
+          if (lane + 32 < kRow) dst[32 + lane] = slab[r * kRow + 32 + lane];
+        }
+      }
+      if (has) {
+        const float q[4] = {q4.x, q4.y, q4.z, q4.w};
+        const GeoGrads gg = project_backward(mu, ls, q, logit, cam, gb.x, gb.y, gb.z, gb.w, gc.x, ga.w, gd);
+        store3(a.g_means, i, gg.mu[0], gg.mu[1], gg.mu[2]);
+        store3(a.g_log_scales, i, gg.ls[0], gg.ls[1], gg.ls[2]);
+        reinterpret_cast<float4 *>(a.g_quats)[i] = make_float4(gg.q[0], gg.q[1], gg.q[2], gg.q[3]);
+        a.g_logits[i] = gg.logit;
+        store3(a.g_base, i, gp[0], gp[1], gp[2]);
+      }
+    }
+  }
+  if (lane == 0) {
+    bulk::wait_stores_done();
+    if (gave_up) atomicExch(a.timeout, 1ull);             // reported by gs_async_status
+  }
+  if (gave_up) bulk::wait(bar, parity);       // the copy may still be on its way into the slab: the same bounded time again
 }
 
 // ---- separate-pass appearance kernels of the neural model (the explicit models follow, with bulk copies) ------
@@ -1288,10 +1410,21 @@ int launch_bwd_sparse(size_t smem, const PreprocessBwdArgs &a, const CamDev &cam
 }
 }  // namespace
 
+namespace {
+template <int APP>
+int launch_bwd_explicit(const PreprocessBwdArgs &a, const CamDev &cam, cudaStream_t st) {
+  constexpr size_t smem = sizeof(float) * kWarps * SlabOf<APP>::value;
+  opt_in_smem(k_preprocess_bwd_explicit<APP>, smem);
+  const int wave = resident_blocks<k_preprocess_bwd_explicit<APP>>(smem, 1 << 20), chunks = grid_for(a.n);
+  launch_chained(k_preprocess_bwd_explicit<APP>, chunks < wave ? chunks : wave, kBlock, smem, st, a, cam);
+  return 1;
+}
+}  // namespace
+
 int launch_preprocess_bwd(int app, const PreprocessBwdArgs &a, const CamDev &cam, cudaStream_t st) {
   if (a.n == 0) return 0;
-  if (app == GS_APP_SH) return launch_bwd_sparse<GS_APP_SH>(kBwdSmemSH, a, cam, st);
-  if (app == GS_APP_SV) return launch_bwd_sparse<GS_APP_SV>(kBwdSmemSV, a, cam, st);
+  if (app == GS_APP_SH) return launch_bwd_explicit<GS_APP_SH>(a, cam, st);
+  if (app == GS_APP_SV) return launch_bwd_explicit<GS_APP_SV>(a, cam, st);
   if (app == kAppExternal) return launch_bwd_sparse<kAppExternal>(sizeof(mlp::Weights), a, cam, st);
   if (app == kAppNeuralHalf) return launch_bwd_sparse<kAppNeuralHalf>(kBwdSmemNN, a, cam, st);
   return launch_bwd_sparse<GS_APP_NEURAL>(kBwdSmemNN, a, cam, st);
