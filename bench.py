@@ -1,11 +1,12 @@
 #!/usr/bin/env python
 """Benchmark of the splatting training step (forward + backward, 8 views of a 1M-Gaussian scene).
 
-`python bench.py --gpus N --steps K --warmup W` prints ONE JSON line on rank 0.
+`python bench.py --gpus N --steps K --warmup W` prints ONE JSON line on rank 0; `--details FILE` also writes the full record
+(stages, rooflines, sweeps) as JSON.
 A "step" is one pass of the whole hot path over one batch: for each of the 8 orbit cameras,
 gs_preprocess -> gs_render_forward -> gs_render_backward on the 1M-Gaussian clustered scene
 (the 1M configuration of the benchmark list) with the neural appearance model; the SH model and
-the appearance-decode sweep are timed beside it and reported in extra keys.
+the appearance-decode sweep are timed beside it.
 
 `--impl reference` times the CPU oracle (the plain double-precision restatement of the method) on
 the host cores on a bounded sample of the same workload.
@@ -403,7 +404,8 @@ def run_ours(args):
         "ms_per_step_single_stream": neural["ms_one"], "ms_per_step_streams_no_graph": neural["ms_streams"],
         "cuda_graph": neural["graph"],
         "streams": 1 if views == 1 else n_lanes,
-        "clocks": clocks, "e2e": e2e, "e2e_gradients_to_host": e2e_host, "gpu_launches": launches_per_step,
+        "clocks": clocks, "e2e": e2e, "e2e_gradients_to_host": e2e_host,
+        "gpu_launches": launches_per_step * args.steps,      # of this library, inside the timed region
         "roofline": roof,
         "rooflines": {k: stage_roofline(k, neural, views, n, peaks, alu_peak)
                       for k in ("preprocess_fwd", "depth_sort", "keygen", "tile_sort", "tile_ranges", "blend_fwd",
@@ -431,7 +433,29 @@ def run_ours(args):
     }
     if not args.skip_cpu:
         out["cpu_baseline"] = cpu_baseline(neural["host"], cams_host, n)
-    print(json.dumps(out))
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(out, f, indent=1)
+    print(json.dumps(headline(out)))
+
+
+def headline(out):
+    """The line on stdout: what was measured, under which conditions, and the figures that the metric names, in less than
+    2000 characters, so that whoever captures the end of the output has all of it.  The full record (stages, rooflines,
+    sweeps, the other arms' breakdowns) is what --details writes."""
+    def pick(d, *keys):
+        return None if d is None else {k: round(d[k], 4) if isinstance(d[k], float) else d[k] for k in keys if k in d}
+    line = {k: out[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                                "vs_baseline", "dtype", "data", "config", "clocks", "gpu_launches")}
+    line["e2e"] = pick(out["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    line["ms_per_step_single_stream"] = round(out["ms_per_step_single_stream"], 4)
+    line["roofline"] = pick(out["roofline"], "kernel", "bound", "achieved", "peak", "unit", "frac")
+    line["arms_ms_per_step"] = {k: round(out[k]["ms_per_step"], 4) for k in ("sh", "sv") if out.get(k)}
+    line["appearance_decode"] = {k: pick(v, "GBps", "frac_of_hbm_peak") for k, v in (out["appearance_decode"] or {}).items()
+                                 if k in ("neural_1M", "neural_10M", "sh_1M", "sh_10M")}
+    if "cpu_baseline" in out:
+        line["cpu_baseline"] = pick(out["cpu_baseline"], "value", "unit", "cores", "kind")
+    return line
 
 
 # Figures read from ncu captures of single launches (orbit view 0 of the default workload) live in
@@ -456,7 +480,8 @@ STAGE_KERNELS = {
     "tile_sort": "k_radix_hist, k_radix_scatter<9>: one stable pass on the cell id, cell ranges and chunks from its totals",
     "tile_ranges": "k_chunk_counts, k_cell_prefix, k_tile_scan, k_expand: records -> per-tile lists",
     "blend_fwd": "k_blend_fwd", "blend_bwd": "k_blend_bwd",
-    "preprocess_bwd": "k_preprocess_bwd_sparse (the Gaussians with a gradient in full batches; the zero rows are written by k_blend_bwd) + k_wgrad_reduce"}
+    "preprocess_bwd": "neural: k_preprocess_bwd_sparse + k_wgrad_reduce, explicit models: k_preprocess_bwd_explicit (the Gaussians "
+                      "with a gradient; the zero rows are written by k_blend_bwd)"}
 
 
 def stage_roofline(stage, arm, views, n, peaks, alu_peak):
@@ -961,6 +986,7 @@ def main():
                     help="workload (3 = the headline: 1M Gaussians, 8 views; the others fill the results table)")
     ap.add_argument("--n", type=int, default=None, help="override the Gaussian count of config 3")
     ap.add_argument("--views", type=int, default=None, help="override the number of views of configs 3 and 4")
+    ap.add_argument("--details", default=None, metavar="FILE", help="write the full record, with stages, rooflines and sweeps, as JSON")
     ap.add_argument("--quick", action="store_true", help="decode sweep at 1M only")
     ap.add_argument("--skip-decode", action="store_true")
     ap.add_argument("--skip-cpu", action="store_true")
