@@ -287,7 +287,7 @@ GsStatus gs_create(int device, GsContext **out) {
   ctx->d_counter = nullptr; ctx->h_counter = nullptr; ctx->d_w_partials = nullptr;
   ctx->profiling = false;
   ctx->views = 0; ctx->reports = false;
-  ctx->cluster_limit = bin_cluster_limit();
+  ctx->cluster_limit = bin_cluster_limit(device);
   ctx->decoder_engine = GS_ENGINE_AUTO;
   if (cudaMalloc(&ctx->d_counter, 8 * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMemset(ctx->d_counter, 0, 8 * sizeof(unsigned long long)) != cudaSuccess ||

@@ -9,6 +9,8 @@
 // The results are the same bits as those of the grid-wide chain: both are stable sorts.
 // The same kernel as a cooperative grid of one CTA per SM, for larger scenes, was no faster than the chain (barriers of
 // 2 us, and every CTA reads every other's digits): a step on 100 000 Gaussians 212 against 217 us, on a million 642 against 604.
+#include <mutex>
+
 #include "gs_bin.cuh"
 
 namespace gs {
@@ -455,20 +457,25 @@ cudaLaunchConfig_t cluster_config(int ctas, cudaLaunchAttribute attr[2], cudaStr
 }
 }  // namespace
 
-int bin_cluster_limit() {
-  int limit = 0;
-  if (cudaFuncSetAttribute(k_bin_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared)) == cudaSuccess &&
-      cudaFuncSetAttribute(k_bin_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-    for (int ctas = kClusterCtas; ctas >= 1 && !limit; ctas /= 2) {
-      cudaLaunchAttribute attr[2];
-      cudaLaunchConfig_t cfg = cluster_config(ctas, attr, nullptr);
-      cfg.numAttrs = 1;
-      int active = 0;
-      if (cudaOccupancyMaxActiveClusters(&active, k_bin_cluster, &cfg) == cudaSuccess && active > 0) limit = ctas;
+int bin_cluster_limit(int device) {
+  // asked once per process and device, whose share of a GPU does not change (the question takes 2 ms)
+  static std::once_flag asked[64];
+  static int limits[64] = {};
+  if (device < 0 || device >= 64) return 0;
+  std::call_once(asked[device], [device] {
+    if (cudaFuncSetAttribute(k_bin_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared)) == cudaSuccess &&
+        cudaFuncSetAttribute(k_bin_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+      for (int ctas = kClusterCtas; ctas >= 1 && !limits[device]; ctas /= 2) {
+        cudaLaunchAttribute attr[2];
+        cudaLaunchConfig_t cfg = cluster_config(ctas, attr, nullptr);
+        cfg.numAttrs = 1;
+        int active = 0;
+        if (cudaOccupancyMaxActiveClusters(&active, k_bin_cluster, &cfg) == cudaSuccess && active > 0) limits[device] = ctas;
+      }
     }
-  }
-  cudaGetLastError();                          // a refusal is an answer
-  return limit;
+    cudaGetLastError();                        // a refusal is an answer
+  });
+  return limits[device];
 }
 
 int launch_bin_cluster(const ClusterBinArgs &a, int ctas, int64_t record_bound, cudaStream_t st) {

@@ -200,7 +200,7 @@ struct ClusterBinArgs {
 };
 // CTAs of the cluster for n Gaussians, one for every 64 up to 16 (1000 Gaussians: 33 us on 16 CTAs, 36 on 4), each alone on
 // its SM; 0: the grid-wide kernels.  `limit`: the largest cluster that the device, or the share of it that the process has,
-// can hold at all (bin_cluster_limit, asked once per context).
+// can hold at all (bin_cluster_limit, with that device current).
 constexpr int kClusterCtas = 16;
 inline int cluster_ctas(int64_t n, int num_cells, int limit) {
   if (n > kClusterMax || num_cells > (1 << kClusterDigit)) return 0;
@@ -208,7 +208,7 @@ inline int cluster_ctas(int64_t n, int num_cells, int limit) {
   while (ctas < kClusterCtas && (int64_t)ctas * 64 < n) ctas *= 2;
   return ctas <= limit ? ctas : 0;
 }
-int bin_cluster_limit();
+int bin_cluster_limit(int device);
 // Returns 0, with nothing launched, if the cluster is refused (a stream with fewer SMs than the context had).
 int launch_bin_cluster(const ClusterBinArgs &a, int ctas, int64_t record_bound, cudaStream_t st);
 int launch_empty_binning(uint32_t *tile_ranges, uint32_t *tile_order, int num_tiles, const CountReport &report, cudaStream_t st);
