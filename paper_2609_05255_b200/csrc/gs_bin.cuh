@@ -8,16 +8,6 @@ namespace bin {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// Inclusive prefix sum over a warp.
-__device__ __forceinline__ uint32_t warp_inclusive(uint32_t v, int lane) {
-#pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const uint32_t t = __shfl_up_sync(kFull, v, s);
-    if (lane >= s) v += t;
-  }
-  return v;
-}
-
 // Stable rank of a row of 32 elements inside its warp, for a radix sort: `count` and `lanes` point to the words of this
 // lane's digit in arrays that belong to the warp alone, both zero at the start of a tile.  Every lane sets its bit in the
 // digit's word, reads back which lanes share the digit, and takes the count so far plus the sharing lanes below it; the

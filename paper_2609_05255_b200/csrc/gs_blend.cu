@@ -83,10 +83,6 @@ __device__ __forceinline__ void copy_async16(void *dst, const void *src) {
 __device__ __forceinline__ void copy_async8(void *dst, const void *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ void copy_async4(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ void fetch_entry(RawEntries &raw, int lane, uint32_t g, const float *mean2d, const float *conic_opacity,
                                             const float *color) {

@@ -413,6 +413,23 @@ __device__ __forceinline__ float tanh_fast(float y) {
   return fmaf(-2.f, r, 1.f);
 }
 
+// Inclusive prefix sum over a warp.
+template <class T>
+__device__ __forceinline__ T warp_inclusive(T v, int lane) {
+#pragma unroll
+  for (int s = 1; s < 32; s <<= 1) {
+    const T t = __shfl_up_sync(0xffffffffu, v, s);
+    if (lane >= s) v += t;
+  }
+  return v;
+}
+
+// A float on its own way into shared memory, no register held.
+__device__ __forceinline__ void copy_async4(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Programmatic dependent launch.  The kernels of the binning (gs_sort.cu) form chains of short, dependent launches (12 per view, 16 of a
 // large scene).
 // Launched with the attribute below, a kernel may be placed on the SMs as soon as the CTAs of its predecessor in the

@@ -55,12 +55,6 @@ __device__ __forceinline__ void warp_store_rows(float *g, int64_t row0, int64_t 
   __syncwarp();
 }
 
-// A float on its own way into shared memory, no register held.
-__device__ __forceinline__ void copy_async4(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // ---- 1D bulk copies (tensor memory accelerator) with bounded waits ------------------------------------------
 // load(): one lane arms the warp's mbarrier with the byte count and starts the copy; wait(): every lane polls the
 // barrier's phase, at most about a second in all; store(): shared -> global as a bulk group of the issuing lane.
@@ -519,12 +513,7 @@ __global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_prepro
     // and round: lanes own very different numbers of rows (1 to 12), and a loop per lane would idle most of them.
     // A row's tiles go into the owner's cell masks with shared-memory ORs (any order gives the same bits).
     const int rows = stored ? rect.w - rect.y : 0;
-    int incl = rows;
-#pragma unroll
-    for (int sft = 1; sft < 32; sft <<= 1) {
-      const int t = __shfl_up_sync(kFull, incl, sft);
-      if (lane >= sft) incl += t;
-    }
+    const int incl = warp_inclusive(rows, lane);
     const int total = __shfl_sync(kFull, incl, 31);
     if (in) {
       TileSpans sp;
@@ -938,12 +927,7 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
     const int64_t w = w0 + (tid >> 2);
     const uint32_t byte = w < w_end ? (__ldg(a.flags + w) >> (8 * (tid & 3))) & 255u : 0u;
     const int cnt = __popc(byte);
-    int incl = cnt;
-#pragma unroll
-    for (int sft = 1; sft < 32; sft <<= 1) {
-      const int t = __shfl_up_sync(kFull, incl, sft);
-      if (lane >= sft) incl += t;
-    }
+    const int incl = warp_inclusive(cnt, lane);
     if (lane == 31) s_warp_count[warp] = incl;
     __syncthreads();
     int offset = incl - cnt, total = 0;
@@ -1012,12 +996,7 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_explicit(PreprocessBw
     const uint32_t word = w < end ? __ldg(a.flags + w) : 0u;
     const bool dense = a.deg > 0 && __popc(word) >= kDenseWord && 32 * w + 32 <= a.n;
     const int own = dense ? 1 << 16 : __popc(word);
-    int incl = own;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const int t = __shfl_up_sync(kFull, incl, s);
-      if (lane >= s) incl += t;
-    }
+    const int incl = warp_inclusive(own, lane);
     if (lane == 31) s_counts[warp] = incl;
     __syncthreads();                // (the round before is over, too)
     int first = incl - own, all = 0;

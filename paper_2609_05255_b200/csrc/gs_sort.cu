@@ -151,12 +151,7 @@ __device__ __forceinline__ void block_exclusive_scan(const uint32_t v[DPT], uint
   uint32_t sum = 0;
 #pragma unroll
   for (int j = 0; j < DPT; ++j) { out[j] = sum; sum += v[j]; }
-  uint32_t inc = sum;
-#pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const uint32_t t = __shfl_up_sync(kFull, inc, s);
-    if (lane >= s) inc += t;
-  }
+  const uint32_t inc = warp_inclusive(sum, lane);
   if (lane == 31) s_warp_tot[warp] = inc;
   __syncthreads();
   uint32_t off = inc - sum;
@@ -476,12 +471,7 @@ __global__ void __launch_bounds__(kScanBlock, 8) k_emit_records(
     cc = __ldg(sorted_count + i);
   }
   const uint32_t cnt = cc & ~kCellBig;
-  uint32_t inc = cnt;
-#pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const uint32_t t = __shfl_up_sync(kFull, inc, s);
-    if (lane >= s) inc += t;
-  }
+  const uint32_t inc = warp_inclusive(cnt, lane);
   if (lane == 31) s_w[warp] = inc;
   // records of all CTAs before this one: the sums per kScanBlock Gaussians come from the last pass of the depth
   // sort; every CTA adds up its own prefix (a few loads per thread) instead of a scan kernel doing it for all
@@ -535,22 +525,12 @@ __global__ void __launch_bounds__(1024) k_cell_chunks(const uint32_t *__restrict
       const uint32_t s0 = cell_ranges[2 * c], e0 = cell_ranges[2 * c + 1];
       v = e0 > s0 ? (e0 - s0 + kCellChunk - 1) / kCellChunk : 0u;
     }
-    uint32_t inc = v;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const uint32_t t = __shfl_up_sync(kFull, inc, s);
-      if (lane >= s) inc += t;
-    }
+    const uint32_t inc = warp_inclusive(v, lane);
     if (lane == 31) s_w[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-      uint32_t w = s_w[lane], winc = w;
-#pragma unroll
-      for (int s = 1; s < 32; s <<= 1) {
-        const uint32_t t = __shfl_up_sync(kFull, winc, s);
-        if (lane >= s) winc += t;
-      }
-      s_w[lane] = winc - w;
+      const uint32_t w = s_w[lane];
+      s_w[lane] = warp_inclusive(w, lane) - w;
     }
     __syncthreads();
     const uint32_t carry = s_carry;

@@ -425,12 +425,7 @@ __global__ void __launch_bounds__(tc::kTile, H == 16 ? 4 : 2) k_variant_bwd_tc(A
       const int64_t w = w0 + (tid >> 2);
       const uint32_t byte = w < w_end ? (__ldg(a.flags + w) >> (8 * (tid & 3))) & 255u : 0u;
       const int cnt = __popc(byte);
-      int incl = cnt;
-#pragma unroll
-      for (int sft = 1; sft < 32; sft <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, sft);
-        if (lane >= sft) incl += t;
-      }
+      const int incl = warp_inclusive(cnt, lane);
       if (lane == 31) s_warp_count[warp] = incl;
       __syncthreads();
       int offset = incl - cnt, total = 0;
