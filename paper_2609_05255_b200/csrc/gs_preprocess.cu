@@ -957,7 +957,7 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
 
 // ---- the same for the explicit models, SH and Spherical Voronoi ----
 // Bound by memory: a Gaussian with a gradient reads and writes its parameter row of 45 or 49 floats and as much again of
-// geometry.  A CTA takes 128 flag words of its run at a time, one per thread.  Where a word has at least kDenseWord
+// geometry.  A CTA takes 128 flag words of its run at a time.  Where a word has at least kDenseWord
 // Gaussians with a gradient (a view of a scene that is not opaque yet: all words), its 32 rows come in by one bulk copy and
 // their gradients leave by one, zeros among them; the Gaussians of the thinner words are listed, and gathered and scattered
 // row by row, 32 at a time.  The four warps take the words and the batches in turn, on their own.
@@ -992,23 +992,25 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_explicit(PreprocessBw
   const int64_t words = (a.n + 31) / 32;
   const int64_t begin = words * blockIdx.x / gridDim.x, end = words * (blockIdx.x + 1) / gridDim.x;
   for (int64_t w0 = begin; w0 < end; w0 += kBlock) {
-    const int64_t w = w0 + tid;
+    // a word per thread, or, in a short round, a byte of one
+    const bool bytes = end - w0 <= kBlock / 4;
+    const int mine = bytes ? tid >> 2 : tid, part = bytes ? tid & 3 : 0;
+    const int64_t w = w0 + mine;
     const uint32_t word = w < end ? __ldg(a.flags + w) : 0u;
     const bool dense = a.deg > 0 && __popc(word) >= kDenseWord && 32 * w + 32 <= a.n;
-    const int own = dense ? 1 << 16 : __popc(word);
+    uint32_t bits = dense ? 0u : bytes ? word & (255u << (8 * part)) : word;
+    const int own = dense && part == 0 ? 1 << 16 : __popc(bits);
     const int incl = warp_inclusive(own, lane);
     if (lane == 31) s_counts[warp] = incl;
     __syncthreads();                // (the round before is over, too)
     int first = incl - own, all = 0;
 #pragma unroll
     for (int k = 0; k < kWarps; ++k) { const int c = s_counts[k]; first += k < warp ? c : 0; all += c; }
-    if (dense) {
+    if (dense && part == 0) {
       s_dense[first >> 16] = word;
-      s_which[first >> 16] = (unsigned char)tid;
-    } else {
-      int at = first & 0xffff;
-      for (uint32_t bits = word; bits; bits &= bits - 1u) s_list[at++] = (unsigned short)(32 * tid + __ffs(bits) - 1);
+      s_which[first >> 16] = (unsigned char)mine;
     }
+    for (int at = first & 0xffff; bits; bits &= bits - 1u) s_list[at++] = (unsigned short)(32 * mine + __ffs(bits) - 1);
     __syncthreads();
     const int num_dense = all >> 16, listed = all & 0xffff, jobs = num_dense + (listed + 31) / 32;
     for (int job = warp; job < jobs && !gave_up; job += kWarps) {
