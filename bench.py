@@ -31,7 +31,7 @@ N_GAUSS, WIDTH, HEIGHT, VIEWS = 1_000_000, 1256, 828, 8
 # the per-Gaussian kernels.
 # Blend kernels (fp32 ALU bound): flops per list entry evaluated for a pixel (the alpha test) and per
 # pair composited, counted from the kernels' arithmetic.
-BLEND_FLOPS_PER_EVALUATED = 8.0       # 3.5 (quad falloff, shared by 4 pixels) + ex2 + mul + min + compare
+BLEND_FLOPS_PER_EVALUATED = 8.0       # 3.5 (falloff, the row's terms shared by four pixels) + ex2 + mul + min + compare
 BLEND_FWD_FLOPS_PER_COMPOSITED = 10.0  # 1-a, T(1-a), compare, aT, three FMAs
 BLEND_BWD_FLOPS_PER_COMPOSITED = 45.0  # reciprocal, T and S recovery, d/d alpha, nine gradient FMAs
 FP32_LANES_PER_SM, NUM_SMS = 128, 148

@@ -180,9 +180,9 @@ __device__ __forceinline__ void composite(float alpha, float n, float w, const f
 }
 
 // Forward.  Entries are taken four at a time: their alphas do not depend on one another, only the chain through T does.
-// 8 x 8 pixels per warp measured best from 16 tiles to 8160 (16 x 8 ties at 8160, 97 against 102 us at 4108, 66 against
-// 77 at 2550; two entries at a time: 1 to 2 us more where a launch is only a few warps per scheduler).
-// 1M Gaussians, 1256 x 828: 150 -> 97 us; 92 M -> 72 M warp instructions.
+// 8 x 8 pixels per warp measured best from 16 tiles to 8160 (16 x 8 ties at 8160, 5 us more at 4108 tiles, 11 at 2550; two
+// entries at a time: 1 to 2 us more where a launch is only a few warps per scheduler).
+// 1M Gaussians, 1256 x 828: 152 -> 105 us; 92 M -> 81 M warp instructions, 76 % of the issue slots.
 constexpr int kFwdPixels = 2, kFwdGroup = 4;
 __global__ void __launch_bounds__(32) k_blend_fwd(
     CamDev cam, const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ order, const uint32_t *__restrict__ vals,
@@ -399,13 +399,14 @@ struct __align__(16) BwdArea {
 // (d colour r, g, b, d opacity) (d conic A, B, C, d mean u) (d mean v, -, -, -).
 // Per entry that is 3 stores and about 20 instructions, where a butterfly of the nine sums over the warp took 19 shuffles
 // (4 cycles each), as many adds and 14 selects, and the same sums as products on the tensor cores (tf32 operands in two
-// terms) took fewer instructions but 105 register operands instead of 55: 215 against 181 us.
+// terms) took fewer instructions but 105 register operands instead of 55: 215 against 181 us (neither writing zero rows, below).
 //
 // The kernel leaves the memory idle, so its warps also write what needs no arithmetic: every gradient row that is zero
 // because its Gaussian received nothing (in a scene with occlusion most of them: 94 % of the listed Gaussians of a view of
-// 1M).  All rows are zeroed here, each warp a slice on its way out
-// (on its way in, the first wave writes them all at once and the others' reads wait behind that: 23 us more at 1M); a bit per Gaussian says who received a gradient, and the
-// projection and appearance backward gathers those alone.
+// 1M).  All rows are zeroed here, each warp a slice on its way out (on its way in, the first wave writes them all at once
+// and the others' reads wait behind that: 23 us more at 1M); a bit per Gaussian says who received a gradient, and the
+// projection and appearance backward works on those alone.  1M Gaussians, 1256 x 828: 259 us without the zero rows -> 207
+// with those of the neural model, 62 % of the issue slots, FMA pipe 55 % busy.
 //
 // 16 x 8 pixels per warp is best where the launch fills the chip; smaller regions give more warps and cull more where it
 // does not, and where a few long lists make the time.  Measured with all three (4 x 8, 8 x 8, 16 x 8; us, zero rows

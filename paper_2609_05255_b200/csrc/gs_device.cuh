@@ -430,13 +430,13 @@ __device__ __forceinline__ void copy_async4(void *dst, const void *src) {
 }
 __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Programmatic dependent launch.  The kernels of the binning (gs_sort.cu) form chains of short, dependent launches (12 per view, 16 of a
-// large scene).
+// Programmatic dependent launch.  The kernels of the binning (gs_sort.cu) form chains of short, dependent launches (12 per view,
+// 16 of a large scene).
 // Launched with the attribute below, a kernel may be placed on the SMs as soon as the CTAs of its predecessor in the
 // stream have exited, without waiting for the predecessor's completion to be processed; dependency_wait() returns once
 // the predecessor has completed and its writes are visible, and every kernel here calls it before its first access to
 // global memory, so the order of all reads and writes is the stream's.  Launched without the attribute it is a no-op.
-// Measured on one stream: 214 instead of 248 us of binning per view.  Letting the successor in earlier
+// When it came in, the binning of a view of 1M took 214 instead of 248 us on one stream (180 by now).  Letting the successor in earlier
 // (griddepcontrol.launch_dependents at the top of every kernel) gained no more on one stream and cost 4 % with
 // several views in flight: the successor's CTAs then sit on the SMs for the whole run of the predecessor, in the
 // places of the other streams' kernels.

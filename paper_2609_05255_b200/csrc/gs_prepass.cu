@@ -72,7 +72,8 @@ __device__ __forceinline__ uint32_t pack_weights(const __half *w, int idx) {   /
 // One warp per 32 Gaussians at a time.  Lane L prepares row L (direction, SH basis, base colour, alpha byte);
 // the rows reach the tensor-core fragment layout through a small shared-memory tile; the weights
 // live in ten registers per lane for the whole kernel.
-// Bound by instruction issue (70 % of the slots, ALU pipe 63 %; 192 MB need 29 us): the warps are persistent, so that the weights
+// Bound by instruction issue and the loads that start every trip (353 warp instructions per 32 Gaussians on 62 % of the slots,
+// ALU pipe 39 %; 192 MB need 29 us): the warps are persistent, so that the weights
 // are read once, all addresses are 32-bit offsets from the warp's rows, the rectifiers work on packed halves, and degree 3
 // has an instance without the selects of the others.  3M Gaussians: 61.3 us before, 56.0 now.  Prefetching the next rows
 // takes registers that are worth more as warps (64.5).

@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t *__restrict__
 
 // Per chunk: write its instances.  The running positions of the tiles start from the tile's range, the chunk's offset
 // inside it and what the warps before this one hold.
-// Bound by the instructions of the ranking (ALU pipe 70 % busy, issue 67 %): a warp whose positions all lie inside the
+// Bound by the instructions of the ranking (issue 67 %, ALU pipe 57 % busy): a warp whose positions all lie inside the
 // buffers stores by the mask bits alone.  Before, a CTA also searched its chunk's cell (eight dependent loads), and two of
 // three CTAs found that they had no chunk.  1M Gaussians, 2.0M records, 7.9M instances: the expansion 55 us, with the chunk
 // list 50, with the stores 44.5.

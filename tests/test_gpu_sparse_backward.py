@@ -1,10 +1,10 @@
-"""The preprocess backward of the neural model spends arithmetic only on the Gaussians that received a gradient
-(k_bwd_flags + k_preprocess_bwd_sparse): the others - culled, or listed in tiles but composited by no pixel - get
-exact zeros.  Checked here: an upstream gradient that is zero outside a small window, so that almost every visible
-Gaussian is skipped and the few that are not fill less than one batch per CTA; an upstream gradient that is zero
-everywhere; a visible Gaussian with a zero gradient and non-finite appearance parameters; sizes around the batch and
-flag-word boundaries (128 Gaussians per batch, 32 per flag word, 4096 per scan round); the same through the unfused
-path, whose projection-only backward uses the same two kernels.  Every case against the oracle by the literal rule,
+"""The preprocess backward of the neural model (k_preprocess_bwd_sparse) spends arithmetic only on the Gaussians that
+received a gradient, which the blend backward flags: the others - culled, or listed in tiles but composited by no pixel - get
+exact zeros, from the blend backward too.  Checked here: an upstream gradient that is zero outside a small window, so that
+almost every visible Gaussian is skipped and the few that are not fill less than one batch per CTA; an upstream gradient that
+is zero everywhere; a visible Gaussian with a zero gradient and non-finite appearance parameters; sizes around the batch and
+flag-word boundaries (128 Gaussians per batch, 32 per flag word; a CTA has a second scan round of 1024 Gaussians from
+454 656 on, which the full-size parity tests reach); the same through the unfused path, whose projection-only backward is the same kernel.  Every case against the oracle by the literal rule,
 with exact zeros where the oracle has zeros."""
 import copy
 
