@@ -181,8 +181,8 @@ typedef struct {
   float *sv_sites;        /* SV:     [n,7,7] with respect to the raw site parameters            */
 } GsGrads;
 
-/* Create / destroy a context on CUDA device `device`.  The context owns 64 bytes of counters
- * (device and pinned host) and 7.5 MB of device memory for the per-CTA partial sums of the decoder
+/* Create / destroy a context on CUDA device `device`.  The context owns 64 bytes of counters on
+ * the device, 128 in pinned host memory and 7.5 MB of device memory for the per-CTA partial sums of the decoder
  * gradient.  Not thread safe: use one context per host thread, and one per stream whose calls may
  * overlap on the GPU.  Returns GS_ERR_CUDA if the device cannot be used. */
 GsStatus gs_create(int device, GsContext **ctx);
