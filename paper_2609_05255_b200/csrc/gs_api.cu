@@ -588,7 +588,7 @@ GsStatus gs_render_backward(GsContext *ctx, const GsScene *scene, const GsCamera
     }
     if (num_pairs > 0) {
       StageTimer t(ctx, GS_STAGE_BLEND_BWD, s);
-      t.done(launch_blend_bwd(cd, bin->tile_ranges, bin->tile_order, bin->sorted_vals, proj->mean2d, proj->conic_opacity, proj->color,
+      t.done(launch_blend_bwd(n, cd, bin->tile_ranges, bin->tile_order, bin->sorted_vals, proj->mean2d, proj->conic_opacity, proj->color,
                               final_T, n_contrib, dL_dimage, g2d, bw.flags, zeros, s));
     } else {
       for (int k = 0; k < zeros.count; ++k)

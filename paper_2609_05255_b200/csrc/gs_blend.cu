@@ -418,8 +418,9 @@ struct __align__(16) BwdArea {
 //    3200                                       clusters of 1M 260 182 188    deep 363 301 530
 //    4108                                       clusters of 1M 303 207 205    deep 404 303 459
 //    7500                                       clusters of 1M 483 313 289    deep 611 408 414
-// So 4 x 8 up to 100 tiles, where all scenes agree, and 8 x 8 up to 4000, where those in clusters change over (the deep one
-// changes over at 7500, the box of 100 000 at 1200, by 10 % at most; 5000 Gaussians at 400: 74 against 53 us at 960 tiles).
+//    3600         box of 100 000 246 160 141    clusters of 300 000 250 170 172, of 20 000 in the box 199 129 113
+// So 4 x 8 up to 100 tiles, where all scenes agree, 8 x 8 up to 3000, and up to 4000 where a scene has many Gaussians for its
+// tiles, 50 and more: there the clusters change over (the deep scene at 7500), the boxes at 1200 to 2000, by 10 % at most.
 // In the two smaller ones, what does not depend on the carried state is worked out for four entries at a time (2 to 4 us
 // less); with 16 x 8 pixels the registers it takes cost more than it gives.
 template <int NPX>
@@ -644,7 +645,7 @@ int launch_blend_fwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *
   return 1;
 }
 
-int launch_blend_bwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
+int launch_blend_bwd(int64_t n, const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
                      const float *mean2d,
                      const float *conic_opacity, const float *color, const float *final_T,
                      const uint32_t *n_contrib, const float *dL_dimage, float *g2d, uint32_t *flags, const ZeroRows &zeros,
@@ -665,7 +666,7 @@ int launch_blend_bwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *
   };
   // (the measurements behind the two lines are at the kernel)
   if (tiles <= 100) launch(k_blend_bwd<1>, Share<1>::kWarps);
-  else if (tiles <= 4000) launch(k_blend_bwd<2>, Share<2>::kWarps);
+  else if (tiles <= 3000 || (tiles <= 4000 && n >= (int64_t)50 * tiles)) launch(k_blend_bwd<2>, Share<2>::kWarps);
   else launch(k_blend_bwd<4>, Share<4>::kWarps);
   return 1;
 }

@@ -229,7 +229,7 @@ struct ZeroRows {
   void add(float *p, uint64_t n) { if (n) { ptr[count] = p; floats[count++] = n; } }
 };
 // Also sets the flag bit of every Gaussian that received a gradient, and fills `zeros`.
-int launch_blend_bwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
+int launch_blend_bwd(int64_t n, const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
                       const float *mean2d, const float *conic_opacity, const float *color,
                       const float *final_T, const uint32_t *n_contrib, const float *dL_dimage,
                       float *g2d, uint32_t *flags, const ZeroRows &zeros, cudaStream_t st);

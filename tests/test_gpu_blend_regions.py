@@ -1,6 +1,6 @@
 """The blend kernels give every warp a region of a tile and choose its size by the number of tiles (backward: 4 x 8 pixels
-up to 100 tiles, 8 x 8 up to 4000, 16 x 8 beyond); lists go through shared memory 32 entries at a time, in groups of four,
-and what the lanes park is summed every eight entries.  Checked against the oracle at the edges of all of these: tile
+up to 100 tiles, 8 x 8 up to 3000, and up to 4000 with 50 Gaussians per tile, 16 x 8 beyond); lists go through shared memory
+32 entries at a time, in groups of four, and what the lanes park is summed every eight entries.  Checked against the oracle at the edges of all of these: tile
 counts on either side of the two lines, ragged images, lists of about 32 and 64 entries, opacities above the alpha clamp."""
 import numpy as np
 import pytest
@@ -34,6 +34,19 @@ def test_image_sizes_at_the_lines_between_region_sizes(oracle, width, height):
 def test_on_either_side_of_the_lines(oracle, width, height):
     sc = scenes.box_scene(3000, 2.0, 2.0, 6.0, -3.0, 0.5, 1.0, scenes.APP_SH, seed=32)
     _check(oracle, sc, scenes.identity_camera(width, height, float(max(width, height)), background=(0.2, 0.1, 0.3)))
+
+
+@pytest.mark.parametrize("n", [150_399, 150_400])                # 3008 tiles: 16 x 8 pixels, 8 x 8 pixels
+def test_many_gaussians_for_their_tiles(oracle, n):
+    sc = scenes.box_scene(n, 2.0, 2.0, 6.0, -5.0, 0.5, 1.0, scenes.APP_SH, seed=33)
+    cam = scenes.identity_camera(1021, 752, 1000.0)
+    G = scenes.upstream_gradient(cam, 5)
+    gpu = run_gpu(sc, cam, G)
+    fwd, ref = oracle.render(sc, cam, G)
+    assert image_mismatch(gpu.image, fwd.image, fwd.fragile).mean() <= 1e-4
+    for nm in grad_names(sc.app):
+        bad = grad_mismatch(getattr(gpu.grads, nm), getattr(ref, nm))
+        assert bad.mean() <= 0.01, (nm, int(bad.sum()))
 
 
 @pytest.mark.parametrize("n", [1, 3, 4, 5, 7, 8, 9, 31, 32, 33, 40, 63, 64, 65])
