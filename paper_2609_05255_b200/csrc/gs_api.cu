@@ -246,13 +246,14 @@ FwdWorkspace carve_fwd(void *ws, int64_t n, int64_t cap, int width, int height) 
 
 // Backward scratch: the 2D gradients [n,12] and the flags of the Gaussians that received one (cleared together), then (used
 // by the separate-pass path only) directions, dL/dcolor and dL/dd as [n,3] each.
-struct BwdWorkspace { float *g2d, *dirs, *g_color, *g_dirs; uint32_t *flags; size_t cleared, bytes; };
+struct BwdWorkspace { float *g2d, *dirs, *g_color, *g_dirs; GradFlags flags; size_t cleared, bytes; };
 BwdWorkspace carve_bwd(void *ws, int64_t n) {
   Carver c{static_cast<char *>(ws), 0};
   const size_t nn = (size_t)(n > 0 ? n : 1);
   BwdWorkspace w;
   w.g2d = c.take<float>(nn * 12);
-  w.flags = c.take<uint32_t>((nn + 31) / 32);     // one bit per Gaussian
+  w.flags.layout((int64_t)nn);
+  w.flags.words = c.take<uint32_t>((size_t)w.flags.stride * w.flags.copies);
   w.cleared = c.used;
   w.dirs = c.take<float>(nn * 3);
   w.g_color = c.take<float>(nn * 3);
@@ -568,7 +569,8 @@ GsStatus gs_render_backward(GsContext *ctx, const GsScene *scene, const GsCamera
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaSetDevice(ctx->device);
   const CamDev cd = make_cam(cam);
-  const BwdWorkspace bw = carve_bwd(workspace, n);
+  BwdWorkspace bw = carve_bwd(workspace, n);
+  if (cd.gx * cd.gy < 320) bw.flags.copies = 1;    // few warps: nobody waits, and the copies' reading costs a little (20 011: 1 us)
   float *g2d = bw.g2d;
   const bool ext = unfused(scene);
   // A decoder variant on the tcgen05 kernels works on the Gaussians that received a gradient only

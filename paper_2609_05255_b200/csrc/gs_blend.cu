@@ -423,12 +423,13 @@ struct __align__(16) BwdArea {
 // tiles, 50 and more: there the clusters change over (the deep scene at 7500), the boxes at 1200 to 2000, by 10 % at most.
 // In the two smaller ones, what does not depend on the carried state is worked out for four entries at a time (2 to 4 us
 // less); with 16 x 8 pixels the registers it takes cost more than it gives.
-template <int NPX>
+// kCopies: the flags exist several times (0.6 us more for 300 000 Gaussians, where they do not, if it is asked here).
+template <int NPX, bool kCopies>
 __global__ void __launch_bounds__(32) k_blend_bwd(
     CamDev cam, const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ order, const uint32_t *__restrict__ vals,
     const float *__restrict__ mean2d, const float *__restrict__ conic_opacity, const float *__restrict__ color,
     const float *__restrict__ final_T, const uint32_t *__restrict__ n_contrib, const float *__restrict__ dL_dimage,
-    float *__restrict__ g2d, uint32_t *__restrict__ flags, ZeroRows zeros) {
+    float *__restrict__ g2d, GradFlags flags, ZeroRows zeros) {
   using V = typename Share<NPX>::V;
   constexpr int kVecs = Share<NPX>::kVecs, kLanes = Lanes<V>::value, kWarps = Share<NPX>::kWarps, kGroup = NPX == 4 ? 1 : 4;
   __shared__ BwdArea<NPX> area;
@@ -556,7 +557,7 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
           if (t == 0) red_add4(dst, s.r, s.g, s.b, __fdividef(s.m, re.y));
           if (t == 1) red_add4(dst + 4, -0.5f * sxx, -sxy, -0.5f * syy, fmaf(A, sx, B * sy));
           if (t == 2) atomicAdd(dst + 8, fmaf(B, sx, C * sy));
-          if (t == 3) atomicOr(flags + (gid >> 5), 1u << (gid & 31u));
+          if (t == 3) flags.set<kCopies>(blockIdx.x, gid);
         }
       }
       __syncwarp();                              // the parked values have been read
@@ -648,7 +649,7 @@ int launch_blend_fwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *
 int launch_blend_bwd(int64_t n, const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
                      const float *mean2d,
                      const float *conic_opacity, const float *color, const float *final_T,
-                     const uint32_t *n_contrib, const float *dL_dimage, float *g2d, uint32_t *flags, const ZeroRows &zeros,
+                     const uint32_t *n_contrib, const float *dL_dimage, float *g2d, const GradFlags &flags, const ZeroRows &zeros,
                      cudaStream_t st) {
   const int tiles = cam.gx * cam.gy;
   // The rows that start as zeros are shared out over all warps of the grid.  An image of few tiles does not have the warps
@@ -664,10 +665,14 @@ int launch_blend_bwd(int64_t n, const CamDev &cam, const uint32_t *ranges, const
     for (int k = 0; k < z.count; ++k) z.slice[k] = (uint32_t)(((z.floats[k] >> 2) + ctas - 1) / ctas);
     kernel<<<ctas, 32, 0, st>>>(cam, ranges, order, vals, mean2d, conic_opacity, color, final_T, n_contrib, dL_dimage, g2d, flags, z);
   };
-  // (the measurements behind the two lines are at the kernel)
-  if (tiles <= 100) launch(k_blend_bwd<1>, Share<1>::kWarps);
-  else if (tiles <= 3000 || (tiles <= 4000 && n >= (int64_t)50 * tiles)) launch(k_blend_bwd<2>, Share<2>::kWarps);
-  else launch(k_blend_bwd<4>, Share<4>::kWarps);
+  // (the measurements behind the lines are at the kernel)
+  auto pick = [&](auto copies) {
+    constexpr bool kCopies = decltype(copies)::value;
+    if (tiles <= 100) launch(k_blend_bwd<1, kCopies>, Share<1>::kWarps);
+    else if (tiles <= 3000 || (tiles <= 4000 && n >= (int64_t)50 * tiles)) launch(k_blend_bwd<2, kCopies>, Share<2>::kWarps);
+    else launch(k_blend_bwd<4, kCopies>, Share<4>::kWarps);
+  };
+  if (flags.copies > 1) pick(Flag<true>()); else pick(Flag<false>());
   return 1;
 }
 

@@ -355,7 +355,7 @@ template <int H, int L>
 int run_bwd_tc(const AppearanceArgs &a, int nfeat, cudaStream_t st) {
   using D = VarDims<H, L>;
   const size_t smem = sizeof(vtc::SmemBwd<H, L>);
-  const bool gather = a.flags != nullptr;
+  const bool gather = a.flags.words != nullptr;
   opt_in(vtc::k_variant_bwd_tc<H, L, false>, smem);
   opt_in(vtc::k_variant_bwd_tc<H, L, true>, smem);
   int per_sm = 512 / vtc::Shape<H, L>::kColsAlloc;

@@ -61,6 +61,37 @@ struct PreprocessArgs {
 };
 int launch_preprocess_fwd(int app, const PreprocessArgs &a, const CamDev &cam, cudaStream_t st);
 
+// Who received a gradient in a view: a bit per Gaussian, set by the warps of the blend backward.  With few Gaussians in a large
+// image all warps are at the same few words, which the L2 serves one after another: the blend backward of 5000 Gaussians at
+// 1280 x 720 took 242 us (8 x 8 pixels per warp), 118 without the bits.  So the bits of less than 65 536 Gaussians exist up to 16 times, a warp sets
+// those of one copy, and a reader takes the copies together: 120 us; 1000 Gaussians at 640 x 480 45 -> 24, 5000 at 3840 x 2160
+// 1000 -> 668, 20 011 at 640 x 480 79 -> 67.  (A byte per Gaussian, stored, is no better than the atomics on bits; looking at
+// what an addition to the Gaussian's row finds there waits for the answer, 10 to 30 % more below 1000 tiles.)
+struct GradFlags {
+  static constexpr int kMostCopies = 16;
+  uint32_t *words;              // [copies, stride]
+  uint32_t stride;
+  int copies;                   // a power of two
+  void layout(int64_t n) {
+    copies = 1;
+    while (copies < kMostCopies && n * copies < 65536) copies *= 2;
+    stride = (uint32_t)((n + 31) / 32 + 31) & ~31u;      // whole lines of 128 bytes
+  }
+#ifdef __CUDACC__
+  template <bool kCopies>
+  __device__ __forceinline__ void set(uint32_t warp, uint32_t id) const {
+    atomicOr(words + (kCopies ? (warp & (uint32_t)(copies - 1)) * stride : 0u) + (id >> 5), 1u << (id & 31u));
+  }
+  __device__ __forceinline__ uint32_t word(int64_t w) const {
+    uint32_t v = __ldg(words + w);
+    if (copies > 1)
+#pragma unroll
+      for (int c = 1; c < kMostCopies; ++c)            // (all in flight together)
+        if (c < copies) v |= __ldg(words + c * stride + w);
+    return v;
+  }
+#endif
+};
 struct PreprocessBwdArgs {
   int64_t n;
   const float *means, *log_scales, *quats, *logits, *base_color, *sh_rest;
@@ -68,7 +99,7 @@ struct PreprocessBwdArgs {
   int deg, act;
   const float *g2d;            // [n,12]: dL/dcolor(3), dL/dopacity, dL/dconic(3), dL/dmean2d(2), pad
   const float *gd_in;          // kAppExternal only: [n,3] dL/dd from the separate appearance backward
-  const uint32_t *flags;       // one bit per Gaussian: it received a gradient in this view (only their rows are written)
+  GradFlags flags;             // who received a gradient in this view (only their rows are written)
   float *g_means, *g_log_scales, *g_quats, *g_logits, *g_base, *g_sh_rest, *g_features;
   float *w_partials;           // [kWgradBlocks, 816]
   float *g_weights;            // [816]
@@ -89,7 +120,7 @@ struct AppearanceArgs {
   int engine;                  // GsDecoderEngine for the default neural decoder: warp-level MMA, tcgen05, or per kernel the faster
   const uint32_t *mask;        // optional [n]: Gaussians with a zero here are skipped (no colour written; zero
                                // gradient rows written); the tiles-touched array in the unfused step
-  const uint32_t *flags;       // optional, backward of the decoder variants on tcgen05: one bit per Gaussian; only the
+  GradFlags flags;             // optional, backward of the decoder variants on tcgen05: only the
                                // flagged ones are worked on (gathered into full tiles) and written
   const float *means, *g2d;    // optional, with flags (the unfused step): view directions from the means and the camera
   float oc[3];                 // centre oc, dL/dcolor from columns 0..2 of the [n,12] rows g2d, instead of dirs / g_color
@@ -228,11 +259,11 @@ struct ZeroRows {
   int count;
   void add(float *p, uint64_t n) { if (n) { ptr[count] = p; floats[count++] = n; } }
 };
-// Also sets the flag bit of every Gaussian that received a gradient, and fills `zeros`.
+// Also sets the flag bit of every Gaussian (of n) that received a gradient, and fills `zeros`.
 int launch_blend_bwd(int64_t n, const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
                       const float *mean2d, const float *conic_opacity, const float *color,
                       const float *final_T, const uint32_t *n_contrib, const float *dL_dimage,
-                      float *g2d, uint32_t *flags, const ZeroRows &zeros, cudaStream_t st);
+                      float *g2d, const GradFlags &flags, const ZeroRows &zeros, cudaStream_t st);
 
 int launch_neural_fold(int64_t n, const __half *features, const __half *weights, __half *preact, cudaStream_t st);
 int launch_neural_prepass(int64_t n, int deg, int act, const float *means, const float *logits, const float *base_color,

@@ -925,7 +925,7 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_sparse(PreprocessBwdA
   for (int64_t w0 = w_begin; w0 < w_end; w0 += kWordsPerRound) {
     reload_fence();
     const int64_t w = w0 + (tid >> 2);
-    const uint32_t byte = w < w_end ? (__ldg(a.flags + w) >> (8 * (tid & 3))) & 255u : 0u;
+    const uint32_t byte = w < w_end ? (a.flags.word(w) >> (8 * (tid & 3))) & 255u : 0u;
     const int cnt = __popc(byte);
     const int incl = warp_inclusive(cnt, lane);
     if (lane == 31) s_warp_count[warp] = incl;
@@ -996,7 +996,7 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_explicit(PreprocessBw
     const bool bytes = end - w0 <= kBlock / 4;
     const int mine = bytes ? tid >> 2 : tid, part = bytes ? tid & 3 : 0;
     const int64_t w = w0 + mine;
-    const uint32_t word = w < end ? __ldg(a.flags + w) : 0u;
+    const uint32_t word = w < end ? a.flags.word(w) : 0u;
     const bool dense = a.deg > 0 && __popc(word) >= kDenseWord && 32 * w + 32 <= a.n;
     uint32_t bits = dense ? 0u : bytes ? word & (255u << (8 * part)) : word;
     const int own = dense && part == 0 ? 1 << 16 : __popc(bits);

@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(tc::kTile, H == 16 ? 4 : 2) k_variant_bwd_tc(A
     const int64_t w_begin = min(nwords, (int64_t)blockIdx.x * per_cta), w_end = min(nwords, w_begin + per_cta);
     for (int64_t w0 = w_begin; w0 < w_end; w0 += kGatherWords) {
       const int64_t w = w0 + (tid >> 2);
-      const uint32_t byte = w < w_end ? (__ldg(a.flags + w) >> (8 * (tid & 3))) & 255u : 0u;
+      const uint32_t byte = w < w_end ? (a.flags.word(w) >> (8 * (tid & 3))) & 255u : 0u;
       const int cnt = __popc(byte);
       const int incl = warp_inclusive(cnt, lane);
       if (lane == 31) s_warp_count[warp] = incl;
