@@ -419,8 +419,10 @@ struct __align__(16) BwdArea {
 //    4108                                       clusters of 1M 303 207 205    deep 404 303 459
 //    7500                                       clusters of 1M 483 313 289    deep 611 408 414
 //    3600         box of 100 000 246 160 141    clusters of 300 000 250 170 172, of 20 000 in the box 199 129 113
-// So 4 x 8 up to 100 tiles, where all scenes agree, 8 x 8 up to 3000, and up to 4000 where a scene has many Gaussians for its
-// tiles, 50 and more: there the clusters change over (the deep scene at 7500), the boxes at 1200 to 2000, by 10 % at most.
+// So 4 x 8 up to 64 tiles, and up to 100 with 50 Gaussians per tile (1870 in 91 tiles: 4 % more for the step), 8 x 8 up to 3000,
+// where the boxes have changed over (at 1200 to 2000, by 10 % at most), and up to 4000 with 400 per tile: the deep scene
+// changes over at 7500, clusters at 4000 when a view runs alone, but with four views in flight, which fill the chip together,
+// 16 x 8 does less work: 1842 against 1881 us for an iteration on 800 000 in clusters, 3240 tiles.
 // In the two smaller ones, what does not depend on the carried state is worked out for four entries at a time (2 to 4 us
 // less); with 16 x 8 pixels the registers it takes cost more than it gives.
 // kCopies: the flags exist several times (0.6 us more for 300 000 Gaussians, where they do not, if it is asked here).
@@ -668,8 +670,8 @@ int launch_blend_bwd(int64_t n, const CamDev &cam, const uint32_t *ranges, const
   // (the measurements behind the lines are at the kernel)
   auto pick = [&](auto copies) {
     constexpr bool kCopies = decltype(copies)::value;
-    if (tiles <= 100) launch(k_blend_bwd<1, kCopies>, Share<1>::kWarps);
-    else if (tiles <= 3000 || (tiles <= 4000 && n >= (int64_t)50 * tiles)) launch(k_blend_bwd<2, kCopies>, Share<2>::kWarps);
+    if (tiles <= 64 || (tiles <= 100 && n >= (int64_t)50 * tiles)) launch(k_blend_bwd<1, kCopies>, Share<1>::kWarps);
+    else if (tiles <= 3000 || (tiles <= 4000 && n >= (int64_t)400 * tiles)) launch(k_blend_bwd<2, kCopies>, Share<2>::kWarps);
     else launch(k_blend_bwd<4, kCopies>, Share<4>::kWarps);
   };
   if (flags.copies > 1) pick(Flag<true>()); else pick(Flag<false>());

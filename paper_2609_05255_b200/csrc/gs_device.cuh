@@ -63,18 +63,16 @@ int launch_preprocess_fwd(int app, const PreprocessArgs &a, const CamDev &cam, c
 
 // Who received a gradient in a view: a bit per Gaussian, set by the warps of the blend backward.  With few Gaussians in a large
 // image all warps are at the same few words, which the L2 serves one after another: the blend backward of 5000 Gaussians at
-// 1280 x 720 took 242 us (8 x 8 pixels per warp), 118 without the bits.  So the bits of less than 65 536 Gaussians exist up to 16 times, a warp sets
+// 1280 x 720 took 242 us (8 x 8 pixels per warp), 118 without the bits.  So the bits of less than 65 536 Gaussians exist up to 16 times, if there is a tile for every 20 of them; a warp sets
 // those of one copy, and a reader takes the copies together: 120 us; 1000 Gaussians at 640 x 480 45 -> 24, 5000 at 3840 x 2160
 // 1000 -> 668, 20 011 at 640 x 480 79 -> 67.  (A byte per Gaussian, stored, is no better than the atomics on bits; looking at
 // what an addition to the Gaussian's row finds there waits for the answer, 10 to 30 % more below 1000 tiles.)
 struct GradFlags {
-  static constexpr int kMostCopies = 16;
   uint32_t *words;              // [copies, stride]
   uint32_t stride;
-  int copies;                   // a power of two
+  int copies;                   // 1, 4 or 16
   void layout(int64_t n) {
-    copies = 1;
-    while (copies < kMostCopies && n * copies < 65536) copies *= 2;
+    copies = n < 16384 ? 16 : n < 65536 ? 4 : 1;
     stride = (uint32_t)((n + 31) / 32 + 31) & ~31u;      // whole lines of 128 bytes
   }
 #ifdef __CUDACC__
@@ -84,10 +82,10 @@ struct GradFlags {
   }
   __device__ __forceinline__ uint32_t word(int64_t w) const {
     uint32_t v = __ldg(words + w);
-    if (copies > 1)
-#pragma unroll
-      for (int c = 1; c < kMostCopies; ++c)            // (all in flight together)
-        if (c < copies) v |= __ldg(words + c * stride + w);
+    for (int c = 1; c < copies; c += 3) {              // (more at a time is more code, which costs where there are no copies)
+      const uint32_t *p = words + c * stride + w;
+      v |= __ldg(p) | __ldg(p + stride) | __ldg(p + 2 * stride);
+    }
     return v;
   }
 #endif

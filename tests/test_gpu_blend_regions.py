@@ -1,7 +1,9 @@
 """The blend kernels give every warp a region of a tile and choose its size by the number of tiles (backward: 4 x 8 pixels
-up to 100 tiles, 8 x 8 up to 3000, and up to 4000 with 50 Gaussians per tile, 16 x 8 beyond); lists go through shared memory
-32 entries at a time, in groups of four, and what the lanes park is summed every eight entries.  Checked against the oracle at the edges of all of these: tile
+up to 64 tiles, and up to 100 with 50 Gaussians per tile, 8 x 8 up to 3000, and up to 4000 with 400, 16 x 8 beyond); lists go
+through shared memory 32 entries at a time, in groups of four, and what the lanes park is summed every eight entries.  Checked against the oracle at the edges of all of these: tile
 counts on either side of the two lines, ragged images, lists of about 32 and 64 entries, opacities above the alpha clamp."""
+import copy
+
 import numpy as np
 import pytest
 
@@ -36,16 +38,27 @@ def test_on_either_side_of_the_lines(oracle, width, height):
     _check(oracle, sc, scenes.identity_camera(width, height, float(max(width, height)), background=(0.2, 0.1, 0.3)))
 
 
-@pytest.mark.parametrize("n", [150_399, 150_400])                # 3008 tiles: 16 x 8 pixels, 8 x 8 pixels
-def test_many_gaussians_for_their_tiles(oracle, n):
-    sc = scenes.box_scene(n, 2.0, 2.0, 6.0, -5.0, 0.5, 1.0, scenes.APP_SH, seed=33)
-    cam = scenes.identity_camera(1021, 752, 1000.0)
+@pytest.mark.parametrize("n,width,height", [(4_999, 160, 160), (5_000, 160, 160),                  # 100 tiles: 8 x 8 pixels, 4 x 8
+                                            (1_203_199, 1021, 752), (1_203_200, 1021, 752)])       # 3008 tiles: 16 x 8, 8 x 8
+def test_many_gaussians_for_their_tiles(oracle, n, width, height):
+    """3000 Gaussians in view, the others behind the camera: the size of the scene alone chooses the kernel."""
+    few = scenes.box_scene(3000, 2.0, 2.0, 6.0, -3.0, 0.5, 1.0, scenes.APP_NEURAL, seed=33)
+    cam = scenes.identity_camera(width, height, float(width))
     G = scenes.upstream_gradient(cam, 5)
-    gpu = run_gpu(sc, cam, G)
-    fwd, ref = oracle.render(sc, cam, G)
+    many = copy.copy(few)
+    for name in ("means", "log_scales", "quats", "opacity_logits", "base_color", "features"):
+        a = getattr(few, name)
+        setattr(many, name, np.concatenate([a, np.repeat(a[:1], n - 3000, 0)]))
+    many.means[3000:, 2] = -3.0
+    gpu = run_gpu(many, cam, G)
+    fwd, ref = oracle.render(few, cam, G)
     assert image_mismatch(gpu.image, fwd.image, fwd.fragile).mean() <= 1e-4
-    for nm in grad_names(sc.app):
-        bad = grad_mismatch(getattr(gpu.grads, nm), getattr(ref, nm))
+    for nm in grad_names(few.app):
+        got = getattr(gpu.grads, nm)
+        if nm != "mlp_weights":
+            assert not got[3000:].any(), nm
+            got = got[:3000]
+        bad = grad_mismatch(got, getattr(ref, nm))
         assert bad.mean() <= 0.01, (nm, int(bad.sum()))
 
 
