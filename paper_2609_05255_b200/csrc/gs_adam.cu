@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(kAdamThreads) k_adam(const __grid_constant__ A
   // the per-column step sizes of the chunk's tensor, in shared memory: the lanes of a warp want
   // different columns, which the constant bank would serve one address at a time
   __shared__ float s_step[GS_ADAM_MAX_COLS];
+  dependency_wait();
   const uint32_t total_chunks = a.chunk_start[a.num_tensors];
   for (uint32_t chunk = blockIdx.x; chunk < total_chunks; chunk += gridDim.x) {
     int ti = 0;
@@ -139,7 +140,7 @@ int launch_adam(const GsAdamTensor *tensors, int num_tensors, int64_t step, int 
   const uint32_t chunks = a.chunk_start[a.num_tensors];
   if (chunks == 0) return 0;
   const uint32_t wave = (uint32_t)num_sms * 8u;
-  k_adam<<<chunks < wave ? chunks : wave, kAdamThreads, 0, st>>>(a);
+  launch_chained(k_adam, chunks < wave ? chunks : wave, kAdamThreads, 0, st, a);
   return 1;
 }
 

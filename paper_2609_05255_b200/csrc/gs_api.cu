@@ -579,7 +579,6 @@ GsStatus gs_render_backward(GsContext *ctx, const GsScene *scene, const GsCamera
                         scene->active_degree > 0;
   if (ext && n > 0 && bad_ptr(proj->tiles_touched)) return fail(ctx, GS_ERR_INVALID_ARG, "proj->tiles_touched is NULL or misaligned");
   if (n > 0) {
-    if ((st = check_cuda(ctx, cudaMemsetAsync(g2d, 0, bw.cleared, s), "memset")) != GS_OK) return st;
     ZeroRows zeros = {};
     const uint64_t m = (uint64_t)n;
     zeros.add(grads->means, 3 * m); zeros.add(grads->log_scales, 3 * m); zeros.add(grads->quats, 4 * m); zeros.add(grads->opacity_logits, m);
@@ -591,9 +590,11 @@ GsStatus gs_render_backward(GsContext *ctx, const GsScene *scene, const GsCamera
     }
     if (num_pairs > 0) {
       StageTimer t(ctx, GS_STAGE_BLEND_BWD, s);
-      t.done(launch_blend_bwd(n, cd, bin->tile_ranges, bin->tile_order, bin->sorted_vals, proj->mean2d, proj->conic_opacity, proj->color,
+      const int clears = launch_clear(g2d, bw.cleared, s);
+      t.done(clears + launch_blend_bwd(n, cd, bin->tile_ranges, bin->tile_order, bin->sorted_vals, proj->mean2d, proj->conic_opacity, proj->color,
                               final_T, n_contrib, dL_dimage, g2d, bw.flags, zeros, s));
     } else {
+      if ((st = check_cuda(ctx, cudaMemsetAsync(g2d, 0, bw.cleared, s), "memset")) != GS_OK) return st;
       for (int k = 0; k < zeros.count; ++k)
         if ((st = check_cuda(ctx, cudaMemsetAsync(zeros.ptr[k], 0, zeros.floats[k] * sizeof(float), s), "memset")) != GS_OK) return st;
     }

@@ -301,6 +301,18 @@ __device__ __forceinline__ float select_alpha(float alpha, uint32_t pos, uint32_
   return r;
 }
 
+// The 2D gradients and flags start from zero.  The blend backward is let in at once and waits for the zeros only before it
+// walks its lists, so that a warp's first loads overlap them.  (As a memset, which neither kernel can be chained to, 2 to 5 us
+// of the stream passed around it.)
+constexpr int kClearThreads = 256, kClearBlocks = 148 * 4;
+__global__ void __launch_bounds__(kClearThreads) k_clear(float4 *__restrict__ rows, size_t quads) {
+  dependency_wait();
+  dependents_start();
+#pragma unroll 4
+  for (size_t i = (size_t)blockIdx.x * kClearThreads + threadIdx.x; i < quads; i += (size_t)gridDim.x * kClearThreads)
+    rows[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 // One warp's slice of the rows that start as zeros.
 constexpr int kZeroWarps = 148 * 2;           // at least; see launch_blend_bwd
 __device__ __forceinline__ void zero_rows(const ZeroRows &z, int lane) {
@@ -437,6 +449,7 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
   __shared__ BwdArea<NPX> area;
   const int lane = threadIdx.x;
   if (blockIdx.x >= (unsigned)(cam.gx * cam.gy * kWarps)) {      // a warp without a region, see launch_blend_bwd
+    dependency_wait();
     zero_rows(zeros, lane);
     return;
   }
@@ -471,6 +484,7 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) wmax = max(wmax, __shfl_xor_sync(kFull, wmax, s));
   if (wmax == 0 || wmax > __ldg(ranges + 2 * tile + 1) - start) {   // nothing composited in this region
+    dependency_wait();
     zero_rows(zeros, lane);
     return;
   }
@@ -481,6 +495,7 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
     fetch_entry(raw, lane, id, mean2d, conic_opacity, color);
   }
   uint32_t id_next = base >= 32u ? __ldg(vals + start + base - 32u + lane) : 0u;
+  dependency_wait();                           // k_clear lets this kernel in early; all it has read so far was there before that
   for (;; base -= 32u) {
     copies_wait();
     bool clamp;
@@ -648,6 +663,13 @@ int launch_blend_fwd(const CamDev &cam, const uint32_t *ranges, const uint32_t *
   return 1;
 }
 
+int launch_clear(void *p, size_t bytes, cudaStream_t st) {
+  const size_t quads = bytes / 16;
+  const int blocks = (int)std::min<size_t>(kClearBlocks, (quads + 4 * kClearThreads - 1) / (4 * kClearThreads));
+  launch_chained(k_clear, blocks, kClearThreads, 0, st, static_cast<float4 *>(p), quads);
+  return 1;
+}
+
 int launch_blend_bwd(int64_t n, const CamDev &cam, const uint32_t *ranges, const uint32_t *order, const uint32_t *vals,
                      const float *mean2d,
                      const float *conic_opacity, const float *color, const float *final_T,
@@ -665,7 +687,7 @@ int launch_blend_bwd(int64_t n, const CamDev &cam, const uint32_t *ranges, const
     ZeroRows z = zeros;
     const int ctas = std::max(tiles * warps, zero_warps);
     for (int k = 0; k < z.count; ++k) z.slice[k] = (uint32_t)(((z.floats[k] >> 2) + ctas - 1) / ctas);
-    kernel<<<ctas, 32, 0, st>>>(cam, ranges, order, vals, mean2d, conic_opacity, color, final_T, n_contrib, dL_dimage, g2d, flags, z);
+    launch_chained(kernel, ctas, 32, 0, st, cam, ranges, order, vals, mean2d, conic_opacity, color, final_T, n_contrib, dL_dimage, g2d, flags, z);
   };
   // (the measurements behind the lines are at the kernel)
   auto pick = [&](auto copies) {

@@ -51,6 +51,7 @@ struct __align__(128) Smem {
 
 template <bool kSplit>
 __global__ void __launch_bounds__(kTile) k_appearance_fwd_tc(AppearanceArgs a) {
+  dependency_wait();
   extern __shared__ __align__(128) unsigned char tc_smem[];
   Smem &S = *reinterpret_cast<Smem *>(tc_smem);
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -194,6 +195,7 @@ struct __align__(128) SmemBwd {
 
 template <bool kSplit>
 __global__ void __launch_bounds__(kTile) k_appearance_bwd_tc(AppearanceArgs a) {
+  dependency_wait();
   extern __shared__ __align__(128) unsigned char tc_smem[];
   SmemBwd &S = *reinterpret_cast<SmemBwd *>(tc_smem);
   const int tid = threadIdx.x, warp = tid >> 5;

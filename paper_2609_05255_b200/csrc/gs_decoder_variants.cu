@@ -102,6 +102,7 @@ __device__ __forceinline__ void variant_forward(const float *sW, VarState<H, L> 
 
 template <int H, int L>
 __global__ void __launch_bounds__(kVarBlock) k_variant_fwd(AppearanceArgs a, int nfeat) {
+  dependency_wait();
   extern __shared__ __align__(16) float sW[];
   for (int k = threadIdx.x; k < VarDims<H, L>::kNumW; k += kVarBlock) sW[k] = __half2float(a.weights[k]);
   __syncthreads();
@@ -156,6 +157,7 @@ __device__ __forceinline__ void warp_weight_grad(const float *sX, const float *s
 
 template <int H, int L>
 __global__ void __launch_bounds__(kVarBlock) k_variant_bwd(AppearanceArgs a, int nfeat) {
+  dependency_wait();
   using D = VarDims<H, L>;
   extern __shared__ __align__(16) float smem[];
   float *sW = smem;                                             // [kNumW]
@@ -280,6 +282,7 @@ __global__ void __launch_bounds__(kVarBlock) k_variant_bwd(AppearanceArgs a, int
 constexpr int kVarReduceGroups = 16;
 __global__ void __launch_bounds__(32 * kVarReduceGroups) k_variant_wreduce(const float *__restrict__ partials, int nblocks, int nw,
                                                                            float *__restrict__ out) {
+  dependency_wait();
   __shared__ float s_part[kVarReduceGroups][32];
   const int k = blockIdx.x * 32 + threadIdx.x, grp = threadIdx.y;
   float s = 0.f;
@@ -302,7 +305,7 @@ __global__ void __launch_bounds__(32 * kVarReduceGroups) k_variant_wreduce(const
   }
 }
 inline void launch_variant_wreduce(const float *partials, int nblocks, int nw, float *out, cudaStream_t st) {
-  k_variant_wreduce<<<(nw + 31) / 32, dim3(32, kVarReduceGroups), 0, st>>>(partials, nblocks, nw, out);
+  launch_chained(k_variant_wreduce, (nw + 31) / 32, dim3(32, kVarReduceGroups), 0, st, partials, nblocks, nw, out);
 }
 
 template <class K>
@@ -312,7 +315,7 @@ template <int H, int L>
 int run_fwd(const AppearanceArgs &a, int nfeat, cudaStream_t st) {
   const size_t smem = sizeof(float) * VarDims<H, L>::kNumW;
   opt_in(k_variant_fwd<H, L>, smem);
-  k_variant_fwd<H, L><<<(unsigned)((a.n + kVarBlock - 1) / kVarBlock), kVarBlock, smem, st>>>(a, nfeat);
+  launch_chained(k_variant_fwd<H, L>, (unsigned)((a.n + kVarBlock - 1) / kVarBlock), kVarBlock, smem, st, a, nfeat);
   return 1;
 }
 template <int H, int L>
@@ -328,7 +331,7 @@ int run_bwd(const AppearanceArgs &a, int nfeat, cudaStream_t st) {
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && per_sm > 0 && sms > 0)
     wave = per_sm * sms < kVarPartialBlocks ? per_sm * sms : kVarPartialBlocks;
   const int blocks = (int)(chunks < wave ? chunks : wave);
-  k_variant_bwd<H, L><<<blocks, kVarBlock, smem, st>>>(a, nfeat);
+  launch_chained(k_variant_bwd<H, L>, blocks, kVarBlock, smem, st, a, nfeat);
   launch_variant_wreduce(a.w_partials, blocks, D::kNumW, a.g_weights, st);
   return 2;
 }
@@ -348,7 +351,7 @@ int run_fwd_tc(const AppearanceArgs &a, int nfeat, cudaStream_t st) {
   opt_in(vtc::k_variant_fwd_tc<H, L>, smem);
   const int64_t tiles = (a.n + tc::kTile - 1) / tc::kTile;
   const int64_t wave = (int64_t)(H == 16 ? 8 : 7) * sm_count();   // 59 and 71 registers per thread
-  vtc::k_variant_fwd_tc<H, L><<<(unsigned)(tiles < wave ? tiles : wave), tc::kTile, smem, st>>>(a, nfeat);
+  launch_chained(vtc::k_variant_fwd_tc<H, L>, (unsigned)(tiles < wave ? tiles : wave), tc::kTile, smem, st, a, nfeat);
   return 1;
 }
 template <int H, int L>
@@ -367,8 +370,7 @@ int run_bwd_tc(const AppearanceArgs &a, int nfeat, cudaStream_t st) {
   int64_t wave = (int64_t)per_sm * sm_count();
   if (wave > kVarPartialBlocks) wave = kVarPartialBlocks;
   const int blocks = (int)(tiles < wave ? tiles : wave);
-  if (gather) vtc::k_variant_bwd_tc<H, L, true><<<blocks, tc::kTile, smem, st>>>(a, nfeat);
-  else vtc::k_variant_bwd_tc<H, L, false><<<blocks, tc::kTile, smem, st>>>(a, nfeat);
+  launch_chained(gather ? vtc::k_variant_bwd_tc<H, L, true> : vtc::k_variant_bwd_tc<H, L, false>, blocks, tc::kTile, smem, st, a, nfeat);
   launch_variant_wreduce(a.w_partials, blocks, D::kNumW, a.g_weights, st);
   return 2;
 }

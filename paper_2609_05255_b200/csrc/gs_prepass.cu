@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(kFoldThreads) k_neural_fold(int64_t n, const _
                                                               const __half *__restrict__ weights,
                                                               __half *__restrict__ preact) {
   __shared__ float s_w[GS_MLP_HIDDEN][17];   // column 0 and the 16 feature columns of the first layer
+  dependency_wait();
   for (int k = threadIdx.x; k < GS_MLP_HIDDEN * 17; k += kFoldThreads) {
     const int o = k / 17, c = k % 17;
     s_w[o][c] = __half2float(weights[kMlpW1 + o * GS_MLP_IN + (c == 0 ? 0 : 15 + c)]);
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(kPrepassThreads, kPrepassBlocks) k_neural_prep
                                                                     float *__restrict__ color) {
   __shared__ uint32_t s_x[kPrepassWarps][32][kXRow];
   __shared__ float s_y[kPrepassWarps][32][3];
+  dependency_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   // B fragments: B[k][nn] = W[nn][k]; b0 holds k = 2t, 2t+1 and b1 k = 2t+8, 2t+9 of column nn = 8 nt + g.
   // Layer 1 keeps only the direction columns 1..15 (column 0 is the folded constant: its weight is dropped).
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(kPrepassThreads, kPrepassBlocks) k_neural_prep
 
 int launch_neural_fold(int64_t n, const __half *features, const __half *weights, __half *preact, cudaStream_t st) {
   if (n <= 0) return 0;
-  k_neural_fold<<<(unsigned)((n + kFoldThreads - 1) / kFoldThreads), kFoldThreads, 0, st>>>(n, features, weights, preact);
+  launch_chained(k_neural_fold, (unsigned)((n + kFoldThreads - 1) / kFoldThreads), kFoldThreads, 0, st, n, features, weights, preact);
   return 1;
 }
 
@@ -212,8 +214,8 @@ int launch_neural_prepass(int64_t n, int deg, int act, const float *means, const
                           cudaStream_t st) {
   if (n <= 0) return 0;
   const int64_t blocks = std::min<int64_t>((n + kPrepassThreads - 1) / kPrepassThreads, 148 * kPrepassBlocks);
-  (deg >= 3 ? k_neural_prepass<true> : k_neural_prepass<false>)<<<(unsigned)blocks, kPrepassThreads, 0, st>>>(
-      n, deg, act, means, logits, base_color, preact, weights, eye[0], eye[1], eye[2], reinterpret_cast<uchar4 *>(rgba), color);
+  launch_chained(deg >= 3 ? k_neural_prepass<true> : k_neural_prepass<false>, (unsigned)blocks, kPrepassThreads, 0, st, n, deg, act, means, logits,
+                 base_color, preact, weights, eye[0], eye[1], eye[2], reinterpret_cast<uchar4 *>(rgba), color);
   return 1;
 }
 

@@ -1118,6 +1118,7 @@ __global__ void __launch_bounds__(kBlock) k_preprocess_bwd_explicit(PreprocessBw
 
 template <int APP>
 __global__ void __launch_bounds__(kBlock) k_appearance_fwd(AppearanceArgs a) {
+  dependency_wait();
   static_assert(IsNeural<APP>::value, "the neural model in either decoder precision");
   __shared__ __align__(16) StageFwd sStage[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1152,6 +1153,7 @@ __global__ void __launch_bounds__(kBlock) k_appearance_fwd(AppearanceArgs a) {
 
 template <int APP>
 __global__ void __launch_bounds__(kBlock) k_appearance_bwd(AppearanceArgs a) {
+  dependency_wait();
   static_assert(IsNeural<APP>::value, "the neural model in either decoder precision");
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1214,6 +1216,7 @@ template <int APP> constexpr size_t bulk_smem_bytes() {
 // BWD = false: colours.  BWD = true: gradient rows (written in place over the parameter rows), dL/dc0, dL/dd.
 template <int APP, bool BWD>
 __global__ void __launch_bounds__(kBlock) k_appearance_bulk(AppearanceArgs a) {
+  dependency_wait();
   static_assert(Explicit<APP>::value, "the explicit models only");
   constexpr int kRow = RowOf<APP>::value, kSlab = SlabOf<APP>::value;
   constexpr uint32_t kBytes = kSlab * sizeof(float);
@@ -1309,6 +1312,7 @@ __global__ void __launch_bounds__(kBlock) k_appearance_bulk(AppearanceArgs a) {
 __global__ void __launch_bounds__(kBlock) k_unfused_prepare(int64_t n, const float *__restrict__ means, CamDev cam,
                                                             const float *__restrict__ g2d, const uint32_t *__restrict__ mask,
                                                             float *__restrict__ dirs, float *__restrict__ g_color) {
+  dependency_wait();
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   if (i >= n) return;
   float d[3] = {0.f, 0.f, 1.f}, g[3] = {0.f, 0.f, 0.f};
@@ -1374,7 +1378,7 @@ int launch_preprocess_fwd(int app, const PreprocessArgs &a, const CamDev &cam, c
 int launch_unfused_prepare(int64_t n, const float *means, const CamDev &cam, const float *g2d, const uint32_t *mask,
                            float *dirs, float *g_color, cudaStream_t st) {
   if (n == 0) return 0;
-  k_unfused_prepare<<<grid_for(n), kBlock, 0, st>>>(n, means, cam, g2d, mask, dirs, g_color);
+  launch_chained(k_unfused_prepare, grid_for(n), kBlock, 0, st, n, means, cam, g2d, mask, dirs, g_color);
   return 1;
 }
 
@@ -1416,7 +1420,7 @@ int launch_bulk(const AppearanceArgs &a, cudaStream_t st) {
   constexpr size_t smem = bulk_smem_bytes<APP>();
   opt_in_smem(k_appearance_bulk<APP, BWD>, smem);
   const int wave = resident_blocks<k_appearance_bulk<APP, BWD>>(smem), chunks = grid_for(a.n);
-  k_appearance_bulk<APP, BWD><<<chunks < wave ? chunks : wave, kBlock, smem, st>>>(a);
+  launch_chained(k_appearance_bulk<APP, BWD>, chunks < wave ? chunks : wave, kBlock, smem, st, a);
   return 1;
 }
 
@@ -1441,19 +1445,19 @@ int launch_appearance_fwd(int app, const AppearanceArgs &a, cudaStream_t st) {
     constexpr size_t smem = sizeof(tc::Smem);
     if (app == kAppNeuralHalf) {
       const int wave = tc_wave();
-      tc::k_appearance_fwd_tc<false><<<chunks < wave ? chunks : wave, kBlock, smem, st>>>(a);
+      launch_chained(tc::k_appearance_fwd_tc<false>, chunks < wave ? chunks : wave, kBlock, smem, st, a);
     } else {
       const int wave = tc_wave();
-      tc::k_appearance_fwd_tc<true><<<chunks < wave ? chunks : wave, kBlock, smem, st>>>(a);
+      launch_chained(tc::k_appearance_fwd_tc<true>, chunks < wave ? chunks : wave, kBlock, smem, st, a);
     }
     return 1;
   }
   if (app == kAppNeuralHalf) {
     const int wave = resident_blocks<k_appearance_fwd<kAppNeuralHalf>>(0, 1 << 20);
-    k_appearance_fwd<kAppNeuralHalf><<<chunks < wave ? chunks : wave, kBlock, 0, st>>>(a);
+    launch_chained(k_appearance_fwd<kAppNeuralHalf>, chunks < wave ? chunks : wave, kBlock, 0, st, a);
   } else {
     const int wave = resident_blocks<k_appearance_fwd<GS_APP_NEURAL>>(0, 1 << 20);
-    k_appearance_fwd<GS_APP_NEURAL><<<chunks < wave ? chunks : wave, kBlock, 0, st>>>(a);
+    launch_chained(k_appearance_fwd<GS_APP_NEURAL>, chunks < wave ? chunks : wave, kBlock, 0, st, a);
   }
   return 1;
 }
@@ -1478,10 +1482,10 @@ int launch_appearance_bwd(int app, const AppearanceArgs &a, cudaStream_t st) {
       if (blocks > grid_for(a.n)) blocks = grid_for(a.n);
       if (app == kAppNeuralHalf) {
         opt_in_smem(tc::k_appearance_bwd_tc<false>, smem);
-        tc::k_appearance_bwd_tc<false><<<blocks, kBlock, smem, st>>>(a);
+        launch_chained(tc::k_appearance_bwd_tc<false>, blocks, kBlock, smem, st, a);
       } else {
         opt_in_smem(tc::k_appearance_bwd_tc<true>, smem);
-        tc::k_appearance_bwd_tc<true><<<blocks, kBlock, smem, st>>>(a);
+        launch_chained(tc::k_appearance_bwd_tc<true>, blocks, kBlock, smem, st, a);
       }
       launch_wgrad_reduce(a.w_partials, blocks, a.g_weights, st);
       return 2;
@@ -1489,13 +1493,13 @@ int launch_appearance_bwd(int app, const AppearanceArgs &a, cudaStream_t st) {
     if (app == kAppNeuralHalf) {
       opt_in_smem(k_appearance_bwd<kAppNeuralHalf>, kBwdSmemNN);
       const int blocks = resident_blocks<k_appearance_bwd<kAppNeuralHalf>>(kBwdSmemNN);
-      k_appearance_bwd<kAppNeuralHalf><<<blocks, kBlock, kBwdSmemNN, st>>>(a);
+      launch_chained(k_appearance_bwd<kAppNeuralHalf>, blocks, kBlock, kBwdSmemNN, st, a);
       launch_wgrad_reduce(a.w_partials, blocks, a.g_weights, st);
       return 2;
     }
     opt_in_smem(k_appearance_bwd<GS_APP_NEURAL>, kBwdSmemNN);
     const int blocks = resident_blocks<k_appearance_bwd<GS_APP_NEURAL>>(kBwdSmemNN);
-    k_appearance_bwd<GS_APP_NEURAL><<<blocks, kBlock, kBwdSmemNN, st>>>(a);
+    launch_chained(k_appearance_bwd<GS_APP_NEURAL>, blocks, kBlock, kBwdSmemNN, st, a);
     launch_wgrad_reduce(a.w_partials, blocks, a.g_weights, st);
     return 2;
   }
@@ -1586,10 +1590,10 @@ extern "C" GsStatus gs_appearance_backward_noalloc(const GsScene *scene, const f
   const int blocks = (int)(chunks < kNoAllocMaxBlocks ? chunks : kNoAllocMaxBlocks);
   if (scene->decoder_precision == GS_DECODER_HALF) {   // same dispatch as gs_appearance_backward
     opt_in_smem(k_appearance_bwd<kAppNeuralHalf>, kBwdSmemNN);
-    k_appearance_bwd<kAppNeuralHalf><<<blocks, kBlock, kBwdSmemNN, st>>>(a);
+    launch_chained(k_appearance_bwd<kAppNeuralHalf>, blocks, kBlock, kBwdSmemNN, st, a);
   } else {
     opt_in_smem(k_appearance_bwd<GS_APP_NEURAL>, kBwdSmemNN);
-    k_appearance_bwd<GS_APP_NEURAL><<<blocks, kBlock, kBwdSmemNN, st>>>(a);
+    launch_chained(k_appearance_bwd<GS_APP_NEURAL>, blocks, kBlock, kBwdSmemNN, st, a);
   }
   launch_wgrad_reduce(scratch, blocks, a.g_weights, st);
   const cudaError_t e = cudaGetLastError();

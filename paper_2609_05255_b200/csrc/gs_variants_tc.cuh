@@ -135,6 +135,7 @@ struct __align__(128) SmemFwd {
 
 template <int H, int L>
 __global__ void __launch_bounds__(tc::kTile) k_variant_fwd_tc(AppearanceArgs a, int nfeat) {
+  dependency_wait();
   using S_t = SmemFwd<H, L>;
   using Sh = Shape<H, L>;
   extern __shared__ __align__(128) unsigned char vtc_smem[];
@@ -242,6 +243,7 @@ constexpr int kGatherQueue = 2 * 32 * kGatherWords;       // a power of two abov
 
 template <int H, int L, bool kGather>
 __global__ void __launch_bounds__(tc::kTile, H == 16 ? 4 : 2) k_variant_bwd_tc(AppearanceArgs a, int nfeat) {
+  dependency_wait();
   using S_t = SmemBwd<H, L>;
   using Sh = Shape<H, L>;
   using D = VarDims<H, L>;
