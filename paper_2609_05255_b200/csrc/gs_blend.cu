@@ -301,13 +301,12 @@ __device__ __forceinline__ float select_alpha(float alpha, uint32_t pos, uint32_
   return r;
 }
 
-// The 2D gradients and flags start from zero.  The blend backward is let in at once and waits for the zeros only before it
-// walks its lists, so that a warp's first loads overlap them.  (As a memset, which neither kernel can be chained to, 2 to 5 us
-// of the stream passed around it.)
+// The 2D gradients and flags start from zero.  (As a memset, which neither neighbour can be chained to, 2 to 5 us of the stream
+// passed around it.  Letting the blend backward in early, to overlap its first loads, is no gain and a trap: the few warps of a
+// small image then pile up on the SMs that this kernel leaves first, 49 -> 60 to 160 us for 30 tiles.)
 constexpr int kClearThreads = 256, kClearBlocks = 148 * 4;
 __global__ void __launch_bounds__(kClearThreads) k_clear(float4 *__restrict__ rows, size_t quads) {
   dependency_wait();
-  dependents_start();
 #pragma unroll 4
   for (size_t i = (size_t)blockIdx.x * kClearThreads + threadIdx.x; i < quads; i += (size_t)gridDim.x * kClearThreads)
     rows[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -446,10 +445,10 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
     float *__restrict__ g2d, GradFlags flags, ZeroRows zeros) {
   using V = typename Share<NPX>::V;
   constexpr int kVecs = Share<NPX>::kVecs, kLanes = Lanes<V>::value, kWarps = Share<NPX>::kWarps, kGroup = NPX == 4 ? 1 : 4;
+  dependency_wait();
   __shared__ BwdArea<NPX> area;
   const int lane = threadIdx.x;
   if (blockIdx.x >= (unsigned)(cam.gx * cam.gy * kWarps)) {      // a warp without a region, see launch_blend_bwd
-    dependency_wait();
     zero_rows(zeros, lane);
     return;
   }
@@ -484,7 +483,6 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) wmax = max(wmax, __shfl_xor_sync(kFull, wmax, s));
   if (wmax == 0 || wmax > __ldg(ranges + 2 * tile + 1) - start) {   // nothing composited in this region
-    dependency_wait();
     zero_rows(zeros, lane);
     return;
   }
@@ -495,7 +493,6 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
     fetch_entry(raw, lane, id, mean2d, conic_opacity, color);
   }
   uint32_t id_next = base >= 32u ? __ldg(vals + start + base - 32u + lane) : 0u;
-  dependency_wait();                           // k_clear lets this kernel in early; all it has read so far was there before that
   for (;; base -= 32u) {
     copies_wait();
     bool clamp;
