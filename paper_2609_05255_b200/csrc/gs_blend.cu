@@ -182,9 +182,10 @@ __device__ __forceinline__ void composite(float alpha, float n, float w, const f
 // Forward.  Entries are taken four at a time: their alphas do not depend on one another, only the chain through T does.
 // 8 x 8 pixels per warp measured best from 16 tiles to 8160 (16 x 8 ties at 8160, 5 us more at 4108 tiles, 11 at 2550; two
 // entries at a time: 1 to 2 us more where a launch is only a few warps per scheduler).
-// 1M Gaussians, 1256 x 828: 152 -> 105 us; 92 M -> 81 M warp instructions, 76 % of the issue slots.
+// 1M Gaussians, 1256 x 828: 152 -> 105 us; 92 M -> 81 M warp instructions, 76 % of the issue slots.  With 32 warps per SM, the
+// most there can be of one-warp CTAs, instead of 28 -> 101, and 201 -> 193 in a view of 3M: one word spilled, before the loop.
 constexpr int kFwdPixels = 2, kFwdGroup = 4;
-__global__ void __launch_bounds__(32) k_blend_fwd(
+__global__ void __launch_bounds__(32, 32) k_blend_fwd(
     CamDev cam, const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ order, const uint32_t *__restrict__ vals,
     const float *__restrict__ mean2d, const float *__restrict__ conic_opacity, const float *__restrict__ color,
     uint32_t *__restrict__ sorted_tiles, float *__restrict__ image, float *__restrict__ final_T, uint32_t *__restrict__ n_contrib) {
