@@ -417,35 +417,43 @@ struct __align__(16) BwdArea {
 // because its Gaussian received nothing (in a scene with occlusion most of them: 94 % of the listed Gaussians of a view of
 // 1M).  All rows are zeroed here, each warp a slice on its way out (on its way in, the first wave writes them all at once
 // and the others' reads wait behind that: 23 us more at 1M); a bit per Gaussian says who received a gradient, and the
-// projection and appearance backward works on those alone.  1M Gaussians, 1256 x 828: 259 us without the zero rows -> 207
+// projection and appearance backward works on those alone.  1M Gaussians, 1256 x 828: 259 us without the zero rows -> 217
 // with those of the neural model, 62 % of the issue slots, FMA pipe 55 % busy.
+//
+// What does not depend on the carried state is worked out for four entries at a time, so that the reciprocals, exponentials and
+// products of one entry fill the waits of another: 217 -> 201 us at 1M (4108 tiles), 436 -> 381 in a view of 3M over depths of
+// 1 to 50 (8160), with 16 warps per SM.  More warps do not help: 24 of 80 registers take as long as 19 of 96, and so do 15
+// (padded shared memory); batches of four entries, which would make room for 28, cost 15 to 30 % for their longer sums.
 //
 // 16 x 8 pixels per warp is best where the launch fills the chip; smaller regions give more warps and cull more where it
 // does not, and where a few long lists make the time.  Measured with all three (4 x 8, 8 x 8, 16 x 8; us, zero rows
-// included) from 25 to 9600 tiles, for scenes of 5000 to 100 000 Gaussians in a box, 300 000 and 1M in clusters, drawn and
-// with all opacities 0.1, and 2M over depths of 1 to 50:
-//     100 tiles   box of 100 000  45  51  92    of 5000  35  41  74    (128: 37 41 70, but 45 33 55; clusters 86 125 332)
-//     361         box of 100 000  55  49  74    clusters of 300 000  90 102 217
-//    2700         box of 100 000 197 129 119    clusters of 1M 234 166 178    deep 336 330 469
-//    3200                                       clusters of 1M 260 182 188    deep 363 301 530
-//    4108                                       clusters of 1M 303 207 205    deep 404 303 459
-//    7500                                       clusters of 1M 483 313 289    deep 611 408 414
-//    3600         box of 100 000 246 160 141    clusters of 300 000 250 170 172, of 20 000 in the box 199 129 113
-// So 4 x 8 up to 64 tiles, and up to 100 with 50 Gaussians per tile (1870 in 91 tiles: 4 % more for the step), 8 x 8 up to 3000,
-// where the boxes have changed over (at 1200 to 2000, by 10 % at most), and up to 4000 with 400 per tile: the deep scene
-// changes over at 7500, clusters at 4000 when a view runs alone, but with four views in flight, which fill the chip together,
-// 16 x 8 does less work: 1842 against 1881 us for an iteration on 800 000 in clusters, 3240 tiles.
-// In the two smaller ones, what does not depend on the carried state is worked out for four entries at a time (2 to 4 us
-// less); with 16 x 8 pixels the registers it takes cost more than it gives.
+// included) for scenes of 5000 to 100 000 Gaussians in a box, 300 000 and 1M in clusters and 2M over depths of 1 to 50:
+//     tiles    box of 5000     box of 100 000      clusters of 300 000   of 1M             deep
+//       64     32  39  69       54  52  84
+//      100     33  36  59       83  75 118
+//      256     30  31  44       58  55  87
+//      576     43  34  40       67  53  75         109 127 195           135 127 227
+//     1024     58  40  44       94  69  67         114  98 160           141 110 173
+//     1600     78  53  49      133  89  84         139 106 141           169 123 132
+//     2500    113  73  64      183 121 108         177 120 128           214 147 153       334 336 642
+//     3025    132  84  71      213 138 119         202 134 147           239 159 164       358 395 663
+//     3600    154  97  80      248 157 133         228 149 148           268 175 173       361 348 681
+//     4225    176 110  89      282 179 151         256 164 157           299 193 185       394 291 579
+//     5625                                         317 203 182           370 235 216       475 305 501
+// So 4 x 8 up to 64 tiles, and up to 100 with 50 Gaussians per tile; 8 x 8 up to 1000, where the boxes change over, up to 3200
+// with 50 per tile, for the clusters (154 000 in 2632: 105 against 122), and up to 6000 with 350, for the deep scenes (3M in
+// 8160: 415 against 381).  With
+// four views in flight, which fill the chip together, 16 x 8 does less work in all of them: 2126 against 2176 us for an
+// iteration on 300 000 in clusters, 2500 tiles.
 // kCopies: the flags exist several times (0.6 us more for 300 000 Gaussians, where they do not, if it is asked here).
 template <int NPX, bool kCopies>
-__global__ void __launch_bounds__(32) k_blend_bwd(
+__global__ void __launch_bounds__(32, NPX == 1 ? 28 : 16) k_blend_bwd(
     CamDev cam, const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ order, const uint32_t *__restrict__ vals,
     const float *__restrict__ mean2d, const float *__restrict__ conic_opacity, const float *__restrict__ color,
     const float *__restrict__ final_T, const uint32_t *__restrict__ n_contrib, const float *__restrict__ dL_dimage,
     float *__restrict__ g2d, GradFlags flags, ZeroRows zeros) {
   using V = typename Share<NPX>::V;
-  constexpr int kVecs = Share<NPX>::kVecs, kLanes = Lanes<V>::value, kWarps = Share<NPX>::kWarps, kGroup = NPX == 4 ? 1 : 4;
+  constexpr int kVecs = Share<NPX>::kVecs, kLanes = Lanes<V>::value, kWarps = Share<NPX>::kWarps, kGroup = 4;
   dependency_wait();
   __shared__ BwdArea<NPX> area;
   const int lane = threadIdx.x;
@@ -511,7 +519,7 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
           // What does not depend on the carried state, for a group of entries.  A pixel that did not composite an entry (it
           // lies beyond the pixel's walk, or alpha < 1/255) enters with alpha = 0, for which the reciprocal is 1, every
           // product below is 0 and its carried state is unchanged.
-          V a[kGroup][kVecs], inv[kGroup][kVecs], gc[kGroup][kVecs], free[kGroup][kVecs];
+          V a[kGroup][kVecs], odds[kGroup][kVecs], gc[kGroup][kVecs], free[kGroup][kVecs];   // odds: alpha / (1 - alpha)
 #pragma unroll
           for (int e = kGroup - 1; e >= 0; --e) {
             const float4 b = st.rest[j + e], c = st.rgb[j + e];
@@ -527,7 +535,8 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
               }
               const V d = add(bc<V>(1.f), neg(a[e][k]));
 #pragma unroll
-              for (int i = 0; i < kLanes; ++i) put(inv[e][k], i, rcp_approx(get(d, i)));
+              for (int i = 0; i < kLanes; ++i) put(odds[e][k], i, rcp_approx(get(d, i)));
+              odds[e][k] = mul(a[e][k], odds[e][k]);
               gc[e][k] = mad(Gb[k], bc<V>(c.z), mad(Gg[k], bc<V>(c.y), mul(Gr[k], bc<V>(c.x))));
             }
           }
@@ -536,14 +545,15 @@ __global__ void __launch_bounds__(32) k_blend_bwd(
           for (int e = kGroup - 1; e >= 0; --e)
 #pragma unroll
             for (int k = 0; k < kVecs; ++k) {
-              const V Tb = mul(T[k], inv[e][k]), w = mul(a[e][k], Tb);   // transmittance in front of this entry; its weight
+              const V w = mul(T[k], odds[e][k]);                // the entry's weight: alpha T / (1 - alpha), T behind it
               if (k == 0) { cr[e] = mul(w, Gr[k]); cg[e] = mul(w, Gg[k]); cb[e] = mul(w, Gb[k]); }
               else { cr[e] = mad(w, Gr[k], cr[e]); cg[e] = mad(w, Gg[k], cg[e]); cb[e] = mad(w, Gb[k], cb[e]); }
-              // d pixel / d alpha = T c - S / (1 - alpha), S = everything composited behind this entry
-              dp[e][k] = mul(a[e][k], mul(mad(T[k], gc[e][k], neg(S[k])), inv[e][k]));
+              // alpha times d pixel / d alpha = (T c - S) / (1 - alpha), S = everything composited behind this entry.  (The difference
+              // first, in one rounding: as w c - odds S it loses what the two have in common, ten times as much in the 3M view.)
+              dp[e][k] = mul(odds[e][k], mad(T[k], gc[e][k], neg(S[k])));
               if (kClamp) dp[e][k] = mul(dp[e][k], free[e][k]);     // clamped at 0.99: alpha does not depend on opacity and power
               S[k] = mad(w, gc[e][k], S[k]);
-              T[k] = Tb;
+              T[k] = add(T[k], w);                       // in front of it: T / (1 - alpha) = T + w
             }
 #pragma unroll
           for (int e = kGroup - 1; e >= 0; --e) park<NPX>(area.parked, j + e - bottom, lane, dp[e], hsum(cr[e]), hsum(cg[e]), hsum(cb[e]));
@@ -690,8 +700,9 @@ int launch_blend_bwd(int64_t n, const CamDev &cam, const uint32_t *ranges, const
   // (the measurements behind the lines are at the kernel)
   auto pick = [&](auto copies) {
     constexpr bool kCopies = decltype(copies)::value;
-    if (tiles <= 64 || (tiles <= 100 && n >= (int64_t)50 * tiles)) launch(k_blend_bwd<1, kCopies>, Share<1>::kWarps);
-    else if (tiles <= 3000 || (tiles <= 4000 && n >= (int64_t)400 * tiles)) launch(k_blend_bwd<2, kCopies>, Share<2>::kWarps);
+    const auto per_tile = [&](int64_t least) { return n >= least * tiles; };
+    if (tiles <= 64 || (tiles <= 100 && per_tile(50))) launch(k_blend_bwd<1, kCopies>, Share<1>::kWarps);
+    else if (tiles <= 1000 || (tiles <= 3200 && per_tile(50)) || (tiles <= 6000 && per_tile(350))) launch(k_blend_bwd<2, kCopies>, Share<2>::kWarps);
     else launch(k_blend_bwd<4, kCopies>, Share<4>::kWarps);
   };
   if (flags.copies > 1) pick(Flag<true>()); else pick(Flag<false>());

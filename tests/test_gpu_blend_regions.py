@@ -1,5 +1,5 @@
 """The blend kernels give every warp a region of a tile and choose its size by the number of tiles (backward: 4 x 8 pixels
-up to 64 tiles, and up to 100 with 50 Gaussians per tile, 8 x 8 up to 3000, and up to 4000 with 400, 16 x 8 beyond); lists go
+up to 64 tiles, and up to 100 with 50 Gaussians per tile, 8 x 8 up to 1000, up to 3200 with 50 and up to 6000 with 350, 16 x 8 beyond); lists go
 through shared memory 32 entries at a time, in groups of four, and what the lanes park is summed every eight entries.  Checked against the oracle at the edges of all of these: tile
 counts on either side of the two lines, ragged images, lists of about 32 and 64 entries, opacities above the alpha clamp."""
 import copy
@@ -11,6 +11,11 @@ from paper_2609_05255_b200 import scenes
 from gpu_helpers import grad_mismatch, grad_names, image_mismatch, run_gpu
 
 pytestmark = pytest.mark.gpu
+
+
+LINES = [(3_000, 640, 400), (3_000, 1025, 247),                                  # 1000, 1040 tiles
+         (159_999, 800, 1024), (160_000, 800, 1024), (170_000, 1617, 512),       # 3200 tiles and 50 per tile; 3264
+         (2_099_999, 960, 1600), (2_100_000, 960, 1600), (2_200_000, 961, 1600)] # 6000 tiles and 350 per tile; 6100
 
 
 def _check(oracle, sc, cam, allow=0.01):   # sums over 800 x 950 pixels, of both signs: 0.3 % miss the literal rule
@@ -60,6 +65,11 @@ def test_many_gaussians_for_their_tiles(oracle, n, width, height):
             got = got[:3000]
         bad = grad_mismatch(got, getattr(ref, nm))
         assert bad.mean() <= 0.01, (nm, int(bad.sum()))
+
+
+@pytest.mark.parametrize("n,width,height", LINES)
+def test_the_lines_for_larger_images(oracle, n, width, height):
+    test_many_gaussians_for_their_tiles(oracle, n, width, height)
 
 
 @pytest.mark.parametrize("n", [1, 3, 4, 5, 7, 8, 9, 31, 32, 33, 40, 63, 64, 65])
