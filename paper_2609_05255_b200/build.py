@@ -9,7 +9,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libgs_b200.so")
-SOURCES = ["gs_api.cu", "gs_preprocess.cu", "gs_sort.cu", "gs_bin_cluster.cu", "gs_blend.cu", "gs_adam.cu", "gs_prepass.cu",
+SOURCES = ["gs_api.cu", "gs_preprocess.cu", "gs_sort.cu", "gs_depth_sort.cu", "gs_bin_cluster.cu", "gs_blend.cu", "gs_adam.cu", "gs_prepass.cu",
            "gs_decoder_variants.cu"]
 HEADERS = [os.path.join(CSRC, h) for h in ("gs_device.cuh", "gs_bin.cuh", "gs_mlp_mma.cuh", "gs_decoder_tc.cuh", "gs_tcgen05.cuh", "gs_variants_tc.cuh")] + [os.path.join(_ROOT, "include", "gs.h")]
 

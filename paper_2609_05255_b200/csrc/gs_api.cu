@@ -222,8 +222,8 @@ FwdWorkspace carve_fwd(void *ws, int64_t n, int64_t cap, int width, int height) 
   const int cells = ((gx + 3) / 4) * ((gy + 3) / 4);
   const size_t pieces = (size_t)max_pieces((int64_t)cc, cells);
   w.sorted_depth = c.take<uint32_t>(nn);
-  w.tmp_keys = c.take<uint32_t>(nn);
-  w.tmp_vals = c.take<uint32_t>(nn);
+  w.tmp_keys = c.take<uint32_t>(2 * ((nn + 63) & ~(size_t)63));      // (one array of pairs to the bucket sort)
+  w.tmp_vals = w.tmp_keys + ((nn + 63) & ~(size_t)63);
   w.block_sums = reinterpret_cast<uint32_t *>(c.take<char>(scan_scratch_bytes((int64_t)nn)));
   w.rec_keys = c.take<uint32_t>(cc);
   w.rec_vals = c.take<uint32_t>(cc);
@@ -239,7 +239,7 @@ FwdWorkspace carve_fwd(void *ws, int64_t n, int64_t cap, int width, int height) 
   w.rec_total = c.take<unsigned long long>(1);
   w.num_visible = c.take<unsigned long long>(1);
   w.num_big = c.take<uint32_t>(1);
-  w.sort_table = c.take<char>(sort_scratch_bytes((int64_t)(nn > cc ? nn : cc)));
+  w.sort_table = c.take<char>(sort_scratch_bytes((int64_t)nn, (int64_t)cc));
   w.bytes = c.used;
   return w;
 }

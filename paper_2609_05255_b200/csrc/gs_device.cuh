@@ -181,7 +181,7 @@ struct SortEpilogue {
   unsigned long long *visible;
   uint32_t *final_vals;
 };
-size_t sort_scratch_bytes(int64_t count);
+size_t sort_scratch_bytes(int64_t n, int64_t records);
 // Stable sort of the cell records (keys: cell << 16 | tile mask) by cell, in radix_passes() passes: an odd number ends in
 // other_keys / other_vals, an even one in keys / vals.  `count` bounds the number of records (and sizes the grid), the true
 // number is read on the device.  With one pass it also leaves the chunks of the expansion.  Comes after launch_depth_sort,
@@ -194,6 +194,14 @@ int radix_passes(int num_bits);
 // the number of Gaussians that are not culled, and the epilogue's block sums cover those.
 int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order, uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t n,
                       unsigned long long *visible, void *scratch, const SortEpilogue &epilogue, const CountReport &report, cudaStream_t st);
+// The same by buckets (gs_depth_sort.cu), for cameras that cull every depth of zero and below: pairs [n] is scratch, `clear` is
+// cleared on the way.
+constexpr int64_t kBucketSortMost = 1 << 22;  // Gaussians
+bool bucket_sort_takes(int64_t n);
+size_t bucket_scratch_bytes();
+int launch_bucket_sort(const uint32_t *depth_key, uint32_t *counts_out, uint32_t *order, unsigned long long *pairs, int64_t n,
+                       unsigned long long *visible, void *scratch, uint32_t *clear, int clear_words, const SortEpilogue &ep,
+                       const CountReport &report, cudaStream_t st);
 size_t scan_scratch_bytes(int64_t n);
 int num_scan_blocks(int64_t n);   // entries of the block sums that launch_emit_records reads
 int launch_emit_records(const uint32_t *depth_order, const uint32_t *sorted_count, const uint32_t *cell_records,

@@ -1,7 +1,8 @@
 // Ordering and binning: a stable LSD radix sort (digits of 4 to 9 bits, keys staged and ranked in shared
 // memory, no inter-block waiting) and the kernels that turn its output into per-tile lists.
 //
-// (1) The Gaussians are sorted once by their 32-bit depth key (ties keep the index order: the sort is stable), culled ones
+// (1) The Gaussians are sorted once by their 32-bit depth key (ties keep the index order), by buckets (gs_depth_sort.cu) or, beyond 4M
+//     and where the near plane lets depths be zero or negative, by the radix sort; culled ones
 //     leaving after the first of the four passes.
 // (2) In that order every Gaussian emits one record per CELL of 4 x 4 tiles that its footprint reaches - the cell id
 //     and a 16-bit mask of the tiles met inside the cell, as the preprocess left them - and the records are sorted by
@@ -87,7 +88,6 @@ __device__ __forceinline__ uint32_t rotated(uint32_t key) { return __funnelshift
 constexpr int kMaxGroups = 22;                   // ceil(sqrt(kMaxSortBlocks)), also the largest group
 constexpr int kGroupTables = 6;                  // four passes of the depth sort, two of the record sort
 static_assert(kMaxGroups * kMaxGroups >= kMaxSortBlocks, "groups");
-constexpr int kDirectBlocks = 148;               // up to this many blocks (one per SM) the depth sort needs no groups, see there
 int group_size(int blocks) { int g = 1; while (g * g < blocks) ++g; return g; }
 
 // Digit histogram of each block's contiguous range: table[block][digit], added to groups[block / group][digit] unless
@@ -177,16 +177,11 @@ template <int BITS> constexpr size_t scatter_smem_bytes() {
 // is a boundary; the two ends of a run may continue in another block and enter with an atomic min / max), 3 the first
 // pass of the depth sort: keys come as they are, the largest digit's elements go to their final place and are counted out,
 // 4 the record sort in a single pass: the digits' totals are the ranges, and the chunks of the expansion follow from them.
-// DIRECT: the depth sort of up to kDirectBlocks blocks of one tile each.  A block reads the whole digit table, and as the
-// place of every element in the next pass is known when it is written, it is counted into that pass's table there and
-// then: one launch per pass.  50 000 Gaussians 44.9 us before, 30.1 now, 100 000 46.6 and 37.1.  With more blocks the atomics
-// and the table's reading cost more than the launches they save: 150 000 41.3 either way, 300 000 53 against 50.
-template <int BITS, int EP, bool DIRECT = false>
+template <int BITS, int EP>
 __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
     const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in, uint32_t *__restrict__ keys_out,
     uint32_t *__restrict__ vals_out, int64_t count, const unsigned long long *__restrict__ count_dev, int shift,
-    const uint32_t *__restrict__ table, const uint32_t *__restrict__ groups, int group, uint32_t *__restrict__ next_table,
-    SortEpilogue ep) {
+    const uint32_t *__restrict__ table, const uint32_t *__restrict__ groups, int group, SortEpilogue ep) {
   dependency_wait();
   constexpr int NB = BITS <= 8 ? 256 : (1 << BITS);   // entries of the digit arrays
   constexpr int DPT = NB / kSortThreads;              // digits per thread
@@ -202,31 +197,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
   // global base of every digit for this block: all smaller digits everywhere + the same digit in the blocks before
   {
     uint32_t tot[DPT] = {}, before[DPT] = {}, start[DPT];
-    if (DIRECT) {
-      // thread: four digits of every fourth block
-      const int part = tid >> 6, rows = (int)gridDim.x, own = (int)blockIdx.x;
-      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-      for (int r0 = part; r0 < rows; r0 += 4 * 16) {
-        uint4 v[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-          v[k] = r0 + 4 * k < rows ? __ldg(reinterpret_cast<const uint4 *>(table) + (r0 + 4 * k) * 64 + (tid & 63)) : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          const uint32_t m = r0 + 4 * k < own ? 0xffffffffu : 0u;
-          a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w;
-          b.x += v[k].x & m; b.y += v[k].y & m; b.z += v[k].z & m; b.w += v[k].w & m;
-        }
-      }
-      reinterpret_cast<uint4 *>(s_warp_cnt)[tid] = a;
-      reinterpret_cast<uint4 *>(s_warp_cnt)[kSortThreads + tid] = b;
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        tot[0] += s_warp_cnt[256 * k + tid];
-        before[0] += s_warp_cnt[256 * (4 + k) + tid];
-      }
-    } else if (tid * DPT <= (int)kDigitMask) {
+    if (tid * DPT <= (int)kDigitMask) {
       const int own = (int)blockIdx.x / group, num = ((int)gridDim.x + group - 1) / group, in_group = (int)blockIdx.x - own * group;
       uint32_t v[kMaxGroups][DPT], u[kMaxGroups][DPT];     // all in flight together: in two halves the pass took 3 us more
 #pragma unroll
@@ -250,7 +221,6 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
       const int d = tid * DPT + j;
       s_base[d] = start[j] + before[j];
       if (EP == 3 && blockIdx.x == 0 && d == (int)kDigitMask) *ep.visible = start[j];
-      if (EP == 3 && DIRECT && d == (int)kDigitMask) s_warp_tot[kSortWarps] = start[j];
     }
     if (EP == 4 && blockIdx.x == gridDim.x - 1) {       // (its range is the shortest)
       uint32_t chunks[DPT], first[DPT];
@@ -355,12 +325,6 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
       s_vals[pos] = val[it];
     }
     __syncthreads();
-    uint32_t per_shift = 0;                             // 2^32 over the blocks of 256 that a block of the next pass takes
-    if (DIRECT && EP != 1) {
-      const uint32_t next_count = EP == 3 ? s_warp_tot[kSortWarps] : (uint32_t)count;
-      const uint32_t per = ((next_count + gridDim.x - 1) / gridDim.x + kSortThreads - 1) / kSortThreads;
-      per_shift = 0xffffffffu / max(per, 1u) + 1u;      // exact for places below 2^24 x 256 (0: every place over one is itself)
-    }
     constexpr int kOut = 4;                             // rows written together, so that what they wait for overlaps
     for (int j0 = 0; j0 < valid_count; j0 += kOut * kSortThreads) {
       uint32_t gpos[kOut], count_of[kOut];
@@ -382,10 +346,6 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
         } else {
           keys_out[gpos[h]] = k;
           vals_out[gpos[h]] = v;
-          if (DIRECT && EP != 1) {
-            const uint32_t place = gpos[h] / kSortThreads, block = per_shift ? __umulhi(place, per_shift) : place;
-            atomicAdd(next_table + (block << BITS) + ((k >> (shift + BITS)) & kDigitMask), 1u);
-          }
         }
         if (EP == 2) {
           const uint32_t run_end = d == kDigitMask ? (uint32_t)valid_count : s_digit_start[d + 1];   // slots past the input hold no run
@@ -673,8 +633,9 @@ __global__ void __launch_bounds__(kExpandThreads, 4) k_expand(const uint32_t *__
 
 }  // namespace
 
-size_t sort_scratch_bytes(int64_t count) {
-  return (2 * (size_t)sort_blocks(count) + kGroupTables * kMaxGroups) * (1 << kMaxDigitBits) * sizeof(uint32_t);
+size_t sort_scratch_bytes(int64_t n, int64_t records) {
+  constexpr size_t kTable = (1 << kMaxDigitBits) * sizeof(uint32_t);
+  return kGroupTables * kMaxGroups * kTable + std::max(2 * sort_blocks(std::max(n, records)) * kTable, bucket_scratch_bytes());
 }
 
 namespace {
@@ -682,20 +643,20 @@ namespace {
 uint32_t *group_table(void *scratch, int p) { return static_cast<uint32_t *>(scratch) + ((size_t)p * kMaxGroups << kMaxDigitBits); }
 uint32_t *block_table(void *scratch) { return group_table(scratch, kGroupTables); }
 
-template <int BITS, int EP, bool DIRECT = false>
+template <int BITS, int EP>
 void launch_scatter(int blocks, const uint32_t *src_k, const uint32_t *src_v, uint32_t *dst_k, uint32_t *dst_v, int64_t count,
                     const unsigned long long *count_dev, int shift, const uint32_t *table, const uint32_t *groups,
-                    const SortEpilogue &ep, cudaStream_t st, uint32_t *next_table = nullptr) {
+                    const SortEpilogue &ep, cudaStream_t st) {
   constexpr size_t smem = scatter_smem_bytes<BITS>();
   static bool opted[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (smem > 48 * 1024 && dev >= 0 && dev < 64 && !opted[dev]) {
-    cudaFuncSetAttribute(k_radix_scatter<BITS, EP, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_radix_scatter<BITS, EP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     opted[dev] = true;
   }
-  launch_chained(k_radix_scatter<BITS, EP, DIRECT>, blocks, kSortThreads, smem, st, src_k, src_v, dst_k, dst_v, count, count_dev, shift, table,
-                 groups, group_size(blocks), next_table, ep);
+  launch_chained(k_radix_scatter<BITS, EP>, blocks, kSortThreads, smem, st, src_k, src_v, dst_k, dst_v, count, count_dev, shift, table,
+                 groups, group_size(blocks), ep);
 }
 }  // namespace
 
@@ -735,6 +696,9 @@ int launch_record_sort(uint32_t *keys, uint32_t *vals, uint32_t *other_keys, uin
 
 int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order, uint32_t *tmp_keys, uint32_t *tmp_vals, int64_t n,
                       unsigned long long *visible, void *scratch, const SortEpilogue &epilogue, const CountReport &report, cudaStream_t st) {
+  if (visible && bucket_sort_takes(n))             // (the record sort's groups are cleared by the way)
+    return launch_bucket_sort(depth_key, keys, order, reinterpret_cast<unsigned long long *>(tmp_keys), n, visible, block_table(scratch),
+                              group_table(scratch, 4), 2 * kMaxGroups << kMaxDigitBits, epilogue, report, st);
   const int blocks = sort_blocks(n), group = group_size(blocks);
   uint32_t *table = block_table(scratch);
   SortEpilogue ep[4] = {};
@@ -746,30 +710,20 @@ int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order
     ep[0].counts = epilogue.counts;
     ep[0].id_mask = ep[3].id_mask = n <= (int64_t)1 << kIdBits ? (1u << kIdBits) - 1u : ~0u;
   }
-  const bool direct = blocks <= kDirectBlocks && visible;
-  // digit tables of the passes, where each has its own: those of the passes to come lie together, after the groups' tables
-  const auto pass_table = [&](int p) { return table + ((size_t)((p + 3) & 3) * blocks << 8); };
   for (int p = 0; p < 4; ++p) {
     const uint32_t *src_k = p == 0 ? depth_key : p & 1 ? tmp_keys : keys, *src_v = p == 0 ? nullptr : p & 1 ? tmp_vals : order;
     uint32_t *dst_k = p & 1 ? keys : tmp_keys, *dst_v = p & 1 ? order : tmp_vals, *groups = group_table(scratch, p);
     const unsigned long long *count = p == 0 ? nullptr : visible;
-    uint32_t *own = direct ? pass_table(p) : table, *next = pass_table(p + 1);
-    if (p == 0 || !direct) {
-      uint32_t *clear = group_table(scratch, direct ? 4 : 1);
-      const int clear_words = p == 0 ? (int)((direct ? pass_table(0) : table) - clear) : 0;
-      launch_chained(p == 0 && visible ? k_radix_hist<true> : k_radix_hist<false>, blocks, kSortThreads, 0, st, src_k, n, count, 8 * p, 8, own,
-                     p == 0 ? (uint32_t *)nullptr : groups, group, clear, clear_words, ep[direct ? 3 : p], p == 0 ? report : CountReport{});
-      if (p == 0 && !direct) launch_chained(k_group_sums, (blocks + group - 1) / group, 256, 0, st, table, blocks, group, groups);
-    }
-#define GS_SCATTER(EP, DIRECT) launch_scatter<8, EP, DIRECT>(blocks, src_k, src_v, dst_k, dst_v, n, count, 8 * p, own, groups, ep[p], st, next)
-    if (direct) {
-      if (p == 0) GS_SCATTER(3, true); else if (p < 3) GS_SCATTER(0, true); else GS_SCATTER(1, true);
-    } else {
-      if (p == 0 && visible) GS_SCATTER(3, false); else if (p < 3) GS_SCATTER(0, false); else GS_SCATTER(1, false);
-    }
+    uint32_t *clear = group_table(scratch, 1);
+    const int clear_words = p == 0 ? (int)(table - clear) : 0;
+    launch_chained(p == 0 && visible ? k_radix_hist<true> : k_radix_hist<false>, blocks, kSortThreads, 0, st, src_k, n, count, 8 * p, 8, table,
+                   p == 0 ? (uint32_t *)nullptr : groups, group, clear, clear_words, ep[p], p == 0 ? report : CountReport{});
+    if (p == 0) launch_chained(k_group_sums, (blocks + group - 1) / group, 256, 0, st, table, blocks, group, groups);
+#define GS_SCATTER(EP) launch_scatter<8, EP>(blocks, src_k, src_v, dst_k, dst_v, n, count, 8 * p, table, groups, ep[p], st)
+    if (p == 0 && visible) GS_SCATTER(3); else if (p < 3) GS_SCATTER(0); else GS_SCATTER(1);
 #undef GS_SCATTER
   }
-  return direct ? 5 : 9;
+  return 9;
 }
 
 size_t scan_scratch_bytes(int64_t n) { return (size_t)((n + kScanBlock - 1) / kScanBlock + 1) * sizeof(uint32_t); }
