@@ -139,33 +139,41 @@ __device__ __forceinline__ void expand_rows(const uint32_t mask[8], const uint32
 #pragma unroll
   for (int t = 0; t < 16; ++t) cur[t] = __shfl_sync(kFull, mine, t);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const uint32_t m = mask[k];
-    if (__ballot_sync(kFull, m != 0u) == 0u) continue;
-    uint32_t incl[4], own[4], tot[4];
+  for (int half = 0; half < 2; ++half) {
+    // instances of the rows before, as bytes like the ranks (96 at most): the running positions move on once in four rows
+    uint32_t before[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      own[r] = spread_row(m, r);
-      incl[r] = own[r];
-    }
-#pragma unroll
-    for (int sft = 1; sft < 32; sft <<= 1) {
+    for (int k = 4 * half; k < 4 * half + 4; ++k) {
+      const uint32_t m = mask[k];
+      if (__ballot_sync(kFull, m != 0u) == 0u) continue;
+      uint32_t incl[4], at[4];
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        const uint32_t u = __shfl_up_sync(kFull, incl[r], sft);
-        if (lane >= sft) incl[r] += u;
+        incl[r] = spread_row(m, r);
+        at[r] = before[r] - incl[r];
+      }
+#pragma unroll
+      for (int sft = 1; sft < 32; sft <<= 1) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const uint32_t u = __shfl_up_sync(kFull, incl[r], sft);
+          if (lane >= sft) incl[r] += u;
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        at[r] += incl[r];
+        before[r] += __shfl_sync(kFull, incl[r], 31);
+      }
+#pragma unroll
+      for (int t = 0; t < 16; ++t) {
+        // one predicated store (no branch): the lane lists tile t and the slot lies inside the buffer
+        const uint32_t pos = cur[t] + __byte_perm(at[t >> 2], 0u, 0x4440 | (t & 3));
+        store_if(kInside || pos < capacity ? m & (1u << t) : 0u, out_vals + pos, gid[k]);
       }
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) tot[r] = __shfl_sync(kFull, incl[r], 31);
-#pragma unroll
-    for (int t = 0; t < 16; ++t) {
-      const int r = t >> 2, sh = 8 * (t & 3);
-      // one predicated store (no branch): the lane lists tile t and the slot lies inside the buffer
-      const uint32_t pos = cur[t] + (((incl[r] - own[r]) >> sh) & 0xffu);
-      store_if(kInside || pos < capacity ? m & (1u << t) : 0u, out_vals + pos, gid[k]);
-      cur[t] += (tot[r] >> sh) & 0xffu;
-    }
+    for (int t = 0; t < 16; ++t) cur[t] += __byte_perm(before[t >> 2], 0u, 0x4440 | (t & 3));
   }
 }
 // `count`: instances that the warp writes for tile `lane` (lanes below 16).
