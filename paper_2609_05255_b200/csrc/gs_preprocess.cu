@@ -436,7 +436,7 @@ __device__ __forceinline__ void load3(const float *p, int64_t i, float v[3]) {
 // wait until there are 32, or 32 where every lane goes on with its own.
 template <int kSlots>
 struct Projections {
-  float la[kSlots], lb[kSlots], lc[kSlots], tau[kSlots];   // la and tau become TileSpans' ila and taup
+  float4 form[kSlots];                     // la, lb, lc, tau; la and tau become TileSpans' ila and taup
   float2 centre[kSlots];
   ushort4 rect[kSlots];                    // (tx0, ty0, tx1, ty1)
   uint32_t id[kSlots];
@@ -444,16 +444,17 @@ struct Projections {
 // Per-warp shared memory of the second half's tile rows: what else TileSpans needs of the 32 owners, their
 // cell masks (sixteen bits per cell), and the owners of the rows in order, with the place of everyone's first.
 struct RowStage {
-  float dys[32], eyp[32];
+  float4 middle[32];                       // u, v, dys, eyp
   uint32_t mask[32][5];
-  unsigned short first[32];
+  short first[32];                         // the owner's first tile row, less the place of its first row in the list
   unsigned char list[32 * 12];
 };
 template <int kSlots>
 __device__ __forceinline__ TileSpans spans_of(const Projections<kSlots> &w, const RowStage &rs, int slot, int owner, const CamDev &cam) {
   TileSpans sp;
-  sp.u = w.centre[slot].x; sp.v = w.centre[slot].y; sp.dys = rs.dys[owner]; sp.eyp = rs.eyp[owner];
-  sp.ila = w.la[slot]; sp.lb = w.lb[slot]; sp.lc = w.lc[slot]; sp.taup = w.tau[slot];
+  const float4 f = w.form[slot], m = rs.middle[owner];
+  sp.u = m.x; sp.v = m.y; sp.dys = m.z; sp.eyp = m.w;
+  sp.ila = f.x; sp.lb = f.y; sp.lc = f.z; sp.taup = f.w;
   sp.W = cam.W; sp.H = cam.H;
   return sp;
 }
@@ -517,10 +518,11 @@ __global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_prepro
     const int total = __shfl_sync(kFull, incl, 31);
     if (in) {
       TileSpans sp;
-      sp.setup(wait.centre[mine].x, wait.centre[mine].y, wait.la[mine], wait.lb[mine], wait.lc[mine], wait.tau[mine], cam.W, cam.H);
-      wait.la[mine] = sp.ila; wait.tau[mine] = sp.taup;
-      rs.dys[lane] = sp.dys; rs.eyp[lane] = sp.eyp;
-      rs.first[lane] = (unsigned short)(incl - rows);
+      const float4 f = wait.form[mine];
+      sp.setup(wait.centre[mine].x, wait.centre[mine].y, f.x, f.y, f.z, f.w, cam.W, cam.H);
+      wait.form[mine] = make_float4(sp.ila, sp.lb, sp.lc, sp.taup);
+      rs.middle[lane] = make_float4(sp.u, sp.v, sp.dys, sp.eyp);
+      rs.first[lane] = (short)((int)rect.y - (incl - rows));
 #pragma unroll
       for (int j = 0; j < 5; ++j) rs.mask[lane][j] = 0u;
       for (int k = 0; k < rows; ++k) rs.list[incl - rows + k] = (unsigned char)lane;
@@ -529,7 +531,7 @@ __global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_prepro
     for (int at = lane; at < total; at += 32) {
       const int o = rs.list[at];
       const ushort4 r = wait.rect[head + o];
-      const int ty = r.y + at - rs.first[o];
+      const int ty = rs.first[o] + at;
       int xa, xb;
       if (spans_of(wait, rs, head + o, o, cam).row(ty, r.x, r.z, xa, xb)) {
         // the row's tiles as bits counted from the first column of the first cell (at most 12), a nibble per cell
@@ -565,10 +567,15 @@ __global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_prepro
     __syncwarp();
     if (stored) {
       uint32_t *slot = a.cell_records + (size_t)i * kCellSlots;
+      uint32_t w[5];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        w[j] = rs.mask[lane][j];
+        tiles += (unsigned)__popc(w[j]);
+      }
 #pragma unroll
       for (int j = 0; j < 9; ++j) {
-        const uint32_t m = (rs.mask[lane][j >> 1] >> (16 * (j & 1))) & 0xffffu;
-        tiles += (unsigned)__popc(m);
+        const uint32_t m = (w[j >> 1] >> (16 * (j & 1))) & 0xffffu;
         if (m) slot[nrec++] = ((uint32_t)((cy0 + j / 3) * cam.cgx + cx0 + j % 3) << 16) | m;
       }
     }
@@ -680,7 +687,7 @@ __global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_prepro
     const uint32_t found = __ballot_sync(kFull, vis);
     if (vis) {
       const int slot = kQueue ? (head + waiting + __popc(found & ((1u << lane) - 1u))) & 63 : lane;
-      wait.la[slot] = g.A; wait.lb[slot] = g.B; wait.lc[slot] = g.C; wait.tau[slot] = g.tau;
+      wait.form[slot] = make_float4(g.A, g.B, g.C, g.tau);
       wait.centre[slot] = make_float2(g.u, g.v); wait.rect[slot] = tiles4; wait.id[slot] = (uint32_t)i;
     }
     __syncwarp();
