@@ -114,3 +114,15 @@ def test_prepass_with_other_colour_activations(oracle, act):
     assert np.abs(want - np.maximum(sc.base_color + 0.5, 0)).max() > 1e-2
     texel = oracle.rgba8(want, 1 / (1 + np.exp(-sc.opacity_logits.astype(np.float64))))
     assert np.abs(rgba.astype(int) - texel.astype(int)).max() <= 1
+
+
+@pytest.mark.parametrize("n", [1, 5, 31, 32, 33, 132_608 + 19, 2 * 132_608 + 33])
+def test_prepass_ends_inside_a_trip(n):
+    """Rows come in pieces of 16 bytes, a trip of the warps ahead: the last ones must be those of the Gaussians' own."""
+    sc, cam = _scene(n, 41)
+    pre, rgba, color = _run(sc, cam, 3)
+    rows = ("means", "log_scales", "quats", "opacity_logits", "base_color", "features")
+    for first in sorted({0, (n - 1) // 32 * 32, max(n - 70, 0)}):
+        sub = scenes.Scene(**{k: (getattr(sc, k)[first:first + 64] if k in rows else getattr(sc, k)) for k in sc.__dataclass_fields__})
+        _, own_rgba, own_color = _run(sub, cam, 3)
+        assert np.array_equal(own_rgba, rgba[first:first + 64]) and np.array_equal(own_color, color[first:first + 64])
