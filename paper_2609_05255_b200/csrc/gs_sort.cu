@@ -179,14 +179,13 @@ __device__ __forceinline__ void block_exclusive_scan(const uint32_t v[DPT], uint
 }
 
 template <int BITS> constexpr size_t scatter_smem_bytes() {
-  return sizeof(uint32_t) * (2 * kSortTile + (size_t)(2 * kSortWarps + 2) * (BITS <= 8 ? 256 : (1 << BITS)) + kSortWarps + 1);
+  return sizeof(uint32_t) * (2 * kSortTile + (size_t)(kSortWarps + 2) * (BITS <= 8 ? 256 : (1 << BITS)) + kSortWarps + 1);
 }
 
 // One pass: stable scatter of this block's range by the BITS-wide digit at `shift` (BITS up to kMaxDigitBits; the
 // digit arrays hold max(256, 2^BITS) entries, thread t looking after digits t * DPT ..).  Slots past the
-// end of the input are not ranked.
-// Ranked by rank_row where finding a row's equal digits took a ballot per bit: eight bits 26.9 -> 22.8 us for 2.9M records, 8.6 -> 7.5 for
-// 0.6M, nine bits 22.0 -> 20.5 for 2.0M, five and six bits 2 to 8 % less.
+// end of the input carry the largest digit and sit at the end of the last tile, so they rank after
+// every real key and are never written.
 // EP selects the epilogue: 0 none, 1 the last pass of the depth sort: leaves the Gaussians' record counts in place of the
 // keys, and their sums per block of sorted positions, 2 ranges of
 // equal ids = key >> key_shift (last pass of the record sort: inside a block's run of one digit the keys are
@@ -205,9 +204,9 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
   extern __shared__ __align__(16) uint32_t s_dyn[];
   uint32_t *s_keys = s_dyn, *s_vals = s_keys + kSortTile;
   uint32_t *s_warp_cnt = s_vals + kSortTile;          // [kSortWarps][NB]
-  uint32_t *s_lanes = s_warp_cnt + kSortWarps * NB;   // [kSortWarps][NB], zero between rows
-  uint32_t *s_digit_start = s_lanes + kSortWarps * NB, *s_base = s_digit_start + NB, *s_warp_tot = s_base + NB;
+  uint32_t *s_digit_start = s_warp_cnt + kSortWarps * NB, *s_base = s_digit_start + NB, *s_warp_tot = s_base + NB;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t lt_mask = (1u << lane) - 1u;
   if (count_dev) count = min(count, (int64_t)__ldg(count_dev));
   constexpr uint32_t kDigitMask = (1u << BITS) - 1u;
 
@@ -265,7 +264,6 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
     }
   }
 
-  for (int k = tid; k < kSortWarps * NB / 4; k += kSortThreads) reinterpret_cast<uint4 *>(s_lanes)[k] = make_uint4(0u, 0u, 0u, 0u);
   const BlockRange r = block_range(count);
   const int span = r.tile_len / kSortWarps;           // consecutive elements of a tile that one warp ranks
   const int items = span / 32;                        // ... as this many rows of 32 (at most kItems)
@@ -273,7 +271,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
     const int64_t tile_begin = r.begin + (int64_t)t * r.tile_len;
     if (tile_begin >= r.end) break;
     const int valid_count = (int)min((int64_t)r.tile_len, r.end - tile_begin);
-    for (int k = tid; k < kSortWarps * NB / 4; k += kSortThreads) reinterpret_cast<uint4 *>(s_warp_cnt)[k] = make_uint4(0u, 0u, 0u, 0u);
+    for (int k = tid; k < kSortWarps * NB; k += kSortThreads) s_warp_cnt[k] = 0;
     __syncthreads();
     uint32_t key[kItems], val[kItems];
     unsigned short rank[kItems];
@@ -295,8 +293,24 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
       if (it >= items) break;                         // the same for every thread of the CTA
       const int local = warp * span + it * 32 + lane;
       const bool ok = local < valid_count;
-      const uint32_t d = (key[it] >> shift) & kDigitMask;
-      rank[it] = (unsigned short)rank_row(s_warp_cnt + warp * NB + d, s_lanes + warp * NB + d, ok, lane);
+      const uint32_t d = ok ? ((key[it] >> shift) & kDigitMask) : kDigitMask;
+      // lanes with the same digit form a group; its first lane bumps the warp's counter once and
+      // hands the old value to the group.  A warp's shared-memory atomics execute in program order,
+      // so the 16 items need no barrier between them and their latencies overlap.
+      // The group comes from one ballot per digit bit: a fixed cost, where the match instruction
+      // takes time in proportion to the number of different digits in the warp.
+      uint32_t peers = kFull;
+#pragma unroll
+      for (int b = 0; b < BITS; ++b) {
+        const bool bit = (d >> b) & 1u;
+        const uint32_t m = __ballot_sync(kFull, bit);
+        peers &= bit ? m : ~m;
+      }
+      const int leader = __ffs(peers) - 1;
+      uint32_t prior = 0;
+      if (lane == leader) prior = atomicAdd(&s_warp_cnt[warp * NB + d], (uint32_t)__popc(peers));
+      prior = __shfl_sync(kFull, prior, leader);
+      rank[it] = (unsigned short)(prior + __popc(peers & lt_mask));
     }
     __syncthreads();
     // per digit: exclusive scan over warps, then over digits
@@ -321,8 +335,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
     for (int it = 0; it < kItems; ++it) {
       if (it >= items) break;
       const int local = warp * span + it * 32 + lane;
-      if (local >= valid_count) continue;
-      const uint32_t d = (key[it] >> shift) & kDigitMask;
+      const uint32_t d = (local < valid_count) ? ((key[it] >> shift) & kDigitMask) : kDigitMask;
       const uint32_t pos = s_digit_start[d] + s_warp_cnt[warp * NB + d] + rank[it];
       s_keys[pos] = key[it];
       s_vals[pos] = val[it];
