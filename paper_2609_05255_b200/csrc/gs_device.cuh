@@ -469,7 +469,7 @@ __device__ __forceinline__ void copy_async4(void *dst, const void *src) {
 }
 __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Programmatic dependent launch.  A step is a chain of short, dependent launches (17 to 22 per view), a decode or a viewer frame one or
+// Programmatic dependent launch.  A step is a chain of short, dependent launches (8 to 18 per view), a decode or a viewer frame one or
 // two, repeated.
 // Launched with the attribute below, a kernel may be placed on the SMs as soon as the CTAs of its predecessor in the
 // stream have exited, without waiting for the predecessor's completion to be processed; dependency_wait() returns once

@@ -35,7 +35,7 @@ constexpr int kScanBlock = 256;   // Gaussians per block of the tiles-touched pr
 // tiles in a few blocks measured faster than two half tiles in every block (0.40 against 0.45 ms per 8 views on
 // 2 M records).  The grid is sized by the host's bound on the count; the ranges follow the count the kernels see
 // (which may live on the device), so the work stays balanced either way.
-constexpr int kMinPerBlock = 1024;   // (2048: the depth sort of 100 000 Gaussians 39 us instead of 37, of 300 000 50 instead of 47)
+constexpr int kMinPerBlock = 1024;
 int sort_blocks(int64_t count) {
   const int64_t b = (count + kMinPerBlock - 1) / kMinPerBlock;
   return (int)(b < 1 ? 1 : b < kMaxSortBlocks ? b : kMaxSortBlocks);
