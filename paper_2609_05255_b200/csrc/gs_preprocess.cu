@@ -446,7 +446,7 @@ struct Projections {
 struct RowStage {
   float4 middle[32];                       // u, v, dys, eyp
   uint32_t mask[32][5];
-  short first[32];                         // the owner's first tile row, less the place of its first row in the list
+  unsigned short first[32];                // the owner's first tile row, less the place of its first row in the list, modulo 2^16
   unsigned char list[32 * 12];
 };
 template <int kSlots>
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_prepro
       sp.setup(wait.centre[mine].x, wait.centre[mine].y, f.x, f.y, f.z, f.w, cam.W, cam.H);
       wait.form[mine] = make_float4(sp.ila, sp.lb, sp.lc, sp.taup);
       rs.middle[lane] = make_float4(sp.u, sp.v, sp.dys, sp.eyp);
-      rs.first[lane] = (short)((int)rect.y - (incl - rows));
+      rs.first[lane] = (unsigned short)((int)rect.y - (incl - rows));
 #pragma unroll
       for (int j = 0; j < 5; ++j) rs.mask[lane][j] = 0u;
       for (int k = 0; k < rows; ++k) rs.list[incl - rows + k] = (unsigned char)lane;
@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(kBlock, IsNeural<APP>::value ? 5 : 6) k_prepro
     for (int at = lane; at < total; at += 32) {
       const int o = rs.list[at];
       const ushort4 r = wait.rect[head + o];
-      const int ty = rs.first[o] + at;
+      const int ty = (rs.first[o] + at) & 0xffff;          // (there are 65535 tile rows at most)
       int xa, xb;
       if (spans_of(wait, rs, head + o, o, cam).row(ty, r.x, r.z, xa, xb)) {
         // the row's tiles as bits counted from the first column of the first cell (at most 12), a nibble per cell
