@@ -10,9 +10,16 @@
 //     20 011     25.8 -> 18.2     5.4   4.4   4.2   4.2        1M (878 000 visible)     76 -> 50     12.3   9.4  10.9  17.8
 //    100 000     31.5 -> 22.4     6.7   5.3   4.9   5.5        1.5M (1.26 visible)      93 -> 65     14.4  11.5  16.8  22.6
 //    300 007     48.5 -> 30.3     7.1   6.3   6.4  10.5        3M (1.1 visible)        114 -> 74     16.7  15.4  19.1  23.0
+// Where the keys do not spread, crowded bins cost a second split or a sort by digits, us in all (the radix sort; evenly spread;
+// 95 % in a tenth of a depth unit, the others from 0.3 to 300; 42 depths and a few far ones; 3, 1000, 20 000 planes):
+//    100 000     37   26   36   37   38   30   27                3M         160  119  155  158  128  161  161
+//    300 007     44   33   47   49   42   41   34                4.2M       201  159  219  214  168  210  211
+//         1M     72   55   76   76   70   72   79
+// and a bucket that the sample missed (its places depend on the indices alone, so an order in memory can hide from it) is shared
+// by all CTAs: of 65 000 elements 80, of 260 000 155 (the radix sort 51, 58), of 1M 700, of 4.2M, all there can be, 5400.
 // What bounds them: the sample one SM's shared memory, the passes the latency of their few loads per thread (two CTAs per SM, the
 // first loads sent ahead of the prologue) and the scattered stores of 8 bytes, the buckets the chain of load, bins, scan, place,
-// rank and write (two CTAs of 80 KB per SM, 1.7 waves at 1M).
+// rank and write (two CTAs of 81 KB per SM, 1.7 waves at 1M).
 #include <algorithm>
 #include "gs_bin.cuh"
 
@@ -22,7 +29,7 @@ namespace {
 using namespace bin;
 typedef unsigned long long u64;
 
-constexpr int kOversample = 8;                   // samples per bucket: four times the mean, what a CTA sorts, is exceeded once in 10^7 buckets
+constexpr int kOversample = 8;                   // samples per bucket: 3.75 times the mean, what a CTA sorts, is exceeded once in 2 10^6 buckets
 constexpr int kMeanLeast = 256, kMeanMost = 2048;
 constexpr int kSamplesMost = 16384;              // shared memory of k_splitters
 constexpr int kBucketsMost = kSamplesMost / kOversample + 1;
@@ -30,7 +37,8 @@ constexpr int kSampleThreads = 1024, kSampleBins = 8192;
 constexpr int kGuideBins = kSampleBins / 2;
 constexpr int kThreads = 512, kWarps = kThreads / 32;
 constexpr int kBlocksMost = 148 * 2;             // CTAs of the two passes over the keys
-constexpr int kPer = 16, kBucketMost = kPer * kThreads;    // elements that a CTA sorts in shared memory
+constexpr int kPer = 15, kBucketMost = kPer * kThreads;    // elements that a CTA sorts in shared memory, of which two CTAs leave 92 KB of L1
+constexpr int kLargeMost = (int)(kBucketSortMost / kBucketMost) + 1;
 constexpr int kBins = 4096;
 constexpr int kCrowded = 48;                     // elements of one bin
 constexpr uint32_t kCountUnknown = 15u;          // a large footprint: to be looked up
@@ -63,6 +71,7 @@ struct Scratch {
   uint32_t *totals, *starts;                     // [kBucketsMost + 1]: elements of a bucket, elements before it
   uint32_t *before;                              // [kBlocksMost, kBucketsMost]: elements of the bucket from blocks served earlier
   uint32_t *culled, *culled_before;              // [kBlocksMost]; [kBlocksMost, kWarps]: those of the block's warps before
+  uint32_t *large;                               // number of the buckets of more than kBucketMost elements, then which
   size_t bytes;
 };
 Scratch carve(void *base) {
@@ -78,37 +87,12 @@ Scratch carve(void *base) {
   s.before = reinterpret_cast<uint32_t *>(take(4 * (size_t)kBlocksMost * kBucketsMost));
   s.culled = reinterpret_cast<uint32_t *>(take(4 * kBlocksMost));
   s.culled_before = reinterpret_cast<uint32_t *>(take(4 * kBlocksMost * kWarps));
+  s.large = reinterpret_cast<uint32_t *>(take(4 * (1 + kLargeMost)));
   s.bytes = (size_t)(p - static_cast<char *>(base));
   return s;
 }
 
 __device__ __forceinline__ u64 element(uint32_t key, uint32_t id) { return (u64)key << 32 | (u64)(id << 4); }
-
-// Sorts a[0, m) by the threads of the CTA: comparators that all point the same way, so that what lies past the end need not
-// exist.  For the rare inputs that the bins below do not spread, and, in global memory, buckets beyond shared memory.
-__device__ void sort_by_comparators(u64 *a, uint32_t m, int tid, int threads) {
-  auto compare = [&](uint32_t i, uint32_t p) {
-    if (p < m) {
-      const u64 x = a[i], y = a[p];
-      if (x > y) { a[i] = y; a[p] = x; }
-    }
-  };
-  for (uint32_t k = 2; k < 2 * m; k *= 2) {
-    const uint32_t pairs = (m + k - 1) / k * (k / 2);
-    for (uint32_t t = tid; t < pairs; t += threads) {
-      const uint32_t i = t / (k / 2) * k + t % (k / 2);
-      compare(i, i ^ (k - 1));
-    }
-    __syncthreads();
-    for (uint32_t j = k / 4; j > 0; j /= 2) {
-      for (uint32_t t = tid; t < pairs; t += threads) {
-        const uint32_t i = t / j * (2 * j) + t % j;
-        compare(i, i + j);
-      }
-      __syncthreads();
-    }
-  }
-}
 
 // In place, exclusive: thread t holds values [t per, (t + 1) per).  Returns the total.
 template <int T, int PER>
@@ -135,6 +119,69 @@ __device__ __forceinline__ uint32_t scan_in_place(uint32_t *v, uint32_t *s_warp,
   return all;
 }
 
+// For what the bins below do not spread (planes of Gaussians at one depth, a narrow range of depths with a few far ones): m <= T PER
+// elements in shared memory by digits of seven bits, in stable passes whose time does not depend on the keys.  Key, less the
+// smallest, and index are one number without the bits between them (id_bits of index), of which the bits [from, to) count.
+// Not inlined: the kernels' own paths keep their registers.
+constexpr int kDigitBits = 7, kDigits = 1 << kDigitBits;
+struct DigitArea { uint32_t elements, tables, sums; };   // byte offsets; tables: [2, T / 32, kDigits] words; sums: kDigitSums words
+constexpr int kDigitSums = kDigits + 32;
+template <int T, int PER>
+__device__ __noinline__ void sort_by_digits(DigitArea area, uint32_t m, uint32_t least, int id_bits, int from, int to) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  constexpr int W = T / 32;
+  typedef uint32_t Table[kDigits];
+  u64 *a = reinterpret_cast<u64 *>(raw + area.elements);
+  Table *counts = reinterpret_cast<Table *>(raw + area.tables), *all_lanes = counts + W;
+  uint32_t *base = reinterpret_cast<uint32_t *>(raw + area.sums), *sums = base + kDigits;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rows = (int)((m + T - 1) / T);
+  uint32_t *count = counts[warp], *lanes = all_lanes[warp];       // see rank_row
+#pragma unroll 1
+  for (int shift = from; shift < to; shift += kDigitBits) {
+#pragma unroll
+    for (int d = 0; d < kDigits; d += 32) { count[d + lane] = 0u; lanes[d + lane] = 0u; }
+    u64 x[PER];
+    uint32_t at[PER];
+#pragma unroll
+    for (int h = 0; h < PER; ++h) {
+      if (h >= rows) break;
+      const uint32_t i = (warp * rows + h) * 32 + lane;
+      x[h] = i < m ? a[i] : 0ull;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < PER; ++h) {
+      if (h >= rows) break;
+      const u64 v = (u64)((uint32_t)(x[h] >> 32) - least) << id_bits | (uint32_t)x[h] >> 4;
+      const uint32_t d = (uint32_t)(v >> shift) & (kDigits - 1u);
+      at[h] = d << 16 | rank_row(count + d, lanes + d, (warp * rows + h) * 32 + lane < m, lane);
+    }
+    __syncthreads();
+    uint32_t total = 0;                          // of the digit tid; the warps' counts become what is in the warps before
+    if (tid < kDigits) {
+      uint32_t c[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w) c[w] = counts[w][tid];
+#pragma unroll
+      for (int w = 0; w < W; ++w) { counts[w][tid] = total; total += c[w]; }
+    }
+    const uint32_t inc = warp_inclusive(total, lane);
+    if (lane == 31) sums[warp] = inc;
+    __syncthreads();
+    const uint32_t before = __reduce_add_sync(kFull, lane < warp && lane < kDigits / 32 ? sums[lane] : 0u);
+    if (tid < kDigits) base[tid] = before + inc - total;
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < PER; ++h) {
+      if (h >= rows) break;
+      const uint32_t d = at[h] >> 16;
+      if ((warp * rows + h) * 32 + lane < m) a[base[d] + count[d] + (at[h] & 0xffffu)] = x[h];
+    }
+    __syncthreads();
+  }
+}
+__device__ __forceinline__ int bits_of(uint32_t v) { return 32 - __clz(v); }
+
 // Where sample j lies: one in every `stride` elements, at a place that varies.
 __device__ __forceinline__ uint32_t sample_place(uint32_t j, uint32_t stride) { return j * stride + __umulhi(j * 2654435761u, stride); }
 
@@ -154,7 +201,11 @@ struct SampleArea {
   uint32_t *bins, *key, *sorted_key;             // sorted: by bin
   uint16_t *sorted;                              // which sample
   uint8_t *slot;                                 // place in the bin
-  static constexpr size_t bytes(int samples) { return kSampleBins * 4 + (size_t)((samples + 15) & ~15) * 11; }
+  // (the digit passes have 64-bit elements over both arrays of keys, their tables in the bins and their sums past the elements)
+  static constexpr size_t bytes(int samples) {
+    const size_t padded = (samples + 15) & ~15;
+    return kSampleBins * 4 + std::max(padded * 11, padded * 8 + kDigitSums * 4);
+  }
   __device__ __forceinline__ SampleArea(unsigned char *raw, uint32_t samples) {
     samples = (samples + 15) & ~15u;
     bins = reinterpret_cast<uint32_t *>(raw);
@@ -165,7 +216,7 @@ struct SampleArea {
   }
 };
 __global__ void __launch_bounds__(kSampleThreads) k_splitters(const uint32_t *__restrict__ keys, uint32_t n, uint32_t stride, uint32_t samples,
-                                                              Scratch s, int fetched, CountReport report) {
+                                                              Scratch s, int fetched, int id_bits, CountReport report) {
   dependency_wait();
   extern __shared__ __align__(16) unsigned char raw[];
   __shared__ uint32_t s_least[kSampleThreads / 32], s_largest[kSampleThreads / 32], s_warp[kSampleThreads / 32];
@@ -206,13 +257,18 @@ __global__ void __launch_bounds__(kSampleThreads) k_splitters(const uint32_t *__
     uint32_t key[kSamplesMost / kSampleThreads];
 #pragma unroll
     for (int h = 0; h < kSamplesMost / kSampleThreads; ++h) key[h] = h * kSampleThreads + tid < (int)samples ? m.key[h * kSampleThreads + tid] : 0u;
-    u64 *a = reinterpret_cast<u64 *>(m.key);     // over both arrays of keys
+    u64 *a = reinterpret_cast<u64 *>(m.key);
     __syncthreads();
 #pragma unroll
-    for (int h = 0; h < kSamplesMost / kSampleThreads; ++h)
-      if (h * kSampleThreads + tid < (int)samples) a[h * kSampleThreads + tid] = element(key[h], place(h * kSampleThreads + tid));
+    for (int h = 0; h < kSamplesMost / kSampleThreads; ++h) {           // (culled ones last; the places rise as they stand)
+      const uint32_t j = h * kSampleThreads + tid;
+      if (j < samples) a[j] = element(min(key[h], largest + 1), place(j));
+    }
     __syncthreads();
-    sort_by_comparators(a, samples, tid, kSampleThreads);       // (culled ones last)
+    static_assert(kSampleBins >= 2 * kSampleThreads / 32 * kDigits, "the tables fit the bins");
+    const uint32_t elements = kSampleBins * 4;
+    sort_by_digits<kSampleThreads, kSamplesMost / kSampleThreads>({elements, 0u, elements + ((samples + 15) & ~15u) * 8}, samples, least, id_bits,
+                                                                  id_bits, id_bits + bits_of(largest + 1 - least));
     for (uint32_t j = tid; j < count / kOversample; j += kSampleThreads) s.splitters[j] = a[(j + 1) * kOversample - 1];
   } else {
 #pragma unroll 4
@@ -333,7 +389,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bucket_scatter(const uint32_t *
   dependency_wait();
   constexpr int kScan = (kBucketsMost + kThreads * 4 - 1) / (kThreads * 4) * 4;
   __shared__ __align__(16) uint32_t s_base[kScan * kThreads];
-  __shared__ uint32_t s_warp[kWarps], s_culled;
+  __shared__ uint32_t s_warp[kWarps], s_culled, s_large;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kRows = 4;
   const uint32_t span = (uint32_t)per / kWarps;
@@ -350,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bucket_scatter(const uint32_t *
   };
   load(begin);
   const int num = (int)__ldg(s.head);
-  if (tid == 0) s_culled = 0u;
+  if (tid == 0) s_culled = s_large = 0u;
   for (int i = tid; i < kScan * kThreads; i += kThreads) s_base[i] = i <= num ? __ldg(s.totals + i) : 0u;
   __syncthreads();
   uint32_t culled = 0;
@@ -359,9 +415,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_bucket_scatter(const uint32_t *
   if (lane == 0 && culled) atomicAdd(&s_culled, culled);
   const uint32_t all = scan_in_place<kThreads, kScan>(s_base, s_warp, tid);
   if (blockIdx.x == 0) {
-    for (int i = tid; i <= num + 1; i += kThreads) s.starts[i] = s_base[i];
-    if (tid == 0) *visible = all;
+    for (int i = tid; i <= num + 1; i += kThreads) {
+      s.starts[i] = s_base[i];
+      if (i <= num && s_base[i + 1] - s_base[i] > kBucketMost) s.large[1 + atomicAdd(&s_large, 1u)] = (uint32_t)i;
+    }
     __syncthreads();
+    if (tid == 0) { *visible = all; s.large[0] = s_large; }
   }
   const uint32_t *row = s.before + (size_t)blockIdx.x * kBucketsMost;
   for (int i = tid; i <= num; i += kThreads) s_base[i] += __ldg(row + i);     // (of a bucket without elements here: not read)
@@ -384,28 +443,202 @@ __global__ void __launch_bounds__(kThreads, 2) k_bucket_scatter(const uint32_t *
 // One CTA per bucket: its elements into bins by their keys (by their indices where the keys are all the same), two
 // bins or more per element, and each to its place among the few of its bin.  Leaves the Gaussians' ids and record counts in order, and
 // the counts' sums per 256 positions.
+constexpr int kSegmentsMost = kBucketMost / kCrowded + 1;
 struct __align__(16) BucketArea {
   u64 a[kBucketMost];
-  uint32_t bins[kBins], warp[kWarps], range[4];
+  uint32_t bins[kBins], sums[kDigitSums], warp[kWarps], range[4];
+  uint32_t segment[4][kSegmentsMost];            // complements of the smallest key and index, largest key and index
 };
-__global__ void __launch_bounds__(kThreads, 2) k_bucket_sort(u64 *__restrict__ in, Scratch s, const uint32_t *__restrict__ counts,
+static_assert(2 * (sizeof(BucketArea) + 1024) <= 164 * 1024, "two CTAs in the carve-out of 164 KB");
+static_assert(kBins >= 2 * kWarps * kDigits, "the tables fit the bins");
+constexpr DigitArea kBucketDigits = {0u, kBucketMost * 8, kBucketMost * 8 + kBins * 4};
+
+// Where bins hold many elements (few different depths, or a few far from the others): m.a[0, count) stands in the order of the
+// bins, which begin at m.bins.  A crowded bin is split once more between its own smallest and largest key, or index where the
+// keys are the same, two elements to a part; what is crowded even then goes by digits.
+// 1M Gaussians in 1000 planes, every bucket crowded: the kernel 35 us, by digits alone 62, evenly spread 22.
+__device__ __noinline__ void sort_crowded(uint32_t count, u64 first, u64 last, int id_bits) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  BucketArea &m = *reinterpret_cast<BucketArea *>(raw);
+  constexpr int T = kThreads;
+  const int tid = threadIdx.x, lane = tid & 31, shift = first >> 32 == last >> 32 ? 0 : 32;
+  const BinMap bin((uint32_t)(first >> shift), (uint32_t)(last >> shift), kBins);
+  for (int i = tid; i < 4 * kSegmentsMost; i += T) m.segment[0][i] = 0u;
+  __syncthreads();
+  u64 x[kPer];
+  uint32_t at[kPer];                             // begin of the bin, elements in it; then part, place in the part
+#pragma unroll
+  for (int h = 0; h < kPer; ++h) {
+    if (h * T >= (int)count) break;
+    const bool ok = h * T + tid < (int)count;
+    x[h] = ok ? m.a[h * T + tid] : 0ull;
+    at[h] = 0u;
+    if (ok) {
+      const uint32_t b = bin((uint32_t)(x[h] >> shift)), begin = m.bins[b], end = b + 1 < kBins ? m.bins[b + 1] : count;
+      at[h] = begin << 16 | (end - begin);
+    }
+    const bool split = (at[h] & 0xffffu) > (uint32_t)kCrowded;
+    const uint32_t key = (uint32_t)(x[h] >> 32), id = (uint32_t)x[h], slot = (at[h] >> 16) / kCrowded;
+    const uint32_t v[4] = {~key, ~id, key, id};
+    const uint32_t voters = __ballot_sync(kFull, split);
+    if (voters == 0u) continue;
+    const uint32_t one = __shfl_sync(kFull, slot, __ffs(voters) - 1);
+    if (__all_sync(kFull, !split || slot == one)) {               // (most warps lie inside one bin)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t most = __reduce_max_sync(kFull, split ? v[k] : 0u);
+        if (lane == 0) atomicMax(&m.segment[k][one], most);
+      }
+    } else if (split) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) atomicMax(&m.segment[k][slot], v[k]);
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < kBins / 4; i += T) reinterpret_cast<uint4 *>(m.bins)[i] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  uint32_t most = 0;
+#pragma unroll
+  for (int h = 0; h < kPer; ++h) {
+    if (h * T >= (int)count) break;
+    if (h * T + tid < (int)count) {
+      const uint32_t begin = at[h] >> 16, size = at[h] & 0xffffu;
+      uint32_t part = begin;
+      if (size > (uint32_t)kCrowded) {
+        const uint32_t seg = begin / kCrowded, k0 = ~m.segment[0][seg], k1 = m.segment[2][seg];
+        const bool same = k0 == k1;
+        const BinMap inner(same ? ~m.segment[1][seg] : k0, same ? m.segment[3][seg] : k1, (int)size);
+        part += inner(same ? (uint32_t)x[h] : (uint32_t)(x[h] >> 32));
+      }
+      part /= 2;
+      const uint32_t slot = atomicAdd(&m.bins[part], 1u);
+      most = max(most, slot);
+      at[h] = part << 16 | slot;
+    }
+  }
+  if (__syncthreads_or(most >= 2 * kCrowded)) {
+    const uint32_t least = (uint32_t)(first >> 32);
+    sort_by_digits<T, kPer>(kBucketDigits, count, least, id_bits, 0, bits_of((uint32_t)(last >> 32) - least) + id_bits);
+    return;
+  }
+  scan_in_place<T, kBins / T>(m.bins, m.warp, tid);
+#pragma unroll
+  for (int h = 0; h < kPer; ++h) {
+    if (h * T >= (int)count) break;
+    if (h * T + tid < (int)count) m.a[m.bins[at[h] >> 16] + (at[h] & 0xffffu)] = x[h];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < kPer; ++h) {
+    if (h * T >= (int)count) break;
+    if (h * T + tid < (int)count) {
+      const uint32_t part = at[h] >> 16, end = part + 1 < kBins ? m.bins[part + 1] : count;
+      uint32_t rank = m.bins[part];
+      for (uint32_t q = rank; q < end; ++q) rank += m.a[q] < x[h];
+      at[h] = rank;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < kPer; ++h) {
+    if (h * T >= (int)count) break;
+    if (h * T + tid < (int)count) m.a[at[h]] = x[h];
+  }
+  __syncthreads();
+}
+
+// Ids, record counts and the counts' sums of the elements m.a[0, count), which come at `start` in the order.
+__device__ __forceinline__ void leave(const BucketArea &m, uint32_t start, uint32_t count, const uint32_t *counts, uint32_t *counts_out,
+                                      uint32_t *order, uint32_t *block_sums, int tid) {
+  for (uint32_t j0 = 0; j0 < count; j0 += kThreads) {
+    const uint32_t j = j0 + tid, pos = start + j;
+    uint32_t c = 0;
+    if (j < count) {
+      const uint32_t v = (uint32_t)m.a[j], id = v >> 4;
+      c = v & 15u;
+      if (c == kCountUnknown) c = __ldg(counts + id);
+      counts_out[pos] = c;
+      order[pos] = id;
+      c &= ~kCellBig;
+    }
+    // a warp's 32 positions lie in two blocks of 256 at most
+    const uint32_t first = __shfl_sync(kFull, pos, 0) / 256u;
+    const uint32_t sum0 = __reduce_add_sync(kFull, pos / 256u == first ? c : 0u), sum1 = __reduce_add_sync(kFull, pos / 256u == first ? 0u : c);
+    if ((tid & 31) == 0 && sum0) atomicAdd(block_sums + first, sum0);
+    if ((tid & 31) == 0 && sum1) atomicAdd(block_sums + first + 1, sum1);
+  }
+}
+
+// Buckets beyond shared memory (the sample missed what the bucket holds): all CTAs take parts of them.  A part lies between two
+// samples of the bucket; a CTA reads the whole bucket, keeps what is in its part and counts what comes before.  What is more
+// than it can keep it takes in several turns, each up to the middle of those that it kept.
+constexpr uint32_t kPartMean = 2048, kPartsMost = 512, kPartOversample = kBucketMost / kPartsMost;
+__device__ __noinline__ void sort_large_buckets(const u64 *in, const Scratch &s, uint32_t large, const uint32_t *counts, uint32_t *counts_out,
+                                                uint32_t *order, uint32_t *block_sums, int id_bits) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  BucketArea &m = *reinterpret_cast<BucketArea *>(raw);
+  const int tid = threadIdx.x, lane = tid & 31;
+  uint32_t part = blockIdx.x;
+  for (uint32_t e = 0; e < large; ++e) {
+    const uint32_t bucket = s.large[1 + e], start = s.starts[bucket], total = s.starts[bucket + 1] - start;
+    const uint32_t parts = min((total + kPartMean - 1) / kPartMean, kPartsMost), samples = parts * kPartOversample;
+    for (; part < parts; part += gridDim.x) {
+      __syncthreads();
+      for (uint32_t j = tid; j < samples; j += kThreads) m.a[j] = in[start + (uint32_t)((u64)j * total / samples)];
+      __syncthreads();
+      sort_by_digits<kThreads, kPer>(kBucketDigits, samples, 0u, id_bits, 0, 32 + id_bits);
+      u64 lo = part == 0 ? 0ull : m.a[part * kPartOversample];
+      const u64 end = part + 1 == parts ? ~0ull : m.a[(part + 1) * kPartOversample];
+      u64 hi = end;
+      while (lo < end) {
+        __syncthreads();
+        if (tid < 2) m.range[tid] = 0u;
+        __syncthreads();
+        uint32_t before = 0;
+        constexpr int kLoads = 8;
+        for (uint32_t i0 = tid; i0 < total; i0 += kLoads * kThreads) {
+          u64 x[kLoads];
+#pragma unroll
+          for (int h = 0; h < kLoads; ++h) x[h] = i0 + h * kThreads < total ? in[start + i0 + h * kThreads] : ~0ull;
+#pragma unroll
+          for (int h = 0; h < kLoads; ++h) {
+            before += x[h] < lo;
+            if (x[h] >= lo && x[h] < hi) {
+              const uint32_t at = atomicAdd(&m.range[0], 1u);
+              if (at < (uint32_t)kBucketMost) m.a[at] = x[h];
+            }
+          }
+        }
+        before = __reduce_add_sync(kFull, before);
+        if (lane == 0) atomicAdd(&m.range[1], before);
+        __syncthreads();
+        const uint32_t found = m.range[0], have = min(found, (uint32_t)kBucketMost);
+        sort_by_digits<kThreads, kPer>(kBucketDigits, have, 0u, id_bits, 0, 32 + id_bits);
+        if (found > have) {
+          hi = m.a[kBucketMost / 2];
+        } else {
+          leave(m, start + m.range[1], have, counts, counts_out, order, block_sums, tid);
+          lo = hi;
+          hi = end;
+        }
+      }
+    }
+    part -= parts;
+  }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) k_bucket_sort(const u64 *__restrict__ in, Scratch s, const uint32_t *__restrict__ counts,
                                                              uint32_t *__restrict__ counts_out, uint32_t *__restrict__ order,
-                                                             uint32_t *__restrict__ block_sums) {
+                                                             uint32_t *__restrict__ block_sums, int id_bits) {
   dependency_wait();
   extern __shared__ __align__(16) unsigned char raw[];
   BucketArea &m = *reinterpret_cast<BucketArea *>(raw);
   constexpr int T = kThreads;
   const int tid = threadIdx.x, lane = tid & 31;
   const uint4 head = __ldg(reinterpret_cast<const uint4 *>(s.head));
-  const uint32_t start = __ldg(s.starts + blockIdx.x), count = __ldg(s.starts + blockIdx.x + 1) - start;
+  const uint32_t start = __ldg(s.starts + blockIdx.x), count = __ldg(s.starts + blockIdx.x + 1) - start, large = __ldg(s.large);
   u64 first = __ldg(s.splitters + max((int)blockIdx.x, 1) - 1), last = __ldg(s.splitters + blockIdx.x);
-  if (blockIdx.x > head.x) return;
-  if (count == 0) return;
-  u64 *sorted = m.a;
-  if (count > kBucketMost) {
-    sorted = in + start;
-    sort_by_comparators(sorted, count, tid, T);
-  } else {
+  if (blockIdx.x <= head.x && count - 1u < (uint32_t)kBucketMost) {
     u64 x[kPer];
     uint32_t at[kPer];
 #pragma unroll
@@ -452,22 +685,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_bucket_sort(u64 *__restrict__ i
         at[h] = b << 16 | slot;
       }
     }
-    if (__syncthreads_or(most >= kCrowded)) {
+    const bool crowded = __syncthreads_or(most >= kCrowded);
+    scan_in_place<T, kBins / T>(m.bins, m.warp, tid);
 #pragma unroll
-      for (int h = 0; h < kPer; ++h) {
-        if (h * T >= (int)count) break;
-        if (h * T + tid < (int)count) m.a[h * T + tid] = x[h];
-      }
-      __syncthreads();
-      sort_by_comparators(m.a, count, tid, T);
+    for (int h = 0; h < kPer; ++h) {
+      if (h * T >= (int)count) break;
+      if (h * T + tid < (int)count) m.a[m.bins[at[h] >> 16] + (at[h] & 0xffffu)] = x[h];
+    }
+    __syncthreads();
+    if (crowded) {
+      sort_crowded(count, first, last, id_bits);
     } else {
-      scan_in_place<T, kBins / T>(m.bins, m.warp, tid);
-#pragma unroll
-      for (int h = 0; h < kPer; ++h) {
-        if (h * T >= (int)count) break;
-        if (h * T + tid < (int)count) m.a[m.bins[at[h] >> 16] + (at[h] & 0xffffu)] = x[h];
-      }
-      __syncthreads();
 #pragma unroll
       for (int h = 0; h < kPer; ++h) {
         if (h * T >= (int)count) break;
@@ -488,25 +716,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_bucket_sort(u64 *__restrict__ i
       }
       __syncthreads();
     }
+    leave(m, start, count, counts, counts_out, order, block_sums, tid);
   }
-  for (uint32_t j0 = 0; j0 < count; j0 += T) {
-    const uint32_t j = j0 + tid, pos = start + j;
-    const bool ok = j < count;
-    uint32_t c = 0;
-    if (ok) {
-      const uint32_t v = (uint32_t)sorted[j], id = v >> 4;
-      c = v & 15u;
-      if (c == kCountUnknown) c = __ldg(counts + id);
-      counts_out[pos] = c;
-      order[pos] = id;
-      c &= ~kCellBig;
-    }
-    // a warp's 32 positions lie in two blocks of 256 at most
-    const uint32_t first = __shfl_sync(kFull, pos, 0) / 256u;
-    const uint32_t sum0 = __reduce_add_sync(kFull, pos / 256u == first ? c : 0u), sum1 = __reduce_add_sync(kFull, pos / 256u == first ? 0u : c);
-    if (lane == 0 && sum0) atomicAdd(block_sums + first, sum0);
-    if (lane == 0 && sum1) atomicAdd(block_sums + first + 1, sum1);
-  }
+  if (large > 0) sort_large_buckets(in, s, large, counts, counts_out, order, block_sums, id_bits);
 }
 
 template <auto Kernel>
@@ -533,16 +745,19 @@ int launch_bucket_sort(const uint32_t *depth_key, uint32_t *counts_out, uint32_t
   const Scratch s = carve(scratch);
   allow_smem<k_splitters>(SampleArea::bytes(kSamplesMost));
   const bool fetch = samples >= kFetchFrom;
+  int id_bits = 1;
+  while ((n - 1) >> id_bits) ++id_bits;
   if (fetch)
     launch_chained(k_fetch_samples, (samples + kFetchThreads - 1) / kFetchThreads, kFetchThreads, 0, st, depth_key, (uint32_t)n, (uint32_t)stride,
                    (uint32_t)samples, s.sampled);
   launch_chained(k_splitters, 1, kSampleThreads, SampleArea::bytes(samples), st, depth_key, (uint32_t)n, (uint32_t)stride, (uint32_t)samples, s,
-                 (int)fetch, report);
+                 (int)fetch, id_bits, report);
   launch_chained(k_bucket_count, blocks, kThreads, 0, st, depth_key, (uint32_t)n, per, s, counts_out, ep.block_sums, ep.num_block_sums, clear,
                  clear_words);
   launch_chained(k_bucket_scatter, blocks, kThreads, 0, st, depth_key, counts_out, ep.counts, (uint32_t)n, per, s, pairs, order, visible);
   allow_smem<k_bucket_sort>(sizeof(BucketArea));
-  launch_chained(k_bucket_sort, samples / kOversample + 1, kThreads, sizeof(BucketArea), st, pairs, s, ep.counts, counts_out, order, ep.block_sums);
+  launch_chained(k_bucket_sort, samples / kOversample + 1, kThreads, sizeof(BucketArea), st, pairs, s, ep.counts, counts_out, order, ep.block_sums,
+                 id_bits);
   return fetch ? 5 : 4;
 }
 
