@@ -38,7 +38,6 @@ constexpr int kGuideBins = kSampleBins / 2;
 constexpr int kThreads = 512, kWarps = kThreads / 32;
 constexpr int kBlocksMost = 148 * 2;             // CTAs of the two passes over the keys
 constexpr int kPer = 15, kBucketMost = kPer * kThreads;    // elements that a CTA sorts in shared memory, of which two CTAs leave 92 KB of L1
-constexpr int kLargeMost = (int)(kBucketSortMost / kBucketMost) + 1;
 constexpr int kBins = 4096;
 constexpr int kCrowded = 48;                     // elements of one bin
 constexpr uint32_t kCountUnknown = 15u;          // a large footprint: to be looked up
@@ -63,31 +62,40 @@ struct BinMap {
   __device__ __forceinline__ uint32_t operator()(uint32_t v) const { return (uint32_t)((float)(v - lo) * scale); }
 };
 
+// Sample and blocks of up to n Gaussians, at most: sizes that never fall as n grows, so that a workspace also serves smaller scenes.
+// (Between 39 072 and 303 104 the stride is n / 1184 rounded down, 33 and more: at most 1184 + 1184 / 33 samples.)
+int samples_most(int64_t n) { return (int)std::max<int64_t>(std::min<int64_t>((n + 31) / 32, 1232), (n + 255) / 256); }
+int blocks_most(int64_t n) { return (int)std::min<int64_t>(kBlocksMost, (n + kThreads - 1) / kThreads); }
+
 struct Scratch {
-  u64 *splitters;                                // [kBucketsMost]
+  u64 *splitters;                                // [buckets]
   uint32_t *head;                                // number of splitters; smallest and largest sampled key; are they the same?
-  uint32_t *sampled;                             // [kSamplesMost] keys
+  uint32_t *sampled;                             // keys of the sample
   uint16_t *guide;                               // [kGuideBins + 1]: splitters in the bins before
-  uint32_t *totals, *starts;                     // [kBucketsMost + 1]: elements of a bucket, elements before it
-  uint32_t *before;                              // [kBlocksMost, kBucketsMost]: elements of the bucket from blocks served earlier
-  uint32_t *culled, *culled_before;              // [kBlocksMost]; [kBlocksMost, kWarps]: those of the block's warps before
+  uint32_t *totals, *starts;                     // [buckets + 1]: elements of a bucket, elements before it
+  uint32_t *before;                              // [blocks, buckets]: elements of the bucket from blocks served earlier
+  uint32_t *culled, *culled_before;              // [blocks]; [blocks, kWarps]: those of the block's warps before
   uint32_t *large;                               // number of the buckets of more than kBucketMost elements, then which
+  uint32_t buckets;                              // at most
   size_t bytes;
 };
-Scratch carve(void *base) {
+Scratch carve(void *base, int64_t n) {
+  n = std::min<int64_t>(n, kBucketSortMost);
   Scratch s;
   char *p = static_cast<char *>(base);
   auto take = [&](size_t bytes) { char *q = p; p += (bytes + 255) & ~(size_t)255; return q; };
-  s.splitters = reinterpret_cast<u64 *>(take(sizeof(u64) * kBucketsMost));
+  const size_t samples = samples_most(n), buckets = samples / kOversample + 1, blocks = blocks_most(n);
+  s.buckets = (uint32_t)buckets;
+  s.splitters = reinterpret_cast<u64 *>(take(sizeof(u64) * buckets));
   s.head = reinterpret_cast<uint32_t *>(take(16));
-  s.sampled = reinterpret_cast<uint32_t *>(take(4 * kSamplesMost));
+  s.sampled = reinterpret_cast<uint32_t *>(take(4 * samples));
   s.guide = reinterpret_cast<uint16_t *>(take(2 * (kGuideBins + 8)));
-  s.totals = reinterpret_cast<uint32_t *>(take(4 * (kBucketsMost + 1)));
-  s.starts = reinterpret_cast<uint32_t *>(take(4 * (kBucketsMost + 1)));
-  s.before = reinterpret_cast<uint32_t *>(take(4 * (size_t)kBlocksMost * kBucketsMost));
-  s.culled = reinterpret_cast<uint32_t *>(take(4 * kBlocksMost));
-  s.culled_before = reinterpret_cast<uint32_t *>(take(4 * kBlocksMost * kWarps));
-  s.large = reinterpret_cast<uint32_t *>(take(4 * (1 + kLargeMost)));
+  s.totals = reinterpret_cast<uint32_t *>(take(4 * (buckets + 1)));
+  s.starts = reinterpret_cast<uint32_t *>(take(4 * (buckets + 1)));
+  s.before = reinterpret_cast<uint32_t *>(take(4 * blocks * buckets));
+  s.culled = reinterpret_cast<uint32_t *>(take(4 * blocks));
+  s.culled_before = reinterpret_cast<uint32_t *>(take(4 * blocks * kWarps));
+  s.large = reinterpret_cast<uint32_t *>(take(4 * (1 + (n / kBucketMost))));
   s.bytes = (size_t)(p - static_cast<char *>(base));
   return s;
 }
@@ -225,7 +233,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_splitters(const uint32_t *__
   auto place = [&](uint32_t j) { return sample_place(j, stride); };
   if (tid == 0) report.send();
   for (int i = tid; i < kSampleBins / 4; i += kSampleThreads) reinterpret_cast<uint4 *>(m.bins)[i] = make_uint4(0u, 0u, 0u, 0u);
-  for (int i = tid; i <= kBucketsMost; i += kSampleThreads) s.totals[i] = 0u;
+  for (uint32_t i = tid; i <= s.buckets; i += kSampleThreads) s.totals[i] = 0u;
   uint32_t least = 0xffffffffu, largest = 0u;
 #pragma unroll 4
   for (uint32_t j = tid; j < samples; j += kSampleThreads) {
@@ -375,7 +383,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bucket_count(const uint32_t *__
     if (lane < kWarps) s.culled_before[blockIdx.x * kWarps + lane] = inc - c;
     if (lane == 31) s.culled[blockIdx.x] = inc;
   }
-  uint32_t *row = s.before + (size_t)blockIdx.x * kBucketsMost;
+  uint32_t *row = s.before + (size_t)blockIdx.x * s.buckets;
   for (int i = tid; i <= num; i += kThreads) {
     const uint32_t c = s_hist[i];
     if (c) row[i] = atomicAdd(s.totals + i, c);
@@ -422,7 +430,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bucket_scatter(const uint32_t *
     __syncthreads();
     if (tid == 0) { *visible = all; s.large[0] = s_large; }
   }
-  const uint32_t *row = s.before + (size_t)blockIdx.x * kBucketsMost;
+  const uint32_t *row = s.before + (size_t)blockIdx.x * s.buckets;
   for (int i = tid; i <= num; i += kThreads) s_base[i] += __ldg(row + i);     // (of a bucket without elements here: not read)
   __syncthreads();
   uint32_t last = all + s_culled + __ldg(s.culled_before + blockIdx.x * kWarps + warp);
@@ -734,7 +742,7 @@ void allow_smem(size_t bytes) {
 
 bool bucket_sort_takes(int64_t n) { return n <= kBucketSortMost; }
 
-size_t bucket_scratch_bytes() { return carve(nullptr).bytes; }
+size_t bucket_scratch_bytes(int64_t n) { return carve(nullptr, n).bytes; }
 
 int launch_bucket_sort(const uint32_t *depth_key, uint32_t *counts_out, uint32_t *order, unsigned long long *pairs, int64_t n,
                        unsigned long long *visible, void *scratch, uint32_t *clear, int clear_words, const SortEpilogue &ep,
@@ -742,7 +750,7 @@ int launch_bucket_sort(const uint32_t *depth_key, uint32_t *counts_out, uint32_t
   static_assert((int64_t)kBucketSortMost * kOversample <= (int64_t)kSamplesMost * kMeanMost, "samples fit");
   const int per = block_elements(n), blocks = (int)((n + per - 1) / per), stride = sample_stride(n);
   const int samples = (int)((n + stride - 1) / stride);
-  const Scratch s = carve(scratch);
+  const Scratch s = carve(scratch, n);
   allow_smem<k_splitters>(SampleArea::bytes(kSamplesMost));
   const bool fetch = samples >= kFetchFrom;
   int id_bits = 1;

@@ -198,7 +198,7 @@ int launch_depth_sort(const uint32_t *depth_key, uint32_t *keys, uint32_t *order
 // cleared on the way.
 constexpr int64_t kBucketSortMost = 1 << 22;  // Gaussians
 bool bucket_sort_takes(int64_t n);
-size_t bucket_scratch_bytes();
+size_t bucket_scratch_bytes(int64_t n);
 int launch_bucket_sort(const uint32_t *depth_key, uint32_t *counts_out, uint32_t *order, unsigned long long *pairs, int64_t n,
                        unsigned long long *visible, void *scratch, uint32_t *clear, int clear_words, const SortEpilogue &ep,
                        const CountReport &report, cudaStream_t st);

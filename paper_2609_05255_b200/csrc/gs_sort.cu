@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(kExpandThreads, 4) k_expand(const uint32_t *__
 
 size_t sort_scratch_bytes(int64_t n, int64_t records) {
   constexpr size_t kTable = (1 << kMaxDigitBits) * sizeof(uint32_t);
-  return kGroupTables * kMaxGroups * kTable + std::max(2 * sort_blocks(std::max(n, records)) * kTable, bucket_scratch_bytes());
+  return kGroupTables * kMaxGroups * kTable + std::max(2 * sort_blocks(std::max(n, records)) * kTable, bucket_scratch_bytes(n));
 }
 
 namespace {

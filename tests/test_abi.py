@@ -46,6 +46,15 @@ def test_workspace_size_is_monotone_and_rejects_bad_arguments(lib_path):
     assert f(1_000_000, 1256, 828, 0) >= 48 * 1_000_000  # the backward's per-Gaussian 2D gradients
 
 
+@pytest.mark.parametrize("n,width,height,pairs,most", [(1, 16, 16, 1, 300e3), (1000, 64, 64, 5000, 400e3), (8192, 512, 512, 100_000, 2.5e6),
+                                                       (20_000, 333, 217, 200_000, 4.7e6)])
+def test_workspace_of_a_small_scene_is_small(lib_path, n, width, height, pairs, most):
+    """Tables of the depth order are as long as the scene needs, not as long as the largest one does."""
+    f = ctypes.CDLL(lib_path).gs_workspace_bytes
+    f.argtypes, f.restype = [ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_int64], ctypes.c_size_t
+    assert f(n, width, height, pairs) <= most
+
+
 def test_binding_struct_fields_follow_the_header():
     import importlib.util
     text = re.sub(r"/\*.*?\*/", "", open(HEADER).read(), flags=re.S)
