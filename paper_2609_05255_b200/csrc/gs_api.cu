@@ -253,8 +253,8 @@ BwdWorkspace carve_bwd(void *ws, int64_t n) {
   BwdWorkspace w;
   w.g2d = c.take<float>(nn * 12);
   w.flags.layout((int64_t)nn);
-  w.flags.words = c.take<uint32_t>((size_t)w.flags.stride * w.flags.copies);
-  w.cleared = c.used;
+  w.cleared = c.used + (size_t)w.flags.stride * w.flags.copies * sizeof(uint32_t);
+  w.flags.words = c.take<uint32_t>(GradFlags::room((int64_t)nn));
   w.dirs = c.take<float>(nn * 3);
   w.g_color = c.take<float>(nn * 3);
   w.g_dirs = c.take<float>(nn * 3);

@@ -75,6 +75,11 @@ struct GradFlags {
     copies = n < 16384 ? 16 : n < 65536 ? 4 : 1;
     stride = (uint32_t)((n + 31) / 32 + 31) & ~31u;      // whole lines of 128 bytes
   }
+  // Words for the copies of up to n Gaussians: never less than a smaller scene's.
+  static size_t room(int64_t n) {
+    const size_t stride = (size_t)((n + 31) / 32 + 31) & ~(size_t)31, copied = 16 * stride;
+    return copied < 8192 ? copied : stride < 8192 ? 8192 : stride;
+  }
 #ifdef __CUDACC__
   template <bool kCopies>
   __device__ __forceinline__ void set(uint32_t warp, uint32_t id) const {

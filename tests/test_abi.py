@@ -55,6 +55,15 @@ def test_workspace_of_a_small_scene_is_small(lib_path, n, width, height, pairs, 
     assert f(n, width, height, pairs) <= most
 
 
+@pytest.mark.parametrize("pairs", [1000, 1_000_000])
+def test_a_workspace_serves_every_smaller_scene(lib_path, pairs):
+    """Renderers keep the workspace of their largest scene while Gaussians are added and pruned."""
+    f = ctypes.CDLL(lib_path).gs_workspace_bytes
+    f.argtypes, f.restype = [ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_int64], ctypes.c_size_t
+    sizes = [f(n, 640, 480, pairs) for n in [*range(1, 70_000), *range(70_000, 4_400_000, 499)]]
+    assert all(a <= b for a, b in zip(sizes, sizes[1:]))
+
+
 def test_binding_struct_fields_follow_the_header():
     import importlib.util
     text = re.sub(r"/\*.*?\*/", "", open(HEADER).read(), flags=re.S)
