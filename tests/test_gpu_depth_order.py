@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("near", [0.2, 0.0, -2.5])
-@pytest.mark.parametrize("n,z_lo", [(32769, 2.0), (40001, -6.0), (33000, -300.0), (151552, -6.0), (151553, -6.0)])  # none, half, nearly all culled; block limit
+@pytest.mark.parametrize("n,z_lo", [(32769, 2.0), (40001, -6.0), (33000, -300.0), (151552, -6.0), (151553, -6.0)])  # none, half, nearly all culled; blocks of 512 and 1024
 def test_order_with_culled_gaussians(n, z_lo, near):
     sc = scenes.box_scene(n, 3.0, z_lo, 8.0, -3.5, 0.8, 1.0, scenes.APP_SH, seed=n)
     cam = dataclasses.replace(scenes.identity_camera(333, 217, 300.0), near_plane=near)
