@@ -72,8 +72,8 @@ typedef enum { GS_DECODER_SPLIT = 0, GS_DECODER_HALF = 1 } GsDecoderPrecision;
 
 /* Pinhole camera (host struct). */
 typedef struct {
-  int32_t width, height;        /* pixels; at most 65535 tiles of 16 pixels per axis and 2^24
-                                   tiles in all (GS_ERR_INVALID_ARG beyond)                    */
+  int32_t width, height;        /* pixels; at most 65535 tiles of 16 pixels per axis and 65536
+                                   cells of 4 x 4 tiles (GS_ERR_INVALID_ARG beyond)            */
   float fx, fy, cx, cy;         /* intrinsics in pixel units                                   */
   float w2c[12];                /* row-major [R|t]: x_cam = R x_world + t                      */
   float near_plane, far_plane;  /* depth cull, typically 0.2 and 1e10                          */
@@ -359,14 +359,14 @@ GsStatus gs_neural_prepass(GsContext *ctx, const GsScene *scene, const uint16_t 
  * At most 4096 stage records are kept between two collects; further ones are dropped. */
 typedef enum {
   GS_STAGE_PREPROCESS_FWD = 0, /* projection + fused colour decode                              */
-  GS_STAGE_DEPTH_SORT,         /* radix sort of the Gaussians by depth key (scenes of up to 8192 Gaussians: the
+  GS_STAGE_DEPTH_SORT,         /* the Gaussians ordered by depth key (scenes of up to 8192 Gaussians: the
                                   whole binning, which is one kernel and the expansion there)   */
   GS_STAGE_TILE_OFFSETS,       /* (the sums of tiles touched are taken by the depth sort's last pass: no time of its own) */
   GS_STAGE_KEYGEN,             /* instance emission                                             */
   GS_STAGE_TILE_SORT,          /* radix sort of the instances by tile id                        */
   GS_STAGE_TILE_RANGES,
   GS_STAGE_BLEND_FWD,
-  GS_STAGE_BLEND_BWD,
+  GS_STAGE_BLEND_BWD,          /* the 2D gradients cleared, and the blend's backward            */
   GS_STAGE_PREPROCESS_BWD,     /* projection backward + fused appearance backward               */
   GS_STAGE_APPEARANCE_FWD,     /* separate-pass decode                                          */
   GS_STAGE_APPEARANCE_BWD,

@@ -466,9 +466,11 @@ GsStatus gs_render_forward(GsContext *ctx, int64_t n, const GsProjected *proj, c
   }
   const int num_cells = cd.cgx * cd.cgy;
   const uint32_t cap32 = pair_capacity > 0xffffffffll ? 0xffffffffu : (uint32_t)pair_capacity;
-  // Up to 8192 Gaussians the whole binning is one cluster's work: 16 SMs, but two launches instead of 12.  Steps measured
-  // with the cluster and with the chain: 2100 Gaussians 115.0 and 118.5 us, 8000 in a small image 87.6 and 88.3, in one of
-  // 640 x 480 113.5 and 112.3, 12 000 143.7 and 142.8, 16 000 137.0 and 131.3, 32 000 138.5 and 132.0.
+  // Up to 8192 Gaussians the whole binning is one cluster's work: 16 SMs, but two launches instead of 11.  Views in flight want few
+  // launches: an iteration of four views on two streams takes 240 to 330 us with the cluster and 320 to 350 with the chain, eight on four
+  // 430 to 530 and 590 to 650, at 1000 to 8000 Gaussians in 64 x 64 to 640 x 480 pixels alike.  A view alone is faster with the
+  // cluster up to 2000 (1000: 72 and 97 us for the step, 2000: 104 and 108) and slower beyond, by 1 to 6 us (3000: 98.9 and
+  // 94.3, 8000: 104.3 and 99.0).  The line is drawn for the views in flight; above 8192 the chain was ahead even when it was longer.
   const int ctas = sorted ? cluster_ctas(n, num_cells, ctx->cluster_limit) : 0;
   bool binned = !sorted;
   if (ctas > 0) {

@@ -254,9 +254,9 @@ __global__ void __launch_bounds__(32, 32) k_blend_fwd(
             const uint32_t pos1 = __float_as_uint(st.rest[j + e].z);
 #pragma unroll
             for (int k = 0; k < kVecs; ++k) {
-              // transmittance behind the entry as T (1 - alpha), both roundings included: the backward recovers T by dividing
-              // (1 - alpha) out again and drifts if the forward rounds another expression (T - alpha T in one rounding: 2.4
-              // times as many gradients of a 1M scene miss 1e-3)
+              // transmittance behind the entry as T (1 - alpha), both roundings included: the backward takes T in front as T + w with
+              // w = T alpha / (1 - alpha), the same 1 - alpha, and drifts if the forward rounds another expression (T - alpha T in one
+              // rounding: 2.4 times as many gradients of a 1M scene missed 1e-3 when the backward divided by 1 - alpha)
               V t;
 #pragma unroll
               for (int i = 0; i < kLanes; ++i) put(t, i, T[kLanes * k + i]);
@@ -417,11 +417,11 @@ struct __align__(16) BwdArea {
 // because its Gaussian received nothing (in a scene with occlusion most of them: 94 % of the listed Gaussians of a view of
 // 1M).  All rows are zeroed here, each warp a slice on its way out (on its way in, the first wave writes them all at once
 // and the others' reads wait behind that: 23 us more at 1M); a bit per Gaussian says who received a gradient, and the
-// projection and appearance backward works on those alone.  1M Gaussians, 1256 x 828: 259 us without the zero rows -> 217
+// projection and appearance backward works on those alone.  1M Gaussians, 1256 x 828: 259 us without the zero rows -> 207
 // with those of the neural model, 62 % of the issue slots, FMA pipe 55 % busy.
 //
 // What does not depend on the carried state is worked out for four entries at a time, so that the reciprocals, exponentials and
-// products of one entry fill the waits of another: 217 -> 201 us at 1M (4108 tiles), 436 -> 381 in a view of 3M over depths of
+// products of one entry fill the waits of another: 209 -> 199 us at 1M (4108 tiles), 436 -> 381 in a view of 3M over depths of
 // 1 to 50 (8160), with 16 warps per SM.  More warps do not help: 24 of 80 registers take as long as 19 of 96, and so do 15
 // (padded shared memory); batches of four entries, which would make room for 28, cost 15 to 30 % for their longer sums.
 //

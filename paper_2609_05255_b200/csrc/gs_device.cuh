@@ -484,7 +484,7 @@ __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;
 // (griddepcontrol.launch_dependents at the top of every kernel) gained no more on one stream and cost 4 % with
 // several views in flight: the successor's CTAs then sit on the SMs for the whole run of the predecessor, in the
 // places of the other streams' kernels.
-// With the blend backward and the kernels outside the step launched like this too: the forward and backward decode of 1M
+// With the blend backward and the kernels outside the step launched like this too, between repeated calls: the forward and backward decode of 1M
 // Gaussians 108.5 -> 103.5 us, a viewer frame of 3M 55.4 -> 53.6, steps 71.1 -> 67.4 (1000 Gaussians) and 587.9 -> 581.9 (1M SH).
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... KArgs, class... Args>

@@ -113,8 +113,8 @@ static_assert(sizeof(PrepassRows) == 120 * 16, "pieces");
 // Bound by instruction issue (192 MB need 29 us): the warps are persistent, so that the weights are read once, the rectifiers
 // work on packed halves, degree 3 has an instance without the selects of the others, the rows come in asynchronous copies a
 // trip ahead and reach the fragments through ldmatrix, and the activation is chosen once.  3M Gaussians: 61.3 us at first,
-// 53.2 with loads at the start of every trip (62 % of the issue slots) and fragments word by word, 52.5 with the copies alone
-// (74 %, of more instructions), 50.7 with ldmatrix and vector stores, 48.1 with one branch for the activation.
+// 53.2 with loads at the start of every trip (62 % of the issue slots) and fragments word by word, 52.5 with the copies alone,
+// 50.7 with ldmatrix and vector stores, 48.1 with one branch for the activation (75 % of the slots).
 template <bool kFull3>   // degree 3: all direction inputs in use
 __global__ void __launch_bounds__(kPrepassThreads, kPrepassBlocks) k_neural_prepass(int64_t n, int deg, int act, const float *__restrict__ means,
                                                                     const float *__restrict__ logits,

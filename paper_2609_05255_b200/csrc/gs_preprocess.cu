@@ -1467,8 +1467,9 @@ int launch_appearance_fwd(int app, const AppearanceArgs &a, cudaStream_t st) {
   const int chunks = grid_for(a.n);
   // The tensor-memory path (tiles of 128 Gaussians = kBlock): on request, and by default from 2M Gaussians on.  The warp-level
   // kernel is the faster one at any size since it fetches a trip ahead (3M 71.5 against 80.2 us, with plain operands 50.5 and 70.0), but
-  // it multiplies the output layer in half-precision operands, too: its errors are 2 % larger (plain 26 %), and a caller
-  // with large scenes keeps what it had.
+  // it multiplies the output layer in half-precision operands, too: root mean square errors against 64 bits at 1M 8.9e-8 against 8.4e-8
+  // (plain 8.3e-5 against 6.6e-5), the largest 4.7e-7 both (5.1e-4, 4.1e-4).  The line is kept for that, not for speed: a caller with
+  // large scenes keeps the errors that it had, one with small scenes, which always ran on the warp-level kernel, too.
   if (a.deg > 0 && (a.engine == GS_ENGINE_TCGEN05 || (a.engine == GS_ENGINE_AUTO && a.n >= 2000000))) {
     constexpr size_t smem = sizeof(tc::Smem);
     if (app == kAppNeuralHalf) {
